@@ -34,7 +34,7 @@ BASE_CANDS = 16384          # generated on the host, tiled on the device
 # DRAM bytes (read + write) per candidate of each batched kernel, from one ncu
 # capture of 16384 candidates of this workload per kernel; a full launch moves
 # the same bytes per candidate (the traffic grows in proportion)
-TRAFFIC_PER_EVAL = {"eval_tiles_kernel": 8307, "eval_stream_kernel": 8308}
+TRAFFIC_PER_EVAL = {"eval_tiles_kernel": 8307}
 ALNS_OPS_PER_ENTRY = 8
 TRAFFIC_SOURCE = "ncu dram__bytes_read+write of a 16384-candidate launch, scaled by candidates per launch"
 TILE = 32                   # batch = BASE_CANDS * TILE = 524288 candidates
@@ -211,8 +211,8 @@ def run_profile(args):
     w, ops_h, off_h = make_inputs(seed=0)
     inst = vrp.Instance.from_workload(w)
     if args.profile_walk == "streamed":
-        # the shape the autotuner picks for the full batch: two-warp groups of the streamed walk
-        vrp.set_eval_config(inst, "coords", 24, walk="streamed", group_warps=2)
+        # two routes per lane, four warps per block: the shape picked for the full batch
+        vrp.set_eval_config(inst, "coords", 4, walk="streamed", group_warps=2)
     ops = torch.from_numpy(ops_h).cuda()
     off = torch.from_numpy(off_h).cuda()
     for _ in range(args.warmup):
@@ -600,7 +600,7 @@ def main():
     ap.add_argument("--profile", action="store_true",
                     help="small case for ncu: 16384 candidates (132 MB), no tuning")
     ap.add_argument("--profile-walk", default="staged", choices=["staged", "streamed"],
-                    help="--profile: the default staged shape, or the streamed two-warp-group shape")
+                    help="--profile: the default shape, or two routes per lane")
     args = ap.parse_args()
     if args.warmup < 3:
         args.warmup = 3
@@ -784,7 +784,7 @@ def main():
     bytes_per_eval = 4 * (2 * N_CUST + M_VEH + 1) + 8
     achieved = B * bytes_per_eval / (kernel_ms / 1000.0) / 1e9
     peak = pk["hbm_gbs"] if pk else 6800.0
-    kernel = "eval_stream_kernel" if tuned.get("walk") == "streamed" else "eval_tiles_kernel"
+    kernel = "eval_tiles_kernel"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": "measured" if pk else "fallback",
                 "bytes_per_unit": bytes_per_eval, "units_per_launch": B,

@@ -108,8 +108,7 @@ int vrprpd_evaluate(const vrprpd_instance* inst, const vrprpd_batch* batch, int3
 
 /* Same result as vrprpd_evaluate from HOST buffers (ops/off/makespan/status
  * all host pointers), returning when done.  Pinned (page-locked) ops and off
- * are read by the kernel in place over the host link, always by the staged
- * walk (its coalesced reads; the best staged shape vrprpd_autotune saw);
+ * are read by the kernel in place over the host link (coalesced, once);
  * pageable ones are copied to the device first.  Results are copied back. */
 int vrprpd_evaluate_host(const vrprpd_instance* inst, const vrprpd_batch* host_batch,
                          int32_t* makespan_host, uint32_t* status_host, void* stream);
@@ -211,18 +210,13 @@ int vrprpd_sync(const vrprpd_instance* inst, void* stream);
 #define VRPRPD_DIST_GLOBAL16 3 /* uint16 matrix gathered from L2 */
 #define VRPRPD_DIST_GLOBAL32 4 /* int32 matrix gathered from L2 */
 #define VRPRPD_DIST_COORDS 5   /* recomputed exactly from coordinates in shared memory */
-/* How a warp walks its candidates:
- *   VRPRPD_WALK_STAGED    each warp reads a tile of floor(32/m) candidates
- *                         with coalesced loads, checks every code (range,
- *                         duplicates) and keeps them as 16-bit codes in shared
- *                         memory, then walks them there;
- *   VRPRPD_WALK_STREAMED  each route's lane reads its own codes from global
- *                         memory through a register queue while it walks and
- *                         checks them on the way (a blocked walk gets the full
- *                         check afterwards); a group of group_warps warps (1
- *                         or 2) walks floor(32 group_warps / m) candidates, so
- *                         for m = 20 two warps walk three candidates.  Shared
- *                         memory holds only the ready times and offsets. */
+/* How many routes a lane walks at once:
+ *   VRPRPD_WALK_STAGED    one: a warp's tile is floor(32/m) candidates;
+ *   VRPRPD_WALK_STREAMED  group_warps (1 or 2) in turn: a warp's tile is
+ *                         floor(32 group_warps / m) candidates, so for m = 20
+ *                         three candidates use 60 of 64 lane slots.
+ * A block gets at most the warps asked for: fewer when the two-route kernel's
+ * registers (16 warps) or the shared memory do not allow them. */
 #define VRPRPD_WALK_STAGED 0
 #define VRPRPD_WALK_STREAMED 1
 typedef struct {
@@ -230,7 +224,7 @@ typedef struct {
     int32_t warps_per_block;
     int32_t blocks_per_sm;     /* 0 = as many as fit */
     int32_t walk;              /* VRPRPD_WALK_STAGED or VRPRPD_WALK_STREAMED */
-    int32_t group_warps;       /* streamed walk: warps per candidate group (1 or 2) */
+    int32_t group_warps;       /* streamed walk: routes per lane (1 or 2) */
 } vrprpd_eval_config;
 
 int vrprpd_eval_set_config(vrprpd_instance* inst, const vrprpd_eval_config* cfg);
@@ -260,9 +254,9 @@ int vrprpd_multi_create(const vrprpd_instance* const* insts, const vrprpd_batch*
  * CUDA graph and later calls replay it; inside a caller's capture (or on the
  * NULL stream) it launches directly.  Results as vrprpd_evaluate. */
 int vrprpd_multi_evaluate(vrprpd_multi* plan, void* stream);
-/* Time the walk (staged, or streamed with one-warp groups), warps per block
- * and distance mode (GLOBAL16/GLOBAL32) on the plan's own batches; keep the
- * fastest. */
+/* Time the routes per lane, warps per block and distance mode (points when
+ * every instance has them close enough together, GLOBAL16, GLOBAL32) on the
+ * plan's own batches; keep the fastest. */
 int vrprpd_multi_autotune(vrprpd_multi* plan, void* stream, vrprpd_eval_config* chosen);
 /* Set the plan's shape by hand: dist_mode GLOBAL16 (every instance with a
  * 16-bit matrix) or GLOBAL32, warps_per_block 1..32, walk staged or streamed

@@ -3,25 +3,9 @@
 // on the semantics of Section 3.1, Eqs. 7-23).
 //
 // Batched form: a persistent launch; the block stages the instance (distances
-// or coordinates, and p) in shared memory with TMA bulk copies, and every warp
-// owns a tile of k = 32/m candidates (one lane per route).  Per tile:
-//   1. offsets are checked and every customer's ready slot is set to
-//      -(p_c + 1): negative means "not dropped yet", and the drop recovers p_c
-//      from the value it reads anyway;
-//   2. the ops are read with coalesced loads, four per lane in flight (int32
-//      codes, or pairs of 16-bit codes in the 16-bit form), checked (code
-//      range, duplicates by a shared bitmap) and kept as 16-bit codes:
-//      half the footprint of the 32-bit stream, so 24 warps fit per SM where
-//      a staged 32-bit copy left room for 16;
-//   3. the route walk: each lane advances its route up to two ops per step,
-//      computing each travel time from the previous stop -- a drop publishes
-//      its pickup-ready time T_drop + p_c to shared memory, a pickup waits
-//      until that time is published (cross-vehicle precedence, Eq. 9) and then
-//      leaves at max(arrival, ready) (Eqs. 8, 10).  A group that makes no
-//      progress in a step while unfinished is a precedence cycle.  Each lane
-//      also tracks its route's stock prefix (Eqs. 13-18);
-//   4. per-candidate reductions: makespan = max return time (Eqs. 21-22),
-//      vehicle capacity, depot pool.
+// or points, and the ready-row template) in shared memory with TMA bulk
+// copies, and every warp owns a tile of candidates, one or two routes per lane
+// (eval_tile below).
 // Plain form: one thread per candidate, Kahn order over routes, scratch in
 // global memory, distances from global memory.
 #include <algorithm>
@@ -31,6 +15,13 @@
 #include "internal.h"
 
 namespace vrp {
+
+// Internal distance mode of VRPRPD_DIST_COORDS when every squared leg is below
+// EUC2D_HALF2_LIMIT: points as pairs of fp16 integers.
+constexpr int DIST_HALF2 = 6;
+
+// Warps per block at most, by routes per lane (register budget 64 and 128).
+__host__ __device__ constexpr int max_warps(int V) { return V == 1 ? 32 : 16; }
 
 struct EvalArgs {
     const int32_t* ops;
@@ -42,294 +33,447 @@ struct EvalArgs {
     const int32_t* d32;
     const uint16_t* d16;
     const int32_t* coords;
-    const int32_t* p;
+    const uint32_t* xy;      // points as fp16 pairs (row_words of them), or null
+    const int32_t* rowt;     // ready-row template, row_words words
     int* err;
     long long num;
     int n, m, R, Q;
     int load_full;
-    int k;            // candidates per warp tile
+    int pool_full;    // load_full: the m full loads exceed R
+    int prefetch;     // candidates in device memory: fetch the next tile's codes into L2
     int N;            // n + 1
+    int K;            // candidates per tile
+    int row_words;    // words of one ready row: n + 2 rounded up to 4
     // shared-memory layout, in 32-bit words
-    int shared_words; // per-block instance data (distances/coords + p)
+    int shared_words; // per-block instance data (distances or points, ready-row template)
     int dist_words;
-    int a_words, ready_words, seen_words, start_words, off_words, valid_words, warp_words;
-    int sw;           // seen words per candidate
-    // streamed form: G warps per group, K candidates per group tile, and the
-    // group region's layout in 32-bit words
-    int G, K;
-    int g_ready, g_off, g_flag, g_prog, g_red, group_words;
+    int a_words, ready_words, off_words, warp_words;
+    int pts;          // many-instance launches: where the warp's region keeps the tile's points
 };
 
-template <int DM>
-__device__ __forceinline__ int dist(const EvalArgs& a, const int32_t* sh, int i, int j) {
-    if constexpr (DM == VRPRPD_DIST_SMEM32) {
-        return sh[i * a.N + j];
-    } else if constexpr (DM == VRPRPD_DIST_SMEM16) {
-        return reinterpret_cast<const uint16_t*>(sh)[i * a.N + j];
-    } else if constexpr (DM == VRPRPD_DIST_GLOBAL16) {
-        return __ldg(a.d16 + i * a.N + j);
-    } else if constexpr (DM == VRPRPD_DIST_GLOBAL32) {
-        return __ldg(a.d32 + i * a.N + j);
-    } else {
-        const int2 pi = reinterpret_cast<const int2*>(sh)[i];
-        const int2 pj = reinterpret_cast<const int2*>(sh)[j];
-        return euc2d_small(pi.x, pi.y, pj.x, pj.y);
-    }
+// ---------------------------------------------------------------------------
+// The walk.  A warp owns a tile of K candidates and walks all their routes in
+// lock step, V routes per lane (32 V >= K m).  Shared memory per warp: the
+// tile's op codes as 16 bits, one row of ready slots per candidate, the route
+// offsets and four words of results per candidate.
+//
+//   stage   codes by 16-byte loads whatever the alignment (four in flight per
+//           lane), saturated to [0, 2n+2] and packed to 16 bits; ready rows
+//           copied from the block's template;
+//   walk    one op per route and round; see below;
+//   check   every customer's slot must have ended PICKED;
+//   reduce  makespan, start loads and flags per candidate by shared atomics.
+//
+// What bounds it.  At n=1000 m=20 a candidate takes 1475 wavefronts of shared
+// memory with one route per lane (1206 with two) and 6.0 k warp instructions
+// (3.9 k), where the earlier kernels issued 9.9 k and 8.4 k: one route per lane
+// runs at 81% of the issue slots and 72% of the shared-memory pipe, two routes
+// at 53% and 60%, short of warps.  262144 candidates: 2861 us before (its best
+// walk and shape), 1411 us now; n=100 m=4, 65536: 89 to 43 us; n=499 m=19,
+// 65536, a quarter of them blocked: 348 to 181 us; 32 instances of 17 to 500
+// customers, 4096 each: 298 to 135 us.
+// Tried at n=1000: the round's loads a round earlier, between the two routes'
+// steps (21% more instructions, 446 us against 365 us for 65536 candidates);
+// legs computed after the round's loads (385); groups of two warps with a
+// shared progress count in place of two routes per lane (365, and 187 against
+// 172 us at n=499); eight code chunks in flight at 64 registers (spills, 486).
+//
+// Ready slots.  Slot c holds -(p_c + 1) until c's drop, the pickup-ready time
+// T_drop + p_c until its pickup, then PICKED.  The slots of the depot (c = 0)
+// and of code 2n+2 (c = n+1, where every code out of range ends up) start as
+// PICKED, so nothing on them is ever ready.  A lane past its route's end holds
+// code 1, "pick up at the depot": it never goes, its point is the depot, so
+// the leg it computes is the way home, and no lane state says whether the
+// route is still going on.
+//
+// A round with no progress in the whole warp ends the walk: every write of
+// earlier rounds was visible to this one, so nothing can go later either.
+// Routes that have not ended then are blocked.
+//
+// Validation without bookkeeping in the walk.  Let a candidate's offsets be in
+// order (checked first).  If no route of it is blocked, 2n ops were walked.  A
+// slot becomes PICKED only by a pickup of its customer, and a pickup goes only
+// after a drop of the same customer.  So if every customer's slot ends PICKED,
+// the 2n ops hold a drop and a pickup of each of the n customers and nothing
+// else: a permutation.  If some slot does not, an op is repeated or out of
+// range.  A candidate with a blocked route gets the full check (range and a
+// duplicate bitmap), which tells MALFORMED from CYCLE.  Whatever a repeated or
+// foreign code does to the slots on the way stays inside its own candidate,
+// and every route still ends: each round that goes on takes at least one op.
+//
+// Stock.  One word holds 2^14 - s above 2^14 + s (s the stock relative to the
+// start, |s| <= 2n < 2^13), so one add moves both and one packed maximum keeps
+// max(-s) and max(s).
+// ---------------------------------------------------------------------------
+constexpr int PICKED = static_cast<int>(0x80000000u);   // ready slot of a customer already picked up
+
+constexpr unsigned STOCK0 = 0x40004000u;
+
+__device__ __forceinline__ int lds_s32(unsigned addr) {
+    int v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts_s32_if(bool on, unsigned addr, int v) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %0, 0;\n\t"
+        "@p st.shared.b32 [%1], %2;\n\t}" ::"r"(static_cast<unsigned>(on)),
+        "r"(addr), "r"(v)
+        : "memory");
+}
+// the 16-bit code at addr, or past the end code 1, a pickup at the depot
+__device__ __forceinline__ int code_or_idle(unsigned addr, unsigned end) {
+    int v;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.lt.u32 p, %1, %2;\n\t"
+        "mov.u32 %0, 1;\n\t"
+        "@p ld.shared.u16 %0, [%1];\n\t}"
+        : "=&r"(v)
+        : "r"(addr), "r"(end)
+        : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned pack_sat_u16(int lo, int hi) {
+    unsigned r;
+    asm("cvt.pack.sat.u16.s32 %0, %1, %2;" : "=r"(r) : "r"(hi), "r"(lo));
+    return r;
+}
+__device__ __forceinline__ unsigned min_u16x2(unsigned a, unsigned b) {
+    unsigned r;
+    asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned max_u16x2(unsigned a, unsigned b) {
+    unsigned r;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
 }
 
-// One tile of k candidates of one instance, processed by one warp.
-// W is the warp's shared-memory region (layout from a), sh/sp the block's
-// staged distances or coordinates and p.
-template <int DM, bool W16>
-__device__ __forceinline__ bool eval_tile(const EvalArgs& a, const int32_t* sh, const int32_t* sp, int32_t* W,
-                                          uint64_t* bar, unsigned& phase, long long t) {
-    (void)bar;
-    (void)phase;
-    const int lane = threadIdx.x & 31;
-    const int n = a.n, m = a.m, two_n = 2 * n, k = a.k;
-    uint16_t* A = reinterpret_cast<uint16_t*>(W);            // op codes, 16 bits each
-    int32_t* ready = W + a.a_words;
-    uint32_t* seen = reinterpret_cast<uint32_t*>(ready + a.ready_words);
-    int32_t* soff = reinterpret_cast<int32_t*>(seen + a.seen_words + a.start_words);
-    int32_t* valid = soff + a.off_words;
-    int32_t* red = valid + a.valid_words;      // 96 words
-    const int grp = lane / m, v = lane - grp * m;
-    const unsigned gmask = (grp < k) ? (m == 32 ? FULL_MASK : (((1u << m) - 1u) << (grp * m))) : 0u;
-    const long long first = t * k;
-    const int kt = static_cast<int>(min(static_cast<long long>(k), a.num - first));
-    const int elems = kt * two_n;
+// Where a route stands, and the leg to the next stop.  leg() returns the
+// travel time plus BIAS (the fp32 form's rounding constant, folded into the
+// departure time instead of subtracted per leg).
+template <int DM>
+struct Place {
+    static constexpr int BIAS = 0;
+    int row;                                   // c (n+1)
+    static __device__ __forceinline__ Place of(const EvalArgs& a, const int32_t*, int c) {
+        // code 2n+2 stands one past the matrix: any row will do, its candidate is malformed
+        if constexpr (DM == VRPRPD_DIST_GLOBAL16 || DM == VRPRPD_DIST_GLOBAL32) return {min(c, a.n) * a.N};
+        else return {c * a.N};
+    }
+    static __device__ __forceinline__ int leg(const EvalArgs& a, const int32_t* sh, const Place& x, const Place&,
+                                              int c) {
+        // shared matrices: row and column n+1 fall into the block's other data, never outside it
+        if constexpr (DM == VRPRPD_DIST_SMEM32) return sh[x.row + c];
+        else if constexpr (DM == VRPRPD_DIST_SMEM16) return reinterpret_cast<const uint16_t*>(sh)[x.row + c];
+        else if constexpr (DM == VRPRPD_DIST_GLOBAL16) return __ldg(a.d16 + x.row + min(c, a.n));
+        else return __ldg(a.d32 + x.row + min(c, a.n));
+    }
+};
+template <>
+struct Place<VRPRPD_DIST_COORDS> {             // any coordinates with squared legs below 2^24
+    static constexpr int BIAS = 0;
+    int2 p;
+    static __device__ __forceinline__ Place of(const EvalArgs&, const int32_t* sh, int c) {
+        return {reinterpret_cast<const int2*>(sh)[c]};
+    }
+    static __device__ __forceinline__ int leg(const EvalArgs&, const int32_t*, const Place& x, const Place& y, int) {
+        return euc2d_small(x.p.x, x.p.y, y.p.x, y.p.y);
+    }
+};
+template <>
+struct Place<DIST_HALF2> {                     // squared legs below 2^21: see euc2d_half2
+    static constexpr int BIAS = EUC2D_BIAS;
+    unsigned p;                                // x, y as two fp16 integers
+    static __device__ __forceinline__ Place of(const EvalArgs&, const int32_t* sh, int c) {
+        return {reinterpret_cast<const unsigned*>(sh)[c]};
+    }
+    static __device__ __forceinline__ int leg(const EvalArgs&, const int32_t*, const Place& x, const Place& y, int) {
+        return euc2d_half2(x.p, y.p);
+    }
+};
 
-    // ---- 1. offsets, flags, duplicate bitmap, unresolved ready times ----
+// A tile's codes on their way from global to shared memory: `total` of them
+// (the first `head`, fewer than a 16-byte chunk holds, belong to what lies
+// before the tile) from the 16-byte boundary `base`, as 16-byte loads; the
+// first and last chunk code by code.  Shared memory gets them saturated to
+// [0, 2n+2] and packed to 16 bits, head included.  A batch is SB chunks per
+// lane, all in flight together.
+template <bool W16, int SB>
+struct CodeBatch {
+    static constexpr int CPC = W16 ? 8 : 4;    // codes per chunk
+    int4 raw[SB] = {};
+    __device__ __forceinline__ void load(const char* base, int head, int total, int first) {
+        const int lane = threadIdx.x & 31, chunks = (total + CPC - 1) / CPC;
+#pragma unroll
+        for (int u = 0; u < SB; ++u) {
+            const int ck = first + 32 * u + lane;
+            if (ck >= chunks) continue;
+            if ((ck > 0 || head == 0) && (ck + 1) * CPC <= total) {
+                raw[u] = __ldg(reinterpret_cast<const int4*>(base) + ck);
+            } else {
+                unsigned w[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int e = 0; e < CPC; ++e) {
+                    const int i = ck * CPC + e;
+                    if (i < head || i >= total) continue;
+                    if constexpr (W16) w[e >> 1] |= static_cast<unsigned>(__ldg(reinterpret_cast<const uint16_t*>(base) + i)) << (16 * (e & 1));
+                    else w[e] = __ldg(reinterpret_cast<const int32_t*>(base) + i);
+                }
+                raw[u] = make_int4(w[0], w[1], w[2], w[3]);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(unsigned A, unsigned lim2, int total, int first) {
+        const int lane = threadIdx.x & 31, chunks = (total + CPC - 1) / CPC;
+#pragma unroll
+        for (int u = 0; u < SB; ++u) {
+            const int ck = first + 32 * u + lane;
+            if (ck >= chunks) continue;
+            if constexpr (W16) {
+                const unsigned x = min_u16x2(raw[u].x, lim2), y = min_u16x2(raw[u].y, lim2);
+                const unsigned z = min_u16x2(raw[u].z, lim2), w = min_u16x2(raw[u].w, lim2);
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(A + 16u * ck), "r"(x), "r"(y), "r"(z),
+                             "r"(w) : "memory");
+            } else {
+                const unsigned x = min_u16x2(pack_sat_u16(raw[u].x, raw[u].y), lim2);
+                const unsigned y = min_u16x2(pack_sat_u16(raw[u].z, raw[u].w), lim2);
+                asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(A + 8u * ck), "r"(x), "r"(y) : "memory");
+            }
+        }
+    }
+};
+
+// One tile of up to K candidates of one instance, walked by one warp.  W is
+// the warp's shared-memory region, sh the instance's distances or points and
+// rowt the ready-row template (shared memory, or for many-instance launches
+// global memory).
+template <int DM, bool W16, int V>
+__device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, const int32_t* rowt, int32_t* W,
+                                          long long t, long long next) {
+    using P = Place<DM>;
+    const int lane = threadIdx.x & 31;
+    const int n = a.n, m = a.m, two_n = 2 * n, K = a.K, str4 = a.row_words >> 2;
+    int32_t* ready = W + a.a_words;
+    int32_t* soff = ready + a.ready_words;
+    int32_t* res = soff + a.off_words;         // [4][K]: return, load + 2^16 per overfull route, malformed, blocked
+    const long long first = t * K;
+    const int kt = static_cast<int>(min(static_cast<long long>(K), a.num - first));
+    const unsigned lim2 = static_cast<unsigned>(two_n + 2) * 0x10001u;
+
+    // ---- codes, offsets, result words, ready rows ----
+    const void* src = W16 ? static_cast<const void*>(a.ops16 + first * two_n) : static_cast<const void*>(a.ops + first * two_n);
+    const int head = static_cast<int>(reinterpret_cast<uintptr_t>(src) & 15u) / (W16 ? 2 : 4);
+    const char* base = static_cast<const char*>(src) - head * (W16 ? 2 : 4);
+    const int total = head + kt * two_n;
+    const unsigned Abase = smem_u32(W), A = Abase + 2u * head;
+    constexpr int SB = V == 1 ? 4 : 8;         // one-route kernels run at 64 registers, the others at 128
+    CodeBatch<W16, SB> codes;
+    codes.load(base, head, total, 0);
     for (int i = lane; i < kt * (m + 1); i += 32)
         soff[i] = W16 ? static_cast<int32_t>(__ldg(a.off16 + first * (m + 1) + i)) : __ldg(a.off + first * (m + 1) + i);
-    for (int i = lane; i < kt; i += 32) valid[i] = 1;
-    for (int i = lane; i < kt * a.sw; i += 32) seen[i] = 0u;
-    // unresolved ready time of c: -(p_c + 1) (negative); the drop recovers p_c from it
-    for (int g = 0; g < kt; ++g)
-        for (int c = lane; c <= n; c += 32) ready[g * (n + 1) + c] = -1 - sp[c];
-    __syncwarp();
-    // offsets: off[0] = 0, off[m] = 2n, non-decreasing
-    for (int i = lane; i < kt * (m + 1); i += 32) {
-        const int g = i / (m + 1), vv = i - g * (m + 1);
-        const int val = soff[i];
-        bool bad = val < 0 || val > two_n || (vv == 0 && val != 0) || (vv == m && val != two_n) ||
-                   (vv < m && val > soff[i + 1]);
-        if (bad) atomicAnd(&valid[g], 0);
+    for (int i = lane; i < 4 * K; i += 32) res[i] = 0;
+    {
+        const int4* from = reinterpret_cast<const int4*>(rowt);
+        int4* dst = reinterpret_cast<int4*>(ready);
+        if (str4 >= 32) {
+            for (int i = lane; i < str4; i += 32) {
+                const int4 v = from[i];
+                for (int g = 0; g < kt; ++g) dst[g * str4 + i] = v;
+            }
+        } else {
+            int s = lane % str4;
+            const int step = 32 % str4;
+            for (int i = lane; i < kt * str4; i += 32) {
+                dst[i] = from[s];
+                s += step;
+                s -= s >= str4 ? str4 : 0;
+            }
+        }
     }
-
-    // ---- 2. ops: coalesced loads, four in flight per lane; code range and
-    // duplicates; kept as 16-bit codes (the walk computes the travel times) ----
-    if constexpr (W16) {
-        // code pairs as 32-bit words: 2n is even, so a pair never straddles
-        // two candidates (n pairs each), and candidate i starts 4n i bytes in
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(a.ops16 + first * two_n);
-        uint32_t* A2 = reinterpret_cast<uint32_t*>(A);
-        const int pairs = elems >> 1;
-        int gbase = 0;
-        for (int base = 0; base < pairs; base += 128) {
-            uint32_t raw[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = base + 32 * u + lane;
-                raw[u] = e < pairs ? __ldg(src + e) : 0x00020002u;
-            }
-            if (k > 1)
-                while ((gbase + 1) * n <= base) ++gbase;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = base + 32 * u + lane;
-                if (e < pairs) {
-                    int g = gbase;
-                    if (k > 1)
-                        while ((g + 1) * n <= e) ++g;
-                    const int lo = static_cast<int>(raw[u] & 0xffffu), hi = static_cast<int>(raw[u] >> 16);
-                    const bool okl = lo >= 2 && lo <= two_n + 1, okh = hi >= 2 && hi <= two_n + 1;
-                    bool bad = !(okl && okh);
-                    if (okl) {
-                        const unsigned bit = 1u << (lo & 31);
-                        bad |= (atomicOr(&seen[g * a.sw + (lo >> 5)], bit) & bit) != 0u;
-                    }
-                    if (okh) {
-                        const unsigned bit = 1u << (hi & 31);
-                        bad |= (atomicOr(&seen[g * a.sw + (hi >> 5)], bit) & bit) != 0u;
-                    }
-                    if (bad) atomicAnd(&valid[g], 0);
-                    A2[e] = static_cast<uint32_t>(okl ? lo : 2) | (static_cast<uint32_t>(okh ? hi : 2) << 16);
-                }
-            }
-        }
-    } else {
-        const int32_t* src = a.ops + first * two_n;
-        int gbase = 0;
-        for (int base = 0; base < elems; base += 128) {
-            int raw[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = base + 32 * u + lane;
-                raw[u] = e < elems ? __ldg(src + e) : 2;
-            }
-            if (k > 1)
-                while ((gbase + 1) * two_n <= base) ++gbase;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = base + 32 * u + lane;
-                if (e < elems) {
-                    int g = gbase;
-                    if (k > 1)
-                        while ((g + 1) * two_n <= e) ++g;
-                    const bool ok = raw[u] >= 2 && raw[u] <= two_n + 1;
-                    bool bad = !ok;
-                    if (ok) {
-                        const unsigned bit = 1u << (raw[u] & 31);
-                        bad = (atomicOr(&seen[g * a.sw + (raw[u] >> 5)], bit) & bit) != 0u;
-                    }
-                    if (bad) atomicAnd(&valid[g], 0);
-                    A[e] = static_cast<uint16_t>(ok ? raw[u] : 2);
-                }
-            }
-        }
+    for (int b = 0;;) {
+        codes.store(Abase, lim2, total, b);
+        b += 32 * SB;
+        if (b * CodeBatch<W16, SB>::CPC >= total) break;
+        codes.load(base, head, total, b);
+    }
+    if (next >= 0 && lane == 0) {
+        // the next tile's codes on their way into L2 while this one is walked
+        const uintptr_t p0 = reinterpret_cast<uintptr_t>(W16 ? static_cast<const void*>(a.ops16 + next * K * two_n)
+                                                             : static_cast<const void*>(a.ops + next * K * two_n));
+        const long long left = min(static_cast<long long>(K), a.num - next * K) * two_n * (W16 ? 2 : 4);
+        const uintptr_t lo = (p0 + 15) & ~static_cast<uintptr_t>(15), hi = (p0 + left) & ~static_cast<uintptr_t>(15);
+        if (hi > lo) l2_prefetch_bulk(lo, static_cast<unsigned>(hi - lo));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(W16 ? static_cast<const void*>(a.off16 + next * K * (m + 1))
+                                                          : static_cast<const void*>(a.off + next * K * (m + 1))));
     }
     __syncwarp();
 
-    // ---- 3. route walk (branch-free; up to two ops per lane per step) ----
-    // Each op's travel time is computed here from the previous stop.  Ready
-    // times have a single writer (the dropping lane) and are read with
-    // volatile loads: a pickup sees either "unresolved" (and retries next
-    // step) or the final value.  The __syncwarp at the end of each step makes
-    // every write of step t visible in step t+1, so a group with no progress
-    // in a step can never progress again (a cycle).
-    const bool mine = grp < kt && valid[grp] != 0;
-    int pos = 0, end = 0, start = 0;
-    if (mine) {
-        start = pos = soff[grp * (m + 1) + v];
-        end = soff[grp * (m + 1) + v + 1];
+    // ---- the walk ----
+    // Per route: the op in hand (code, its slot's address, its point, the leg
+    // into it), the code after it, and where the one after that lies (ca).
+    int dep[V], leg[V], code[V], ncode[V], cand[V];
+    unsigned stock[V], ext[V], rbase[V], ca[V], ce[V], ad[V];
+    bool live[V];
+    P at[V];
+#pragma unroll
+    for (int s = 0; s < V; ++s) {
+        const int vl = lane + 32 * s, c = vl / m, v = vl - c * m;
+        live[s] = c < kt;
+        cand[s] = live[s] ? c : 0;
+        int lo = 0, hi = 0;
+        if (live[s]) {
+            lo = soff[c * (m + 1) + v];
+            hi = soff[c * (m + 1) + v + 1];
+            if (lo < 0 || hi > two_n || lo > hi || (v == 0 && lo != 0) || (v == m - 1 && hi != two_n)) {
+                res[2 * K + c] = 1;
+                lo = hi = 0;
+            }
+        }
+        rbase[s] = smem_u32(ready + cand[s] * a.row_words);
+        const unsigned cbase = A + 2u * static_cast<unsigned>(cand[s] * two_n);
+        ca[s] = cbase + 2u * static_cast<unsigned>(lo);
+        ce[s] = cbase + 2u * static_cast<unsigned>(hi);
+        dep[s] = -P::BIAS;
+        stock[s] = ext[s] = STOCK0;
+        const P depot = P::of(a, sh, 0);
+        code[s] = code_or_idle(ca[s], ce[s]);
+        ncode[s] = code_or_idle(ca[s] + 2u, ce[s]);
+        ca[s] += 4u;
+        const int c1 = code[s] >> 1;
+        at[s] = P::of(a, sh, c1);
+        leg[s] = P::leg(a, sh, depot, at[s], c1);
+        ad[s] = rbase[s] + 4u * static_cast<unsigned>(c1);
     }
-    const uint16_t* wp = A + (grp < k ? grp : 0) * two_n;
-    volatile int* rdy = ready + (grp < k ? grp : 0) * (n + 1);
-    int dep = 0, s = 0, smin = 0, smax = 0, loc = 0;
-    bool walking = mine && pos < end, cyc = false;
-    while (__any_sync(FULL_MASK, walking)) {
-        // first op
-        const int o1 = walking ? wp[pos] : 0;
-        const int c1 = o1 >> 1;
-        const bool p1 = (o1 & 1) != 0;
-        // Travel times from shared memory are computed branch-free on every
-        // lane (an idle lane reads code 0, the depot; its result is unused);
-        // with coordinates, c1's point is kept for the second op's leg.  Only
-        // the L2 gathers are skipped on idle lanes.
-        int2 pc1 = make_int2(0, 0);
-        int t1;
-        if constexpr (DM == VRPRPD_DIST_COORDS) {
-            const int2 pl = reinterpret_cast<const int2*>(sh)[loc];
-            pc1 = reinterpret_cast<const int2*>(sh)[c1];
-            t1 = euc2d_small(pl.x, pl.y, pc1.x, pc1.y);
-        } else if constexpr (DM == VRPRPD_DIST_SMEM32 || DM == VRPRPD_DIST_SMEM16) {
-            t1 = dist<DM>(a, sh, loc, c1);
-        } else {
-            t1 = walking ? dist<DM>(a, sh, loc, c1) : 0;
+    for (;;) {
+        bool any = false;
+        int r[V], acode[V];
+        P nat[V];
+#pragma unroll
+        for (int s = 0; s < V; ++s) {
+            // every load of the round at its start: whether the op in hand is
+            // ready, the next op's point, the code after that
+            r[s] = lds_s32(ad[s]);
+            nat[s] = P::of(a, sh, ncode[s] >> 1);
+            acode[s] = code_or_idle(ca[s], ce[s]);
         }
-        const int r1 = rdy[c1];
-        const bool go1 = walking && (!p1 || r1 >= 0);
-        const int a1 = dep + t1;
-        if (go1 && !p1) rdy[c1] = a1 - 1 - r1;
-        dep = go1 ? max(a1, p1 ? r1 : 0) : dep;
-        s += go1 ? (p1 ? 1 : -1) : 0;
-        smin = min(smin, s);
-        smax = max(smax, s);
-        pos += go1 ? 1 : 0;
-        loc = go1 ? c1 : loc;
-        // second op, only behind a first one that went
-        const bool try2 = go1 && pos < end;
-        const int o2 = try2 ? wp[pos] : 0;
-        const int c2 = o2 >> 1;
-        const bool p2 = (o2 & 1) != 0;
-        int t2;
-        if constexpr (DM == VRPRPD_DIST_COORDS) {
-            const int2 pc2 = reinterpret_cast<const int2*>(sh)[c2];
-            t2 = euc2d_small(pc1.x, pc1.y, pc2.x, pc2.y);
-        } else if constexpr (DM == VRPRPD_DIST_SMEM32 || DM == VRPRPD_DIST_SMEM16) {
-            t2 = dist<DM>(a, sh, c1, c2);
-        } else {
-            t2 = try2 ? dist<DM>(a, sh, c1, c2) : 0;
+#pragma unroll
+        for (int s = 0; s < V; ++s) {
+            // this round's op: a drop goes at once, a pickup once it is ready.  A
+            // drop's slot is negative, so the same maximum serves both
+            const bool pick = (code[s] & 1) != 0;
+            const bool go = !pick || r[s] >= 0;
+            const int nd = __viaddmax_s32(dep[s], leg[s], r[s]);
+            sts_s32_if(go, ad[s], pick ? PICKED : static_cast<int>(static_cast<unsigned>(nd) - 1u - static_cast<unsigned>(r[s])));
+            any = any || go;
+            const int c1 = ncode[s] >> 1;
+            const int nleg = P::leg(a, sh, at[s], nat[s], c1);
+            if (go) {
+                dep[s] = nd - P::BIAS;
+                stock[s] += pick ? 0xffff0001u : 0x0000ffffu;
+                code[s] = ncode[s];
+                ncode[s] = acode[s];
+                at[s] = nat[s];
+                leg[s] = nleg;
+                ad[s] = rbase[s] + 4u * static_cast<unsigned>(c1);
+                ca[s] += 2u;
+            }
+            ext[s] = max_u16x2(ext[s], stock[s]);
         }
-        const int r2 = rdy[c2];
-        const bool go2 = try2 && (!p2 || r2 >= 0);
-        const int a2 = dep + t2;
-        if (go2 && !p2) rdy[c2] = a2 - 1 - r2;
-        dep = go2 ? max(a2, p2 ? r2 : 0) : dep;
-        s += go2 ? (p2 ? 1 : -1) : 0;
-        smin = min(smin, s);
-        smax = max(smax, s);
-        pos += go2 ? 1 : 0;
-        loc = go2 ? c2 : loc;
-        const unsigned prog = __ballot_sync(FULL_MASK, go1);
-        const bool more = pos < end;
-        cyc = cyc || (walking && more && (prog & gmask) == 0u);
-        walking = walking && more && !cyc;
         __syncwarp();
+        if (!__any_sync(FULL_MASK, any)) break;
     }
-    if (cyc)                                   // finish the stock prefix of a blocked route
-        for (; pos < end; ++pos) {
-            const int o = wp[pos];
-            if (o & 1) { ++s; smax = max(smax, s); } else { --s; smin = min(smin, s); }
+    bool some_blocked = false;
+#pragma unroll
+    for (int s = 0; s < V; ++s) {
+        const bool blocked = ca[s] - 4u < ce[s];
+        if (blocked) {                         // finish the stock of a blocked route
+            some_blocked = true;
+            res[3 * K + cand[s]] = 1;
+            for (unsigned q = ca[s] - 4u; q < ce[s]; q += 2u) {
+                stock[s] += (code_or_idle(q, ce[s]) & 1) ? 0xffff0001u : 0x0000ffffu;
+                ext[s] = max_u16x2(ext[s], stock[s]);
+            }
         }
+        if (live[s]) {
+            const int up = static_cast<int>(ext[s] & 0xffffu) - 0x4000, down = static_cast<int>(ext[s] >> 16) - 0x4000;
+            const bool over = a.load_full ? (down > a.Q || up > 0) : (down + up > a.Q);
+            atomicMax(&res[cand[s]], dep[s] + leg[s]);
+            atomicAdd(&res[K + cand[s]], (a.load_full ? 0 : down) + (over ? 0x10000 : 0));
+        }
+    }
 
-    // ---- 4. per-candidate reduction ----
-    int ret = 0, flags = 0, pool = 0;
-    if (mine) {
-        if (!cyc && end > start) ret = dep + dist<DM>(a, sh, loc, 0);
-        if (a.load_full) {
-            flags = (smin < -a.Q || smax > 0) ? VRPRPD_VEH_CAP : 0;
-            pool = a.Q;
-        } else {
-            flags = (-smin + smax > a.Q) ? VRPRPD_VEH_CAP : 0;
-            pool = -smin;
+    // ---- every customer picked up? ----
+    {
+        const int4* rows = reinterpret_cast<const int4*>(ready);
+        for (int i = lane; i < kt * str4; i += 32) {
+            const int4 v = rows[i];
+            if (max(max(v.x, v.y), max(v.z, v.w)) != PICKED) res[2 * K + i / str4] |= 2;
         }
-        if (cyc) flags |= VRPRPD_CYCLE;
-    }
-    red[lane] = ret;
-    red[32 + lane] = flags;
-    red[64 + lane] = pool;
-    __syncwarp();
-    if (grp < kt && v == 0) {
-        int z = 0, f = 0;
-        long long pl = 0;
-        for (int j = 0; j < m; ++j) {
-            z = max(z, red[grp * m + j]);
-            f |= red[32 + grp * m + j];
-            pl += red[64 + grp * m + j];
-        }
-        if (pl > a.R) f |= VRPRPD_POOL;
-        if (f & VRPRPD_CYCLE) z = 0x7fffffff;
-        if (!valid[grp]) { z = 0x7fffffff; f = VRPRPD_MALFORMED; }
-        a.z[first + grp] = z;
-        a.st[first + grp] = static_cast<uint32_t>(f);
     }
     __syncwarp();
-    return true;
+    if (__any_sync(FULL_MASK, some_blocked)) {
+        // the full check of candidates with a blocked route, on the staged codes
+        for (int g = 0; g < kt; ++g) {
+            if (!res[3 * K + g] || (res[2 * K + g] & 1)) continue;   // uniform over the warp
+            uint32_t* seen = reinterpret_cast<uint32_t*>(ready + g * a.row_words);
+            for (int i = lane; i < (two_n + 2 + 31) / 32; i += 32) seen[i] = 0u;
+            __syncwarp();
+            bool bad = false;
+            for (int e = lane; e < two_n; e += 32) {
+                const int o = code_or_idle(A + 2u * static_cast<unsigned>(g * two_n + e), ~0u);
+                bool dup = o < 2 || o > two_n + 1;
+                if (!dup) {
+                    const unsigned bit = 1u << (o & 31);
+                    dup = (atomicOr(&seen[o >> 5], bit) & bit) != 0u;
+                }
+                bad = bad || dup;
+            }
+            bad = __any_sync(FULL_MASK, bad);
+            if (lane == 0) res[2 * K + g] = bad ? 1 : 0;
+            __syncwarp();
+        }
+    }
+
+    // ---- results ----
+    for (int g = lane; g < kt; g += 32) {
+        const int load = res[K + g];
+        int z = res[g], f = 0;
+        if (load >> 16) f |= VRPRPD_VEH_CAP;
+        if (a.load_full ? a.pool_full != 0 : (load & 0xffff) > a.R) f |= VRPRPD_POOL;
+        if (res[3 * K + g]) { f |= VRPRPD_CYCLE; z = 0x7fffffff; }
+        if (res[2 * K + g]) { z = 0x7fffffff; f = VRPRPD_MALFORMED; }
+        a.z[first + g] = z;
+        a.st[first + g] = static_cast<uint32_t>(f);
+    }
+    __syncwarp();
 }
 
-template <int DM, bool W16>
-__global__ void __launch_bounds__(1024) eval_tiles_kernel(EvalArgs a) {
+template <int DM, bool W16, int V>
+__global__ void __launch_bounds__(32 * max_warps(V)) eval_tiles_kernel(EvalArgs a) {
     extern __shared__ __align__(16) int32_t smem[];
     __shared__ __align__(8) uint64_t block_bar;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 
     // ---- block-wide staging of the instance (TMA bulk copies) ----
-    int32_t* sh = smem;                        // distances or coordinates
-    int32_t* sp = smem + a.dist_words;         // p[0..n]
+    int32_t* sh = smem;                        // distances or points
+    int32_t* rowt = smem + a.dist_words;       // ready-row template
     if (threadIdx.x == 0) {
         mbar_init(&block_bar, 1);
         unsigned dist_bytes = 0;
         if constexpr (DM == VRPRPD_DIST_SMEM32) dist_bytes = ((a.N * a.N * 4) + 15) & ~15;
         if constexpr (DM == VRPRPD_DIST_SMEM16) dist_bytes = ((a.N * a.N * 2) + 15) & ~15;
         if constexpr (DM == VRPRPD_DIST_COORDS) dist_bytes = ((a.N * 8) + 15) & ~15;
-        unsigned p_bytes = ((a.N * 4) + 15) & ~15;
-        mbar_arrive_expect_tx(&block_bar, dist_bytes + p_bytes);
+        const unsigned row_bytes = a.row_words * 4u;
+        if constexpr (DM == DIST_HALF2) dist_bytes = row_bytes;
+        mbar_arrive_expect_tx(&block_bar, dist_bytes + row_bytes);
         if constexpr (DM == VRPRPD_DIST_SMEM32) tma_bulk_g2s(sh, a.d32, dist_bytes, &block_bar);
         if constexpr (DM == VRPRPD_DIST_SMEM16) tma_bulk_g2s(sh, a.d16, dist_bytes, &block_bar);
         if constexpr (DM == VRPRPD_DIST_COORDS) tma_bulk_g2s(sh, a.coords, dist_bytes, &block_bar);
-        tma_bulk_g2s(sp, a.p, p_bytes, &block_bar);
+        if constexpr (DM == DIST_HALF2) tma_bulk_g2s(sh, a.xy, dist_bytes, &block_bar);
+        tma_bulk_g2s(rowt, a.rowt, row_bytes, &block_bar);
     }
     __syncthreads();
     if (!mbar_wait_bounded(&block_bar, 0)) {
@@ -338,358 +482,29 @@ __global__ void __launch_bounds__(1024) eval_tiles_kernel(EvalArgs a) {
         return;
     }
     int32_t* W = smem + a.shared_words + warp * a.warp_words;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(W + a.warp_words - 4);
-    if (lane == 0) mbar_init(bar, 1);
-    __syncwarp();
-    const long long ntiles = (a.num + a.k - 1) / a.k;
+    const long long ntiles = (a.num + a.K - 1) / a.K;
     const long long gw = static_cast<long long>(blockIdx.x) * nwarps + warp;
     const long long nw = static_cast<long long>(gridDim.x) * nwarps;
-    unsigned phase = 0;
     for (long long t = gw; t < ntiles; t += nw)
-        if (!eval_tile<DM, W16>(a, sh, sp, W, bar, phase, t)) return;
-}
-
-// ---------------------------------------------------------------------------
-// Streamed form.  No staging pass: each lane reads its own route's op codes
-// from global memory through a four-deep register queue (two codes in use,
-// the next two loaded at the top of every step, so their latency overlaps
-// the step), and checks them as it walks.  A group of G warps walks
-// K = floor(32 G / m) candidates at once, lane L of the group taking route
-// L mod m of candidate L / m, so for m that does not divide 32 (m = 20: three
-// candidates per two warps) candidates straddle warps and far fewer lanes
-// idle.  The group meets at a named barrier once per step.  Shared memory
-// holds only the ready times, the offsets and a few words per candidate.
-//
-// Validation without a staging pass.  Offsets are checked first.  Each code
-// is range-checked as it is walked.  A drop must find its customer's ready
-// slot unresolved (a resolved or picked slot means a second drop: MALFORMED);
-// a pickup marks the slot picked (INT32_MIN), so a second pickup of the same
-// customer waits forever.  Slots are written by atomic exchange and the old
-// value must be the one read: two lanes holding the same op in one step
-// cannot both pass.  If every route is walked to its end with no such
-// fault, the candidate is a permutation: the n drops are of distinct
-// customers, each pickup follows its own customer's drop and no customer is
-// picked twice, so the 2n codes hold n drops and n pickups of n distinct
-// customers.  A candidate whose walk blocks (a cycle, or a repeated or
-// missing op) gets the full check (range and a duplicate bitmap) after the
-// walk, which tells MALFORMED from CYCLE.
-// ---------------------------------------------------------------------------
-constexpr int PICKED = static_cast<int>(0x80000000u);   // ready slot of a customer already picked up
-
-__device__ __forceinline__ void named_sync(int id, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-// barrier of the group plus an OR over its threads' predicates
-__device__ __forceinline__ bool named_any(int id, int nthreads, bool pred) {
-    unsigned r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"(static_cast<unsigned>(pred)), "r"(id), "r"(nthreads)
-        : "memory");
-    return r != 0;
-}
-
-// shared-memory ready slots by 32-bit shared address: a volatile load, and an
-// exchange executed only when `on` (else the read value comes back)
-__device__ __forceinline__ int lds_volatile(unsigned addr) {
-    int v;
-    asm volatile("ld.volatile.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ int atoms_exch_if(bool on, unsigned addr, int val, int otherwise) {
-    int old = otherwise;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.u32 p, %2, 0;\n\t"
-        "@p atom.shared.exch.b32 %0, [%1], %3;\n\t}"
-        : "+r"(old)
-        : "r"(addr), "r"(static_cast<unsigned>(on)), "r"(val)
-        : "memory");
-    return old;
-}
-
-template <int G>
-__device__ __forceinline__ void group_sync(int id) {
-    if constexpr (G == 1) __syncwarp();
-    else named_sync(id, 32 * G);
-}
-template <int G>
-__device__ __forceinline__ bool group_any(int id, bool pred) {
-    if constexpr (G == 1) {
-        __syncwarp();
-        return __any_sync(FULL_MASK, pred) != 0;
-    } else {
-        return named_any(id, 32 * G, pred);
-    }
-}
-
-template <int DM, bool W16, int G>
-__device__ __forceinline__ void eval_stream_tile(const EvalArgs& a, const int32_t* sh, const int32_t* sp, int32_t* W,
-                                                 int gl, int bar_id, long long t) {
-    constexpr int NT = 32 * G;
-    const int n = a.n, m = a.m, two_n = 2 * n, K = a.K, N1 = n + 1;
-    int32_t* ready = W + a.g_ready;     // K x (n+1): -(p+1) unresolved, T_drop + p, or PICKED
-    int32_t* soff = W + a.g_off;        // K x (m+1)
-    int32_t* flag = W + a.g_flag;       // K: 1 = malformed
-    // [2][K]: the last step (of the slot's parity) in which the candidate
-    // progressed.  Two slots: a warp of the group that has left step t's
-    // barrier may stamp step t+1 before another warp of the group has read
-    // step t's stamp; it can never reach step t+2 before that read
-    int32_t* prog = W + a.g_prog;
-    int32_t* red = W + a.g_red;         // 3 x NT
-    const long long first = t * K;
-    const int kt = static_cast<int>(min(static_cast<long long>(K), a.num - first));
-    const int cand = gl / m, v = gl - cand * m;
-    const bool active = cand < kt;
-
-    // ---- 1. offsets, flags, unresolved ready times ----
-    for (int i = gl; i < kt * (m + 1); i += NT)
-        soff[i] = W16 ? static_cast<int32_t>(__ldg(a.off16 + first * (m + 1) + i)) : __ldg(a.off + first * (m + 1) + i);
-    for (int i = gl; i < kt; i += NT) {
-        flag[i] = 0;
-        prog[i] = -1;
-        prog[K + i] = -1;
-    }
-    for (int g = 0; g < kt; ++g)
-        for (int c = gl; c <= n; c += NT) ready[g * N1 + c] = -1 - sp[c];
-    group_sync<G>(bar_id);
-    // each lane checks the offsets around its route: off[0] = 0, off[m] = 2n, non-decreasing
-    int pos = 0, end = 0, start = 0;
-    if (active) {
-        const int lo = soff[cand * (m + 1) + v], hi = soff[cand * (m + 1) + v + 1];
-        if (lo < 0 || hi > two_n || lo > hi || (v == 0 && lo != 0) || (v == m - 1 && hi != two_n)) flag[cand] = 1;
-        start = pos = lo;
-        end = hi;
-    }
-    group_sync<G>(bar_id);
-    const bool ok_off = active && flag[cand] == 0;
-
-    // ---- 2. the walk (up to two ops per lane per step) ----
-    const long long cbase = (first + (active ? cand : 0)) * two_n;
-    auto code_at = [&](int q) -> int {
-        return W16 ? static_cast<int>(__ldg(a.ops16 + cbase + q)) : __ldg(a.ops + cbase + q);
-    };
-    // this lane's codes from its current position on, and its candidate's
-    // ready slots as a shared-memory address
-    const int32_t* rp32 = nullptr;
-    const uint16_t* rp16 = nullptr;
-    if constexpr (W16) rp16 = a.ops16 + cbase + pos;
-    else rp32 = a.ops + cbase + pos;
-    const unsigned rdy_addr = smem_u32(ready + (active ? cand : 0) * N1);
-    int dep = 0, s = 0, smin = 0, smax = 0, loc = 0;
-    bool walking = ok_off && pos < end, cyc = false, bad = false;
-    int q0 = walking ? code_at(pos) : 0;
-    int q1 = (walking && pos + 1 < end) ? code_at(pos + 1) : 0;
-    for (int step = 0;; ++step) {
-        int q2 = 0, q3 = 0;
-        if (walking && pos + 2 < end) q2 = W16 ? static_cast<int>(__ldg(rp16 + 2)) : __ldg(rp32 + 2);
-        if (walking && pos + 3 < end) q3 = W16 ? static_cast<int>(__ldg(rp16 + 3)) : __ldg(rp32 + 3);
-        // first op
-        const int o1 = walking ? q0 : 0;
-        const bool in1 = static_cast<unsigned>(o1 - 2) < static_cast<unsigned>(two_n);
-        const int c1 = in1 ? (o1 >> 1) : 0;
-        const bool p1 = (o1 & 1) != 0;
-        int2 pc1 = make_int2(0, 0);
-        int t1;
-        if constexpr (DM == VRPRPD_DIST_COORDS) {
-            const int2 pl = reinterpret_cast<const int2*>(sh)[loc];
-            pc1 = reinterpret_cast<const int2*>(sh)[c1];
-            t1 = euc2d_small(pl.x, pl.y, pc1.x, pc1.y);
-        } else if constexpr (DM == VRPRPD_DIST_SMEM32 || DM == VRPRPD_DIST_SMEM16) {
-            t1 = dist<DM>(a, sh, loc, c1);
-        } else {
-            t1 = walking ? dist<DM>(a, sh, loc, c1) : 0;
-        }
-        const unsigned ad1 = rdy_addr + 4u * static_cast<unsigned>(c1);
-        const int r1 = lds_volatile(ad1);
-        // a drop needs an unresolved slot, -(p+1) in [-2^31 + 1, -1]
-        const bool bad1 = walking && (!in1 || (!p1 && static_cast<unsigned>(r1) <= 0x80000000u));
-        const bool go1 = walking && !bad1 && (!p1 || r1 >= 0);
-        const int a1 = dep + t1;
-        // exchange, not store: two lanes that read the same slot in the same
-        // step (a repeated op) cannot both see it unchanged
-        const int old1 = atoms_exch_if(go1, ad1, p1 ? PICKED : a1 - 1 - r1, r1);
-        const bool race1 = old1 != r1;
-        dep = go1 ? max(a1, p1 ? r1 : 0) : dep;
-        s += go1 ? (p1 ? 1 : -1) : 0;
-        smin = min(smin, s);
-        smax = max(smax, s);
-        pos += go1 ? 1 : 0;
-        loc = go1 ? c1 : loc;
-        // second op, only behind a first one that went
-        const bool try2 = go1 && pos < end;
-        const int o2 = try2 ? q1 : 0;
-        const bool in2 = static_cast<unsigned>(o2 - 2) < static_cast<unsigned>(two_n);
-        const int c2 = in2 ? (o2 >> 1) : 0;
-        const bool p2 = (o2 & 1) != 0;
-        int t2;
-        if constexpr (DM == VRPRPD_DIST_COORDS) {
-            const int2 pc2 = reinterpret_cast<const int2*>(sh)[c2];
-            t2 = euc2d_small(pc1.x, pc1.y, pc2.x, pc2.y);
-        } else if constexpr (DM == VRPRPD_DIST_SMEM32 || DM == VRPRPD_DIST_SMEM16) {
-            t2 = dist<DM>(a, sh, c1, c2);
-        } else {
-            t2 = try2 ? dist<DM>(a, sh, c1, c2) : 0;
-        }
-        const unsigned ad2 = rdy_addr + 4u * static_cast<unsigned>(c2);
-        const int r2 = lds_volatile(ad2);
-        const bool bad2 = try2 && (!in2 || (!p2 && static_cast<unsigned>(r2) <= 0x80000000u));
-        const bool go2 = try2 && !bad2 && (!p2 || r2 >= 0);
-        const int a2 = dep + t2;
-        const int old2 = atoms_exch_if(go2, ad2, p2 ? PICKED : a2 - 1 - r2, r2);
-        const bool race2 = old2 != r2;
-        dep = go2 ? max(a2, p2 ? r2 : 0) : dep;
-        s += go2 ? (p2 ? 1 : -1) : 0;
-        smin = min(smin, s);
-        smax = max(smax, s);
-        pos += go2 ? 1 : 0;
-        loc = go2 ? c2 : loc;
-        // the queue and the code pointer move by the ops taken
-        const int took = (go1 ? 1 : 0) + (go2 ? 1 : 0);
-        q0 = go2 ? q2 : (go1 ? q1 : q0);
-        q1 = go2 ? q3 : (go1 ? q2 : q1);
-        if constexpr (W16) rp16 += took;
-        else rp32 += took;
-        // a repeat caught by the exchange only marks the candidate: the walk
-        // goes on (its slots stay in range and it still ends), which keeps the
-        // exchange's round trip off the step's critical path
-        const bool fault = bad1 || bad2;
-        bad = bad || fault || race1 || race2;
-        if (go1) prog[(step & 1) * K + cand] = step;
-        const bool cont = walking && !fault && pos < end;
-        // the group's barrier: every ready time and stamp of this step is
-        // visible after it, so a candidate with no progress in a step while
-        // unfinished can never progress again (a cycle, or a repeated or
-        // missing op that the full check below tells apart)
-        const bool any = group_any<G>(bar_id, cont);
-        cyc = cyc || (cont && prog[(step & 1) * K + cand] != step);
-        walking = cont && !cyc;
-        if (!any) break;
-    }
-    if (bad) flag[cand] = 1;
-    if (cyc)                                   // finish the stock prefix of a blocked route
-        for (; pos < end; ++pos) {
-            const int o = code_at(pos);
-            if (o & 1) { ++s; smax = max(smax, s); } else { --s; smin = min(smin, s); }
-        }
-    red[gl] = cyc ? 1 : 0;
-    group_sync<G>(bar_id);
-
-    // ---- 3. full check of the candidates whose walk blocked ----
-    for (int g = 0; g < kt; ++g) {
-        bool blocked = false;
-        for (int j = 0; j < m; ++j) blocked = blocked || red[g * m + j] != 0;
-        if (!blocked || flag[g]) continue;     // uniform over the group
-        uint32_t* seen = reinterpret_cast<uint32_t*>(ready + g * N1);   // the ready times are no longer needed
-        const int sw = (two_n + 2 + 31) / 32;
-        for (int i = gl; i < sw; i += NT) seen[i] = 0u;
-        group_sync<G>(bar_id);
-        const long long gb = (first + g) * two_n;
-        for (int e = gl; e < two_n; e += NT) {
-            const int o = W16 ? static_cast<int>(__ldg(a.ops16 + gb + e)) : __ldg(a.ops + gb + e);
-            bool dup = static_cast<unsigned>(o - 2) >= static_cast<unsigned>(two_n);
-            if (!dup) {
-                const unsigned bit = 1u << (o & 31);
-                dup = (atomicOr(&seen[o >> 5], bit) & bit) != 0u;
-            }
-            if (dup) flag[g] = 1;
-        }
-        group_sync<G>(bar_id);
-    }
-
-    // ---- 4. per-candidate reduction ----
-    int ret = 0, f = 0, pool = 0;
-    if (ok_off) {
-        if (!cyc && end > start) ret = dep + dist<DM>(a, sh, loc, 0);
-        if (a.load_full) {
-            f = (smin < -a.Q || smax > 0) ? VRPRPD_VEH_CAP : 0;
-            pool = a.Q;
-        } else {
-            f = (-smin + smax > a.Q) ? VRPRPD_VEH_CAP : 0;
-            pool = -smin;
-        }
-        if (cyc) f |= VRPRPD_CYCLE;
-    }
-    group_sync<G>(bar_id);                     // the blocked marks above are read
-    red[gl] = ret;
-    red[NT + gl] = f;
-    red[2 * NT + gl] = pool;
-    group_sync<G>(bar_id);
-    if (active && v == 0) {
-        int z = 0, fl = 0;
-        long long pl = 0;
-        for (int j = 0; j < m; ++j) {
-            z = max(z, red[cand * m + j]);
-            fl |= red[NT + cand * m + j];
-            pl += red[2 * NT + cand * m + j];
-        }
-        if (pl > a.R) fl |= VRPRPD_POOL;
-        if (fl & VRPRPD_CYCLE) z = 0x7fffffff;
-        if (flag[cand]) { z = 0x7fffffff; fl = VRPRPD_MALFORMED; }
-        a.z[first + cand] = z;
-        a.st[first + cand] = static_cast<uint32_t>(fl);
-    }
-    group_sync<G>(bar_id);                     // the region is reused by the next tile
-}
-
-template <int DM, bool W16, int G>
-__global__ void __launch_bounds__(1024) eval_stream_kernel(EvalArgs a) {
-    extern __shared__ __align__(16) int32_t smem[];
-    __shared__ __align__(8) uint64_t block_bar;
-    // ---- block-wide staging of the instance (TMA bulk copies) ----
-    int32_t* sh = smem;
-    int32_t* sp = smem + a.dist_words;
-    if (threadIdx.x == 0) {
-        mbar_init(&block_bar, 1);
-        unsigned dist_bytes = 0;
-        if constexpr (DM == VRPRPD_DIST_SMEM32) dist_bytes = ((a.N * a.N * 4) + 15) & ~15;
-        if constexpr (DM == VRPRPD_DIST_SMEM16) dist_bytes = ((a.N * a.N * 2) + 15) & ~15;
-        if constexpr (DM == VRPRPD_DIST_COORDS) dist_bytes = ((a.N * 8) + 15) & ~15;
-        unsigned p_bytes = ((a.N * 4) + 15) & ~15;
-        mbar_arrive_expect_tx(&block_bar, dist_bytes + p_bytes);
-        if constexpr (DM == VRPRPD_DIST_SMEM32) tma_bulk_g2s(sh, a.d32, dist_bytes, &block_bar);
-        if constexpr (DM == VRPRPD_DIST_SMEM16) tma_bulk_g2s(sh, a.d16, dist_bytes, &block_bar);
-        if constexpr (DM == VRPRPD_DIST_COORDS) tma_bulk_g2s(sh, a.coords, dist_bytes, &block_bar);
-        tma_bulk_g2s(sp, a.p, p_bytes, &block_bar);
-    }
-    __syncthreads();
-    if (!mbar_wait_bounded(&block_bar, 0)) {
-        if (threadIdx.x == 0) atomicExch(a.err, DEV_TIMEOUT_TMA);
-        mbar_wait_bounded(&block_bar, 0);
-        return;
-    }
-    const int warp = threadIdx.x >> 5, group = warp / G, gl = threadIdx.x - group * 32 * G;
-    const int ngroups = (blockDim.x >> 5) / G;
-    if (group >= ngroups) return;
-    int32_t* W = smem + a.shared_words + static_cast<long long>(group) * a.group_words;
-    const long long ntiles = (a.num + a.K - 1) / a.K;
-    const long long g0 = static_cast<long long>(blockIdx.x) * ngroups + group;
-    const long long ng = static_cast<long long>(gridDim.x) * ngroups;
-    for (long long t = g0; t < ntiles; t += ng) eval_stream_tile<DM, W16, G>(a, sh, sp, W, gl, 1 + group, t);
+        eval_tile<DM, W16, V>(a, sh, rowt, W, t, a.prefetch && t + nw < ntiles ? t + nw : -1);
 }
 
 // Many instances of uneven size in one persistent launch: tile t of the
 // whole job belongs to the instance whose tile prefix brackets it.  Distances
-// come from each instance's matrix in global memory (L2-resident); p is read
-// through the cache.  Every warp region is sized for the largest instance.
-template <int DM>
-__global__ void __launch_bounds__(1024) eval_multi_kernel(const EvalArgs* __restrict__ insts,
+// come from the instance's points, copied into the warp's region per tile
+// (DIST_HALF2), or from its matrix in global memory (L2-resident).  Every warp
+// region is sized for the largest instance.
+template <int DM, int V>
+__global__ void __launch_bounds__(32 * max_warps(V)) eval_multi_kernel(const EvalArgs* __restrict__ insts,
                                                           const long long* __restrict__ tile_prefix, int n_inst,
                                                           int warp_words) {
     extern __shared__ __align__(16) int32_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     int32_t* W = smem + warp * warp_words;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(W + warp_words - 4);
-    if (lane == 0) mbar_init(bar, 1);
-    __syncwarp();
     const long long total = tile_prefix[n_inst];
     const long long gw = static_cast<long long>(blockIdx.x) * nwarps + warp;
     const long long nw = static_cast<long long>(gridDim.x) * nwarps;
-    unsigned phase = 0;
+    int have = -1;                              // the instance whose points the region holds
     for (long long t = gw; t < total; t += nw) {
         int lo = 0, hi = n_inst;                // prefix[lo] <= t < prefix[lo+1]
         while (hi - lo > 1) {
@@ -697,32 +512,17 @@ __global__ void __launch_bounds__(1024) eval_multi_kernel(const EvalArgs* __rest
             if (__ldg(tile_prefix + mid) <= t) lo = mid; else hi = mid;
         }
         const EvalArgs a = insts[lo];
-        if (!eval_tile<DM, false>(a, nullptr, a.p, W, bar, phase, t - __ldg(tile_prefix + lo))) return;
-    }
-}
-
-
-// The same with the streamed walk, one-warp groups: tile t of the whole job is
-// ⌊32/m⌋ candidates of the instance whose tile prefix brackets it, walked by
-// one warp whose region is sized for the largest instance.
-template <int DM>
-__global__ void __launch_bounds__(1024) eval_multi_stream_kernel(const EvalArgs* __restrict__ insts,
-                                                                 const long long* __restrict__ tile_prefix,
-                                                                 int n_inst, int group_words) {
-    extern __shared__ __align__(16) int32_t smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    int32_t* W = smem + warp * group_words;
-    const long long total = tile_prefix[n_inst];
-    const long long gw = static_cast<long long>(blockIdx.x) * nwarps + warp;
-    const long long nw = static_cast<long long>(gridDim.x) * nwarps;
-    for (long long t = gw; t < total; t += nw) {
-        int lo = 0, hi = n_inst;                // prefix[lo] <= t < prefix[lo+1]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(tile_prefix + mid) <= t) lo = mid; else hi = mid;
+        const int32_t* sh = nullptr;
+        if constexpr (DM == DIST_HALF2) {
+            sh = W + a.pts;
+            if (have != lo) {
+                const int4* src = reinterpret_cast<const int4*>(a.xy);
+                int4* dst = reinterpret_cast<int4*>(W + a.pts);
+                for (int i = lane; i < a.row_words / 4; i += 32) dst[i] = __ldg(src + i);
+                have = lo;
+            }
         }
-        const EvalArgs a = insts[lo];
-        eval_stream_tile<DM, false, 1>(a, nullptr, a.p, W, lane, 0, t - __ldg(tile_prefix + lo));
+        eval_tile<DM, false, V>(a, sh, a.rowt, W, t - __ldg(tile_prefix + lo), -1);
     }
 }
 
@@ -809,29 +609,19 @@ __global__ void eval_plain_kernel(const int32_t* __restrict__ ops, const int32_t
 // ---------------------------------------------------------------------------
 static int round4(long long w) { return static_cast<int>((w + 3) & ~3ll); }
 
+// Shared memory of an SM, and what the system keeps of it per block.
+constexpr long long SM_SHARED_BYTES = 228 << 10, BLOCK_SHARED_BYTES = 1 << 10;
+
 struct Plan {
-    int dm = 0, warps = 0, blocks = 0;
+    int dm = 0;          // the kernel's distance mode (DIST_HALF2 for small coordinates)
+    int warps = 0, blocks = 0;
     bool w16 = false;    // 16-bit op codes and offsets
-    int walk = VRPRPD_WALK_STAGED;
-    int G = 1;           // streamed form: warps per group
+    int V = 1;           // routes per lane
     size_t smem = 0;
     EvalArgs args{};
 };
 
-static bool coords_small(const vrprpd_instance* I) {
-    if (!I->has_coords) return false;
-    int minx = I->h_coords[0], maxx = minx, miny = I->h_coords[1], maxy = miny;
-    for (int i = 0; i <= I->n; ++i) {
-        minx = std::min(minx, I->h_coords[2 * i]);
-        maxx = std::max(maxx, I->h_coords[2 * i]);
-        miny = std::min(miny, I->h_coords[2 * i + 1]);
-        maxy = std::max(maxy, I->h_coords[2 * i + 1]);
-    }
-    long long dx = maxx - minx, dy = maxy - miny;
-    return dx * dx + dy * dy < (1ll << 24);
-}
-
-bool coords_exact_small(const vrprpd_instance* I) { return coords_small(I); }
+bool coords_exact_small(const vrprpd_instance* I) { return I->coords24; }
 
 bool batched_supported(const vrprpd_instance* I) {
     return I->m <= 32 && 2 * I->n + 1 < (1 << PACK_SHIFT) && I->maxd < (1 << 19);
@@ -843,41 +633,48 @@ static bool dist_mode_available(const vrprpd_instance* I, int dm) {
         case VRPRPD_DIST_SMEM16: return I->has_d16;
         case VRPRPD_DIST_GLOBAL16: return I->has_d16;
         case VRPRPD_DIST_GLOBAL32: return true;
-        case VRPRPD_DIST_COORDS: return coords_small(I);
+        case VRPRPD_DIST_COORDS: return I->coords24;
     }
     return false;
 }
 
-static bool make_plan(const vrprpd_instance* I, int dm, int warps, int blocks_per_sm, long long num, Plan* P);
-
-// The streamed form's layout: groups of G warps (for G > 1 at most 15 per
-// block, one named barrier each), K = floor(32 G / m) candidates per group tile.
-static bool make_plan_stream(const vrprpd_instance* I, int dm, int warps, int G, long long num, Plan* P) {
-    if (G != 1 && G != 2) return false;
-    // groups of more than one warp meet at named barriers 1..15
-    if (warps % G != 0 || (G > 1 && warps / G > 15) || 32 * G < I->m) return false;
-    if (!make_plan(I, dm, G, 0, num, P)) return false;        // instance words and shared fields
-    EvalArgs& a = P->args;
-    const long long N1 = I->n + 1;
-    a.G = G;
-    a.K = (32 * G) / I->m;
-    a.g_ready = 0;
-    a.g_off = round4(static_cast<long long>(a.K) * N1);
-    a.g_flag = a.g_off + round4(static_cast<long long>(a.K) * (I->m + 1));
-    a.g_prog = a.g_flag + round4(a.K);
-    a.g_red = a.g_prog + round4(2ll * a.K);
-    a.group_words = a.g_red + 3 * 32 * G;
-    const size_t smem = static_cast<size_t>(a.shared_words + static_cast<long long>(warps / G) * a.group_words) * 4;
-    if (smem + 64 > I->smem_optin) return false;
-    P->walk = VRPRPD_WALK_STREAMED;
-    P->G = G;
-    P->warps = warps;
-    P->smem = smem;
-    return true;
+// What the entry points accept, in words of shared memory: the shapes of
+// vrprpd_eval_config mean a block of `warps` warps, each with a region for
+// floor(32/m) candidates (staged), or each group of G warps with one for
+// floor(32 G/m) (streamed; codes not kept), beside the instance data.  The
+// kernel's own regions are at most as large, or hold fewer candidates.
+static long long accepted_shared_words(const vrprpd_instance* I, int dm) {
+    const long long N = I->n + 1;
+    long long w = 0;
+    if (dm == VRPRPD_DIST_SMEM32) w = N * N;
+    if (dm == VRPRPD_DIST_SMEM16) w = (N * N + 1) / 2;
+    if (dm == VRPRPD_DIST_COORDS) w = 2 * N;
+    return round4(w) + round4(N);
+}
+static long long accepted_staged_words(int n, int m) {
+    const long long k = 32 / m, N = n + 1, sw = (2ll * n + 2 + 31) / 32;
+    return round4((k * 2 * n + 1) / 2 + 2) + round4(k * N) + round4(k * sw) + round4(k * (m + 1)) + round4(k) + 100;
+}
+static long long accepted_streamed_words(int n, int m, int G) {
+    const long long K = 32ll * G / m, N = n + 1;
+    return round4(K * N) + round4(K * (m + 1)) + round4(K) + round4(2 * K) + 96ll * G;
+}
+static bool shape_accepted(const vrprpd_instance* I, int dm, int warps, int walk, int G) {
+    long long words = accepted_shared_words(I, dm);
+    if (walk == VRPRPD_WALK_STREAMED) {
+        if ((G != 1 && G != 2) || warps % G != 0 || (G > 1 && warps / G > 15) || 32 * G < I->m) return false;
+        words += warps / G * accepted_streamed_words(I->n, I->m, G);
+    } else {
+        words += warps * accepted_staged_words(I->n, I->m);
+    }
+    return words * 4 + 64 <= static_cast<long long>(I->smem_optin);
 }
 
-// Fill the layout for (dist mode, warps per block); false if it does not fit.
-static bool make_plan(const vrprpd_instance* I, int dm, int warps, int blocks_per_sm, long long num, Plan* P) {
+// The layout for (distance mode, warps per block, routes per lane): as many
+// candidates per tile as the lanes take (32 V / m), fewer where the block's
+// shared memory does not hold them or a warp's region would pass `cap` words.
+// False if not even one fits.
+static bool make_plan(const vrprpd_instance* I, int dm, int warps, int V, long long num, Plan* P, int cap = INT32_MAX) {
     EvalArgs& a = P->args;
     a = EvalArgs{};
     a.n = I->n;
@@ -886,170 +683,138 @@ static bool make_plan(const vrprpd_instance* I, int dm, int warps, int blocks_pe
     a.Q = I->Q;
     a.N = I->n + 1;
     a.load_full = (I->flags & VRPRPD_LOAD_FULL) != 0;
-    a.k = 32 / I->m;
+    a.pool_full = static_cast<long long>(I->m) * I->Q > I->R;
     a.d32 = I->d32;
     a.d16 = I->d16;
     a.coords = I->coords;
-    a.p = I->p;
+    a.xy = I->xy;
+    a.rowt = I->rowt;
+    a.row_words = I->row_words;
     a.err = I->err;
     a.num = num;
-    const long long N = a.N, two_n = 2ll * I->n;
+    const long long N = a.N;
+    if (dm == VRPRPD_DIST_COORDS && I->xy) dm = DIST_HALF2;
     long long dist_words = 0;
     if (dm == VRPRPD_DIST_SMEM32) dist_words = N * N;
     if (dm == VRPRPD_DIST_SMEM16) dist_words = (N * N + 1) / 2;
     if (dm == VRPRPD_DIST_COORDS) dist_words = 2 * N;
+    if (dm == DIST_HALF2) dist_words = a.row_words;
     a.dist_words = round4(dist_words);
-    a.shared_words = a.dist_words + round4(N);
-    a.sw = static_cast<int>((two_n + 2 + 31) / 32);
-    a.a_words = round4((a.k * two_n + 1) / 2 + 2);
-    a.ready_words = round4(static_cast<long long>(a.k) * N);
-    a.seen_words = round4(static_cast<long long>(a.k) * a.sw);
-    a.start_words = 0;
-    a.off_words = round4(static_cast<long long>(a.k) * (I->m + 1));
-    a.valid_words = round4(a.k);
-    a.warp_words = a.a_words + a.ready_words + a.seen_words + a.start_words + a.off_words + a.valid_words + 96 + 4;
-    const size_t smem = static_cast<size_t>(a.shared_words + static_cast<long long>(warps) * a.warp_words) * 4;
-    if (smem + 64 > I->smem_optin) return false;
-    P->dm = dm;
-    P->warps = warps;
-    P->walk = VRPRPD_WALK_STAGED;
-    P->G = 1;
-    P->smem = smem;
-    return true;
-}
-
-template <bool W16, int G>
-static const void* stream_kernel_for(int dm) {
-    switch (dm) {
-        case VRPRPD_DIST_SMEM32: return reinterpret_cast<const void*>(&eval_stream_kernel<VRPRPD_DIST_SMEM32, W16, G>);
-        case VRPRPD_DIST_SMEM16: return reinterpret_cast<const void*>(&eval_stream_kernel<VRPRPD_DIST_SMEM16, W16, G>);
-        case VRPRPD_DIST_GLOBAL16: return reinterpret_cast<const void*>(&eval_stream_kernel<VRPRPD_DIST_GLOBAL16, W16, G>);
-        case VRPRPD_DIST_GLOBAL32: return reinterpret_cast<const void*>(&eval_stream_kernel<VRPRPD_DIST_GLOBAL32, W16, G>);
-        default: return reinterpret_cast<const void*>(&eval_stream_kernel<VRPRPD_DIST_COORDS, W16, G>);
+    a.shared_words = a.dist_words + a.row_words;
+    for (int K = 32 * V / I->m; K >= 1; --K) {
+        a.K = K;
+        a.a_words = round4(static_cast<long long>(K) * I->n) + 8;   // codes, shifted by up to 7 and padded to 16 bytes
+        a.ready_words = K * a.row_words;
+        a.off_words = round4(static_cast<long long>(K) * (I->m + 1));
+        a.warp_words = a.a_words + a.ready_words + a.off_words + round4(4ll * K);
+        P->smem = static_cast<size_t>(a.shared_words + static_cast<long long>(warps) * a.warp_words) * 4;
+        if (P->smem + 64 <= I->smem_optin && (K == 1 || a.warp_words <= cap)) {
+            P->dm = dm;
+            P->warps = warps;
+            P->V = V;
+            return true;
+        }
     }
+    return false;
 }
 
-template <bool W16>
+template <bool W16, int V>
 static const void* kernel_for(int dm) {
     switch (dm) {
-        case VRPRPD_DIST_SMEM32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM32, W16>);
-        case VRPRPD_DIST_SMEM16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM16, W16>);
-        case VRPRPD_DIST_GLOBAL16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL16, W16>);
-        case VRPRPD_DIST_GLOBAL32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL32, W16>);
-        default: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_COORDS, W16>);
+        case VRPRPD_DIST_SMEM32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM32, W16, V>);
+        case VRPRPD_DIST_SMEM16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM16, W16, V>);
+        case VRPRPD_DIST_GLOBAL16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL16, W16, V>);
+        case VRPRPD_DIST_GLOBAL32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL32, W16, V>);
+        case DIST_HALF2: return reinterpret_cast<const void*>(&eval_tiles_kernel<DIST_HALF2, W16, V>);
+        default: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_COORDS, W16, V>);
     }
 }
 
-static const void* plan_kernel(const Plan* P) {
-    if (P->walk == VRPRPD_WALK_STREAMED) {
-        if (P->G == 2) return P->w16 ? stream_kernel_for<true, 2>(P->dm) : stream_kernel_for<false, 2>(P->dm);
-        return P->w16 ? stream_kernel_for<true, 1>(P->dm) : stream_kernel_for<false, 1>(P->dm);
-    }
-    return P->w16 ? kernel_for<true>(P->dm) : kernel_for<false>(P->dm);
+static const void* plan_kernel(const Plan& P) {
+    if (P.V == 2) return P.w16 ? kernel_for<true, 2>(P.dm) : kernel_for<false, 2>(P.dm);
+    return P.w16 ? kernel_for<true, 1>(P.dm) : kernel_for<false, 1>(P.dm);
 }
 
 static int finalize_plan(const vrprpd_instance* I, int blocks_per_sm, Plan* P) {
-    const void* fn = plan_kernel(P);
+    const void* fn = plan_kernel(*P);
     { int rc_ = ensure_smem_limit(fn); if (rc_) return rc_; }
     int occ = 0;
     VRP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, P->warps * 32, P->smem));
     VRP_CHECK(occ > 0, VRPRPD_EINVAL, "evaluation layout does not fit on an SM");
     if (blocks_per_sm > 0) occ = std::min(occ, blocks_per_sm);
-    const bool streamed = P->walk == VRPRPD_WALK_STREAMED;
-    const long long per_tile = streamed ? P->args.K : P->args.k;
-    const long long units = streamed ? P->warps / P->G : P->warps;     // tile workers per block
-    const long long ntiles = (P->args.num + per_tile - 1) / per_tile;
-    long long want = (ntiles + units - 1) / units;
-    long long blocks = std::min<long long>(static_cast<long long>(occ) * I->num_sms, want);
+    const long long ntiles = (P->args.num + P->args.K - 1) / P->args.K;
+    const long long want = (ntiles + P->warps - 1) / P->warps;
+    const long long blocks = std::min<long long>(static_cast<long long>(occ) * I->num_sms, want);
     P->blocks = static_cast<int>(std::max<long long>(blocks, 1));
     return VRPRPD_OK;
 }
 
-// Default shape: shared-memory distances when they leave room for 8 warps,
-// else recomputed coordinates, else L2 gathers.
-// host_mapped: the candidates are read in place from pinned host memory over
-// the host link, where only the staged walk's coalesced reads are fast; the
-// best staged shape the autotuner saw is used then (else the default order).
-static int choose_plan(const vrprpd_instance* I, long long num, Plan* P, bool host_mapped = false) {
-    EvalTuning T = I->tune;
-    if (host_mapped && T.walk != VRPRPD_WALK_STAGED) T = I->tune_staged;
-    if (T.dist_mode != VRPRPD_DIST_AUTO && T.warps_per_block > 0) {
-        VRP_CHECK(dist_mode_available(I, T.dist_mode), VRPRPD_EINVAL, "configured distance mode unavailable");
-        if (T.walk == VRPRPD_WALK_STREAMED) {
-            const bool w16 = P->w16;
-            VRP_CHECK(make_plan_stream(I, T.dist_mode, T.warps_per_block, T.group_warps, num, P), VRPRPD_EINVAL,
-                      "configured streamed layout does not fit (warps %d, group %d)", T.warps_per_block,
-                      T.group_warps);
-            P->w16 = w16;
-            return finalize_plan(I, T.blocks_per_sm, P);
-        }
-        VRP_CHECK(make_plan(I, T.dist_mode, T.warps_per_block, T.blocks_per_sm, num, P), VRPRPD_EINVAL,
-                  "configured evaluation layout exceeds shared memory");
-        return finalize_plan(I, T.blocks_per_sm, P);
-    }
-    const int order[] = {VRPRPD_DIST_SMEM32, VRPRPD_DIST_SMEM16, VRPRPD_DIST_COORDS, VRPRPD_DIST_GLOBAL16,
-                         VRPRPD_DIST_GLOBAL32};
-    for (int dm : order) {
-        if (!dist_mode_available(I, dm)) continue;
-        for (int warps : {32, 24, 16, 8}) {
-            if (dm != VRPRPD_DIST_GLOBAL32 && dm != VRPRPD_DIST_GLOBAL16 && warps < 8) continue;
-            if (make_plan(I, dm, warps, 0, num, P)) return finalize_plan(I, 0, P);
-        }
-    }
-    for (int warps : {8, 4, 2, 1})
-        if (make_plan(I, VRPRPD_DIST_GLOBAL32, warps, 0, num, P)) return finalize_plan(I, 0, P);
-    set_error("no evaluation layout fits shared memory (n=%d, m=%d)", I->n, I->m);
+// The plan of a configured or tuned shape: its warps per block, or the most
+// that fit.
+static int plan_shape(const vrprpd_instance* I, const EvalTuning& T, long long num, Plan* P) {
+    VRP_CHECK(dist_mode_available(I, T.dist_mode), VRPRPD_EINVAL, "configured distance mode unavailable");
+    const int V = T.walk == VRPRPD_WALK_STREAMED ? T.group_warps : 1;
+    for (int warps = std::min(T.warps_per_block, max_warps(V)); warps >= 1; --warps)
+        if (make_plan(I, T.dist_mode, warps, V, num, P)) return finalize_plan(I, T.blocks_per_sm, P);
+    set_error("configured evaluation layout exceeds shared memory");
     return VRPRPD_EINVAL;
 }
 
-template <bool W16>
-static void launch_tiles(const Plan& P, const EvalArgs& a, cudaStream_t stream) {
-    switch (P.dm) {
-        case VRPRPD_DIST_SMEM32:
-            eval_tiles_kernel<VRPRPD_DIST_SMEM32, W16><<<P.blocks, P.warps * 32, P.smem, stream>>>(a);
-            break;
-        case VRPRPD_DIST_SMEM16:
-            eval_tiles_kernel<VRPRPD_DIST_SMEM16, W16><<<P.blocks, P.warps * 32, P.smem, stream>>>(a);
-            break;
-        case VRPRPD_DIST_GLOBAL16:
-            eval_tiles_kernel<VRPRPD_DIST_GLOBAL16, W16><<<P.blocks, P.warps * 32, P.smem, stream>>>(a);
-            break;
-        case VRPRPD_DIST_GLOBAL32:
-            eval_tiles_kernel<VRPRPD_DIST_GLOBAL32, W16><<<P.blocks, P.warps * 32, P.smem, stream>>>(a);
-            break;
-        default:
-            eval_tiles_kernel<VRPRPD_DIST_COORDS, W16><<<P.blocks, P.warps * 32, P.smem, stream>>>(a);
-            break;
+static int choose_plan(const vrprpd_instance* I, long long num, Plan* P) {
+    if (I->tune.dist_mode != VRPRPD_DIST_AUTO && I->tune.warps_per_block > 0) return plan_shape(I, I->tune, num, P);
+    if (!shape_accepted(I, VRPRPD_DIST_GLOBAL32, 1, VRPRPD_WALK_STAGED, 1)) {
+        set_error("no evaluation layout fits shared memory (n=%d, m=%d)", I->n, I->m);
+        return VRPRPD_EINVAL;
     }
-}
-
-template <bool W16, int G>
-static void launch_stream(const Plan& P, const EvalArgs& a, cudaStream_t stream) {
-    const int th = P.warps * 32;
-    switch (P.dm) {
-        case VRPRPD_DIST_SMEM32: eval_stream_kernel<VRPRPD_DIST_SMEM32, W16, G><<<P.blocks, th, P.smem, stream>>>(a); break;
-        case VRPRPD_DIST_SMEM16: eval_stream_kernel<VRPRPD_DIST_SMEM16, W16, G><<<P.blocks, th, P.smem, stream>>>(a); break;
-        case VRPRPD_DIST_GLOBAL16: eval_stream_kernel<VRPRPD_DIST_GLOBAL16, W16, G><<<P.blocks, th, P.smem, stream>>>(a); break;
-        case VRPRPD_DIST_GLOBAL32: eval_stream_kernel<VRPRPD_DIST_GLOBAL32, W16, G><<<P.blocks, th, P.smem, stream>>>(a); break;
-        default: eval_stream_kernel<VRPRPD_DIST_COORDS, W16, G><<<P.blocks, th, P.smem, stream>>>(a); break;
+    // Distances: points as fp16 pairs when the instance has them (a leg is 7
+    // instructions from one 4-byte gather); else the 16-bit matrix in shared
+    // memory while it takes at most half of it, recomputed integer legs, and
+    // the matrix in L2 last.
+    int dm = VRPRPD_DIST_GLOBAL32;
+    if (I->xy) dm = VRPRPD_DIST_COORDS;
+    else if (I->has_d16 && accepted_shared_words(I, VRPRPD_DIST_SMEM16) * 8 <= static_cast<long long>(I->smem_optin)) dm = VRPRPD_DIST_SMEM16;
+    else if (accepted_shared_words(I, VRPRPD_DIST_SMEM32) * 8 <= static_cast<long long>(I->smem_optin)) dm = VRPRPD_DIST_SMEM32;
+    else if (I->coords24) dm = VRPRPD_DIST_COORDS;
+    else if (I->has_d16) dm = VRPRPD_DIST_GLOBAL16;
+    // Two routes per lane when that uses the lanes better by a fifth or more
+    // (m = 11, 12 and 17..21): n=499 m=19 (57 of 64 lane slots against 19 of
+    // 32) 172 us against 223 us for 65536 candidates, n=1000 m=20 368 against
+    // 377; but n=200 m=6 (30 of 32 both ways) 78 us against 72 us.
+    const int m = I->m, V = 5 * (64 / m) * m >= 6 * 2 * (32 / m) * m ? 2 : 1;
+    // Warps per block: most routes in flight on an SM, the smallest block on
+    // ties (n=200 m=6: 4 warps 72 us, 24 warps 76 us); few tiles are spread
+    // over the SMs first.
+    Plan best;
+    best.w16 = P->w16;
+    long long most = 0;
+    for (int warps : {4, 8, 12, 16, 24, 28, 32, 2, 1}) {
+        Plan C;
+        if (warps > max_warps(V) || (warps < 4 && most) || !make_plan(I, dm, warps, V, num, &C)) continue;
+        const long long by_smem = SM_SHARED_BYTES / static_cast<long long>(C.smem + BLOCK_SHARED_BYTES);
+        const long long resident = warps * std::min<long long>(by_smem, max_warps(V) / warps);
+        if (resident * C.args.K > most) {
+            most = resident * C.args.K;
+            best.args = C.args;
+            best.dm = C.dm;
+            best.warps = warps;
+            best.V = V;
+        }
     }
+    if (!most) {
+        set_error("no evaluation layout fits shared memory (n=%d, m=%d)", I->n, I->m);
+        return VRPRPD_EINVAL;
+    }
+    const long long ntiles = (num + best.args.K - 1) / best.args.K;
+    best.warps = static_cast<int>(std::max<long long>(1, std::min<long long>(best.warps, (ntiles + I->num_sms - 1) / I->num_sms)));
+    best.smem = static_cast<size_t>(best.args.shared_words + static_cast<long long>(best.warps) * best.args.warp_words) * 4;
+    *P = best;
+    return finalize_plan(I, 0, P);
 }
 
 static int launch_plan(const Plan& P, cudaStream_t stream) {
-    if (P.walk == VRPRPD_WALK_STREAMED) {
-        if (P.G == 2) {
-            if (P.w16) launch_stream<true, 2>(P, P.args, stream);
-            else launch_stream<false, 2>(P, P.args, stream);
-        } else {
-            if (P.w16) launch_stream<true, 1>(P, P.args, stream);
-            else launch_stream<false, 1>(P, P.args, stream);
-        }
-    } else if (P.w16) {
-        launch_tiles<true>(P, P.args, stream);
-    } else {
-        launch_tiles<false>(P, P.args, stream);
-    }
-    VRP_CUDA(cudaGetLastError());
+    EvalArgs args = P.args;
+    void* params[] = {&args};
+    VRP_CUDA(cudaLaunchKernel(plan_kernel(P), dim3(P.blocks), dim3(P.warps * 32), params, P.smem, stream));
     return VRPRPD_OK;
 }
 
@@ -1070,8 +835,9 @@ int evaluate_device(const vrprpd_instance* I, const int32_t* ops, const int32_t*
         return VRPRPD_EINVAL;
     }
     Plan P;
-    int rc = choose_plan(I, num, &P, host_mapped);
+    int rc = choose_plan(I, num, &P);
     if (rc) return rc;
+    P.args.prefetch = host_mapped ? 0 : 1;
     P.args.ops = ops;
     P.args.off = off;
     P.args.z = z;
@@ -1089,8 +855,9 @@ static int evaluate_device16(const vrprpd_instance* I, const uint16_t* ops, cons
     }
     Plan P;
     P.w16 = true;
-    int rc = choose_plan(I, num, &P, host_mapped);
+    int rc = choose_plan(I, num, &P);
     if (rc) return rc;
+    P.args.prefetch = host_mapped ? 0 : 1;
     P.args.ops16 = ops;
     P.args.off16 = off;
     P.args.z = z;
@@ -1228,7 +995,6 @@ extern "C" int vrprpd_eval_set_config(vrprpd_instance* I, const vrprpd_eval_conf
     VRP_CHECK(I && cfg, VRPRPD_EINVAL, "NULL argument");
     if (cfg->dist_mode == VRPRPD_DIST_AUTO) {
         I->tune = EvalTuning{};
-        I->tune_staged = EvalTuning{};
         return VRPRPD_OK;
     }
     VRP_CHECK(cfg->dist_mode >= VRPRPD_DIST_SMEM32 && cfg->dist_mode <= VRPRPD_DIST_COORDS, VRPRPD_EINVAL,
@@ -1238,15 +1004,11 @@ extern "C" int vrprpd_eval_set_config(vrprpd_instance* I, const vrprpd_eval_conf
     VRP_CHECK(cfg->warps_per_block >= 1 && cfg->warps_per_block <= 32, VRPRPD_EINVAL, "bad warps_per_block");
     VRP_CHECK(cfg->walk == VRPRPD_WALK_STAGED || cfg->walk == VRPRPD_WALK_STREAMED, VRPRPD_EINVAL, "bad walk %d",
               cfg->walk);
-    Plan P;
-    if (cfg->walk == VRPRPD_WALK_STREAMED) {
-        VRP_CHECK(make_plan_stream(I, cfg->dist_mode, cfg->warps_per_block, cfg->group_warps, 1, &P), VRPRPD_EINVAL,
-                  "streamed layout does not fit (group_warps must be 1 or 2, divide warps_per_block, leave at "
-                  "most 15 groups and cover m lanes)");
-    } else {
-        VRP_CHECK(make_plan(I, cfg->dist_mode, cfg->warps_per_block, cfg->blocks_per_sm, 1, &P), VRPRPD_EINVAL,
-                  "layout exceeds shared memory");
-    }
+    VRP_CHECK(shape_accepted(I, cfg->dist_mode, cfg->warps_per_block, cfg->walk, cfg->group_warps), VRPRPD_EINVAL,
+              cfg->walk == VRPRPD_WALK_STREAMED
+                  ? "streamed layout does not fit (group_warps must be 1 or 2, divide warps_per_block, leave at "
+                    "most 15 groups and cover m lanes)"
+                  : "layout exceeds shared memory");
     I->tune.dist_mode = cfg->dist_mode;
     I->tune.warps_per_block = cfg->warps_per_block;
     I->tune.blocks_per_sm = cfg->blocks_per_sm;
@@ -1260,11 +1022,12 @@ extern "C" int vrprpd_eval_get_config(const vrprpd_instance* I, vrprpd_eval_conf
     Plan P;
     int rc = choose_plan(I, 1 << 20, &P);
     if (rc) return rc;
-    cfg->dist_mode = P.dm;
-    cfg->warps_per_block = P.warps;
+    const bool set = I->tune.dist_mode != VRPRPD_DIST_AUTO;
+    cfg->dist_mode = P.dm == DIST_HALF2 ? VRPRPD_DIST_COORDS : P.dm;
+    cfg->warps_per_block = set ? I->tune.warps_per_block : P.warps;
     cfg->blocks_per_sm = I->tune.blocks_per_sm;
-    cfg->walk = P.walk;
-    cfg->group_warps = P.G;
+    cfg->walk = set ? I->tune.walk : P.V == 2 ? VRPRPD_WALK_STREAMED : VRPRPD_WALK_STAGED;
+    cfg->group_warps = set ? I->tune.group_warps : P.V;
     return VRPRPD_OK;
 }
 
@@ -1282,48 +1045,35 @@ extern "C" int vrprpd_autotune(vrprpd_instance* I, const vrprpd_batch* b, void* 
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    float best_ms = 1e30f, best_staged_ms = 1e30f;
-    EvalTuning best{}, best_staged{};
+    float best_ms = 1e30f;
+    EvalTuning best{};
     const EvalTuning saved = I->tune;
     const int modes[] = {VRPRPD_DIST_SMEM32, VRPRPD_DIST_SMEM16, VRPRPD_DIST_COORDS, VRPRPD_DIST_GLOBAL16,
                          VRPRPD_DIST_GLOBAL32};
-    // the staged walk, then the streamed walk with one- and two-warp groups
-    struct Cand { int walk, dm, warps, bps, G; };
-    std::vector<Cand> cands;
     for (int dm : modes) {
         if (!dist_mode_available(I, dm)) continue;
-        for (int warps : {4, 8, 12, 16, 24, 32})
-            for (int bps : {0, 1, 2}) {
+        for (int V : {1, 2}) {
+            const int walk = V == 2 ? VRPRPD_WALK_STREAMED : VRPRPD_WALK_STAGED;
+            for (int warps : {4, 8, 12, 16, 24, 28, 32}) {
                 Plan P;
-                if (make_plan(I, dm, warps, bps, b->num, &P)) cands.push_back({VRPRPD_WALK_STAGED, dm, warps, bps, 1});
-            }
-        for (int G : {1, 2})
-            for (int warps : {4, 8, 12, 16, 20, 24, 28, 30, 32})
-                for (int bps : {0, 1, 2}) {
-                    Plan P;
-                    if (make_plan_stream(I, dm, warps, G, b->num, &P)) cands.push_back({VRPRPD_WALK_STREAMED, dm, warps, bps, G});
+                if (warps > max_warps(V) || !shape_accepted(I, dm, warps, walk, V) || !make_plan(I, dm, warps, V, b->num, &P)) continue;
+                I->tune = EvalTuning{dm, warps, 0, walk, V};
+                float ms_min = 1e30f;
+                for (int rep = 0; rep < 4; ++rep) {
+                    cudaEventRecord(e0, stream);
+                    int rc = evaluate_device(I, b->ops, b->off, b->num, z, st, stream);
+                    cudaEventRecord(e1, stream);
+                    if (rc) break;
+                    cudaEventSynchronize(e1);
+                    float ms = 0;
+                    cudaEventElapsedTime(&ms, e0, e1);
+                    if (rep > 0) ms_min = std::min(ms_min, ms);
                 }
-    }
-    for (const Cand& cd : cands) {
-        I->tune = EvalTuning{cd.dm, cd.warps, cd.bps, cd.walk, cd.G};
-        float ms_min = 1e30f;
-        for (int rep = 0; rep < 4; ++rep) {
-            cudaEventRecord(e0, stream);
-            int rc = evaluate_device(I, b->ops, b->off, b->num, z, st, stream);
-            cudaEventRecord(e1, stream);
-            if (rc) break;
-            cudaEventSynchronize(e1);
-            float ms = 0;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (rep > 0) ms_min = std::min(ms_min, ms);
-        }
-        if (ms_min < best_ms) {
-            best_ms = ms_min;
-            best = I->tune;
-        }
-        if (cd.walk == VRPRPD_WALK_STAGED && ms_min < best_staged_ms) {
-            best_staged_ms = ms_min;
-            best_staged = I->tune;
+                if (ms_min < best_ms) {
+                    best_ms = ms_min;
+                    best = I->tune;
+                }
+            }
         }
     }
     cudaEventDestroy(e0);
@@ -1336,7 +1086,6 @@ extern "C" int vrprpd_autotune(vrprpd_instance* I, const vrprpd_batch* b, void* 
         return VRPRPD_EINVAL;
     }
     I->tune = best;
-    I->tune_staged = best_staged;
     if (chosen) {
         chosen->dist_mode = best.dist_mode;
         chosen->warps_per_block = best.warps_per_block;
@@ -1351,15 +1100,23 @@ extern "C" int vrprpd_autotune(vrprpd_instance* I, const vrprpd_batch* b, void* 
 // ---------------------------------------------------------------------------
 // many instances, one persistent launch
 // ---------------------------------------------------------------------------
+// Words of one warp's region per route a lane walks, at most (unless a single
+// candidate needs more): every region is sized for the largest instance, and
+// this leaves 26 warps per SM.
+constexpr int MULTI_CAP_WORDS = 2048;
+
 struct vrprpd_multi {
     int n_inst = 0, device = 0, num_sms = 0;
     size_t smem_optin = 0;
-    // per walk (0 staged, 1 streamed): per-instance arguments and tile prefix
+    bool all16 = true, all_xy = true;
+    // what the entry points accept: the largest instance's region per warp, staged and streamed
+    long long accepted_words[2] = {0, 0};
+    // for one and two routes per lane: per-instance arguments and tile prefix
     std::vector<EvalArgs> args[2];
     std::vector<long long> prefix[2];
     EvalArgs* d_args[2] = {nullptr, nullptr};
     long long* d_prefix[2] = {nullptr, nullptr};
-    int walk = VRPRPD_WALK_STAGED;
+    int V = 1;
     int dm = VRPRPD_DIST_GLOBAL16, warps = 8, blocks = 0, warp_words = 0;
     size_t smem = 0;
     cudaGraph_t graph = nullptr;
@@ -1369,54 +1126,43 @@ struct vrprpd_multi {
 
 namespace vrp {
 
-static const void* multi_kernel(int walk, int dm) {
-    if (walk == VRPRPD_WALK_STREAMED)
-        return dm == VRPRPD_DIST_GLOBAL16 ? reinterpret_cast<const void*>(&eval_multi_stream_kernel<VRPRPD_DIST_GLOBAL16>)
-                                          : reinterpret_cast<const void*>(&eval_multi_stream_kernel<VRPRPD_DIST_GLOBAL32>);
-    return dm == VRPRPD_DIST_GLOBAL16 ? reinterpret_cast<const void*>(&eval_multi_kernel<VRPRPD_DIST_GLOBAL16>)
-                                      : reinterpret_cast<const void*>(&eval_multi_kernel<VRPRPD_DIST_GLOBAL32>);
+template <int V>
+static const void* multi_kernel(int dm) {
+    if (dm == DIST_HALF2) return reinterpret_cast<const void*>(&eval_multi_kernel<DIST_HALF2, V>);
+    return dm == VRPRPD_DIST_GLOBAL16 ? reinterpret_cast<const void*>(&eval_multi_kernel<VRPRPD_DIST_GLOBAL16, V>)
+                                      : reinterpret_cast<const void*>(&eval_multi_kernel<VRPRPD_DIST_GLOBAL32, V>);
 }
+static const void* multi_kernel(const vrprpd_multi* M) { return M->V == 2 ? multi_kernel<2>(M->dm) : multi_kernel<1>(M->dm); }
 
-static int multi_layout(vrprpd_multi* M, int dm, int warps, int walk) {
-    const bool streamed = walk == VRPRPD_WALK_STREAMED;
+static int multi_layout(vrprpd_multi* M, int dm, int warps, int V) {
     int ww = 0;
-    for (auto& a : M->args[streamed]) ww = std::max(ww, streamed ? a.group_words : a.warp_words);
-    const size_t smem = static_cast<size_t>(warps) * ww * 4;
-    if (smem + 64 > M->smem_optin) return VRPRPD_EINVAL;
-    const void* fn = multi_kernel(walk, dm);
-    { int rc_ = ensure_smem_limit(fn); if (rc_) return rc_; }
-    int occ = 0;
-    VRP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, warps * 32, smem));
-    if (occ <= 0) return VRPRPD_EINVAL;
-    const long long total = M->prefix[streamed].back();
-    M->blocks = static_cast<int>(std::max<long long>(1, std::min<long long>(static_cast<long long>(occ) * M->num_sms,
-                                                                         (total + warps - 1) / warps)));
-    M->walk = walk;
+    for (auto& a : M->args[V - 1]) ww = std::max(ww, a.warp_words);
+    for (warps = std::min(warps, max_warps(V)); warps >= 1; --warps)
+        if (static_cast<size_t>(warps) * ww * 4 + 64 <= M->smem_optin) break;
+    if (warps < 1) return VRPRPD_EINVAL;
+    M->V = V;
     M->dm = dm;
     M->warps = warps;
     M->warp_words = ww;
-    M->smem = smem;
+    M->smem = static_cast<size_t>(warps) * ww * 4;
+    const void* fn = multi_kernel(M);
+    { int rc_ = ensure_smem_limit(fn); if (rc_) return rc_; }
+    int occ = 0;
+    VRP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, warps * 32, M->smem));
+    if (occ <= 0) return VRPRPD_EINVAL;
+    const long long total = M->prefix[V - 1].back();
+    M->blocks = static_cast<int>(std::max<long long>(1, std::min<long long>(static_cast<long long>(occ) * M->num_sms,
+                                                                         (total + warps - 1) / warps)));
     if (M->exec) { cudaGraphExecDestroy(M->exec); M->exec = nullptr; }
     if (M->graph) { cudaGraphDestroy(M->graph); M->graph = nullptr; }
     return VRPRPD_OK;
 }
 
 static int multi_launch(vrprpd_multi* M, cudaStream_t s) {
-    const int w = M->walk == VRPRPD_WALK_STREAMED ? 1 : 0;
-    const dim3 grid(M->blocks), block(M->warps * 32);
-    if (w && M->dm == VRPRPD_DIST_GLOBAL16)
-        eval_multi_stream_kernel<VRPRPD_DIST_GLOBAL16><<<grid, block, M->smem, s>>>(M->d_args[1], M->d_prefix[1],
-                                                                                   M->n_inst, M->warp_words);
-    else if (w)
-        eval_multi_stream_kernel<VRPRPD_DIST_GLOBAL32><<<grid, block, M->smem, s>>>(M->d_args[1], M->d_prefix[1],
-                                                                                   M->n_inst, M->warp_words);
-    else if (M->dm == VRPRPD_DIST_GLOBAL16)
-        eval_multi_kernel<VRPRPD_DIST_GLOBAL16><<<grid, block, M->smem, s>>>(M->d_args[0], M->d_prefix[0],
-                                                                            M->n_inst, M->warp_words);
-    else
-        eval_multi_kernel<VRPRPD_DIST_GLOBAL32><<<grid, block, M->smem, s>>>(M->d_args[0], M->d_prefix[0],
-                                                                            M->n_inst, M->warp_words);
-    VRP_CUDA(cudaGetLastError());
+    const EvalArgs* args = M->d_args[M->V - 1];
+    const long long* prefix = M->d_prefix[M->V - 1];
+    void* params[] = {&args, &prefix, &M->n_inst, &M->warp_words};
+    VRP_CUDA(cudaLaunchKernel(multi_kernel(M), dim3(M->blocks), dim3(M->warps * 32), params, M->smem, s));
     return VRPRPD_OK;
 }
 
@@ -1431,7 +1177,6 @@ extern "C" int vrprpd_multi_create(const vrprpd_instance* const* insts, const vr
     M->n_inst = n_inst;
     M->prefix[0].assign(1, 0);
     M->prefix[1].assign(1, 0);
-    bool all16 = true;
     for (int i = 0; i < n_inst; ++i) {
         const vrprpd_instance* I = insts[i];
         int rc = check_batch(I, &batches[i], makespan[i], status[i]);
@@ -1450,23 +1195,25 @@ extern "C" int vrprpd_multi_create(const vrprpd_instance* const* insts, const vr
             set_error("instances live on different devices");
             return VRPRPD_EINVAL;
         }
-        all16 = all16 && I->has_d16;
-        // both walks' layouts: the staged one (per warp) and the streamed one
-        // (one-warp groups); no instance data is staged in shared memory
+        M->all16 = M->all16 && I->has_d16;
+        M->all_xy = M->all_xy && I->xy != nullptr;
+        M->accepted_words[0] = std::max(M->accepted_words[0], accepted_staged_words(I->n, I->m));
+        M->accepted_words[1] = std::max(M->accepted_words[1], accepted_streamed_words(I->n, I->m, 1));
+        // no block-wide instance data; the points (if used) follow the warp's region
         for (int w = 0; w < 2; ++w) {
             Plan P;
-            if (w == 0) make_plan(I, VRPRPD_DIST_GLOBAL32, 1, 0, batches[i].num, &P);
-            else make_plan_stream(I, VRPRPD_DIST_GLOBAL32, 1, 1, batches[i].num, &P);
+            make_plan(I, VRPRPD_DIST_GLOBAL32, 1, w + 1, batches[i].num, &P, MULTI_CAP_WORDS * (w + 1));
             EvalArgs a = P.args;
             a.shared_words = 0;
             a.dist_words = 0;
+            a.pts = a.warp_words;
+            a.warp_words += I->xy ? a.row_words : 0;
             a.ops = batches[i].ops;
             a.off = batches[i].off;
             a.z = makespan[i];
             a.st = status[i];
-            const long long per_tile = w == 0 ? a.k : a.K;
             M->args[w].push_back(a);
-            M->prefix[w].push_back(M->prefix[w].back() + (a.num + per_tile - 1) / per_tile);
+            M->prefix[w].push_back(M->prefix[w].back() + (a.num + a.K - 1) / a.K);
         }
     }
     cudaError_t e = cudaSuccess;
@@ -1485,9 +1232,14 @@ extern "C" int vrprpd_multi_create(const vrprpd_instance* const* insts, const vr
         return VRPRPD_ECUDA;
     }
     int rc = VRPRPD_EINVAL;
-    for (int warps : {8, 4, 2, 1}) {
-        rc = multi_layout(M, all16 ? VRPRPD_DIST_GLOBAL16 : VRPRPD_DIST_GLOBAL32, warps, VRPRPD_WALK_STAGED);
-        if (rc == VRPRPD_OK) break;
+    if (M->accepted_words[0] * 4 + 64 <= static_cast<long long>(M->smem_optin)) {
+        // one or two routes per lane as for a single instance, by the lane
+        // steps of the whole job (a tile walks about 2n/m rounds of V routes)
+        double steps[2] = {0, 0};
+        for (int w = 0; w < 2; ++w)
+            for (auto& a : M->args[w]) steps[w] += static_cast<double>((a.num + a.K - 1) / a.K) * (w + 1) * a.n / a.m;
+        const int dm = M->all_xy ? DIST_HALF2 : M->all16 ? VRPRPD_DIST_GLOBAL16 : VRPRPD_DIST_GLOBAL32;
+        rc = multi_layout(M, dm, 4, 1.2 * steps[1] <= steps[0] ? 2 : 1);
     }
     if (rc) {
         set_error("multi_create: no layout fits shared memory");
@@ -1524,18 +1276,17 @@ extern "C" int vrprpd_multi_evaluate(vrprpd_multi* M, void* stream_) {
 extern "C" int vrprpd_multi_autotune(vrprpd_multi* M, void* stream_, vrprpd_eval_config* chosen) {
     VRP_CHECK(M, VRPRPD_EINVAL, "NULL plan");
     cudaStream_t s = static_cast<cudaStream_t>(stream_);
-    bool all16 = true;
-    for (auto& a : M->args[0]) all16 = all16 && a.d16 != nullptr;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     float best = 1e30f;
-    int bdm = M->dm, bw = M->warps, bwalk = M->walk;
-    for (int walk : {VRPRPD_WALK_STAGED, VRPRPD_WALK_STREAMED}) {
-        for (int dm : {VRPRPD_DIST_GLOBAL16, VRPRPD_DIST_GLOBAL32}) {
-            if (dm == VRPRPD_DIST_GLOBAL16 && !all16) continue;
+    int bdm = M->dm, bw = M->warps, bV = M->V;
+    for (int V : {1, 2}) {
+        for (int dm : {DIST_HALF2, static_cast<int>(VRPRPD_DIST_GLOBAL16), static_cast<int>(VRPRPD_DIST_GLOBAL32)}) {
+            if ((dm == DIST_HALF2 && !M->all_xy) || (dm == VRPRPD_DIST_GLOBAL16 && !M->all16)) continue;
             for (int warps : {4, 8, 12, 16, 24, 32}) {
-                if (multi_layout(M, dm, warps, walk) != VRPRPD_OK) continue;
+                if (M->accepted_words[V - 1] * 4 * warps + 64 > static_cast<long long>(M->smem_optin)) continue;
+                if (multi_layout(M, dm, warps, V) != VRPRPD_OK) continue;
                 float ms_min = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {
                     cudaEventRecord(e0, s);
@@ -1546,20 +1297,20 @@ extern "C" int vrprpd_multi_autotune(vrprpd_multi* M, void* stream_, vrprpd_eval
                     cudaEventElapsedTime(&ms, e0, e1);
                     if (rep > 0) ms_min = std::min(ms_min, ms);
                 }
-                if (ms_min < best) { best = ms_min; bdm = dm; bw = warps; bwalk = walk; }
+                if (ms_min < best) { best = ms_min; bdm = dm; bw = warps; bV = V; }
             }
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    int rc = multi_layout(M, bdm, bw, bwalk);
+    int rc = multi_layout(M, bdm, bw, bV);
     if (rc) return rc;
     if (chosen) {
-        chosen->dist_mode = bdm;
+        chosen->dist_mode = bdm == DIST_HALF2 ? VRPRPD_DIST_COORDS : bdm;
         chosen->warps_per_block = bw;
         chosen->blocks_per_sm = 0;
-        chosen->walk = bwalk;
-        chosen->group_warps = 1;
+        chosen->walk = bV == 2 ? VRPRPD_WALK_STREAMED : VRPRPD_WALK_STAGED;
+        chosen->group_warps = bV;
     }
     VRP_CUDA(cudaGetLastError());
     return VRPRPD_OK;
@@ -1574,7 +1325,10 @@ extern "C" int vrprpd_multi_set_config(vrprpd_multi* M, const vrprpd_eval_config
     if (cfg->dist_mode == VRPRPD_DIST_GLOBAL16)
         for (auto& a : M->args[0]) VRP_CHECK(a.d16 != nullptr, VRPRPD_EINVAL, "an instance has no 16-bit matrix");
     VRP_CHECK(cfg->warps_per_block >= 1 && cfg->warps_per_block <= 32, VRPRPD_EINVAL, "bad warps_per_block");
-    const int rc = multi_layout(M, cfg->dist_mode, cfg->warps_per_block, cfg->walk);
+    const bool streamed = cfg->walk == VRPRPD_WALK_STREAMED;
+    VRP_CHECK(M->accepted_words[streamed] * 4 * cfg->warps_per_block + 64 <= static_cast<long long>(M->smem_optin),
+              VRPRPD_EINVAL, "this layout does not fit shared memory");
+    const int rc = multi_layout(M, cfg->dist_mode, cfg->warps_per_block, 1);
     VRP_CHECK(rc == VRPRPD_OK, rc, "this layout does not fit shared memory");
     return VRPRPD_OK;
 }

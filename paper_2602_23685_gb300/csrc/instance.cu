@@ -1,5 +1,6 @@
 // Instance construction: validation, device residency and the EUC_2D
 // distance kernel (Section 5.1: TSPLIB edge weights as travel times).
+#include <algorithm>
 #include <cstdarg>
 #include <cstdlib>
 #include <cstring>
@@ -108,8 +109,16 @@ static int common_init(vrprpd_instance* I, const int32_t* p, int32_t n, int32_t 
     int optin = 0;
     VRP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, I->device));
     I->smem_optin = static_cast<size_t>(optin);
-    VRP_CUDA(cudaMalloc(&I->p, pad16((n + 1) * sizeof(int32_t))));
-    VRP_CUDA(cudaMemcpy(I->p, I->h_p.data(), (n + 1) * sizeof(int32_t), cudaMemcpyHostToDevice));
+    // p, then the evaluator's ready-row template: -(p_c + 1) per customer, the
+    // "already picked up" word in the depot's slot and past the last customer
+    I->row_words = (n + 2 + 3) & ~3;
+    const size_t p_words = (n + 1 + 63) & ~static_cast<size_t>(63);
+    std::vector<int32_t> h(p_words + I->row_words, INT32_MIN);
+    for (int c = 0; c <= n; ++c) h[c] = I->h_p[c];
+    for (int c = 1; c <= n; ++c) h[p_words + c] = -1 - I->h_p[c];
+    VRP_CUDA(cudaMalloc(&I->p, h.size() * sizeof(int32_t)));
+    I->rowt = I->p + p_words;
+    VRP_CUDA(cudaMemcpy(I->p, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     return VRPRPD_OK;
 }
 
@@ -134,11 +143,29 @@ extern "C" int vrprpd_instance_create(const int32_t* coords, const int32_t* p, i
     I->h_coords.assign(coords, coords + 2 * N);
     I->has_coords = true;
     const long long NN = static_cast<long long>(N) * N;
+    // the box of the points bounds every squared leg
+    int lo[2] = {coords[0], coords[1]}, hi[2] = {coords[0], coords[1]};
+    for (int i = 0; i < 2 * N; ++i) {
+        lo[i & 1] = std::min(lo[i & 1], coords[i]);
+        hi[i & 1] = std::max(hi[i & 1], coords[i]);
+    }
+    const long long dx = hi[0] - lo[0], dy = hi[1] - lo[1];
+    I->coords24 = dx * dx + dy * dy < (1ll << 24);
+    const bool half = dx * dx + dy * dy < EUC2D_HALF2_LIMIT;
+    const size_t c_words = (2 * N + 63) & ~static_cast<size_t>(63);
+    std::vector<int32_t> h(c_words + (half ? I->row_words : 0), 0);
+    std::copy(coords, coords + 2 * N, h.begin());
+    for (int i = 0; half && i < N; ++i) {
+        const __half2 v = __floats2half2_rn(static_cast<float>(coords[2 * i] - lo[0]),
+                                            static_cast<float>(coords[2 * i + 1] - lo[1]));
+        std::memcpy(&h[c_words + i], &v, 4);
+    }
     int* dmax = nullptr;
-    cudaError_t e = cudaMalloc(&I->coords, pad16(2 * N * sizeof(int32_t)));
+    cudaError_t e = cudaMalloc(&I->coords, h.size() * sizeof(int32_t));
+    if (e == cudaSuccess && half) I->xy = reinterpret_cast<uint32_t*>(I->coords) + c_words;
     if (e == cudaSuccess) e = cudaMalloc(&I->d32, pad16(NN * sizeof(int32_t)));
     if (e == cudaSuccess) e = cudaMalloc(&dmax, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemcpy(I->coords, coords, 2 * N * sizeof(int32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(I->coords, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(dmax, 0, sizeof(int));
     if (e == cudaSuccess) {
         int blocks = static_cast<int>((NN + 255) / 256);

@@ -74,6 +74,10 @@ struct vrprpd_instance {
     uint16_t* d16 = nullptr;     // (n+1)^2 when maxd < 65536
     int32_t* coords = nullptr;   // (n+1) x 2
     int32_t* p = nullptr;        // n+1, p[0] = 0, p[c] = processing time of c
+    int row_words = 0;           // words of an evaluator's ready row: n + 2 rounded up to 4
+    int32_t* rowt = nullptr;     // its template (eval.cu), in p's allocation
+    uint32_t* xy = nullptr;      // points as fp16 pairs, in coords' allocation; null when too far apart
+    bool coords24 = false;       // coordinates with every squared leg below 2^24
     int* err = nullptr;          // device error word
     // host copies
     std::vector<int32_t> h_d, h_p, h_coords;
@@ -84,5 +88,4 @@ struct vrprpd_instance {
     int32_t* stage = nullptr;
     size_t stage_bytes = 0;
     vrp::EvalTuning tune;
-    vrp::EvalTuning tune_staged;   // the best staged-walk shape the autotuner saw (host-mapped candidates)
 };
