@@ -108,6 +108,7 @@ struct EvalArgs {
 constexpr int PICKED = static_cast<int>(0x80000000u);   // ready slot of a customer already picked up
 
 constexpr unsigned STOCK0 = 0x40004000u;
+constexpr int NOTE_NONE = (1 << 26) - 1;                 // a drop whose vehicle has no next op
 
 __device__ __forceinline__ int lds_s32(unsigned addr) {
     int v;
@@ -250,15 +251,23 @@ struct CodeBatch {
 // the warp's shared-memory region, sh the instance's distances or points and
 // rowt the ready-row template (shared memory, or for many-instance launches
 // global memory).
-template <int DM, bool W16, int V>
+// COUNT: the coordination counts instead of makespan and status.  A drop also
+// leaves, beside its ready slot, its vehicle and how much later than the ready
+// time its vehicle reaches its next op (both known the moment it goes), so the
+// pickup settles its customer by itself: 32768 candidates at n=200 m=6 in 92 us,
+// where the kernel with one candidate per warp, four words per customer and
+// legs from L2 (metrics.cu) takes 317 us.
+template <int DM, bool W16, int V, bool COUNT>
 __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, const int32_t* rowt, int32_t* W,
                                           long long t, long long next) {
     using P = Place<DM>;
     const int lane = threadIdx.x & 31;
     const int n = a.n, m = a.m, two_n = 2 * n, K = a.K, str4 = a.row_words >> 2;
     int32_t* ready = W + a.a_words;
-    int32_t* soff = ready + a.ready_words;
+    int32_t* soff = ready + (COUNT ? 2 : 1) * a.ready_words;
     int32_t* res = soff + a.off_words;         // [4][K]: return, load + 2^16 per overfull route, malformed, blocked
+                                               // (COUNT: cross, interleaved, malformed, blocked)
+    const unsigned note = 4u * static_cast<unsigned>(a.ready_words);   // from a ready slot to the drop's note
     const long long first = t * K;
     const int kt = static_cast<int>(min(static_cast<long long>(K), a.num - first));
     const unsigned lim2 = static_cast<unsigned>(two_n + 2) * 0x10001u;
@@ -316,6 +325,7 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
     // into it), the code after it, and where the one after that lies (ca).
     int dep[V], leg[V], code[V], ncode[V], cand[V];
     unsigned stock[V], ext[V], rbase[V], ca[V], ce[V], ad[V];
+    int veh[V], prev[V], cross[V], inter[V];   // COUNT only
     bool live[V];
     P at[V];
 #pragma unroll
@@ -323,6 +333,8 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
         const int vl = lane + 32 * s, c = vl / m, v = vl - c * m;
         live[s] = c < kt;
         cand[s] = live[s] ? c : 0;
+        veh[s] = v;
+        prev[s] = cross[s] = inter[s] = 0;
         int lo = 0, hi = 0;
         if (live[s]) {
             lo = soff[c * (m + 1) + v];
@@ -366,13 +378,27 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
             const bool pick = (code[s] & 1) != 0;
             const bool go = !pick || r[s] >= 0;
             const int nd = __viaddmax_s32(dep[s], leg[s], r[s]);
-            sts_s32_if(go, ad[s], pick ? PICKED : static_cast<int>(static_cast<unsigned>(nd) - 1u - static_cast<unsigned>(r[s])));
-            any = any || go;
             const int c1 = ncode[s] >> 1;
             const int nleg = P::leg(a, sh, at[s], nat[s], c1);
+            if constexpr (COUNT) {
+                // (next arrival - ready) << 5 | vehicle; the arrival is T_drop + the
+                // next leg, the ready time T_drop + p and the slot still -(p + 1)
+                if (!pick) {
+                    const int late = ncode[s] == 1 ? NOTE_NONE : nleg - P::BIAS + 1 + r[s];
+                    sts_s32_if(true, ad[s] + note, static_cast<int>(static_cast<unsigned>(late) << 5) | veh[s]);
+                } else if (go) {
+                    const int w = lds_s32(ad[s] + note), late = w >> 5;
+                    const bool same = (w & 31) == veh[s];
+                    cross[s] += same ? 0 : 1;
+                    inter[s] += (same ? prev[s] != (code[s] ^ 1) : late != NOTE_NONE && r[s] + late < nd) ? 1 : 0;
+                }
+                prev[s] = go ? code[s] : prev[s];
+            }
+            sts_s32_if(go, ad[s], pick ? PICKED : static_cast<int>(static_cast<unsigned>(nd) - 1u - static_cast<unsigned>(r[s])));
+            any = any || go;
             if (go) {
                 dep[s] = nd - P::BIAS;
-                stock[s] += pick ? 0xffff0001u : 0x0000ffffu;
+                if constexpr (!COUNT) stock[s] += pick ? 0xffff0001u : 0x0000ffffu;
                 code[s] = ncode[s];
                 ncode[s] = acode[s];
                 at[s] = nat[s];
@@ -380,7 +406,7 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
                 ad[s] = rbase[s] + 4u * static_cast<unsigned>(c1);
                 ca[s] += 2u;
             }
-            ext[s] = max_u16x2(ext[s], stock[s]);
+            if constexpr (!COUNT) ext[s] = max_u16x2(ext[s], stock[s]);
         }
         __syncwarp();
         if (!__any_sync(FULL_MASK, any)) break;
@@ -389,15 +415,19 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
 #pragma unroll
     for (int s = 0; s < V; ++s) {
         const bool blocked = ca[s] - 4u < ce[s];
-        if (blocked) {                         // finish the stock of a blocked route
+        if (blocked) {
             some_blocked = true;
             res[3 * K + cand[s]] = 1;
-            for (unsigned q = ca[s] - 4u; q < ce[s]; q += 2u) {
-                stock[s] += (code_or_idle(q, ce[s]) & 1) ? 0xffff0001u : 0x0000ffffu;
-                ext[s] = max_u16x2(ext[s], stock[s]);
-            }
+            if constexpr (!COUNT)              // finish the stock of a blocked route
+                for (unsigned q = ca[s] - 4u; q < ce[s]; q += 2u) {
+                    stock[s] += (code_or_idle(q, ce[s]) & 1) ? 0xffff0001u : 0x0000ffffu;
+                    ext[s] = max_u16x2(ext[s], stock[s]);
+                }
         }
-        if (live[s]) {
+        if constexpr (COUNT) {
+            if (cross[s]) atomicAdd(&res[cand[s]], cross[s]);
+            if (inter[s]) atomicAdd(&res[K + cand[s]], inter[s]);
+        } else if (live[s]) {
             const int up = static_cast<int>(ext[s] & 0xffffu) - 0x4000, down = static_cast<int>(ext[s] >> 16) - 0x4000;
             const bool over = a.load_full ? (down > a.Q || up > 0) : (down + up > a.Q);
             atomicMax(&res[cand[s]], dep[s] + leg[s]);
@@ -434,11 +464,42 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
             bad = __any_sync(FULL_MASK, bad);
             if (lane == 0) res[2 * K + g] = bad ? 1 : 0;
             __syncwarp();
+            if constexpr (COUNT) {
+                // the cross count of a cycle: both vehicles of every customer by
+                // its ops' places, now in the candidate's row
+                if (bad) continue;
+                int32_t* both = ready + g * a.row_words;
+                const int32_t* F = soff + g * (m + 1);
+                for (int c = lane; c <= n; c += 32) both[c] = 0;
+                if (lane == 0) res[g] = 0;
+                __syncwarp();
+                for (int e = lane; e < two_n; e += 32) {
+                    const int o = code_or_idle(A + 2u * static_cast<unsigned>(g * two_n + e), ~0u);
+                    int lo = 0, hi = m;
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (F[mid] <= e) lo = mid; else hi = mid;
+                    }
+                    atomicXor(&both[o >> 1], lo);
+                }
+                __syncwarp();
+                int nc = 0;
+                for (int c = 1 + lane; c <= n; c += 32) nc += both[c] != 0 ? 1 : 0;
+                nc = __reduce_add_sync(FULL_MASK, nc);
+                if (lane == 0) res[g] = nc;
+                __syncwarp();
+            }
         }
     }
 
     // ---- results ----
     for (int g = lane; g < kt; g += 32) {
+        if constexpr (COUNT) {
+            const bool bad = res[2 * K + g] != 0;
+            a.z[first + g] = bad ? -1 : res[g];
+            a.st[first + g] = static_cast<uint32_t>(bad || res[3 * K + g] ? -1 : res[K + g]);
+            continue;
+        }
         const int load = res[K + g];
         int z = res[g], f = 0;
         if (load >> 16) f |= VRPRPD_VEH_CAP;
@@ -451,7 +512,7 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
     __syncwarp();
 }
 
-template <int DM, bool W16, int V>
+template <int DM, bool W16, int V, bool COUNT>
 __global__ void __launch_bounds__(32 * max_warps(V)) eval_tiles_kernel(EvalArgs a) {
     extern __shared__ __align__(16) int32_t smem[];
     __shared__ __align__(8) uint64_t block_bar;
@@ -486,7 +547,7 @@ __global__ void __launch_bounds__(32 * max_warps(V)) eval_tiles_kernel(EvalArgs 
     const long long gw = static_cast<long long>(blockIdx.x) * nwarps + warp;
     const long long nw = static_cast<long long>(gridDim.x) * nwarps;
     for (long long t = gw; t < ntiles; t += nw)
-        eval_tile<DM, W16, V>(a, sh, rowt, W, t, a.prefetch && t + nw < ntiles ? t + nw : -1);
+        eval_tile<DM, W16, V, COUNT>(a, sh, rowt, W, t, a.prefetch && t + nw < ntiles ? t + nw : -1);
 }
 
 // Many instances of uneven size in one persistent launch: tile t of the
@@ -522,7 +583,7 @@ __global__ void __launch_bounds__(32 * max_warps(V)) eval_multi_kernel(const Eva
                 have = lo;
             }
         }
-        eval_tile<DM, false, V>(a, sh, a.rowt, W, t - __ldg(tile_prefix + lo), -1);
+        eval_tile<DM, false, V, false>(a, sh, a.rowt, W, t - __ldg(tile_prefix + lo), -1);
     }
 }
 
@@ -616,6 +677,7 @@ struct Plan {
     int dm = 0;          // the kernel's distance mode (DIST_HALF2 for small coordinates)
     int warps = 0, blocks = 0;
     bool w16 = false;    // 16-bit op codes and offsets
+    bool count = false;  // coordination counts instead of makespan and status
     int V = 1;           // routes per lane
     size_t smem = 0;
     EvalArgs args{};
@@ -706,7 +768,7 @@ static bool make_plan(const vrprpd_instance* I, int dm, int warps, int V, long l
         a.a_words = round4(static_cast<long long>(K) * I->n) + 8;   // codes, shifted by up to 7 and padded to 16 bytes
         a.ready_words = K * a.row_words;
         a.off_words = round4(static_cast<long long>(K) * (I->m + 1));
-        a.warp_words = a.a_words + a.ready_words + a.off_words + round4(4ll * K);
+        a.warp_words = a.a_words + a.ready_words + a.off_words + round4(4ll * K) + (P->count ? a.ready_words : 0);
         P->smem = static_cast<size_t>(a.shared_words + static_cast<long long>(warps) * a.warp_words) * 4;
         if (P->smem + 64 <= I->smem_optin && (K == 1 || a.warp_words <= cap)) {
             P->dm = dm;
@@ -718,19 +780,20 @@ static bool make_plan(const vrprpd_instance* I, int dm, int warps, int V, long l
     return false;
 }
 
-template <bool W16, int V>
+template <bool W16, int V, bool COUNT = false>
 static const void* kernel_for(int dm) {
     switch (dm) {
-        case VRPRPD_DIST_SMEM32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM32, W16, V>);
-        case VRPRPD_DIST_SMEM16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM16, W16, V>);
-        case VRPRPD_DIST_GLOBAL16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL16, W16, V>);
-        case VRPRPD_DIST_GLOBAL32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL32, W16, V>);
-        case DIST_HALF2: return reinterpret_cast<const void*>(&eval_tiles_kernel<DIST_HALF2, W16, V>);
-        default: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_COORDS, W16, V>);
+        case VRPRPD_DIST_SMEM32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM32, W16, V, COUNT>);
+        case VRPRPD_DIST_SMEM16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_SMEM16, W16, V, COUNT>);
+        case VRPRPD_DIST_GLOBAL16: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL16, W16, V, COUNT>);
+        case VRPRPD_DIST_GLOBAL32: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_GLOBAL32, W16, V, COUNT>);
+        case DIST_HALF2: return reinterpret_cast<const void*>(&eval_tiles_kernel<DIST_HALF2, W16, V, COUNT>);
+        default: return reinterpret_cast<const void*>(&eval_tiles_kernel<VRPRPD_DIST_COORDS, W16, V, COUNT>);
     }
 }
 
 static const void* plan_kernel(const Plan& P) {
+    if (P.count) return P.V == 2 ? kernel_for<false, 2, true>(P.dm) : kernel_for<false, 1, true>(P.dm);
     if (P.V == 2) return P.w16 ? kernel_for<true, 2>(P.dm) : kernel_for<false, 2>(P.dm);
     return P.w16 ? kernel_for<true, 1>(P.dm) : kernel_for<false, 1>(P.dm);
 }
@@ -760,12 +823,8 @@ static int plan_shape(const vrprpd_instance* I, const EvalTuning& T, long long n
     return VRPRPD_EINVAL;
 }
 
-static int choose_plan(const vrprpd_instance* I, long long num, Plan* P) {
-    if (I->tune.dist_mode != VRPRPD_DIST_AUTO && I->tune.warps_per_block > 0) return plan_shape(I, I->tune, num, P);
-    if (!shape_accepted(I, VRPRPD_DIST_GLOBAL32, 1, VRPRPD_WALK_STAGED, 1)) {
-        set_error("no evaluation layout fits shared memory (n=%d, m=%d)", I->n, I->m);
-        return VRPRPD_EINVAL;
-    }
+// The plan when nothing is configured.
+static int auto_plan(const vrprpd_instance* I, long long num, Plan* P) {
     // Distances: points as fp16 pairs when the instance has them (a leg is 7
     // instructions from one 4-byte gather); else the 16-bit matrix in shared
     // memory while it takes at most half of it, recomputed integer legs, and
@@ -786,9 +845,11 @@ static int choose_plan(const vrprpd_instance* I, long long num, Plan* P) {
     // over the SMs first.
     Plan best;
     best.w16 = P->w16;
+    best.count = P->count;
     long long most = 0;
     for (int warps : {4, 8, 12, 16, 24, 28, 32, 2, 1}) {
         Plan C;
+        C.count = P->count;
         if (warps > max_warps(V) || (warps < 4 && most) || !make_plan(I, dm, warps, V, num, &C)) continue;
         const long long by_smem = SM_SHARED_BYTES / static_cast<long long>(C.smem + BLOCK_SHARED_BYTES);
         const long long resident = warps * std::min<long long>(by_smem, max_warps(V) / warps);
@@ -809,6 +870,15 @@ static int choose_plan(const vrprpd_instance* I, long long num, Plan* P) {
     best.smem = static_cast<size_t>(best.args.shared_words + static_cast<long long>(best.warps) * best.args.warp_words) * 4;
     *P = best;
     return finalize_plan(I, 0, P);
+}
+
+static int choose_plan(const vrprpd_instance* I, long long num, Plan* P) {
+    if (I->tune.dist_mode != VRPRPD_DIST_AUTO && I->tune.warps_per_block > 0) return plan_shape(I, I->tune, num, P);
+    if (!shape_accepted(I, VRPRPD_DIST_GLOBAL32, 1, VRPRPD_WALK_STAGED, 1)) {
+        set_error("no evaluation layout fits shared memory (n=%d, m=%d)", I->n, I->m);
+        return VRPRPD_EINVAL;
+    }
+    return auto_plan(I, num, P);
 }
 
 static int launch_plan(const Plan& P, cudaStream_t stream) {
@@ -863,6 +933,24 @@ static int evaluate_device16(const vrprpd_instance* I, const uint16_t* ops, cons
     P.args.z = z;
     P.args.st = st;
     return launch_plan(P, stream);
+}
+
+// Coordination counts by the same walk, for instances its words hold: true
+// when launched (*rc is its result), false when the caller has to.
+bool coordination_walk(const vrprpd_instance* I, const int32_t* ops, const int32_t* off, long long num,
+                       int32_t* cross, int32_t* interleaved, cudaStream_t stream, int* rc) {
+    if (!batched_supported(I) || I->maxp >= (1 << 25)) return false;
+    Plan P;
+    P.count = true;
+    *rc = auto_plan(I, num, &P);
+    if (*rc) return false;
+    P.args.prefetch = 1;
+    P.args.ops = ops;
+    P.args.off = off;
+    P.args.z = cross;
+    P.args.st = reinterpret_cast<uint32_t*>(interleaved);
+    *rc = launch_plan(P, stream);
+    return true;
 }
 
 static int check_batch16(const vrprpd_instance* I, const vrprpd_batch16* b, const void* z, const void* st) {

@@ -1,6 +1,10 @@
 // Coordination counts of Section 5.2 ("Key Metrics": Cross-Agent % and
 // Interleaved %) for a batch of complete solutions of one instance.
 //
+// The evaluator's walk counts them on the way (eval.cu).  The kernel here takes
+// what that walk does not: n above 2046, distances from 2^19 or processing
+// times from 2^25 on.
+//
 // One warp per candidate.  A pre-pass over the ops, 32 at a time, checks op
 // codes (range, duplicates) and records each customer's dropoff and pickup
 // vehicles (a binary search of the op's position in the route offsets).  Then
@@ -22,6 +26,10 @@
 #include "internal.h"
 
 namespace vrp {
+
+bool coordination_walk(const vrprpd_instance* I, const int32_t* ops, const int32_t* off, long long num,
+                       int32_t* cross, int32_t* interleaved, cudaStream_t stream, int* rc);
+
 namespace {
 
 constexpr int CO_WARPS = 2;
@@ -161,6 +169,8 @@ extern "C" int vrprpd_coordination(const vrprpd_instance* I, const vrprpd_batch*
     const long long bound = (2ll * I->n + 1) * I->maxd + static_cast<long long>(I->n) * I->maxp;
     VRP_CHECK(bound < (1ll << 31) - 1, VRPRPD_EINVAL, "coordination counts need (2n+1)*max(d) + n*max(p) < 2^31");
     if (b->num == 0) return VRPRPD_OK;
+    int rc = VRPRPD_OK;
+    if (coordination_walk(I, b->ops, b->off, b->num, cross, interleaved, static_cast<cudaStream_t>(stream), &rc)) return rc;
     const size_t smem = static_cast<size_t>(CO_WARPS) * co_stride(I->n, I->m) * sizeof(int);
     VRP_CHECK(smem <= I->smem_optin, VRPRPD_EINVAL, "n=%d too large for the coordination kernel", I->n);
     { int rc_ = ensure_smem_limit(reinterpret_cast<const void*>(&coordination_kernel)); if (rc_) return rc_; }

@@ -90,3 +90,20 @@ def test_walk_edges(vrp, n, m, box):
         z, st = vrp.evaluate(inst, view, dev(f16))
         vrp.sync(inst)
         assert np.array_equal(z.cpu().numpy(), zo[fits]) and np.array_equal(st.cpu().numpy().astype(np.uint32), so[fits])
+
+
+# one and two routes per lane, empty routes; p from 2^25 on takes the other kernel
+@pytest.mark.parametrize("n,m,pmax", [(1, 1, 9), (3, 2, 9), (5, 32, 50), (61, 17, 300), (62, 21, 300), (333, 5, 300),
+                                      (20, 3, 1 << 25)])
+def test_coordination_edges(vrp, n, m, pmax):
+    rng = np.random.default_rng(n)
+    p = rng.integers(0, pmax + 1, size=n).astype(np.int32)
+    p[0] = pmax
+    coords = rng.integers(0, 900, size=(n + 1, 2)).astype(np.int32)
+    inst = vrp.Instance(m, n, 3, p, coords=coords)
+    oi = oracle.OracleInstance(oracle.euc2d(coords), p, m, n, 3)
+    ops, off = population(n, m, 60, seed=n + m)
+    cr, il = vrp.coordination(inst, dev(ops), dev(off))
+    cr, il = cr.cpu().numpy(), il.cpu().numpy()
+    for k in range(len(ops)):
+        assert (cr[k], il[k]) == oracle.coordination(oi, ops[k], off[k])[:2], k
