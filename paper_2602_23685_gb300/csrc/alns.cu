@@ -90,14 +90,9 @@ struct AlnsCtl {
     int upd[16];
     unsigned long long steps_incr, steps_full;
     unsigned long long phase_ns[7];   // begin, prep, gaps, matrix, select, end, local search (rank 0 wall time)
-    // periodic local search: its mode while a candidate's matrix runs (0
-    // otherwise), the pass's candidates, the best move so far (customer,
-    // makespan, travel, flat gap index, drop route/position, pickup
-    // route/position in the solution without the customer)
-    int ls, ls_ncand, ls_moved, ls_have, ls_bott, ls_rt;
-    int ls_c, ls_bz, ls_a, ls_ia, ls_b, ls_jb;
-    int ls_moves, ls_new_best;
-    long long ls_travel, ls_bt, ls_bflat;
+    // periodic local search: the pass's candidates, the bottleneck vehicle,
+    // whether the last pass moved, moves applied and new bests so far
+    int ls_ncand, ls_bott, ls_moved, ls_moves, ls_new_best;
     int imports;                      // best-of-all solutions this replica took at checkpoints
     // Words that the whole team hits with atomics or polls, each group on a
     // cache line of its own: the CTA that selects an insertion while the
@@ -161,9 +156,8 @@ struct AlnsTeam {
     int scw_stride;
     int* scpair;               // [SC_CAP][SC_CAP]: makespan with both stops in two shortcut gaps of one customer
     int* trace;
-    int* gains;                // [n+1]: removal gain z(cur) - z(cur - c), worst removal
+    int* gains;                // [n+1]: removal gain z(cur) - z(cur - c), worst removal; local search: places of the ops
     int* lscand;               // [n+1]: local-search candidates of the current pass
-    int4* lsmask;              // [slots]: allowed drop routes, pickup routes, fixed drop gap (-1 any)
     int* dump_delta;
     int* dump_travel;
 };
@@ -1142,7 +1136,7 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
     // into the keys before any tile runs.
     {
         AlnsCtl* ctl = t.ctl;
-        const int nrem = ctl->nrem, z = ctl->z_work, lsm = ctl->ls;
+        const int nrem = ctl->nrem, z = ctl->z_work;
         const int Gp = (G + 31) & ~31;
         const long long total = static_cast<long long>(nrem) * Gp;
         const int sumL = ctl->sum_load;
@@ -1170,20 +1164,12 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
                 const int dxc = Dx(t, s, x, c), dcy = Dx(t, s, c, y), dcc = Dx(t, s, c, c);
                 const int delta = dxc + dcy;
                 const bool shortcut = delta < w;
-                // a local-search slot allows some drop gaps (rows) and pickup gaps
-                // (columns) only; the others read as excluded
-                bool rok = true, cok = true;
-                if (lsm) {
-                    const int4 mk = t.lsmask[ti];
-                    rok = ((static_cast<unsigned>(mk.x) >> r) & 1u) != 0 && (mk.z < 0 || mk.z == g);
-                    cok = ((static_cast<unsigned>(mk.y) >> r) & 1u) != 0;
-                }
-                vr = make_int4(shortcut || !rok ? SKIPV : max(z, Hx + delta + Ty), Hx + dxc + pc, Hx + delta,
+                vr = make_int4(shortcut ? SKIPV : max(z, Hx + delta + Ty), Hx + dxc + pc, Hx + delta,
                                static_cast<int>(static_cast<unsigned>(delta - w + (1 << 19)) << 12));
-                const int2 va = make_int2(shortcut || !(rok && cok) ? SKIPV : max(z, Hx + dxc + max(dcc, pc) + dcy + Ty),
+                const int2 va = make_int2(shortcut ? SKIPV : max(z, Hx + dxc + max(dcc, pc) + dcy + Ty),
                                           static_cast<int>((static_cast<unsigned>(dxc + dcc + dcy - w + (1 << 19)) << 12) |
                                                            static_cast<unsigned>(g)));
-                vc = make_int4(shortcut || !cok ? SKIPV : Hx + Ty + delta, dcy + Ty, delta + Ty,
+                vc = make_int4(shortcut ? SKIPV : Hx + Ty + delta, dcy + Ty, delta + Ty,
                                static_cast<int>((static_cast<unsigned>(delta - w) << 12) + static_cast<unsigned>(g)));
                 t.vrow[e] = vr;
                 t.vadj[e] = va;
@@ -1389,7 +1375,7 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
     int4 bnd_r = make_int4(0, 0, 0, 0), bnd_c0 = bnd_r, bnd_c1 = make_int4(0, 0, 0x7fffffff, -1);
     unsigned long long gm[4] = {KEY_NONE, KEY_NONE, KEY_NONE, KEY_NONE};
     const bool mine = prune_on && tid < nrem;
-    const int kind = ctl->ls ? 0 : ctl->rj;
+    const int kind = ctl->rj;
     // drop vehicles of the tile's rows: the routes of gaps r0 and min(G, r0 + TR) - 1
     auto route_of_gap = [&](int g) {
         int lo = 0, hi = t.m;
@@ -1738,17 +1724,9 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
     const bool dump = t.mode == 1;
     unsigned cnt = 0;
     auto loc = [&](int pos) { return pos >= 0 ? (s.sW[pos] & PACK_MASK) >> 1 : 0; };
-    // a local-search slot's mask (see the gap phase)
-    const int lsm = ctl->ls;
-    const int4 mk = lsm ? t.lsmask[ti] : make_int4(-1, -1, -1, 0);
-    auto allowed = [&](int row, int col) {
-        return ((static_cast<unsigned>(mk.x) >> t.groute[row]) & 1u) != 0 && (mk.z < 0 || mk.z == row) &&
-               ((static_cast<unsigned>(mk.y) >> t.groute[col]) & 1u) != 0;
-    };
     for (int k = piece * blockDim.x + tid; k < G && z1 != 0x7fffffff; k += FB_SPLIT * blockDim.x) {
         if (k == g || t.sc[scrow + k]) continue;              // both gaps shortcuts: below / elsewhere
         const int row = as_col ? k : g, col = as_col ? g : k;
-        if (lsm && !allowed(row, col)) continue;
         const int a = t.groute[row], i = t.gpos[row], b = t.groute[col], j = t.gpos[col];
         const long long idx = static_cast<long long>(row) * G + col;
         if (a == b && j < i) {
@@ -1792,7 +1770,6 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
             while (todo) {
                 const int col = k0 + __ffs(todo) - 1;
                 todo &= todo - 1;
-                if (lsm && !allowed(g, col)) continue;
                 const int a = ga, i = gi, b = t.groute[col], j = t.gpos[col];
                 const long long idx = static_cast<long long>(g) * G + col;
                 if (a == b && j < i) {
@@ -1837,18 +1814,6 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s) {
     const int nwalks = gap_walk_items(t);
     bool walks_seen = false;
     int* slot = s.misc;
-    // local search: tiles that hold no allowed entry are skipped (pickup
-    // repositioning: one row of tiles; relocation: tiles whose rows and
-    // columns share no route)
-    const int lsm = ctl->ls, ls_rt = ctl->ls_rt;
-    auto ls_skip = [&](int rt, int ct) {
-        if (lsm == 1) return rt != ls_rt;
-        if (lsm == 2) {
-            const int r0 = rt * TR, r1 = min(G, r0 + TR) - 1, c0 = ct * TC, c1 = min(G, c0 + TC) - 1;
-            return t.groute[r1] < t.groute[c0] || t.groute[c1] < t.groute[r0];
-        }
-        return false;
-    };
     // Tiles go out by their distance d = |ct - rt/2| from the diagonal (the
     // column tile that holds the row band's own gaps): the entries near it
     // (drop and pickup on one route or on neighbouring ones) are where a
@@ -1878,7 +1843,7 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s) {
         if (item >= nfb) {
             int rt = 0, ct = 0;
             tile_of(item - nfb, &rt, &ct);
-            if (rt >= 0 && !ls_skip(rt, ct)) matrix_tile(t, s, rt, ct, N, G);
+            if (rt >= 0) matrix_tile(t, s, rt, ct, N, G);
         } else {
             if (!walks_seen) {
                 // the shortcut simulations, still running in other CTAs, must be done (bounded wait)
@@ -2634,26 +2599,67 @@ __device__ __noinline__ void replica_import(const AlnsTeam& t, const Smem& s) {
 // ---------------------------------------------------------------------------
 // periodic local search (Section 4.2.6), on the current solution
 // ---------------------------------------------------------------------------
-// Each candidate customer c runs one team step (prep, gaps, shortcut walks,
-// matrix) on W = cur - c with one or more masked slots for c: pickup
-// repositioning has one slot whose only drop gap is c's own dropoff place;
-// relocation has one slot per vehicle v other than the bottleneck, with both
-// gaps on v.  Taking c out can leave one of its old routes over capacity; the
-// matrix judges the receiving routes only, so a slot is kept only if every
-// such route is one it writes to.  The pass's best move is
-// the least (makespan, travel, customer, flat gap index) over all slots; it
-// is applied if it lowers the makespan.
+// A pass finds, over all its candidate customers c, the least (makespan,
+// travel, customer, gaps) among the moves that lower the makespan, and applies
+// it.  Pickup repositioning takes c's pickup out and puts it into any gap the
+// schedule allows; relocation takes both ops out and puts them into two gaps
+// (or one) of a vehicle other than the bottleneck.  Taking c out can leave one
+// of its old routes over capacity; only the receiving routes are judged, so a
+// move is kept only if every such route is one it writes to.
+//
+// Candidates are independent, so each is one CTA's work (relocation: split by
+// target vehicle while CTAs are idle) and the team meets once per pass.
+//   Pickup repositioning works on cur without the pickup alone: one walk gives
+// every departure H and the makespan z, one backward walk every tail T and
+// which ops lead to c's drop (a pickup before one of those is a cycle).  A gap
+// (x, y) that is no shortcut for c is then exact in O(1),
+//     z' = max(z, max(H(x) + d(x,c), H(drop) + p_c) + d(c,y) + T(y)),
+// since no path gets shorter; a shortcut gap is simulated.
+//   Relocation works on cur without c.  A gap costs H(x) + d(x,c) + d(c,y) + T(y)
+// whether it takes the drop or the pickup, so only gaps below the current
+// makespan (less the route's largest shortcut) can matter; each of those walks
+// W from its next op once, as far as the target route's end, and settles its
+// pairs on the way with the matrix formula.  Pairs with a shortcut gap are
+// simulated.
+// Before, every candidate was a team step of its own (the whole longest-path
+// table walked again, the matrix phase, five team barriers): 167 ms per local
+// search of both kinds at n=1000 m=20, 0.35 ms now; at n=120 m=5, eight
+// replicas, 40 ms of an 81 ms run, 1.0 ms now.
 enum { LS_PICKUP = 1, LS_RELOCATE = 2 };
 
-// Rank 0: the candidates of one pass, in ascending id.  Pickup repositioning:
-// customers whose pickup is on a vehicle returning at 95% of the makespan or
-// later (20 ret >= 19 z); relocation: customers with an op on the bottleneck
-// vehicle (latest return, lower index on ties).
+constexpr int TAIL_BITS = (1 << 29) - 1;       // a tail; the bit above: the op leads to the candidate's drop
+constexpr int TAIL_NONE = INT32_MIN + 1;       // tail of a pickup that is not in the solution
+constexpr int LS_MAX_CTAS = SC_CAP * SC_CAP / 4;
+
+// Scratch of one CTA, in words: H, T, stock after each op, packed prefix and
+// suffix extremes (N each), then one word per gap of a route and a list of its gaps.
+__device__ __forceinline__ int ls_scratch_words(int n) { return 14 * n + 8; }
+// The CTAs that take part: the scratch lies in the buffers of the shortcut
+// simulations and of the longest-path table, which the next step rebuilds.
+__device__ __forceinline__ int ls_active(const AlnsTeam& t, int team_blocks) {
+    const int N = 2 * t.n, w = ls_scratch_words(t.n);
+    const int a0 = SC_CAP * (4 * N + 8) / w, a1 = N * N / w;
+    return min(team_blocks, min(a0 + 2 * a1, LS_MAX_CTAS));
+}
+__device__ __forceinline__ int* ls_scratch(const AlnsTeam& t, int rank) {
+    const int N = 2 * t.n, w = ls_scratch_words(t.n);
+    const int a0 = SC_CAP * (4 * N + 8) / w, a1 = N * N / w;
+    if (rank < a0) return t.scw + static_cast<long long>(rank) * w;
+    rank -= a0;
+    return rank < a1 ? t.Ms + static_cast<long long>(rank) * w : t.Ms2 + static_cast<long long>(rank - a1) * w;
+}
+
+// Rank 0: the candidates of one pass, in ascending id, and where every op of
+// the current solution stands.  Pickup repositioning: customers whose pickup is
+// on a vehicle returning at 95% of the makespan or later (20 ret >= 19 z);
+// relocation: customers with an op on the bottleneck vehicle (latest return,
+// lower index on ties).
 __device__ __noinline__ void ls_candidates(const AlnsTeam& t, const Smem& s, int mode) {
     AlnsCtl* ctl = t.ctl;
     const int n = t.n, m = t.m, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     stage_ops(t, s, t.cur_ops, t.cur_off);
     int* ret = s.misc + 32;                    // [32] return time per route
+    uint16_t* place = reinterpret_cast<uint16_t*>(t.gains);   // [2n+2] by op code
     for (int c = tid; c <= n; c += blockDim.x) s.flags[c] = 0;
     if (warp == 0) {
         int z;
@@ -2672,7 +2678,6 @@ __device__ __noinline__ void ls_candidates(const AlnsTeam& t, const Smem& s, int
             for (int v = 1; v < m; ++v)
                 if (ret[v] > ret[b]) b = v;
             ctl->ls_bott = b;
-            ctl->ls_have = 0;
         }
     }
     __syncthreads();
@@ -2685,6 +2690,7 @@ __device__ __noinline__ void ls_candidates(const AlnsTeam& t, const Smem& s, int
             if (s.sWoff[mid] <= k) lo = mid; else hi = mid;
         }
         const int o = s.sW[k] & PACK_MASK;
+        place[o] = static_cast<uint16_t>(k);
         const bool cand = mode == LS_PICKUP ? ((o & 1) && 20ll * ret[lo] >= 19ll * z) : lo == bott;
         if (cand) s.flags[o >> 1] = 1;
     }
@@ -2703,165 +2709,523 @@ __device__ __noinline__ void ls_candidates(const AlnsTeam& t, const Smem& s, int
     __syncthreads();
 }
 
-// Rank 0: W = cur - c for candidate k, the routes of W over capacity, its
-// travel, and the slots with their masks.
-__device__ __noinline__ void ls_setup(const AlnsTeam& t, const Smem& s, int mode, int k) {
-    AlnsCtl* ctl = t.ctl;
-    const int n = t.n, m = t.m, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int c = t.lscand[k];
-    int* sh = s.misc + 32;                     // [0] drop position of c in cur, [1] bad-route mask
-    unsigned long long* travel = reinterpret_cast<unsigned long long*>(s.misc + 40);
-    for (int x = tid; x <= n; x += blockDim.x) s.flags[x] = x == c ? 1 : 0;
-    for (int q = tid; q < 2 * n; q += blockDim.x)
-        if (t.cur_ops[q] == 2 * c) sh[0] = q;
-    if (tid == 0) {
-        sh[1] = 0;
-        *travel = 0ull;
-        ctl->wsel = 0;
+// Stage cur without the ops at places lo < hi (hi < 0: lo alone): packed legs
+// and ops, route offsets.
+__device__ void stage_without(const AlnsTeam& t, const Smem& s, int lo, int hi) {
+    const int m = t.m, N = 2 * t.n - (hi >= 0 ? 2 : 1);
+    for (int v = threadIdx.x; v <= m; v += blockDim.x) {
+        const int o = t.cur_off[v];
+        s.sWoff[v] = o - (lo < o ? 1 : 0) - (hi >= 0 && hi < o ? 1 : 0);
+    }
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+        int q = k + (k >= lo ? 1 : 0);
+        if (hi >= 0 && q >= hi) ++q;
+        s.sW[k] = t.cur_ops[q];
     }
     __syncthreads();
-    const int pdrop = sh[0];
-    build_W_from_cur(t, s);
-    stage_W(t, s);
+    // a neighbour may already carry its leg: its op bits stay the same
+    volatile int* W = s.sW;
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+        int l = 0, h = m;
+        while (h - l > 1) {
+            const int mid = (l + h) >> 1;
+            if (s.sWoff[mid] <= k) l = mid; else h = mid;
+        }
+        const int o = W[k];
+        const int prev = k == s.sWoff[l] ? 0 : (W[k - 1] & PACK_MASK) >> 1;
+        W[k] = (Dx(t, s, prev, o >> 1) << PACK_SHIFT) | o;
+    }
     __syncthreads();
-    // per route: stock range of W (the minimal or the full start load) and travel
-    for (int r = warp; r < m; r += ALNS_WARPS) {
-        const int st = s.sWoff[r], en = s.sWoff[r + 1];
-        int carry = 0, mn = 0, mx = 0;
-        long long tr = 0;
-        for (int base = st; base < en; base += 32) {
-            const int q = base + lane;
-            const bool in = q < en;
-            const int w = in ? s.sW[q] : 0;
-            int v = in ? (((w & PACK_MASK) & 1) ? 1 : -1) : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(FULL_MASK, v, o);
-                if (lane >= o) v += y;
-            }
-            if (in) {
-                mn = min(mn, carry + v);
-                mx = max(mx, carry + v);
-                tr += w >> PACK_SHIFT;
-            }
-            carry += __shfl_sync(FULL_MASK, v, 31);
+}
+
+// One warp: departures of the staged (acyclic) solution into H; its makespan.
+__device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
+    const int lane = threadIdx.x & 31, n = t.n;
+    volatile int* rdy = rdy_;
+    for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
+    __syncwarp();
+    int pos = lane < t.m ? s.sWoff[lane] : 0;
+    const int start = pos, end = lane < t.m ? s.sWoff[lane + 1] : 0;
+    int dep = 0, last = 0, x = pos < end ? s.sW[pos] : 0;
+    for (;;) {
+        const bool on = pos < end;
+        const int c = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0;
+        const bool pick = (x & 1) != 0;
+        const int r = on && pick ? rdy[c] : 0;
+        const bool go = on && (!pick || r != UNRES);
+        if (go) {
+            dep += x >> PACK_SHIFT;
+            if (pick) dep = max(dep, r);
+            else rdy[c] = dep + s.sp[c];
+            H[pos] = dep;
+            last = c;
+            x = nx;
+            ++pos;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            mn = min(mn, __shfl_xor_sync(FULL_MASK, mn, o));
-            mx = max(mx, __shfl_xor_sync(FULL_MASK, mx, o));
-            tr += __shfl_xor_sync(FULL_MASK, tr, o);
+        __syncwarp();
+        if (!__any_sync(FULL_MASK, go)) break;
+    }
+    int ret = end > start ? dep + Dx(t, s, last, 0) : 0;
+    for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
+    return ret;
+}
+
+// One warp: the tail of every staged op (longest path from its departure to
+// the end of the schedule) into T, with the mark of the ops that lead to the
+// drop of c at dpos.  c > 0: c's pickup is not in the solution.
+__device__ void walk_tails(const AlnsTeam& t, const Smem& s, int* tp_, int* T, int c0, int dpos) {
+    const int lane = threadIdx.x & 31, n = t.n;
+    volatile int* tp = tp_;
+    for (int c = lane; c <= n; c += 32) tp[c] = c0 > 0 && c == c0 ? TAIL_NONE : UNRES;
+    __syncwarp();
+    const int start = lane < t.m ? s.sWoff[lane] : 0;
+    int pos = (lane < t.m ? s.sWoff[lane + 1] : 0) - 1;
+    int x = pos >= start ? s.sW[pos] : 0;
+    int leg = pos >= start ? Dx(t, s, (x & PACK_MASK) >> 1, 0) : 0, acc = 0, mark = 0;
+    for (;;) {
+        const bool on = pos >= start;
+        const int c = (x & PACK_MASK) >> 1, nx = pos - 1 >= start ? s.sW[pos - 1] : 0;
+        const bool drop = !(x & 1);
+        const int r = on && drop ? tp[c] : 0;
+        const bool go = on && (!drop || r != UNRES);
+        if (go) {
+            acc += leg;
+            if (drop && r != TAIL_NONE) {
+                acc = max(acc, s.sp[c] + (r & TAIL_BITS));
+                mark |= r & ~TAIL_BITS;
+            }
+            if (pos == dpos) mark = TAIL_BITS + 1;
+            T[pos] = acc | mark;
+            if (!drop) tp[c] = acc | mark;
+            leg = x >> PACK_SHIFT;
+            x = nx;
+            --pos;
         }
+        __syncwarp();
+        if (!__any_sync(FULL_MASK, go)) break;
+    }
+}
+
+// One warp, route r of the staged solution: stock after every op, its running
+// extremes (the start counts, at 0) and the extremes from every op on, packed
+// as shorts; the route's extremes, start load and length into the CTA's words.
+struct LsRoutes {
+    int mn[32], mx[32], load[32], len[32];
+};
+__device__ __forceinline__ int pack_range(int mn, int mx) { return (mn & 0xffff) | (mx << 16); }
+__device__ __forceinline__ int range_lo(int p) { return static_cast<int>(static_cast<short>(p & 0xffff)); }
+__device__ __forceinline__ int range_hi(int p) { return p >> 16; }
+
+__device__ void ls_scan_route(const AlnsTeam& t, const Smem& s, int r, int* S, int* PM, int* SM, LsRoutes* R) {
+    const int lane = threadIdx.x & 31, st = s.sWoff[r], en = s.sWoff[r + 1];
+    int carry = 0, cmin = 0, cmax = 0, len = 0;
+    for (int base = st; base < en; base += 32) {
+        const int k = base + lane;
+        const bool in = k < en;
+        const int x = in ? s.sW[k] : 0;
+        int v = in ? ((x & 1) ? 1 : -1) : 0;
+        len += x >> PACK_SHIFT;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL_MASK, v, o);
+            if (lane >= o) v += y;
+        }
+        const int sv = carry + v;
+        int mn = in ? sv : INT32_MAX, mx = in ? sv : INT32_MIN;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y1 = __shfl_up_sync(FULL_MASK, mn, o), y2 = __shfl_up_sync(FULL_MASK, mx, o);
+            if (lane >= o) { mn = min(mn, y1); mx = max(mx, y2); }
+        }
+        mn = min(mn, cmin);
+        mx = max(mx, cmax);
+        if (in) { S[k] = sv; PM[k] = pack_range(mn, mx); }
+        carry = __shfl_sync(FULL_MASK, sv, 31);
+        cmin = __shfl_sync(FULL_MASK, mn, 31);
+        cmax = __shfl_sync(FULL_MASK, mx, 31);
+    }
+    __syncwarp();
+    int smn = INT32_MAX, smx = INT32_MIN;
+    for (int top = en - 1; top >= st; top -= 32) {
+        const int k = top - lane;
+        const bool in = k >= st;
+        const int sv = in ? S[k] : 0;
+        int mn = in ? sv : INT32_MAX, mx = in ? sv : INT32_MIN;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y1 = __shfl_up_sync(FULL_MASK, mn, o), y2 = __shfl_up_sync(FULL_MASK, mx, o);
+            if (lane >= o) { mn = min(mn, y1); mx = max(mx, y2); }
+        }
+        mn = min(mn, smn);
+        mx = max(mx, smx);
+        if (in) SM[k] = pack_range(mn, mx);
+        smn = __shfl_sync(FULL_MASK, mn, 31);
+        smx = __shfl_sync(FULL_MASK, mx, 31);
+    }
+    len = __reduce_add_sync(FULL_MASK, len);
+    if (lane == 0) {
+        R->mn[r] = cmin;
+        R->mx[r] = cmax;
+        R->load[r] = t.load_full ? t.Q : -cmin;
+        R->len[r] = len + (en > st ? Dx(t, s, (s.sW[en - 1] & PACK_MASK) >> 1, 0) : 0);
+    }
+}
+
+// A move's key: makespan and travel, then customer, drop gap and pickup gap
+// (route and place in the solution without the customer; the order of gaps by
+// flat index).
+struct LsBest {
+    unsigned long long hi = KEY_NONE, lo = KEY_NONE;
+    __device__ __forceinline__ void take(int z, int tr, int c, int a, int ia, int b, int jb) {
+        const unsigned long long h = (static_cast<unsigned long long>(static_cast<unsigned>(z)) << 32) | static_cast<unsigned>(tr);
+        const unsigned long long l = (static_cast<unsigned long long>(c) << 34) |
+                                     (static_cast<unsigned long long>((a << 12) | ia) << 17) |
+                                     static_cast<unsigned long long>((b << 12) | jb);
+        least(h, l);
+    }
+    __device__ __forceinline__ void least(unsigned long long h, unsigned long long l) {
+        if (h < hi || (h == hi && l < lo)) { hi = h; lo = l; }
+    }
+};
+// The least of all threads' keys, in thread 0 (sh: 2 u64 per warp).
+__device__ void ls_block_least(LsBest& b, unsigned long long* sh) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long h = __shfl_xor_sync(FULL_MASK, b.hi, o), l = __shfl_xor_sync(FULL_MASK, b.lo, o);
+        b.least(h, l);
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        sh[2 * (threadIdx.x >> 5)] = b.hi;
+        sh[2 * (threadIdx.x >> 5) + 1] = b.lo;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < ALNS_WARPS; ++w) b.least(sh[2 * w], sh[2 * w + 1]);
+    __syncthreads();
+}
+
+// One candidate of pickup repositioning, the whole CTA.
+__device__ void ls_pickup_item(const AlnsTeam& t, const Smem& s, int* scr, LsRoutes* rt, int c, LsBest& best,
+                               unsigned& scored, unsigned& simulated) {
+    const int n = t.n, m = t.m, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N0 = 2 * n;
+    const int rw = ((n + 1) + 3) & ~3;
+    const uint16_t* place = reinterpret_cast<const uint16_t*>(t.gains);
+    const int pd = place[2 * c], pp = place[2 * c + 1], zcur = t.ctl->z_cur;
+    int *H = scr, *T = H + N0, *S = T + N0, *PM = S + N0, *SM = PM + N0, *list = SM + N0;   // (an empty route has no shortcut gap: at most 2N)
+    int* sh = s.misc + 32;                     // makespan, shortcut gaps
+    __syncthreads();                           // the previous item is done with the staged solution
+    stage_without(t, s, pp, -1);
+    const int N = N0 - 1, G = N + m, d1 = pd - (pp < pd ? 1 : 0);
+    if (tid == 0) sh[1] = 0;
+    if (warp == 0) {
+        const int z = walk_heads(t, s, s.rdy, H);
+        if (lane == 0) sh[0] = z;
+    } else if (warp == 1) {
+        walk_tails(t, s, s.rdy + rw, T, c, d1);
+    } else {
+        for (int r = warp - 2; r < m; r += ALNS_WARPS - 2) ls_scan_route(t, s, r, S, PM, SM, rt);
+    }
+    __syncthreads();
+    const int z1 = sh[0], hp = H[d1] + s.sp[c];
+    int a = 0, p = 0, sumL = 0, len = 0;
+    for (int v = 0; v < m; ++v) {
+        if (t.cur_off[v] <= pd) a = v;
+        if (t.cur_off[v] <= pp) p = v;
+        sumL += rt->load[v];
+        len += rt->len[v];
+    }
+    const int ia = pd - t.cur_off[a];
+    int tmp = 0;
+    const bool okA = cap_ok(t, rt->mn[a], rt->mx[a], tmp);
+    // the pickup's old route, left over capacity, has to take it back
+    const int only = p != a && !cap_ok(t, rt->mn[p], rt->mx[p], tmp) ? p : -1;
+    auto gap_of = [&](int g, int* pos) {
+        int lo = 0, hi = m;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (s.sWoff[mid] + mid <= g) lo = mid; else hi = mid;
+        }
+        *pos = g - (s.sWoff[lo] + lo);
+        return lo;
+    };
+    auto cust = [&](int k) { return (s.sW[k] & PACK_MASK) >> 1; };
+    for (int g = tid; g < G; g += ALNS_THREADS) {
+        int pos;
+        const int r = gap_of(g, &pos), off = s.sWoff[r], L = s.sWoff[r + 1] - off;
+        if ((only >= 0 && r != only) || (r == a && off + pos <= d1) || (r != a && !okA)) continue;
+        const int xo = pos > 0 ? off + pos - 1 : -1, yo = pos < L ? off + pos : -1;
+        const int Ty = yo >= 0 ? T[yo] : 0;
+        if (Ty > TAIL_BITS) continue;          // the pickup would come before an op that leads to its drop
+        const int pm = xo >= 0 ? PM[xo] : 0, sb = xo >= 0 ? S[xo] : 0;
+        int mn = range_lo(pm), mx = max(range_hi(pm), sb + 1);
+        if (yo >= 0) {
+            const int sm = SM[yo];
+            mn = min(mn, range_lo(sm) + 1);
+            mx = max(mx, range_hi(sm) + 1);
+        }
+        int lb = 0;
+        if (!cap_ok(t, mn, mx, lb) || sumL - rt->load[r] + lb > t.R) continue;
+        const int x = xo >= 0 ? cust(xo) : 0, y = yo >= 0 ? cust(yo) : 0;
+        const int dxc = Dx(t, s, x, c), dcy = Dx(t, s, c, y), w = L == 0 ? 0 : Dx(t, s, x, y);
+        if (dxc + dcy < w) {
+            list[atomicAdd(&sh[1], 1)] = g;
+            continue;
+        }
+        ++scored;
+        const int zn = max(z1, max((xo >= 0 ? H[xo] : 0) + dxc, hp) + dcy + Ty);
+        if (zn < zcur) best.take(zn, len + dxc + dcy - w, c, a, ia, r, pos - (r == a ? 1 : 0));
+    }
+    __syncthreads();
+    const int ns = sh[1];
+    int* rdy = s.rdy + warp * rw;
+    for (int k = warp; k < ns; k += ALNS_WARPS) {
+        int pos;
+        const int r = gap_of(list[k], &pos), off = s.sWoff[r], L = s.sWoff[r + 1] - off;
+        for (int q = lane; q <= n; q += 32) rdy[q] = UNRES;
+        __syncwarp();
+        const int zn = walk_fwd(t, s, rdy, r, pos, 2 * c + 1, -1, 0, 0, nullptr, nullptr);
+        const int x = pos > 0 ? cust(off + pos - 1) : 0, y = pos < L ? cust(off + pos) : 0;
         if (lane == 0) {
-            int load = 0;
-            if (!cap_ok(t, mn, mx, load)) atomicOr(&sh[1], 1 << r);
-            if (en > st) tr += Dx(t, s, (s.sW[en - 1] & PACK_MASK) >> 1, 0);
-            atomicAdd(travel, static_cast<unsigned long long>(tr));
+            ++simulated;
+            if (zn < zcur)
+                best.take(zn, len + Dx(t, s, x, c) + Dx(t, s, c, y) - Dx(t, s, x, y), c, a, ia, r, pos - (r == a ? 1 : 0));
         }
     }
-    __syncthreads();
-    if (tid == 0) {
-        const unsigned bad = static_cast<unsigned>(sh[1]);
-        const unsigned all = m == 32 ? 0xffffffffu : (1u << m) - 1u;
-        int ns = 0;
-        if (mode == LS_PICKUP) {
-            int a = 0;
-            for (int v = 0; v < m; ++v)
-                if (t.cur_off[v] <= pdrop) a = v;
-            const int ia = pdrop - t.cur_off[a];
-            const int g1 = s.sWoff[a] + a + ia;
-            const unsigned rest = bad & ~(1u << a);
-            if (__popc(rest) <= 1) {
-                t.lsmask[0] = make_int4(static_cast<int>(1u << a), static_cast<int>(rest ? rest : all), g1, 0);
-                t.rem[0] = c;
-                ns = 1;
-            }
-            ctl->ls_rt = g1 / TR;
-        } else {
-            for (int v = 0; v < m; ++v) {
-                if (v == ctl->ls_bott || (bad & ~(1u << v)) != 0u) continue;
-                t.lsmask[ns] = make_int4(static_cast<int>(1u << v), static_cast<int>(1u << v), -1, 0);
-                t.rem[ns] = c;
-                ++ns;
-            }
-            ctl->ls_rt = -1;
-        }
-        ctl->nrem = ns;
-        ctl->ls = mode;
-        ctl->ls_travel = static_cast<long long>(*travel);
-        ctl->repair_fail = 0;
-        ctl->n_short = 0;
-        ctl->work_counter = 0;
-        ctl->incr = 0;
-        ctl->sum_load = 0;
-        ctl->walks_done = 0;
-    }
-    __syncthreads();
 }
 
-// Rank 0 after a candidate's matrix: its best entry over the slots against
-// the pass's best move so far.
-__device__ __noinline__ void ls_collect(const AlnsTeam& t, const Smem& s) {
-    AlnsCtl* ctl = t.ctl;
-    const int m = t.m, N = s.sWoff[m], G = N + m, ns = ctl->nrem, lane = threadIdx.x & 31;
-    if ((threadIdx.x >> 5) == 0) {
-        for (int ti = 0; ti < ns; ++ti) {
-            unsigned long long bv = lane < m ? t.rkeys[ti * 32 + lane] : KEY_NONE;
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long other = __shfl_xor_sync(FULL_MASK, bv, o);
-                bv = other < bv ? other : bv;
+// One candidate of relocation onto the vehicles part, part + split, ..., the whole CTA.
+__device__ void ls_relocate_item(const AlnsTeam& t, const Smem& s, int* scr, LsRoutes* rt, int c, int part, int split,
+                                 LsBest& best, unsigned& scored, unsigned& simulated) {
+    const int n = t.n, m = t.m, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N0 = 2 * n;
+    const int rw = ((n + 1) + 3) & ~3;
+    const uint16_t* place = reinterpret_cast<const uint16_t*>(t.gains);
+    const int pd = place[2 * c], pp = place[2 * c + 1], zcur = t.ctl->z_cur, bott = t.ctl->ls_bott, pc = s.sp[c];
+    int *H = scr, *T = H + N0, *S = T + N0, *PM = S + N0, *SM = PM + N0, *gC = SM + N0, *list = gC + N0 + 4;
+    constexpr int SCUT = INT32_MIN;            // gC: a shortcut gap; SKIPV: one that cannot matter; else its path
+    int* sh = s.misc + 32;                     // makespan, largest shortcut, gaps that matter
+    __syncthreads();                           // the previous item is done with the staged solution
+    stage_without(t, s, min(pd, pp), max(pd, pp));
+    if (warp == 0) {
+        const int z = walk_heads(t, s, s.rdy, H);
+        if (lane == 0) sh[0] = z;
+    } else if (warp == 1) {
+        walk_tails(t, s, s.rdy + rw, T, 0, -1);
+    } else {
+        for (int r = warp - 2; r < m; r += ALNS_WARPS - 2) ls_scan_route(t, s, r, S, PM, SM, rt);
+    }
+    __syncthreads();
+    const int z = sh[0], dcc = Dx(t, s, c, c);
+    int sumL = 0, len = 0;
+    unsigned bad = 0;
+    for (int v = 0; v < m; ++v) {
+        int l = 0;
+        sumL += rt->load[v];
+        len += rt->len[v];
+        if (!cap_ok(t, rt->mn[v], rt->mx[v], l)) bad |= 1u << v;
+    }
+    auto cust = [&](int k) { return (s.sW[k] & PACK_MASK) >> 1; };
+    int* rdy_ = s.rdy + warp * rw;
+    volatile int* rdy = rdy_;
+    for (int v = part; v < m; v += split) {
+        if (v == bott || (bad & ~(1u << v)) != 0u) continue;   // uniform over the CTA
+        const int off = s.sWoff[v], L = s.sWoff[v + 1] - off;
+        struct Gap { int Hx, Ty, dxc, dcy, w; };
+        auto gap = [&](int i) {
+            Gap g;
+            const int x = i > 0 ? cust(off + i - 1) : 0, y = i < L ? cust(off + i) : 0;
+            g.Hx = i > 0 ? H[off + i - 1] : 0;
+            g.Ty = i < L ? T[off + i] : 0;
+            g.dxc = Dx(t, s, x, c);
+            g.dcy = Dx(t, s, c, y);
+            g.w = L == 0 ? 0 : Dx(t, s, x, y);
+            return g;
+        };
+        auto fits = [&](int mn, int mx) {
+            int l = 0;
+            return cap_ok(t, mn, mx, l) && sumL - rt->load[v] + l <= t.R;
+        };
+        // both ops into gap i
+        auto fits_adjacent = [&](int i) {
+            const int pm = i > 0 ? PM[off + i - 1] : 0, sb = i > 0 ? S[off + i - 1] : 0;
+            int mn = min(range_lo(pm), sb - 1), mx = range_hi(pm);
+            if (i < L) {
+                mn = min(mn, range_lo(SM[off + i]));
+                mx = max(mx, range_hi(SM[off + i]));
             }
-            if (lane == 0 && bv != KEY_NONE) {
-                const int row = static_cast<int>(bv & 0xFFF);
-                const int col = static_cast<int>(t.keys[static_cast<long long>(ti) * G + row] & 0xFFF);
-                const int dz = static_cast<int>(static_cast<unsigned>(bv >> 32) ^ 0x80000000u);
-                const int dt = static_cast<int>((bv >> 12) & 0xFFFFFull) - (1 << 19);
-                const int zn = ctl->z_work + dz;
-                const long long tn = ctl->ls_travel + dt;
-                const long long flat = static_cast<long long>(row) * G + col;
-                const int c = t.rem[ti];
-                bool better = !ctl->ls_have;
-                if (!better) {
-                    if (zn != ctl->ls_bz) better = zn < ctl->ls_bz;
-                    else if (tn != ctl->ls_bt) better = tn < ctl->ls_bt;
-                    else if (c != ctl->ls_c) better = c < ctl->ls_c;
-                    else better = flat < ctl->ls_bflat;
+            return fits(mn, mx);
+        };
+        __syncthreads();                       // the previous route is done with gC, the list and the words
+        if (tid == 0) { sh[1] = 0; sh[2] = 0; }
+        __syncthreads();
+        for (int i = tid; i <= L; i += ALNS_THREADS) {
+            const Gap g = gap(i);
+            const int cut = g.w - g.dxc - g.dcy;
+            if (cut > 0) atomicMax(&sh[1], cut);
+            gC[i] = cut > 0 ? SCUT : g.Hx + g.dxc + g.dcy + g.Ty;
+        }
+        __syncthreads();
+        // a path through two shortcut gaps loses at most both
+        const int cut = sh[1];
+        if (z - 2 * cut >= zcur) continue;
+        for (int i = tid; i <= L; i += ALNS_THREADS) {
+            const int gc = gC[i];
+            if (gc != SCUT) {
+                const Gap g = gap(i);
+                const int zn = max(z, g.Hx + g.dxc + max(dcc, pc) + g.dcy + g.Ty);
+                ++scored;
+                if (zn < zcur && fits_adjacent(i)) best.take(zn, len + g.dxc + dcc + g.dcy - g.w, c, v, i, v, i);
+                if (gc - cut >= zcur) {
+                    gC[i] = SKIPV;
+                    continue;
                 }
-                if (better) {
-                    ctl->ls_have = 1;
-                    ctl->ls_c = c;
-                    ctl->ls_bz = zn;
-                    ctl->ls_bt = tn;
-                    ctl->ls_bflat = flat;
-                    ctl->ls_a = t.groute[row];
-                    ctl->ls_ia = t.gpos[row];
-                    ctl->ls_b = t.groute[col];
-                    ctl->ls_jb = t.gpos[col];
+            }
+            list[atomicAdd(&sh[2], 1)] = i;
+        }
+        __syncthreads();
+        const int nv = sh[2];
+        for (int k = warp; k < nv; k += ALNS_WARPS) {
+            const int i = list[k];
+            const bool si = gC[i] == SCUT;
+            const Gap gi = gap(i);
+            const int pmi = i > 0 ? PM[off + i - 1] : 0, sbi = i > 0 ? S[off + i - 1] : 0;
+            bool walk = false;
+            for (int q = 0; q < nv; ++q) {
+                const int j = list[q];
+                if (j < i || (j == i && !si)) continue;
+                const int gc = gC[j];
+                if (!si && gc != SCUT) { walk = true; continue; }
+                // a shortcut on either side: simulated
+                const Gap gj = gap(j);
+                bool ok;
+                if (i == j) {
+                    ok = fits_adjacent(i);
+                } else {
+                    int mn = INT32_MAX, mx = INT32_MIN;
+                    for (int e = off + i + lane; e < off + j; e += 32) { mn = min(mn, S[e]); mx = max(mx, S[e]); }
+                    mn = __reduce_min_sync(FULL_MASK, mn);
+                    mx = __reduce_max_sync(FULL_MASK, mx);
+                    mn = min(min(range_lo(pmi), sbi - 1), mn - 1);
+                    mx = max(max(range_hi(pmi), mx - 1), S[off + j - 1]);
+                    if (j < L) {
+                        mn = min(mn, range_lo(SM[off + j]));
+                        mx = max(mx, range_hi(SM[off + j]));
+                    }
+                    ok = fits(mn, mx);
                 }
+                if (!ok) continue;
+                const int zn = walk_insert(t, s, rdy_, c, v, i, v, j);
+                if (lane == 0) {
+                    ++simulated;
+                    const int di = gi.dxc + gi.dcy - gi.w;
+                    if (zn < zcur)
+                        best.take(zn, len + (i == j ? gi.dxc + dcc + gi.dcy - gi.w : di + gj.dxc + gj.dcy - gj.w), c, v, i, v, j);
+                }
+            }
+            if (!walk) continue;
+            // W from op y_i on: the longest path from it to every op of the route
+            const int u = off + i, row = max(z, gC[i]);
+            for (int q = lane; q <= n; q += 32) rdy[q] = UNRES;
+            __syncwarp();
+            int pos = lane < m ? s.sWoff[lane] : 0, val = NEG, sv = sbi, mn = INT32_MAX, mx = INT32_MIN;
+            const int end = lane < m ? s.sWoff[lane + 1] : 0;
+            int x = pos < end ? s.sW[pos] : 0;
+            for (;;) {
+                const bool on = pos < end, at = pos == u;
+                const int cc = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0;
+                const bool pick = (x & 1) != 0;
+                const int r = on && pick && !at ? rdy[cc] : 0;
+                const bool go = on && (!pick || at || r != UNRES);
+                if (go) {
+                    val = at ? 0 : max(val == NEG ? NEG : val + (x >> PACK_SHIFT), pick ? r : NEG);
+                    if (!pick) rdy[cc] = val == NEG ? NEG : val + s.sp[cc];
+                    if (lane == v && pos >= u) {
+                        sv += pick ? 1 : -1;
+                        mn = min(mn, sv);
+                        mx = max(mx, sv);
+                        const int j = pos + 1 - off, gc = gC[j];
+                        if (gc != SCUT && gc != SKIPV) {
+                            const Gap gj = gap(j);
+                            ++scored;
+                            const int zn = max(max(row, gc), max(gi.Hx + gi.dxc + pc + gj.dcy + gj.Ty,
+                                                                 gi.Hx + gi.dxc + gi.dcy + val + gj.dxc + gj.dcy + gj.Ty));
+                            if (zn < zcur) {
+                                int lo = min(min(range_lo(pmi), sbi - 1), mn - 1), hi = max(max(range_hi(pmi), mx - 1), sv);
+                                if (j < L) {
+                                    lo = min(lo, range_lo(SM[off + j]));
+                                    hi = max(hi, range_hi(SM[off + j]));
+                                }
+                                if (fits(lo, hi))
+                                    best.take(zn, len + gi.dxc + gi.dcy - gi.w + gj.dxc + gj.dcy - gj.w, c, v, i, v, j);
+                            }
+                        }
+                    }
+                    x = nx;
+                    ++pos;
+                }
+                __syncwarp();
+                if (!__any_sync(FULL_MASK, go) || __shfl_sync(FULL_MASK, pos >= end, v)) break;
             }
         }
     }
-    __syncthreads();
 }
 
-// Rank 0 at the end of a pass: apply the best move if it lowers the makespan.
-__device__ __noinline__ void ls_apply(const AlnsTeam& t, const Smem& s) {
+// One pass, every CTA of the team between two barriers: its share of the
+// candidates, the CTA's least key to its record.
+__device__ __noinline__ void ls_pass(const AlnsTeam& t, const Smem& s, int rank, int team_blocks, int mode) {
+    const int active = ls_active(t, team_blocks);
+    if (rank >= active) return;
     AlnsCtl* ctl = t.ctl;
-    const bool go = ctl->ls_have && ctl->ls_bz < ctl->z_cur;
+    const int ncand = *reinterpret_cast<volatile int*>(&ctl->ls_ncand);
+    int* scr = ls_scratch(t, rank);
+    LsRoutes* rt = reinterpret_cast<LsRoutes*>(s.rowv);
+    LsBest best;
+    unsigned scored = 0, simulated = 0;
+    if (mode == LS_PICKUP) {
+        for (int k = rank; k < ncand; k += active) ls_pickup_item(t, s, scr, rt, t.lscand[k], best, scored, simulated);
+    } else {
+        const int split = max(1, min(t.m - 1, active / max(ncand, 1)));
+        for (int k = rank; k < ncand * split; k += active)
+            ls_relocate_item(t, s, scr, rt, t.lscand[k / split], k % split, split, best, scored, simulated);
+    }
+    const unsigned ws = __reduce_add_sync(FULL_MASK, scored), wf = __reduce_add_sync(FULL_MASK, simulated);
+    if ((threadIdx.x & 31) == 0) {
+        if (ws) atomicAdd(&ctl->entries, static_cast<unsigned long long>(ws));
+        if (wf) atomicAdd(&ctl->fallback_entries, static_cast<unsigned long long>(wf));
+    }
+    ls_block_least(best, reinterpret_cast<unsigned long long*>(s.colv));
+    if (threadIdx.x == 0) {
+        unsigned long long* rec = reinterpret_cast<unsigned long long*>(t.scpair) + 2 * rank;
+        rec[0] = best.hi;
+        rec[1] = best.lo;
+    }
+}
+
+// Rank 0 at the end of a pass: apply the least move (all in the records lower
+// the makespan).
+__device__ __noinline__ void ls_apply(const AlnsTeam& t, const Smem& s, int team_blocks) {
+    AlnsCtl* ctl = t.ctl;
+    const int active = ls_active(t, team_blocks);
+    const unsigned long long* rec = reinterpret_cast<const unsigned long long*>(t.scpair);
+    LsBest best;
+    for (int k = threadIdx.x; k < active; k += ALNS_THREADS) best.least(__ldcg(rec + 2 * k), __ldcg(rec + 2 * k + 1));
+    unsigned long long* sh = reinterpret_cast<unsigned long long*>(s.colv);
+    ls_block_least(best, sh);
+    if (threadIdx.x == 0) { sh[0] = best.hi; sh[1] = best.lo; }
+    __syncthreads();
+    const unsigned long long hi = sh[0], lo = sh[1];
+    const bool go = hi != KEY_NONE;
     if (go) {
-        const int c = ctl->ls_c;
+        const int c = static_cast<int>(lo >> 34), drop = static_cast<int>(lo >> 17) & 0x1ffff, pick = static_cast<int>(lo) & 0x1ffff;
         for (int x = threadIdx.x; x <= t.n; x += blockDim.x) s.flags[x] = x == c ? 1 : 0;
         if (threadIdx.x == 0) ctl->wsel = 0;
         __syncthreads();
         build_W_from_cur(t, s);
         stage_W(t, s);
         __syncthreads();
-        insert_staged(t, s, c, ctl->ls_a, ctl->ls_ia, ctl->ls_b, ctl->ls_jb, t.cur_ops, t.cur_off);
+        insert_staged(t, s, c, drop >> 12, drop & 0xfff, pick >> 12, pick & 0xfff, t.cur_ops, t.cur_off);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         ctl->ls_moved = go ? 1 : 0;
-        ctl->ls = 0;
         if (go) {
-            ctl->z_cur = ctl->ls_bz;
+            ctl->z_cur = static_cast<int>(hi >> 32);
             ctl->ls_moves += 1;
         }
     }
@@ -2899,22 +3263,9 @@ __device__ __noinline__ bool ls_block(const AlnsTeam& t, const Smem& s, int rank
         for (int pass = 0; pass < 3; ++pass) {
             if (rank == 0) ls_candidates(t, s, mode);
             if (!team_barrier(ctl, team_blocks, gen)) return false;
-            const int ncand = *reinterpret_cast<volatile int*>(&ctl->ls_ncand);
-            for (int k = 0; k < ncand; ++k) {
-                if (rank == 0) ls_setup(t, s, mode, k);
-                if (!team_barrier(ctl, team_blocks, gen)) return false;
-                if (*reinterpret_cast<volatile int*>(&ctl->nrem) == 0) continue;
-                phase_prep(t, s, rank, team_blocks, false);
-                if (!team_barrier(ctl, team_blocks, gen)) return false;
-                phase_gaps(t, s, rank, team_blocks);
-                team_arrive(ctl, team_blocks, gen);
-                gap_walks(t, s, rank, team_blocks);
-                if (!team_wait(ctl, team_blocks, gen)) return false;
-                phase_matrix(t, s);
-                if (!team_barrier(ctl, team_blocks, gen)) return false;
-                if (rank == 0) ls_collect(t, s);
-            }
-            if (rank == 0) ls_apply(t, s);
+            ls_pass(t, s, rank, team_blocks, mode);
+            if (!team_barrier(ctl, team_blocks, gen)) return false;
+            if (rank == 0) ls_apply(t, s, team_blocks);
             if (!team_barrier(ctl, team_blocks, gen)) return false;
             if (!*reinterpret_cast<volatile int*>(&ctl->ls_moved)) break;
         }
@@ -3171,7 +3522,7 @@ static size_t team_bytes(int n, int m, int qmax, int iterations, bool dump) {
     add(static_cast<size_t>(SC_CAP) * SC_CAP, 4);
     add(std::max(iterations, 1), 4);
     add(n + 1, 4);
-    add(n + 1, 4); add(static_cast<size_t>(qmax), 16);
+    add(n + 1, 4);
     if (dump) { add(G * G, 4); add(G * G, 4); }
     return w;
 }
@@ -3213,17 +3564,14 @@ static void carve_team(AlnsTeam& t, DevBuf& B, int n, int m, int qmax, int itera
     t.trace = B.take<int>(std::max(iterations, 1));
     t.gains = B.take<int>(n + 1);
     t.lscand = B.take<int>(n + 1);
-    t.lsmask = B.take<int4>(static_cast<size_t>(qmax));
     t.dump_delta = dump ? B.take<int>(G * G) : nullptr;
     t.dump_travel = dump ? B.take<int>(G * G) : nullptr;
 }
 
 // Rows of the per-customer buffers: a route removal takes a whole route, so
-// with that operator on, up to n customers wait for reinsertion at once; the
-// relocation local search runs up to m - 1 slots for one customer.
+// with that operator on, up to n customers wait for reinsertion at once.
 int alns_row_cap(int n, int m, int qmax, const vrprpd_alns_params* P) {
     int cap = (P->destroy_mask & (1 << D_ROUTE)) ? n : qmax;
-    if (P->ls_relocate_every > 0) cap = std::max(cap, m);
     return std::max(cap, 1);
 }
 
