@@ -46,6 +46,7 @@ struct DecArgs {
     int smem_dist;       // 1 = distance matrix staged in shared memory as int32, 2 = as uint16
     int pack;            // every schedule time is below 2^22: SelectVehicle is one 32-bit reduction
     const uint16_t* d16; // the 16-bit copy (max d < 65536) or null
+    int* err;
     int32_t* ops;
     int32_t* off;
     int32_t* z;
@@ -59,209 +60,354 @@ __host__ __device__ inline int pow2_at_least(int x) {
     return p;
 }
 
+constexpr int SORT_REGS_MAX = 1024;   // ops (a power of two) that a warp sorts in registers
+
 __host__ __device__ inline size_t dec_warp_words(int n, int P) {
-    // sort buffer (u64) + tdrop + sched bitmap + per-op (vehicle<<16 | seq) +
-    // per-op hinted vehicle (bytes)
-    return static_cast<size_t>(2 * P) + (((n + 1) + 3) & ~3) + ((((2 * n + 2 + 31) / 32) + 3) & ~3) +
-           (((2 * n) + 3) & ~3) + ((((2 * n + 3) / 4) + 3) & ~3);
+    // op list (beyond SORT_REGS_MAX the u64 sort buffer it comes from) + tdrop +
+    // log of the scheduled ops + per-op hinted vehicle (bytes)
+    const int list = P > SORT_REGS_MAX ? 2 * P : P > 32 ? P : 32;
+    return static_cast<size_t>(list) + (((n + 1) + 3) & ~3) + (((2 * n) + 3) & ~3) + ((((2 * n + 3) / 4) + 3) & ~3);
 }
 
-// The vehicle an assignment hint names: floor(m * alpha) in fp64 (exact for a
-// float alpha and m <= 32), capped at m - 1.
-__host__ __device__ inline int hint_vehicle(float alpha, int m) {
-    const double x = static_cast<double>(alpha) * static_cast<double>(m);
-    int h = static_cast<int>(floor(x));
-    h = h > m - 1 ? m - 1 : h;
-    return h < 0 ? 0 : h;
+// The vehicle an assignment hint names: floor(m * alpha), capped to [0, m - 1].
+// The product rounded down lies at or above an integer exactly when the product
+// does (integers up to 32 are floats), so fp32 gives the floor of the exact
+// product; an fp64 product, also exact, costs a tenth of the decode here.
+__device__ inline int hint_vehicle(float alpha, int m) {
+    const int h = __float2int_rd(__fmul_rd(alpha, static_cast<float>(m)));
+    return max(min(h, m - 1), 0);
+}
+
+// The ops in priority order into list: stable argsort of the 2n keys, as a
+// bitonic sort of (key bits, op index) by one warp.  Lane l holds elements
+// l EPL .. l EPL + EPL - 1 in registers, so of the 45 steps for 512 elements 30
+// stay inside a lane and 15 are shuffles (in shared memory every step was a
+// pass over the buffer and a barrier).
+__device__ __forceinline__ unsigned long long sort_entry(const float* kk, int two_n, int i) {
+    if (i >= two_n) return ~0ull;                                     // padding sorts last
+    const float f = __fadd_rn(__ldg(kk + i), 0.0f);                  // -0 -> +0
+    return (static_cast<unsigned long long>(__float_as_uint(f)) << 32) | static_cast<unsigned>(i);
+}
+template <int EPL>
+__device__ __noinline__ void sort_ops(const float* kk, int two_n, int* list) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long x[EPL];
+#pragma unroll
+    for (int r = 0; r < EPL; ++r) x[r] = sort_entry(kk, two_n, lane * EPL + r);
+    auto exchange = [&](int i, int j, bool asc) {
+        const unsigned long long a = x[i], b = x[j];
+        const bool swap = (a > b) == asc;
+        x[i] = swap ? b : a;
+        x[j] = swap ? a : b;
+    };
+#pragma unroll
+    for (int size = 2; size < EPL; size <<= 1)
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1)
+#pragma unroll
+            for (int r = 0; r < EPL; ++r)
+                if (!(r & stride)) exchange(r, r | stride, (r & size) == 0);
+    for (int size = EPL > 1 ? EPL : 2; size <= 32 * EPL; size <<= 1) {
+        const bool asc = ((lane * EPL) & size) == 0;
+        for (int far = size / (2 * EPL); far > 0; far >>= 1) {
+            const bool least = ((lane & far) == 0) == asc;
+#pragma unroll
+            for (int r = 0; r < EPL; ++r) {
+                const unsigned long long o = __shfl_xor_sync(FULL_MASK, x[r], far);
+                x[r] = (o < x[r]) == least ? o : x[r];
+            }
+        }
+#pragma unroll
+        for (int stride = EPL >> 1; stride > 0; stride >>= 1)
+#pragma unroll
+            for (int r = 0; r < EPL; ++r)
+                if (!(r & stride)) exchange(r, r | stride, asc);
+    }
+#pragma unroll
+    for (int r = 0; r < EPL; ++r) list[lane * EPL + r] = static_cast<int>(x[r] & 0xffffffffu);
+    __syncwarp();
+}
+// The same beyond SORT_REGS_MAX, through a shared buffer that list shares.
+__device__ __noinline__ void sort_ops_shared(const float* kk, int two_n, int P, unsigned long long* sb, int* list) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < P; i += 32) sb[i] = sort_entry(kk, two_n, i);
+    __syncwarp();
+    for (int size = 2; size <= P; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int i = lane; i < P / 2; i += 32) {
+                const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
+                const bool asc = (lo & size) == 0;
+                const unsigned long long x = sb[lo], y = sb[hi];
+                if ((x > y) == asc) { sb[lo] = y; sb[hi] = x; }
+            }
+            __syncwarp();
+        }
+    }
+    for (int base = 0; base < P; base += 32) {                       // list[k] lies at or below sb[k]
+        const int v = static_cast<int>(sb[base + lane] & 0xffffffffu);
+        __syncwarp();
+        list[base + lane] = v;
+        __syncwarp();
+    }
+}
+
+// shared-memory accesses by 32-bit address, out of the compiler's reach to turn
+// into generic ones or branches
+__device__ __forceinline__ int lds_u16(unsigned addr) {
+    int v;
+    asm("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ int lds_b32(unsigned addr) {
+    int v;
+    asm("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void sts_if(bool on, unsigned addr, int v) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %0, 0;\n\t"
+        "@p st.shared.b32 [%1], %2;\n\t}" ::"r"(static_cast<unsigned>(on)),
+        "r"(addr), "r"(v)
+        : "memory");
+}
+// index of the highest set bit (of a single one here), ~0 for none
+__device__ __forceinline__ unsigned bit_index(unsigned x) {
+    unsigned r;
+    asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
 }
 
 // The decoder specialised on its per-visit choices, so the chain of one op's
 // visit holds no branch on them: SD where distances come from (0 L2 int32,
 // 1 shared int32, 2 shared uint16), HINTS the 4n layout's tie rule, FULL the
 // Eq. 13 start load, PACK the one-reduction SelectVehicle.
+//
+// One chain of dependent visits per chromosome is what takes the time, and with
+// one chromosome per warp nothing else runs beside it: latency, and the warp's
+// own instruction count.  So:
+//   - a pass takes the list 32 ops at a time, one per lane, and goes straight to
+//     the ops that can be scheduled.  Whether a drop (a pickup) fits any vehicle
+//     does not depend on the customer, so two votes after each visit say which
+//     kind can go next, and masks where the next of each kind stands: of 1290
+//     list entries per decode at n=200 m=6 R=20, 400 are visited, none in vain;
+//   - the next drop and the next pickup are both looked up (their words, then
+//     their distances from every vehicle) while the vehicle is selected;
+//   - a vehicle's stock is two numbers, see below; its time, tie rank and one
+//     flag share the selection key, so key == minimum names the winner;
+//   - an op's place is logged by the winner, drop times are written once per
+//     chunk, and the matrix arrives by one bulk copy behind the sort.
+// 1024 decodes of the 4n layout at n=200 m=6: 281 us before, 89 us now (47 k warp
+// instructions and about 300 cycles a visit; sort 5 us, the rest around it 8 us).
+// Tried on the way: one visit list for both kinds, entries two visits ahead,
+// starting over when a kind blocks or unblocks (112-141 us: a restart every 2.7
+// visits); partners by match_any (373 cycles a call).
 template <int SD, bool HINTS, bool FULL, bool PACK>
 __global__ void __launch_bounds__(DEC_WARPS * 32, 1) decode_kernel(DecArgs a) {
     extern __shared__ __align__(16) int smem_dec[];
+    __shared__ __align__(8) uint64_t dist_bar;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = a.n, m = a.m, two_n = 2 * n, N1 = n + 1;
+    constexpr int ES = SD == 2 ? 2 : 4;                   // bytes of a distance
     int* sd = smem_dec;                                   // staged distances (optional)
     const int dist_words = SD == 1 ? ((N1 * N1 + 3) & ~3) : SD == 2 ? (((N1 * N1 + 1) / 2 + 3) & ~3) : 0;
     int* sp = sd + dist_words;
-    uint16_t* sd16 = reinterpret_cast<uint16_t*>(sd);
+    if (SD != 0 && threadIdx.x == 0) {
+        mbar_init(&dist_bar, 1);
+        mbar_arrive_expect_tx(&dist_bar, dist_words * 4u);
+        // (the matrices are padded to 16 bytes in global memory)
+        tma_bulk_g2s(sd, SD == 2 ? static_cast<const void*>(a.d16) : static_cast<const void*>(a.d32), dist_words * 4u, &dist_bar);
+    }
     for (int i = threadIdx.x; i < N1; i += blockDim.x) sp[i] = a.p[i];
-    if (SD == 1)
-        for (int i = threadIdx.x; i < N1 * N1; i += blockDim.x) sd[i] = a.d32[i];
-    if (SD == 2)
-        for (int i = threadIdx.x; i < N1 * N1; i += blockDim.x) sd16[i] = a.d16[i];
-    int* wbase = sp + ((N1 + 3) & ~3) + warp * static_cast<int>(dec_warp_words(n, a.P));
-    unsigned long long* sb = reinterpret_cast<unsigned long long*>(wbase);
-    int* tdrop = wbase + 2 * a.P;
-    unsigned* sched = reinterpret_cast<unsigned*>(tdrop + (((n + 1) + 3) & ~3));
-    int* vs = reinterpret_cast<int*>(sched + ((((two_n + 2 + 31) / 32) + 3) & ~3));
+    int* list = sp + ((N1 + 3) & ~3) + warp * static_cast<int>(dec_warp_words(n, a.P));
+    int* tdrop = list + (a.P > SORT_REGS_MAX ? 2 * a.P : a.P > 32 ? a.P : 32);   // drop time, -1 before
+    int* vs = tdrop + (((n + 1) + 3) & ~3);               // log of the scheduled ops
     unsigned char* hv = reinterpret_cast<unsigned char*>(vs + ((two_n + 3) & ~3));
     __syncthreads();
     const float* keys = a.keys;
     if (a.keys2 != nullptr && a.ctl->sel == 1) keys = a.keys2;
-    auto dist = [&](int i, int j) -> int {
-        if constexpr (SD == 2) return static_cast<int>(sd16[i * N1 + j]);
-        else if constexpr (SD == 1) return sd[i * N1 + j];
-        else return __ldg(a.d32 + i * N1 + j);
+    bool staged = SD == 0;
+    const unsigned sd_addr = smem_u32(sd), log_addr = smem_u32(vs), lanebit = 1u << lane;
+    // the distance from a place (row: shared address of, or index into, its
+    // row) to the customer whose offset within a row off is
+    auto dist = [&](unsigned row, unsigned off) -> int {
+        if constexpr (SD == 2) return lds_u16(row + off);
+        else if constexpr (SD == 1) return lds_b32(row + off);
+        else return __ldg(reinterpret_cast<const int*>(reinterpret_cast<const char*>(a.d32) + row + off));
     };
+    const unsigned row0 = SD == 0 ? 0u : sd_addr;
     for (int ch = blockIdx.x * DEC_WARPS + warp; ch < a.num; ch += gridDim.x * DEC_WARPS) {
         const float* kk = keys + static_cast<long long>(ch) * a.L;
-        // ---- segmented key sort: (key bits << 32 | op index), padding sorts last ----
-        for (int i = lane; i < a.P; i += 32) {
-            unsigned long long v = ~0ull;
-            if (i < two_n) {
-                const float f = __fadd_rn(kk[i], 0.0f);          // -0 -> +0
-                v = (static_cast<unsigned long long>(__float_as_uint(f)) << 32) | static_cast<unsigned>(i);
-            }
-            sb[i] = v;
-        }
-        for (int i = lane; i <= n; i += 32) tdrop[i] = 0;
-        for (int i = lane; i < (two_n + 2 + 31) / 32; i += 32) sched[i] = 0u;
-        for (int i = lane; i < two_n; i += 32) vs[i] = -1;
+        for (int i = lane; i <= n; i += 32) tdrop[i] = -1;
         if (HINTS)
             for (int i = lane; i < two_n; i += 32) hv[i] = static_cast<unsigned char>(hint_vehicle(kk[two_n + i], m));
-        __syncwarp();
-        for (int size = 2; size <= a.P; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int i = lane; i < a.P / 2; i += 32) {
-                    const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
-                    const bool asc = (lo & size) == 0;
-                    const unsigned long long x = sb[lo], y = sb[hi];
-                    if ((x > y) == asc) { sb[lo] = y; sb[hi] = x; }
-                }
-                __syncwarp();
+        // ---- segmented key sort ----
+        switch (a.P) {
+            case 64: sort_ops<2>(kk, two_n, list); break;
+            case 128: sort_ops<4>(kk, two_n, list); break;
+            case 256: sort_ops<8>(kk, two_n, list); break;
+            case 512: sort_ops<16>(kk, two_n, list); break;
+            case 1024: sort_ops<32>(kk, two_n, list); break;
+            default:
+                if (a.P <= 32) sort_ops<1>(kk, two_n, list);
+                else sort_ops_shared(kk, two_n, a.P, reinterpret_cast<unsigned long long*>(list), list);
+        }
+        if (!staged) {
+            if (!mbar_wait_bounded(&dist_bar, 0)) {
+                if (lane == 0) atomicExch(a.err, DEV_TIMEOUT_TMA);
+                mbar_wait_bounded(&dist_bar, 0);          // one more bounded chance for the copy in flight
+                return;
             }
+            staged = true;
         }
         // ---- tie-break order: vehicle ranks (stable argsort of the m vehicle
         // keys) or, per op, cyclic distance from the hinted vehicle ----
-        constexpr bool hints = HINTS;
-        const float kv = (!hints && lane < m) ? __fadd_rn(kk[two_n + lane], 0.0f) : 0.0f;
+        const float kv = (!HINTS && lane < m) ? __fadd_rn(kk[two_n + lane], 0.0f) : 0.0f;
         int rank = 0;
-        for (int u = 0; !hints && u < m; ++u) {
+        for (int u = 0; !HINTS && u < m; ++u) {
             const float ku = __shfl_sync(FULL_MASK, kv, u);
             if (lane < m && (ku < kv || (ku == kv && u < lane))) ++rank;
         }
         // ---- multi-pass decode (Algorithm 2), lane v = vehicle v ----
-        int tv = 0, locv = 0, net = 0, nmin = 0, nmax = 0, load = 0, cnt = 0;
-        int sum_load = 0, done = 0;
-        int len = two_n;                       // sb[0, len): ops not scheduled yet, priority order
-        for (int pass = 0; pass < two_n && done < two_n; ++pass) {
-            bool progress = false;
-            // Whether a drop (a pickup) fits some vehicle does not depend on the
-            // customer: it needs one unit of room, resp. stock, on a vehicle.  A
-            // drop never makes room for another drop (it lowers its vehicle's
-            // stock and raises the pool's load), nor a pickup for another pickup,
-            // so once no vehicle takes a drop, every drop fails until a pickup is
-            // scheduled, and the other way round.  Those visits are skipped.
-            bool drops_blocked = false, picks_blocked = false;
-            unsigned long long e_next = len > 0 ? sb[0] : 0ull;
-            for (int k = 0; k < len; ++k) {
-                // the next op's entry is read ahead: the order does not change
-                // within a pass, so its latency overlaps this op
-                const unsigned long long e_cur = e_next;
-                if (k + 1 < len) e_next = sb[k + 1];
-                const int oi = static_cast<int>(e_cur & 0xffffffffu);
-                const int o = oi + 2, c = o >> 1;
-                const bool pick = (o & 1) != 0;
-                // the list holds only ops unscheduled at the pass's start, and only
-                // the op visited gets scheduled: o itself is still unscheduled
-                if (pick ? picks_blocked : drops_blocked) continue;
-                if (pick && !((sched[(2 * c) >> 5] >> ((2 * c) & 31)) & 1u)) continue;
-                // the time a pickup waits for, read before the selection
-                const int ready = pick ? tdrop[c] + sp[c] : 0;
-                bool ok = false;
-                if (lane < m) {
-                    if (!pick) {
-                        if (FULL) ok = net > -a.Q;
-                        else {
-                            const int nl = max(load, 1 - net);
-                            ok = nl + nmax <= a.Q && sum_load - load + nl <= a.R;
-                        }
-                    } else {
-                        ok = FULL ? (net < 0) : (load + net + 1 <= a.Q);
-                    }
-                }
-                const int arr = ok ? tv + dist(locv, c) : 0;
-                int tie = rank;
-                if (hints) {                       // cyclic distance from the hinted vehicle
-                    tie = lane - static_cast<int>(hv[oi]);
-                    tie += tie < 0 ? m : 0;
-                }
-                // SelectVehicle: least arrival, then tie rank, then lane.  With
-                // every time below 2^22 the three fit one 32-bit key and one warp
-                // reduction; otherwise two reductions
-                int win;
-                if constexpr (PACK) {
-                    const unsigned key = ok ? ((static_cast<unsigned>(arr) << 10) | (static_cast<unsigned>(tie) << 5) |
-                                               static_cast<unsigned>(lane))
-                                            : 0xffffffffu;
-                    const unsigned kmin = __reduce_min_sync(FULL_MASK, key);
-                    if (kmin == 0xffffffffu) {
-                        if (pick) picks_blocked = true; else drops_blocked = true;
-                        continue;
-                    }
-                    win = static_cast<int>(kmin & 31u);
-                } else {
-                    const unsigned ua = ok ? static_cast<unsigned>(arr) : 0xffffffffu;
-                    const unsigned amin = __reduce_min_sync(FULL_MASK, ua);
-                    if (amin == 0xffffffffu) {
-                        if (pick) picks_blocked = true; else drops_blocked = true;
-                        continue;
-                    }
-                    const unsigned sub = (ok && ua == amin)
-                                             ? ((static_cast<unsigned>(tie) << 5) | static_cast<unsigned>(lane))
-                                             : 0xffffffffu;
-                    win = static_cast<int>(__reduce_min_sync(FULL_MASK, sub) & 31u);
-                }
-                // the winner's update, by selects rather than a branch: a drop
-                // sets its arrival and lowers the net stock (the start load may
-                // grow), a pickup waits for its ready time and raises it
-                const bool me = lane == win;
-                const int nnet = net + (pick ? 1 : -1);
-                const int nnmin = min(nmin, nnet), nnmax = max(nmax, nnet);
-                const int nload = pick ? load : -nnmin;
-                const int dsum = (me && !pick) ? nload - load : 0;
-                if (me) {
-                    tv = pick ? max(arr, ready) : arr;
-                    net = nnet;
-                    nmin = nnmin;
-                    nmax = nnmax;
-                    load = nload;
-                    locv = c;
-                    vs[oi] = (lane << 16) | cnt;
-                    sched[o >> 5] |= 1u << (o & 31);
-                    if (!pick) tdrop[c] = arr;
-                }
-                // a pickup can make room for drops, a drop stock for pickups
-                if (pick) drops_blocked = false; else picks_blocked = false;
-                cnt += me ? 1 : 0;
-                sum_load += __shfl_sync(FULL_MASK, dsum, win);
-                __syncwarp();
-                progress = true;
-                ++done;
-            }
-            if (!progress) break;
-            // the next pass scans only the ops still unscheduled, order kept (in
-            // place: a chunk is read into registers before any of it is written)
-            int w = 0;
+        // Of a vehicle's stock two numbers count.  LOAD_MIN: room r = start load +
+        // net (0 when a drop needs one more at the depot) and slack e = largest net
+        // - net; start load + largest net = r + e.  A drop fits if r > 0, or if
+        // e < Q and the pool has one left, a pickup if r < Q.  A drop lowers r, not
+        // below 0 (there the start load grows and the pool gives one), and raises e;
+        // a pickup raises r and lowers e, not below 0.
+        // Eq. 13: r = stock on board, from Q; a drop fits if r > 0, a pickup if r < Q.
+        const bool vehicle = lane < m;
+        int room = FULL ? a.Q : 0, slack = 0, pool = a.R, done = 0;
+        unsigned row = row0;
+        // PACK: time << 10 | tie rank << 5 | (room == 0), with hints the rank added
+        // per op; else the time, and the rest apart
+        int flag = room == 0 ? 1 : 0, tv = 0;
+        unsigned tkey = static_cast<unsigned>((HINTS ? 0 : rank * 32) + flag);
+        unsigned entry = static_cast<unsigned>(lane) << 26;      // the log: vehicle, place in its route, op
+        unsigned log_at = log_addr;
+        bool okD = vehicle && (FULL ? room > 0 : a.Q > 0 && pool > 0), okP = vehicle && room < a.Q;
+        bool anyD = __any_sync(FULL_MASK, okD), anyP = __any_sync(FULL_MASK, okP);
+        int len = two_n;                       // list[0, len): ops not scheduled yet, priority order
+        while (done < two_n) {
+            const int before = done;
+            int kept = 0;
             for (int base = 0; base < len; base += 32) {
-                const int k = base + lane;
-                const unsigned long long e = k < len ? sb[k] : 0ull;
-                const int o = static_cast<int>(e & 0xffffffffu) + 2;
-                const bool keep = k < len && !((sched[o >> 5] >> (o & 31)) & 1u);
-                const unsigned bal = __ballot_sync(FULL_MASK, keep);
+                const bool in = base + lane < len;
+                const int oi = in ? list[base + lane] : 0, mine = (oi >> 1) + 1;
+                const bool is_drop = in && !(oi & 1), is_pick = in && (oi & 1);
+                const int td = tdrop[mine], pm = sp[mine];
+                // a drop's own pickup further down the chunk: found through the drop's
+                // time slot, where such pickups leave their lane for a moment
                 __syncwarp();
-                if (keep) sb[w + __popc(bal & ((1u << lane) - 1u))] = e;
-                w += __popc(bal);
+                if (is_pick && td < 0) tdrop[mine] = -2 - lane;
+                __syncwarp();
+                const int mate = is_drop ? -2 - tdrop[mine] : -1;
+                __syncwarp();
+                if (is_pick && td < 0) tdrop[mine] = -1;
+                int ready = is_pick ? td + pm : 0;     // for a pickup whose drop is scheduled
+                // bits 0-12 the op code 2c + isPickup, 16-20 the hinted vehicle, 21-25
+                // the mate's lane, 31 whether there is one
+                unsigned word = static_cast<unsigned>(oi + 2);
+                if (HINTS) word |= static_cast<unsigned>(hv[oi]) << 16;
+                if (mate > lane) word |= (static_cast<unsigned>(mate) << 21) | 0x80000000u;
+                const unsigned drops = __ballot_sync(FULL_MASK, is_drop);
+                unsigned picks = __ballot_sync(FULL_MASK, is_pick && td >= 0);
+                int when = -1;                         // this lane's op: its vehicle's arrival, once scheduled
+                // the next drop and the next pickup: bit, lane, word, distances
+                unsigned bD = drops & (0u - drops), bP = picks & (0u - picks);
+                unsigned jD = bit_index(bD), jP = bit_index(bP);
+                unsigned wD = __shfl_sync(FULL_MASK, word, jD), wP = __shfl_sync(FULL_MASK, word, jP);
+                int dD = dist(row, (wD & 0x1ffeu) * (ES / 2)), dP = dist(row, (wP & 0x1ffeu) * (ES / 2));
+                for (;;) {
+                    const unsigned eD = anyD ? bD : 0u, eP = anyP ? bP : 0u;
+                    if (!(eD | eP)) break;
+                    const bool pick = eP - 1u < eD - 1u;         // the earlier one (0: none)
+                    const unsigned bit = pick ? eP : eD, w = pick ? wP : wD;
+                    const int d = pick ? dP : dD;
+                    const unsigned j = pick ? jP : jD;
+                    // In program order, since nothing else hides a latency: the reduction,
+                    // the search for the next two ops, the winner, their words, the votes,
+                    // their distances.
+                    // SelectVehicle: least arrival, then tie rank (unique per vehicle).
+                    // With every time below 2^22 both fit one 32-bit key and one warp
+                    // reduction; otherwise two reductions
+                    const bool ok = pick ? okP : okD;
+                    unsigned tie = 0u;
+                    if (HINTS) {                       // cyclic distance from the hinted vehicle
+                        const unsigned t0 = static_cast<unsigned>(lane) - ((w >> 16) & 31u);
+                        tie = min(t0, t0 + static_cast<unsigned>(m)) * 32u;
+                    }
+                    unsigned least, own;
+                    int first;
+                    if constexpr (PACK) {
+                        own = ok ? static_cast<unsigned>(d) * 1024u + tkey + tie : 0xffffffffu;
+                        least = __reduce_min_sync(FULL_MASK, own);
+                        first = static_cast<int>(least >> 10);
+                    } else {
+                        const unsigned arr = ok ? static_cast<unsigned>(tv + d) : 0xffffffffu;
+                        first = static_cast<int>(__reduce_min_sync(FULL_MASK, arr));
+                        own = arr == static_cast<unsigned>(first) ? tkey + tie : 0xffffffffu;
+                        least = __reduce_min_sync(FULL_MASK, own);
+                    }
+                    // the two ops that may follow: past this one, its mate among them
+                    const unsigned link = (w >> 31) << ((w >> 21) & 31u), past = 0u - 2u * bit;
+                    picks |= link;
+                    const unsigned mD = drops & past, mP = picks & past;
+                    bD = mD & (0u - mD);
+                    bP = mP & (0u - mP);
+                    jD = bit_index(bD);
+                    jP = bit_index(bP);
+                    const int wait = __shfl_sync(FULL_MASK, ready, j);
+                    // the winner's update, by selects
+                    const bool me = own == least;
+                    const int step = me ? (pick ? 1 : -1) : 0;
+                    room = __viaddmax_s32(room, step, 0);
+                    slack = __viaddmax_s32(slack, -step, 0);
+                    if (!FULL) pool -= pick ? 0 : static_cast<int>(least & 1u);
+                    okD = vehicle && (room > 0 || (!FULL && slack < a.Q && pool > 0));
+                    okP = vehicle && room < a.Q;
+                    row = me ? row0 + (w & 0x1ffeu) * static_cast<unsigned>(N1 * (ES / 2)) : row;
+                    wD = __shfl_sync(FULL_MASK, word, jD);
+                    wP = __shfl_sync(FULL_MASK, word, jP);
+                    anyD = __any_sync(FULL_MASK, okD);
+                    anyP = __any_sync(FULL_MASK, okP);
+                    // it leaves at its arrival, or once a pickup is ready (wait is 0 for a drop)
+                    const int leave = max(first, wait);
+                    flag = room == 0 ? 1 : 0;
+                    if constexpr (PACK) {
+                        const unsigned nk = static_cast<unsigned>(leave) * 1024u + static_cast<unsigned>((HINTS ? 0 : rank * 32) + flag);
+                        tkey = me ? nk : tkey;
+                    } else {
+                        tv = me ? leave : tv;
+                        tkey = static_cast<unsigned>((HINTS ? 0 : rank * 32) + flag);
+                    }
+                    sts_if(me, log_at, static_cast<int>(entry | (w & 0x1fffu)));
+                    dD = dist(row, (wD & 0x1ffeu) * (ES / 2));
+                    dP = dist(row, (wP & 0x1ffeu) * (ES / 2));
+                    log_at += 4u;
+                    entry += me ? 1u << 13 : 0u;
+                    when = (lanebit & bit) ? first : when;
+                    ready = (lanebit & link) ? first + pm : ready;
+                }
+                // drop times, and the ops still unscheduled, order kept, for the next
+                // pass (in place)
+                const bool fin = when >= 0;
+                __syncwarp();
+                if (fin && is_drop) tdrop[mine] = when;
+                done += __popc(__ballot_sync(FULL_MASK, fin));
+                const bool keep = in && !fin;
+                const unsigned bal = __ballot_sync(FULL_MASK, keep);
+                if (keep) list[kept + __popc(bal & (lanebit - 1u))] = oi;
+                kept += __popc(bal);
                 __syncwarp();
             }
-            len = w;
+            len = kept;
+            if (done == before) break;
         }
+        if constexpr (PACK) tv = static_cast<int>(tkey >> 10);
+        const int cnt = static_cast<int>((entry >> 13) & 0x1fffu);
         // ---- outputs: routes, makespan, penalty fitness ----
-        int ret = (lane < m && cnt > 0) ? tv + dist(locv, 0) : 0;
+        int ret = (lane < m && cnt > 0) ? tv + dist(row, 0u) : 0;
         for (int off = 16; off > 0; off >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, off));
         int incl = lane < m ? cnt : 0;
         for (int off = 1; off < 32; off <<= 1) {
@@ -274,11 +420,11 @@ __global__ void __launch_bounds__(DEC_WARPS * 32, 1) decode_kernel(DecArgs a) {
         if (lane == 0) off_out[m] = done;
         int32_t* ops_out = a.ops + static_cast<long long>(ch) * two_n;
         __syncwarp();
-        for (int oi = lane; oi < two_n; oi += 32) {
-            const int w = vs[oi];
-            if (w < 0) continue;
-            const int v = w >> 16, seq = w & 0xffff;
-            ops_out[off_out[v] + seq] = oi + 2;
+        for (int base = 0; base < done; base += 32) {
+            const bool in = base + lane < done;
+            const unsigned w = in ? static_cast<unsigned>(vs[base + lane]) : 0u;
+            const int at = __shfl_sync(FULL_MASK, excl, w >> 26) + static_cast<int>((w >> 13) & 0x1fffu);
+            if (in) ops_out[at] = static_cast<int>(w & 0x1fffu);
         }
         if (lane == 0) {
             const int un = two_n - done;
@@ -617,6 +763,7 @@ static DecArgs dec_args(const vrprpd_instance* I, const DecPlan& D, int num, int
     a.p = I->p;
     a.smem_dist = D.smem_dist;
     a.d16 = I->d16;
+    a.err = I->err;
     // a decoded schedule is a precedence graph of the instance's ops, so no
     // time exceeds (2n+1) max d + n max p
     const long long bound = (2ll * I->n + 1) * I->maxd + static_cast<long long>(I->n) * I->maxp;
