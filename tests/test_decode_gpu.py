@@ -49,3 +49,18 @@ def test_decode_long_times(vrp, top, pmax, layout):
     p = rng.integers(0, pmax + 1, size=n).astype(np.int32)
     keys = rng.random((6, 4 * n if layout else 2 * n + m)).astype(np.float32)
     check(vrp, n, m, 8, 3, layout, keys, d=d, p=p)
+
+
+@pytest.mark.parametrize("pop,layout", [(2, 0), (63, 1), (65, 0), (2049, 1)])
+def test_generations_over_ranking_tiles(vrp, pop, layout):
+    # populations around the ranking's element groups and key tile: the last
+    # population and every generation's best equal the oracle's
+    import workloads
+    w = workloads.make_instance(9, 2, 3, 2, "2x", seed=pop)
+    inst = vrp.Instance.from_workload(w)
+    oi = oracle.OracleInstance.from_workload(w)
+    g = vrp.brkga_run(inst, vrp.brkga_params(pop, 3, layout=layout), seed=5, final_keys=True)
+    o = oracle.brkga_run(oi, oracle.brkga_params(pop, 3, layout=layout), None, None, 5)
+    assert np.array_equal(g["trace"], o["trace"]) and g["best_fitness"] == o["best_fitness"]
+    assert np.array_equal(g["keys"].cpu().numpy().view(np.uint32), o["keys"].view(np.uint32))
+    assert np.array_equal(g["best_ops"], o["best_ops"])
