@@ -3759,11 +3759,11 @@ static int run_team(const vrprpd_instance* I, const vrprpd_solution* init, const
     DevBuf B;
     const size_t per_team = team_bytes(n, m, qcap, iters, dump);
     B.cap = per_team * R + 4096;
-    VRP_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&B.base), B.cap, stream));
+    VRP_CUDA(pool_alloc(reinterpret_cast<void**>(&B.base), B.cap, stream));
     auto cleanup = [&]() { cudaFreeAsync(B.base, stream); };
     unsigned* gbar = B.take<unsigned>(4);
     AlnsTeam* d_team = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d_team), sizeof(AlnsTeam) * R, stream);
+    cudaError_t e = pool_alloc(reinterpret_cast<void**>(&d_team), sizeof(AlnsTeam) * R, stream);
     if (e != cudaSuccess) { cleanup(); set_error("alns setup: %s", cudaGetErrorString(e)); return VRPRPD_ECUDA; }
     AlnsTeam t{};
     t.n = n;
@@ -3992,7 +3992,7 @@ int initial_solution_paper_tb(const vrprpd_instance* I, int32_t refine_rounds, v
     VRP_CHECK(alns_supported(I, &why), VRPRPD_EINVAL, "%s", why.c_str());
     const int n = I->n, m = I->m;
     int32_t* dops = nullptr;
-    VRP_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&dops), (2 * n + m + 1) * 4, stream));
+    VRP_CUDA(pool_alloc(reinterpret_cast<void**>(&dops), (2 * n + m + 1) * 4, stream));
     int32_t* doff = dops + 2 * n;
     int rc = construct_paper_device(I, dops, doff, stream);
     cudaError_t e = cudaSuccess;

@@ -845,39 +845,50 @@ extern "C" int vrprpd_brkga_run(const vrprpd_instance* I, const vrprpd_brkga_par
     VRP_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     // device buffers
     const size_t keys_b = static_cast<size_t>(pop) * L * 4;
-    std::vector<void*> allocs;
-    bool alloc_failed = false;
-    auto dalloc = [&](size_t bytes) -> void* {
-        void* p = nullptr;
-        if (cudaMallocAsync(&p, std::max<size_t>(bytes, 16), s) != cudaSuccess) {
-            alloc_failed = true;
-            return nullptr;
-        }
-        allocs.push_back(p);
+    char* mem = nullptr;
+    size_t used = 0;
+    auto take = [&](size_t bytes) {            // an offset first, a pointer once mem is there
+        char* p = mem ? mem + used : nullptr;
+        used += (bytes + 255) & ~static_cast<size_t>(255);
         return p;
     };
     auto cleanup = [&]() {
-        for (void* p : allocs) cudaFreeAsync(p, s);
+        if (mem) cudaFreeAsync(mem, s);
         cudaStreamSynchronize(s);
         cudaStreamDestroy(s);
     };
-    float* buf0 = static_cast<float*>(dalloc(keys_b));
-    float* buf1 = static_cast<float*>(dalloc(keys_b));
-    float* base = static_cast<float*>(dalloc(static_cast<size_t>(4) * L * 4));   // ALNS encoding + 3 seeds
-    int32_t* dops = static_cast<int32_t*>(dalloc(static_cast<size_t>(pop) * 2 * n * 4));
-    int32_t* doff = static_cast<int32_t*>(dalloc(static_cast<size_t>(pop) * (m + 1) * 4));
-    int32_t* zdec = static_cast<int32_t*>(dalloc(pop * 4));
-    int32_t* un = static_cast<int32_t*>(dalloc(pop * 4));
-    long long* fitd = static_cast<long long*>(dalloc(pop * 8));
-    int32_t* zev = static_cast<int32_t*>(dalloc(pop * 4));
-    uint32_t* stev = static_cast<uint32_t*>(dalloc(pop * 4));
-    int32_t* rank = static_cast<int32_t*>(dalloc(pop * 4));
-    long long* fit = static_cast<long long*>(dalloc(pop * 8));
-    long long* dtrace = static_cast<long long*>(dalloc(static_cast<size_t>(G) * 8));
-    BrkgaCtl* ctl = static_cast<BrkgaCtl*>(dalloc(sizeof(BrkgaCtl)));
-    int32_t* wops = static_cast<int32_t*>(dalloc(2 * n * 4));
-    int32_t* woff = static_cast<int32_t*>(dalloc((m + 1) * 4));
-    if (alloc_failed) { cleanup(); set_error("BRKGA: device allocation failed"); return VRPRPD_ENOMEM; }
+    float *buf0 = nullptr, *buf1 = nullptr, *base = nullptr;
+    int32_t *dops = nullptr, *doff = nullptr, *zdec = nullptr, *un = nullptr, *zev = nullptr, *rank = nullptr,
+            *wops = nullptr, *woff = nullptr;
+    uint32_t* stev = nullptr;
+    long long *fitd = nullptr, *fit = nullptr, *dtrace = nullptr;
+    BrkgaCtl* ctl = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {     // the total, then the pieces of one allocation
+        if (pass == 1 && pool_alloc(reinterpret_cast<void**>(&mem), used, s) != cudaSuccess) {
+            mem = nullptr;
+            cudaGetLastError();
+            cleanup();
+            set_error("BRKGA: device allocation failed");
+            return VRPRPD_ENOMEM;
+        }
+        used = 0;
+        buf0 = reinterpret_cast<float*>(take(keys_b));
+        buf1 = reinterpret_cast<float*>(take(keys_b));
+        base = reinterpret_cast<float*>(take(static_cast<size_t>(4) * L * 4));   // ALNS encoding + 3 seeds
+        dops = reinterpret_cast<int32_t*>(take(static_cast<size_t>(pop) * 2 * n * 4));
+        doff = reinterpret_cast<int32_t*>(take(static_cast<size_t>(pop) * (m + 1) * 4));
+        zdec = reinterpret_cast<int32_t*>(take(pop * 4));
+        un = reinterpret_cast<int32_t*>(take(pop * 4));
+        fitd = reinterpret_cast<long long*>(take(pop * 8));
+        zev = reinterpret_cast<int32_t*>(take(pop * 4));
+        stev = reinterpret_cast<uint32_t*>(take(pop * 4));
+        rank = reinterpret_cast<int32_t*>(take(pop * 4));
+        fit = reinterpret_cast<long long*>(take(pop * 8));
+        dtrace = reinterpret_cast<long long*>(take(static_cast<size_t>(G) * 8));
+        ctl = reinterpret_cast<BrkgaCtl*>(take(sizeof(BrkgaCtl)));
+        wops = reinterpret_cast<int32_t*>(take(2 * n * 4));
+        woff = reinterpret_cast<int32_t*>(take((m + 1) * 4));
+    }
     const unsigned long long key = stream_key(seed, RNG_STREAM_BRKGA), wkey = stream_key(seed, RNG_STREAM_WARM);
     BrkgaCtl c0{0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(ctl, &c0, sizeof(c0), cudaMemcpyHostToDevice, s);

@@ -18,6 +18,16 @@ void set_error(const char* fmt, ...);
 // so setting it per launch would race between host threads that launch the
 // same kernel with different sizes; the size a launch uses is its own.
 int ensure_smem_limit(const void* kernel);
+// Scratch of one call (or a served request's instance) from the library's own
+// pool of the current device, ordered on stream (instance.cu).
+cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t stream);
+// Instances and servers hold the pool; it goes with the last of them.
+void pool_hold();
+void pool_release();
+// vrprpd_instance_create and _destroy for a caller that has finished all work on
+// the instance when it destroys it, everything ordered on its own stream.
+int instance_create_on(const int32_t* coords, const int32_t* p, int32_t n, int32_t m, int32_t R, int32_t Q,
+                       uint32_t flags, cudaStream_t stream, vrprpd_instance** out);
 // The three-phase start and its refinement by a team of team_blocks CTAs (0:
 // chosen from n); the server passes each request's share (alns.cu).
 int initial_solution_paper_tb(const vrprpd_instance* I, int32_t refine_rounds, vrprpd_solution* out,
@@ -64,6 +74,8 @@ struct vrprpd_instance {
     int32_t n = 0, m = 0, R = 0, Q = 0;
     uint32_t flags = 0;
     int device = 0;
+    bool pooled = false;         // device arrays from the library's pool, ordered on stream
+    cudaStream_t stream = nullptr;
     int num_sms = 0;
     size_t smem_optin = 0;
     int32_t maxd = 0, maxp = 0;

@@ -80,7 +80,7 @@ static size_t request_bytes(const vrprpd_request& r) {
 static void serve_one(vrprpd_server* S, vrprpd_server::Req& q, cudaStream_t stream) {
     const vrprpd_request& r = q.r;
     vrprpd_instance* I = nullptr;
-    int rc = vrprpd_instance_create(q.coords.data(), q.p.data(), r.n, r.m, r.R, r.Q, r.flags, &I);
+    int rc = instance_create_on(q.coords.data(), q.p.data(), r.n, r.m, r.R, r.Q, r.flags, stream, &I);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -194,6 +194,7 @@ extern "C" int vrprpd_server_create(size_t mem_budget, int32_t max_active, vrprp
     S->budget = mem_budget;
     S->max_active = max_active;
     S->t0 = std::chrono::steady_clock::now();
+    pool_hold();
     for (int i = 0; i < max_active; ++i) S->workers.emplace_back(worker_main, S);
     *out = S;
     return VRPRPD_OK;
@@ -336,4 +337,5 @@ extern "C" void vrprpd_server_destroy(vrprpd_server* S) {
     S->cv_work.notify_all();
     for (auto& t : S->workers) t.join();
     delete S;
+    pool_release();
 }
