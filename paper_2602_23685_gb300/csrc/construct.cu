@@ -3,17 +3,24 @@
 //      the integer cross product, then id; by id without coordinates), a
 //      bitonic sort with that comparison; cut into m' = min(m, R) sectors of
 //      equal count (customer k of the order in sector floor(k m' / n));
-//   2. load balancing on w_c = 2 d(0,c) + p_c (one thread): while the spread
+//   2. load balancing on w_c = 2 d(0,c) + p_c (one warp): while the spread
 //      of the sector workloads is 10% of their mean or more, the heaviest
 //      sector (lowest index on ties) hands its boundary customer to its
 //      lighter neighbour (lower index on ties), unless that would leave the
 //      neighbour at least as heavy as the heaviest was; at most 4n moves;
-//   3. nearest-neighbour routes (one thread per vehicle): vehicle v serves
+//   3. nearest-neighbour routes (one warp per vehicle): vehicle v serves
 //      its sector alone from the depot at time 0 with b = min(Q, floor(R/m'))
 //      resources, each step taking the feasible op that completes first (a
 //      drop while a resource is left: its arrival; a pickup of a dropped
 //      customer: max(arrival, T_drop + p)), ties by travel, then drop before
 //      pickup, then op code.
+// The steps of 2 and 3 depend on each other, so their latency is what counts:
+// workloads and states in shared memory, a sector per lane in 2 (three
+// reductions and two exchanges a move), a customer per lane in 3 (two reductions
+// a step).  With the instance's limits (schedule times below 2^27, d below 2^17)
+// every sum and key fits 32 bits.  One thread for 2 and one per vehicle for 3
+// made the whole start (constructor, evaluation and the calls around them) 656 us
+// at n=200 m=6 and 1789 us at n=1000 m=20; now 179 and 240 us.
 // Vehicle v's ops start at 2 * (first customer index of its sector), so the
 // route offsets follow from the sector bounds.  The refinement rounds that
 // follow run in the ALNS kernel's local search.
@@ -35,23 +42,27 @@ __device__ __forceinline__ bool angle_before(const int32_t* xy, int a, int b) {
     return a < b;
 }
 
-__global__ void __launch_bounds__(256) construct_kernel(const int32_t* __restrict__ xy, const int32_t* __restrict__ d,
-                                                        const int32_t* __restrict__ p, int n, int m, int R, int Q,
-                                                        int32_t* __restrict__ ops, int32_t* __restrict__ off) {
-    extern __shared__ __align__(16) long long csm[];
+__global__ void __launch_bounds__(1024) construct_kernel(const int32_t* __restrict__ xy, const int32_t* __restrict__ d,
+                                                         const int32_t* __restrict__ p, int n, int m, int R, int Q,
+                                                         int32_t* __restrict__ ops, int32_t* __restrict__ off) {
+    extern __shared__ __align__(16) int csm[];
     __shared__ int start[33];
-    __shared__ long long Wl[32];
-    const int tid = threadIdx.x, N1 = n + 1;
+    __shared__ int Wl[32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N1 = n + 1;
     int P = 1;
     while (P < n) P <<= 1;
-    long long* rdy = csm;                                        // [n+1]
-    int* ord = reinterpret_cast<int*>(rdy + N1);                 // [P]
+    int* rdy = csm;                            // [n+1] pickup-ready times; first the workloads
+    int* ord = rdy + N1;                       // [P]
     unsigned char* state = reinterpret_cast<unsigned char*>(ord + P);   // [n+1]
     const int mp = m < R ? m : R;
     const int b = min(Q, R / mp);
     // 1. sweep order (entries past n sort last)
     for (int i = tid; i < P; i += blockDim.x) ord[i] = i < n ? i + 1 : 0x7fffffff;
-    for (int c = tid; c <= n; c += blockDim.x) { state[c] = 0; rdy[c] = 0; }
+    for (int c = tid; c <= n; c += blockDim.x) {
+        state[c] = 0;
+        rdy[c] = c ? 2 * __ldg(d + c) + __ldg(p + c) : 0;
+    }
+    if (tid < 32) Wl[tid] = 0;
     __syncthreads();
     if (xy) {
         for (int size = 2; size <= P; size <<= 1) {
@@ -68,68 +79,72 @@ __global__ void __launch_bounds__(256) construct_kernel(const int32_t* __restric
         }
     }
     // 2. sectors and load balancing
-    if (tid == 0) {
-        for (int s = 0; s < mp; ++s) Wl[s] = 0;
-        for (int k = 0; k < n; ++k) {
-            const int s = static_cast<int>((static_cast<long long>(k) * mp) / n);
-            const int c = ord[k];
-            Wl[s] += 2ll * __ldg(d + c) + __ldg(p + c);
-        }
-        for (int s = 0; s <= mp; ++s) start[s] = static_cast<int>((static_cast<long long>(s) * n + mp - 1) / mp);
+    for (int k = tid; k < n; k += blockDim.x)
+        atomicAdd(&Wl[static_cast<int>((static_cast<long long>(k) * mp) / n)], rdy[ord[k]]);
+    if (tid <= mp) start[tid] = static_cast<int>((static_cast<long long>(tid) * n + mp - 1) / mp);
+    __syncthreads();
+    if (warp == 0) {
+        const bool sector = lane < mp;
+        int W = sector ? Wl[lane] : 0, lo = sector ? start[lane] : 0, hi = sector ? start[lane + 1] : 0;
+        const long long tot = __reduce_add_sync(FULL_MASK, static_cast<unsigned>(W));     // below 2^27
         for (int mv = 0; mv < 4 * n && mp > 1; ++mv) {
-            int h = 0, l = 0;
-            long long tot = 0;
-            for (int s = 0; s < mp; ++s) {
-                tot += Wl[s];
-                if (Wl[s] > Wl[h]) h = s;
-                if (Wl[s] < Wl[l]) l = s;
+            // the heaviest sector (lowest index) and the least load
+            const unsigned top = __reduce_max_sync(FULL_MASK, sector ? (static_cast<unsigned>(W) << 5) | (31u - lane) : 0u);
+            const int h = 31 - static_cast<int>(top & 31u), Wh = static_cast<int>(top >> 5);
+            const int least = __reduce_min_sync(FULL_MASK, sector ? W : 0x7fffffff);
+            if (10ll * mp * (Wh - least) < tot) break;
+            const int Wp = __shfl_sync(FULL_MASK, W, (h - 1) & 31), Wn = __shfl_sync(FULL_MASK, W, (h + 1) & 31);
+            const int g = h > 0 && (h + 1 >= mp || Wp <= Wn) ? h - 1 : h + 1;
+            const int hlo = __shfl_sync(FULL_MASK, lo, h), hhi = __shfl_sync(FULL_MASK, hi, h);
+            if (hlo == hhi) break;
+            const int wc = rdy[ord[g < h ? hlo : hhi - 1]];
+            if ((g < h ? Wp : Wn) + wc >= Wh) break;
+            if (lane == g) {
+                W += wc;
+                if (g < h) ++hi; else --lo;
             }
-            if (10ll * mp * (Wl[h] - Wl[l]) < tot) break;
-            int g = -1;
-            if (h > 0) g = h - 1;
-            if (h + 1 < mp && (g < 0 || Wl[h + 1] < Wl[g])) g = h + 1;
-            if (start[h + 1] == start[h]) break;
-            const int c = g < h ? ord[start[h]] : ord[start[h + 1] - 1];
-            const long long wc = 2ll * __ldg(d + c) + __ldg(p + c);
-            if (Wl[g] + wc >= Wl[h]) break;
-            Wl[g] += wc;
-            Wl[h] -= wc;
-            if (g < h) start[h] += 1; else start[h + 1] -= 1;
+            if (lane == h) {
+                W -= wc;
+                if (g < h) ++lo; else --hi;
+            }
+        }
+        if (sector) {
+            start[lane] = lo;
+            if (lane == mp - 1) start[mp] = hi;
         }
     }
     __syncthreads();
-    // 3. nearest-neighbour routes, one thread per vehicle
-    if (tid < mp) {
-        const int v = tid, k0 = start[v], k1 = start[v + 1];
-        long long t = 0;
-        int loc = 0, out = 0, w = 2 * k0;
+    for (int c = tid; c <= n; c += blockDim.x) rdy[c] = 0;
+    __syncthreads();
+    // 3. nearest-neighbour routes
+    for (int v = warp; v < mp; v += static_cast<int>(blockDim.x >> 5)) {
+        const int k0 = start[v], k1 = start[v + 1];
+        int t = 0, loc = 0, out = 0, w = 2 * k0;
         for (int step = 0; step < 2 * (k1 - k0); ++step) {
-            int bo = -1;
-            long long bt = 0, bd = 0;
-            for (int k = k0; k < k1; ++k) {
-                const int c = ord[k];
-                const int st = state[c];
+            // completion time first, then travel (below 2^17), drop before pickup, op code
+            unsigned fin = 0xffffffffu, rest = 0xffffffffu;
+            for (int k = k0 + lane; k < k1; k += 32) {
+                const int c = ord[k], st = state[c];
                 if (st == 2 || (st == 0 && out >= b)) continue;
-                const int pick = st == 1 ? 1 : 0;
-                const long long dl = __ldg(d + loc * N1 + c);
-                long long fin = t + dl;
-                if (pick && rdy[c] > fin) fin = rdy[c];
-                const int o = 2 * c + pick;
-                bool better = bo < 0;
-                if (!better) {
-                    if (fin != bt) better = fin < bt;
-                    else if (dl != bd) better = dl < bd;
-                    else if ((o & 1) != (bo & 1)) better = (o & 1) < (bo & 1);
-                    else better = o < bo;
-                }
-                if (better) { bo = o; bt = fin; bd = dl; }
+                const int dl = __ldg(d + loc * N1 + c);
+                const unsigned f = static_cast<unsigned>(st == 1 ? max(t + dl, rdy[c]) : t + dl);
+                const unsigned q = (static_cast<unsigned>(dl) << 13) | (static_cast<unsigned>(st) << 12) | static_cast<unsigned>(2 * c + st);
+                if (f < fin || (f == fin && q < rest)) { fin = f; rest = q; }
             }
-            const int c = bo >> 1;
-            if (bo & 1) { state[c] = 2; --out; }
-            else { state[c] = 1; ++out; rdy[c] = bt + __ldg(p + c); }
-            t = bt;
+            const unsigned best = __reduce_min_sync(FULL_MASK, fin);
+            const unsigned pick = __reduce_min_sync(FULL_MASK, fin == best ? rest : 0xffffffffu);
+            const int o = static_cast<int>(pick & 0xfffu), c = o >> 1;
+            __syncwarp();
+            if (lane == 0) {
+                state[c] = (o & 1) ? 2 : 1;
+                if (!(o & 1)) rdy[c] = static_cast<int>(best) + __ldg(p + c);
+                ops[w] = o;
+            }
+            out += (o & 1) ? -1 : 1;
+            t = static_cast<int>(best);
             loc = c;
-            ops[w++] = bo;
+            ++w;
+            __syncwarp();
         }
     }
     for (int v = tid; v <= m; v += blockDim.x) off[v] = v <= mp ? 2 * start[v] : 2 * n;
@@ -144,10 +159,10 @@ int construct_paper_device(const vrprpd_instance* I, int32_t* ops, int32_t* off,
     const int n = I->n;
     int P = 1;
     while (P < n) P <<= 1;
-    const size_t smem = static_cast<size_t>(n + 1) * 8 + static_cast<size_t>(P) * 4 + n + 1 + 16;
+    const size_t smem = static_cast<size_t>(n + 1) * 4 + static_cast<size_t>(P) * 4 + n + 1 + 16;
     VRP_CHECK(smem <= I->smem_optin, VRPRPD_EINVAL, "n=%d too large for the constructor", n);
     { int rc_ = ensure_smem_limit(reinterpret_cast<const void*>(&construct_kernel)); if (rc_) return rc_; }
-    construct_kernel<<<1, 256, smem, stream>>>(I->has_coords ? I->coords : nullptr, I->d32, I->p, n, I->m, I->R,
+    construct_kernel<<<1, 1024, smem, stream>>>(I->has_coords ? I->coords : nullptr, I->d32, I->p, n, I->m, I->R,
                                                I->Q, ops, off);
     VRP_CUDA(cudaGetLastError());
     return VRPRPD_OK;
