@@ -71,7 +71,7 @@ constexpr long long REGRET_INF = 1ll << 40;
 
 struct AlnsCtl {
     int iter, q, nrem, di, rj;
-    int z_cur, z_best, z_work;
+    int z_cur, z_best, z_work, z_next;   // z_next: z_work after the insertion just selected
     unsigned st_work;
     int stagnation, repair_fail, wsel, err;
     int pick_t, pick_row, pick_col;
@@ -158,6 +158,7 @@ struct AlnsTeam {
     int* scpair;               // [SC_CAP][SC_CAP]: makespan with both stops in two shortcut gaps of one customer
     int* trace;
     int* gains;                // [n+1]: removal gain z(cur) - z(cur - c), worst removal; local search: places of the ops
+    double* pw;                // [n+1]: prefix sums of the worst removal's weights r^-6
     int* lscand;               // [n+1]: local-search candidates of the current pass
     int* dump_delta;
     int* dump_travel;
@@ -436,6 +437,38 @@ __device__ void walk_depot(const AlnsTeam& t, const Smem& s, int* rdy_, bool wri
     if (anycyc) ret = 0x7fffffff;
     *z_out = ret;
     *st_out = st;
+}
+
+// One warp: departures of the staged (acyclic) solution into H; its makespan.
+__device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
+    const int lane = threadIdx.x & 31, n = t.n;
+    volatile int* rdy = rdy_;
+    for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
+    __syncwarp();
+    int pos = lane < t.m ? s.sWoff[lane] : 0;
+    const int start = pos, end = lane < t.m ? s.sWoff[lane + 1] : 0;
+    int dep = 0, last = 0, x = pos < end ? s.sW[pos] : 0;
+    for (;;) {
+        const bool on = pos < end;
+        const int c = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0;
+        const bool pick = (x & 1) != 0;
+        const int r = on && pick ? rdy[c] : 0;
+        const bool go = on && (!pick || r != UNRES);
+        if (go) {
+            dep += x >> PACK_SHIFT;
+            if (pick) dep = max(dep, r);
+            else rdy[c] = dep + s.sp[c];
+            H[pos] = dep;
+            last = c;
+            x = nx;
+            ++pos;
+        }
+        __syncwarp();
+        if (!__any_sync(FULL_MASK, go)) break;
+    }
+    int ret = end > start ? dep + Dx(t, s, last, 0) : 0;
+    for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
+    return ret;
 }
 
 // From op u: row u of LP (NEG where unreachable) and T(u).  Up to two ops per
@@ -2014,6 +2047,8 @@ __device__ void phase_select(const AlnsTeam& t, const Smem& s) {
             sel[1] = pick;
             sel[2] = static_cast<int>(bestv[pick] & 0xFFF);
             sel[3] = colof(pick);
+            // the entry is exact: the makespan once it is inserted
+            ctl->z_next = ctl->z_work + static_cast<int>(static_cast<unsigned>(bestv[pick] >> 32) ^ 0x80000000u);
             ctl->pick_t = sel[1];
             ctl->pick_row = sel[2];
             ctl->pick_col = sel[3];
@@ -2130,6 +2165,25 @@ __device__ void block_sort(unsigned long long* a, int P) {
     }
 }
 
+// The prefix sums of r^-6, r = 1..n, in order, once per run (rank 0's block):
+// the quotients side by side, then one chain of additions.
+__device__ __noinline__ void worst_weights(const AlnsTeam& t, const Smem& s) {
+    double* x = reinterpret_cast<double*>(s.rdy);
+    for (int r = 1 + threadIdx.x; r <= t.n; r += blockDim.x) {
+        const double y = static_cast<double>(r), y2 = __dmul_rn(y, y);
+        x[r] = __ddiv_rn(1.0, __dmul_rn(__dmul_rn(y2, y2), y2));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double acc = 0.0;
+        for (int r = 1; r <= t.n; ++r) {
+            acc = __dadd_rn(acc, x[r]);
+            t.pw[r] = acc;
+        }
+    }
+    __syncthreads();
+}
+
 // The structured destroy operators (Section 4.2.2), rank 0's block: marks
 // s.flags[c] and leaves the count in ctl->q.  Rankings sort (key << 12 | c),
 // so ties go to the smaller customer id.  Draws: the operator's pick at
@@ -2152,11 +2206,7 @@ __device__ __noinline__ void select_structured(const AlnsTeam& t, const Smem& s)
     // facts of the current solution
     stage_ops(t, s, t.cur_ops, t.cur_off);
     const bool timed = di == D_SHAW || di == D_CRITICAL;
-    if (timed && warp == 0) {
-        int z;
-        unsigned st;
-        walk_depot(t, s, s.rdy, true, &z, &st);
-    }
+    if (timed && warp == 0) walk_heads(t, s, s.rdy, t.H);
     __syncthreads();
     const int N = s.sWoff[m];
     for (int k = tid; k < N; k += blockDim.x) {
@@ -2189,30 +2239,32 @@ __device__ __noinline__ void select_structured(const AlnsTeam& t, const Smem& s)
     if (di == D_WORST) {
         // removal gains from the team phase, largest first; q roulette draws
         // over the remaining ranked list with weight r^-6 on the r-th
-        double* pw = reinterpret_cast<double*>(keys + P);                         // [n+1] prefix weights
         for (int i = tid; i < P; i += blockDim.x)
             keys[i] = i < n ? ((static_cast<unsigned long long>((1ll << 30) - t.gains[i + 1]) << 12) |
                                static_cast<unsigned long long>(i + 1))
                             : KEY_NONE;
         block_sort(keys, P);
-        if (tid == 0) {
-            double acc = 0.0;
-            for (int r = 1; r <= n; ++r) {
-                const double x = static_cast<double>(r), x2 = __dmul_rn(x, x);
-                acc = __dadd_rn(acc, __ddiv_rn(1.0, __dmul_rn(__dmul_rn(x2, x2), x2)));
-                pw[r] = acc;
-            }
+        if (warp == 0) {
+            // the r-th weight's prefix first passes the target, then the r-th
+            // customer of the ranking still there, 32 at a time
             for (int k = 0; k < q; ++k) {
                 const int R = n - k;
-                const double target = __dmul_rn(draw_unit(draw(t.key, base + 16 + static_cast<unsigned long long>(k))), pw[R]);
-                int r = 1;
-                while (r < R && !(pw[r] > target)) ++r;
-                int seen = 0;
-                for (int i = 0; i < n; ++i) {
-                    const int c = static_cast<int>(keys[i] & 0xFFF);
-                    if (s.flags[c]) continue;
-                    if (++seen == r) { s.flags[c] = 1; break; }
+                const double target = __dmul_rn(draw_unit(draw(t.key, base + 16 + static_cast<unsigned long long>(k))), t.pw[R]);
+                int r = R;
+                for (int r0 = 1; r0 < R; r0 += 32) {
+                    const unsigned past = __ballot_sync(FULL_MASK, r0 + lane < R && t.pw[r0 + lane] > target);
+                    if (past) { r = r0 + __ffs(past) - 1; break; }
                 }
+                for (int i0 = 0; i0 < n; i0 += 32) {
+                    const int c = i0 + lane < n ? static_cast<int>(keys[i0 + lane] & 0xFFF) : 0;
+                    const bool there = i0 + lane < n && !s.flags[c];
+                    const unsigned left = __ballot_sync(FULL_MASK, there);
+                    const int cnt = __popc(left);
+                    if (r > cnt) { r -= cnt; continue; }
+                    if (there && __popc(left & ((1u << lane) - 1u)) == r - 1) s.flags[c] = 1;
+                    break;
+                }
+                __syncwarp();
             }
         }
     } else if (di == D_SHAW || di == D_CLUSTER) {
@@ -2240,6 +2292,27 @@ __device__ __noinline__ void select_structured(const AlnsTeam& t, const Smem& s)
         take_sorted(q - 1);
     } else {
         // a random non-empty route, or the bottleneck route's customers
+        if (di == D_CRITICAL && warp == 0) {
+            // latest return, the lower index on ties (times stay below 2^27); its
+            // customers in customer order
+            int rv = 0;
+            if (lane < m && s.sWoff[lane + 1] > s.sWoff[lane]) {
+                const int last = s.sWoff[lane + 1] - 1;
+                rv = t.H[last] + Dx(t, s, (s.sW[last] & PACK_MASK) >> 1, 0);
+            }
+            const unsigned top = __reduce_max_sync(FULL_MASK, lane < m ? (static_cast<unsigned>(rv) << 5) | (31u - lane) : 0u);
+            const int vb = 31 - static_cast<int>(top & 31u);
+            int nl = 0;
+            for (int c0 = 1; c0 <= n; c0 += 32) {
+                const int c = c0 + lane;
+                const bool on = c <= n && (vd[c] == vb || vp[c] == vb);
+                const unsigned bal = __ballot_sync(FULL_MASK, on);
+                if (on) lst[nl + __popc(bal & ((1u << lane) - 1u))] = c;
+                nl += __popc(bal);
+            }
+            if (lane == 0) sh[2] = nl;
+        }
+        __syncthreads();
         if (tid == 0) {
             if (di == D_ROUTE) {
                 int K = 0;
@@ -2250,21 +2323,8 @@ __device__ __noinline__ void select_structured(const AlnsTeam& t, const Smem& s)
                     if (s.sWoff[v + 1] > s.sWoff[v] && kk-- == 0) { vsel = v; break; }
                 sh[0] = vsel;
             } else {
-                // latest return, the lower index on ties; q of its customers by
-                // partial Fisher-Yates in customer order (all if fewer)
-                long long best = -1;
-                int vb = 0;
-                for (int v = 0; v < m; ++v) {
-                    long long rv = 0;
-                    if (s.sWoff[v + 1] > s.sWoff[v]) {
-                        const int last = s.sWoff[v + 1] - 1;
-                        rv = static_cast<long long>(t.H[last]) + Dx(t, s, (s.sW[last] & PACK_MASK) >> 1, 0);
-                    }
-                    if (rv > best) { best = rv; vb = v; }
-                }
-                int nl = 0;
-                for (int c = 1; c <= n; ++c)
-                    if (vd[c] == vb || vp[c] == vb) lst[nl++] = c;
+                // q of the listed customers by partial Fisher-Yates (all if fewer)
+                const int nl = sh[2];
                 const int take = q < nl ? q : nl;
                 for (int k = 0; k < take; ++k) {
                     const int jj = k + draw_below(draw(t.key, base + 16 + static_cast<unsigned long long>(k)), nl - k);
@@ -2391,6 +2451,7 @@ __device__ __noinline__ void phase_begin(const AlnsTeam& t, const Smem& s) {
     if (ctl->di != D_RANDOM) select_structured(t, s);
     if (threadIdx.x == 0) {
         ctl->repair_fail = 0;
+        ctl->z_next = ctl->z_cur;              // should nothing be removed
         ctl->n_short = 0;
         ctl->work_counter = 0;
         ctl->wsel = 0;
@@ -2420,16 +2481,56 @@ __device__ __noinline__ void phase_begin(const AlnsTeam& t, const Smem& s) {
 __device__ __noinline__ void phase_end(const AlnsTeam& t, const Smem& s, bool first) {
     AlnsCtl* ctl = t.ctl;
     const int n = t.n, m = t.m;
-    stage_W(t, s);
-    int* rdy = s.rdy;
-    if ((threadIdx.x >> 5) == 0) {
-        int z;
-        unsigned st;
-        walk_depot(t, s, rdy, false, &z, &st);
-        if ((threadIdx.x & 31) == 0) {
-            if (ctl->repair_fail) { z = 0x7fffffff; st = VRPRPD_MALFORMED; }
-            ctl->z_work = z;
-            ctl->st_work = st;
+    if (first) {
+        stage_W(t, s);
+        if ((threadIdx.x >> 5) == 0) {
+            int z;
+            unsigned st;
+            walk_depot(t, s, s.rdy, false, &z, &st);
+            if ((threadIdx.x & 31) == 0) {
+                ctl->z_work = z;
+                ctl->st_work = st;
+            }
+        }
+    } else {
+        // the last insertion left the makespan; the stock is what it did not
+        // judge as a whole (no insertion closes a cycle)
+        int* sh = s.misc + 32;                 // start loads, vehicles over capacity
+        if (threadIdx.x == 0) { sh[0] = 0; sh[1] = 0; }
+        __syncthreads();
+        const int* W = t.W_ops[ctl->wsel];
+        const int* Wo = t.W_off[ctl->wsel];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int r = warp; r < m && !ctl->repair_fail; r += ALNS_WARPS) {
+            const int en = Wo[r + 1];
+            int carry = 0, mn = 0, mx = 0;
+            for (int base = Wo[r]; base < en; base += 32) {
+                const bool in = base + lane < en;
+                int v = in ? ((W[base + lane] & 1) ? 1 : -1) : 0;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL_MASK, v, o);
+                    if (lane >= o) v += y;
+                }
+                if (in) {
+                    mn = min(mn, carry + v);
+                    mx = max(mx, carry + v);
+                }
+                carry += __shfl_sync(FULL_MASK, v, 31);
+            }
+            mn = __reduce_min_sync(FULL_MASK, mn);
+            mx = __reduce_max_sync(FULL_MASK, mx);
+            int load = 0;
+            const bool ok = cap_ok(t, mn, mx, load);
+            if (lane == 0) {
+                atomicAdd(&sh[0], load);
+                if (!ok) sh[1] = 1;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            ctl->z_work = ctl->repair_fail ? 0x7fffffff : ctl->z_next;
+            ctl->st_work = ctl->repair_fail ? VRPRPD_MALFORMED
+                                            : (sh[1] ? VRPRPD_VEH_CAP : 0u) | (sh[0] > t.R ? VRPRPD_POOL : 0u);
         }
     }
     __syncthreads();
@@ -2665,9 +2766,7 @@ __device__ __noinline__ void ls_candidates(const AlnsTeam& t, const Smem& s, int
     uint16_t* place = reinterpret_cast<uint16_t*>(t.gains);   // [2n+2] by op code
     for (int c = tid; c <= n; c += blockDim.x) s.flags[c] = 0;
     if (warp == 0) {
-        int z;
-        unsigned st;
-        walk_depot(t, s, s.rdy, true, &z, &st);
+        walk_heads(t, s, s.rdy, t.H);
         __syncwarp();
         int rv = 0;
         if (lane < m && s.sWoff[lane + 1] > s.sWoff[lane]) {
@@ -2740,38 +2839,6 @@ __device__ void stage_without(const AlnsTeam& t, const Smem& s, int lo, int hi) 
         W[k] = (Dx(t, s, prev, o >> 1) << PACK_SHIFT) | o;
     }
     __syncthreads();
-}
-
-// One warp: departures of the staged (acyclic) solution into H; its makespan.
-__device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
-    const int lane = threadIdx.x & 31, n = t.n;
-    volatile int* rdy = rdy_;
-    for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
-    __syncwarp();
-    int pos = lane < t.m ? s.sWoff[lane] : 0;
-    const int start = pos, end = lane < t.m ? s.sWoff[lane + 1] : 0;
-    int dep = 0, last = 0, x = pos < end ? s.sW[pos] : 0;
-    for (;;) {
-        const bool on = pos < end;
-        const int c = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0;
-        const bool pick = (x & 1) != 0;
-        const int r = on && pick ? rdy[c] : 0;
-        const bool go = on && (!pick || r != UNRES);
-        if (go) {
-            dep += x >> PACK_SHIFT;
-            if (pick) dep = max(dep, r);
-            else rdy[c] = dep + s.sp[c];
-            H[pos] = dep;
-            last = c;
-            x = nx;
-            ++pos;
-        }
-        __syncwarp();
-        if (!__any_sync(FULL_MASK, go)) break;
-    }
-    int ret = end > start ? dep + Dx(t, s, last, 0) : 0;
-    for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
-    return ret;
 }
 
 // One warp: the tail of every staged op (longest path from its departure to
@@ -3426,6 +3493,7 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
         if (threadIdx.x == 0) ctl->wsel = 0;
         __syncthreads();
         phase_end(t, s, true);
+        if (t.mode == 0 && (t.destroy_mask & (1 << D_WORST))) worst_weights(t, s);
     }
     if (!team_barrier(ctl, team_blocks, gen)) return;
     if (t.mode == 2) {
@@ -3551,6 +3619,7 @@ static size_t team_bytes(int n, int m, int qmax, int iterations, bool dump) {
     add(static_cast<size_t>(SC_CAP) * (4 * N + 8), 4);
     add(static_cast<size_t>(SC_CAP) * SC_CAP, 4);
     add(std::max(iterations, 1), 4);
+    add(n + 1, 8);
     add(n + 1, 4);
     add(n + 1, 4);
     if (dump) { add(G * G, 4); add(G * G, 4); }
@@ -3592,6 +3661,7 @@ static void carve_team(AlnsTeam& t, DevBuf& B, int n, int m, int qmax, int itera
     t.scw = B.take<int>(static_cast<size_t>(SC_CAP) * (4 * N + 8));
     t.scpair = B.take<int>(static_cast<size_t>(SC_CAP) * SC_CAP);
     t.trace = B.take<int>(std::max(iterations, 1));
+    t.pw = B.take<double>(n + 1);
     t.gains = B.take<int>(n + 1);
     t.lscand = B.take<int>(n + 1);
     t.dump_delta = dump ? B.take<int>(G * G) : nullptr;
