@@ -471,65 +471,43 @@ __device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
     return ret;
 }
 
-// From op u: row u of LP (NEG where unreachable) and T(u).  Up to two ops per
-// lane per step; ready times have one writer (the dropping lane) and are read
-// volatile, so a pickup sees "unresolved" (and retries) or the final value,
-// and the __syncwarp closing each step makes every write of a step visible in
-// the next: a step in which no lane moves means a precedence cycle.
+// From op u: row u of LP (NEG where unreachable) and T(u).  One op per lane and
+// round; ready times have one writer (the dropping lane) and are read volatile,
+// so a pickup sees "unresolved" (and retries) or the final value, and the
+// __syncwarp closing each round makes every write of a round visible in the
+// next: a round in which no lane moves ends the walk, and a route not ended then
+// means a precedence cycle.  (Two ops a round, with every choice written out,
+// took more instructions: the preparation of a step 27.8 us at n=1000, 7 of 36
+// steps full, and 26.4 us now; 9.8 and 9.1 us at n=120.)
 __device__ void walk_source(const AlnsTeam& t, const Smem& s, int* rdy_, int u, int N) {
-    const int* __restrict__ sW = s.sW;
-    const int* __restrict__ spp = s.sp;
-
     const int lane = threadIdx.x & 31, m = t.m, n = t.n;
     volatile int* rdy = rdy_;
     for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
     __syncwarp();
-    const bool mine = lane < m;
-    int pos = mine ? s.sWoff[lane] : 0;
-    const int end = mine ? s.sWoff[lane + 1] : 0;
-    int val = NEG, last = 0;
+    int pos = lane < m ? s.sWoff[lane] : 0;
+    const int end = lane < m ? s.sWoff[lane + 1] : 0;
+    int val = NEG, last = 0, x = pos < end ? s.sW[pos] : 0;
     int* row = t.Ms + static_cast<long long>(u) * N;
-    bool walking = mine && pos < end;
-    // each step reads both candidate stops and both ready times first; a
-    // pickup right behind its own drop waits one step
-    bool alive = __any_sync(FULL_MASK, walking);
-    while (alive) {
-        const bool can1 = walking, can2 = walking && pos + 1 < end;
-        const int w1 = can1 ? sW[pos] : 0, w2 = can2 ? sW[pos + 1] : 0;
-        const int c1 = (w1 & PACK_MASK) >> 1, c2 = (w2 & PACK_MASK) >> 1;
-        const bool k1 = (w1 & 1) != 0, k2 = (w2 & 1) != 0;
-        const bool at1 = pos == u, at2 = pos + 1 == u;
-        const int r1 = (can1 && k1 && !at1) ? rdy[c1] : 0;
-        const int r2 = (can2 && k2 && !at2) ? rdy[c2] : 0;
-        const bool go1 = can1 && (!k1 || at1 || r1 != UNRES);
-        const bool go2 = go1 && can2 && (!k2 || at2 || r2 != UNRES);
-        int v1 = (val == NEG) ? NEG : val + (w1 >> PACK_SHIFT);
-        if (k1 && !at1) v1 = max(v1, r1);
-        if (at1) v1 = 0;
-        int v2 = (v1 == NEG) ? NEG : v1 + (w2 >> PACK_SHIFT);
-        if (k2 && !at2) v2 = max(v2, r2);
-        if (at2) v2 = 0;
-        if (go1) {
-            if (!k1) rdy[c1] = (v1 == NEG) ? NEG : v1 + spp[c1];
-            row[pos] = v1;
-            val = v1;
-            last = c1;
+    for (;;) {
+        const bool on = pos < end, at = pos == u;
+        const int c = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0, p = s.sp[c];
+        const bool pick = (x & 1) != 0;
+        int r = NEG;                           // (the source's own time is 0 whatever it waits for)
+        if (pick && !at) r = rdy[c];
+        const bool go = on && r != UNRES;
+        if (go) {
+            val = at ? 0 : max(val == NEG ? val : val + (x >> PACK_SHIFT), r);
+            if (!pick) rdy[c] = val == NEG ? val : val + p;
+            row[pos] = val;
+            last = c;
+            x = nx;
+            ++pos;
         }
-        if (go2) {
-            if (!k2) rdy[c2] = (v2 == NEG) ? NEG : v2 + spp[c2];
-            row[pos + 1] = v2;
-            val = v2;
-            last = c2;
-        }
-        pos += (go1 ? 1 : 0) + (go2 ? 1 : 0);
-        const bool more = pos < end;
-        const unsigned prog = __ballot_sync(FULL_MASK, go1);
-        if (walking && more && prog == 0u) atomicExch(&t.ctl->err, DEV_BAD_STATE);
-        walking = walking && more && prog != 0u;
         __syncwarp();
-        alive = prog != 0u && __any_sync(FULL_MASK, walking);
+        if (!__any_sync(FULL_MASK, go)) break;
     }
-    int tail = (mine && val != NEG) ? val + Dx(t, s, last, 0) : NEG;
+    if (pos < end) atomicExch(&t.ctl->err, DEV_BAD_STATE);
+    int tail = (lane < m && val != NEG) ? val + Dx(t, s, last, 0) : NEG;
     for (int o = 16; o > 0; o >>= 1) tail = max(tail, __shfl_xor_sync(FULL_MASK, tail, o));
     if (lane == 0) t.T[u] = tail;
 }
@@ -1062,10 +1040,8 @@ __device__ void phase_prep(const AlnsTeam& t, const Smem& s, int rank, int team_
     for (int r = team_warps - 1 - gw; r < t.m; r += team_warps) scan_route_stock(t, s, r);
     for (int unit = gw; !incr && unit <= N; unit += team_warps) {
         if (unit == 0) {
-            int z;
-            unsigned st;
-            walk_depot(t, s, rdy, true, &z, &st);
-            if ((threadIdx.x & 31) == 0) { ctl->z_work = z; ctl->st_work = st; }
+            const int z = walk_heads(t, s, rdy, t.H);
+            if ((threadIdx.x & 31) == 0) ctl->z_work = z;
         } else {
             walk_source(t, s, rdy, unit - 1, N);
         }
