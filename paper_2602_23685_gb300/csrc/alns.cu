@@ -439,34 +439,59 @@ __device__ void walk_depot(const AlnsTeam& t, const Smem& s, int* rdy_, bool wri
     *st_out = st;
 }
 
+// What one stop of a walk needs from shared memory, by shared-window addresses.
+// A round is a chain of dependent instructions, and through the generic pointers
+// of Smem the compiler reads those pointers again after every store of a ready
+// time: 0.19 us a round, and 0.08 us so (one warp, n = 1000, m = 20).
+struct WalkMem {
+    unsigned w, p, r;                          // packed ops, processing times, ready times (or tails)
+    __device__ __forceinline__ WalkMem(const Smem& s, const int* rdy) : w(smem_u32(s.sW)), p(smem_u32(s.sp)), r(smem_u32(rdy)) {}
+    static __device__ __forceinline__ int ld(unsigned a) {
+        int v;
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
+        return v;
+    }
+    static __device__ __forceinline__ void st(unsigned a, int v) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+    __device__ __forceinline__ int op(int pos) const { return ld(w + 4u * static_cast<unsigned>(pos)); }
+    // byte offset of the customer of packed op x in a per-customer array
+    static __device__ __forceinline__ unsigned at(int x) { return static_cast<unsigned>(x & (PACK_MASK & ~1)) << 1; }
+};
+constexpr int FREE = INT32_MIN + 1;            // "ready time" of a stop that waits for nothing
+// Rounds between two looks at whether any lane still moves: the vote is as long
+// as a shared-memory load, and rounds in which no lane moves change nothing.
+constexpr int WALK_ROUNDS = 4;
+
 // One warp: departures of the staged (acyclic) solution into H; its makespan.
 __device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
     const int lane = threadIdx.x & 31, n = t.n;
-    volatile int* rdy = rdy_;
-    for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
+    for (int c = lane; c <= n; c += 32) rdy_[c] = UNRES;
     __syncwarp();
+    const WalkMem M(s, rdy_);
     int pos = lane < t.m ? s.sWoff[lane] : 0;
     const int start = pos, end = lane < t.m ? s.sWoff[lane + 1] : 0;
-    int dep = 0, last = 0, x = pos < end ? s.sW[pos] : 0;
-    for (;;) {
-        const bool on = pos < end;
-        const int c = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0;
-        const bool pick = (x & 1) != 0;
-        const int r = on && pick ? rdy[c] : 0;
-        const bool go = on && (!pick || r != UNRES);
-        if (go) {
-            dep += x >> PACK_SHIFT;
-            if (pick) dep = max(dep, r);
-            else rdy[c] = dep + s.sp[c];
-            H[pos] = dep;
-            last = c;
-            x = nx;
-            ++pos;
+    int dep = 0, last = 0, x = pos < end ? M.op(pos) : 0;
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool pick = (x & 1) != 0;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = M.op(pos + 1);
+            const int r = pick ? rv : FREE;
+            const bool go = pos < end && r != UNRES;
+            const int d = max(dep + (x >> PACK_SHIFT), r);
+            if (go && !pick) M.st(M.r + ca, d + p);
+            if (go) H[pos] = d;
+            dep = go ? d : dep;
+            last = go ? x : last;
+            pos += go ? 1 : 0;
+            x = go ? (pos < end ? nx : 0) : x;
+            moved |= go;
+            __syncwarp();
         }
-        __syncwarp();
-        if (!__any_sync(FULL_MASK, go)) break;
-    }
-    int ret = end > start ? dep + Dx(t, s, last, 0) : 0;
+    } while (__any_sync(FULL_MASK, moved));
+    int ret = end > start ? dep + Dx(t, s, (last & PACK_MASK) >> 1, 0) : 0;
     for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
     return ret;
 }
@@ -475,152 +500,137 @@ __device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
 // round; ready times have one writer (the dropping lane) and are read volatile,
 // so a pickup sees "unresolved" (and retries) or the final value, and the
 // __syncwarp closing each round makes every write of a round visible in the
-// next: a round in which no lane moves ends the walk, and a route not ended then
+// next: rounds in which no lane moves end the walk, and a route not ended then
 // means a precedence cycle.  (Two ops a round, with every choice written out,
 // took more instructions: the preparation of a step 27.8 us at n=1000, 7 of 36
-// steps full, and 26.4 us now; 9.8 and 9.1 us at n=120.)
+// steps full; one op a round takes 24 us, bound by the row's scattered stores;
+// 9.8 and 8.3 us at n=120.)
 __device__ void walk_source(const AlnsTeam& t, const Smem& s, int* rdy_, int u, int N) {
     const int lane = threadIdx.x & 31, m = t.m, n = t.n;
-    volatile int* rdy = rdy_;
-    for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
+    for (int c = lane; c <= n; c += 32) rdy_[c] = UNRES;
     __syncwarp();
+    const WalkMem M(s, rdy_);
     int pos = lane < m ? s.sWoff[lane] : 0;
     const int end = lane < m ? s.sWoff[lane + 1] : 0;
-    int val = NEG, last = 0, x = pos < end ? s.sW[pos] : 0;
+    int val = NEG, last = 0, x = pos < end ? M.op(pos) : 0;
     int* row = t.Ms + static_cast<long long>(u) * N;
-    for (;;) {
-        const bool on = pos < end, at = pos == u;
-        const int c = (x & PACK_MASK) >> 1, nx = pos + 1 < end ? s.sW[pos + 1] : 0, p = s.sp[c];
-        const bool pick = (x & 1) != 0;
-        int r = NEG;                           // (the source's own time is 0 whatever it waits for)
-        if (pick && !at) r = rdy[c];
-        const bool go = on && r != UNRES;
-        if (go) {
-            val = at ? 0 : max(val == NEG ? val : val + (x >> PACK_SHIFT), r);
-            if (!pick) rdy[c] = val == NEG ? val : val + p;
-            row[pos] = val;
-            last = c;
-            x = nx;
-            ++pos;
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool pick = (x & 1) != 0, at = pos == u;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = M.op(pos + 1);
+            const int r = pick && !at ? rv : NEG;  // (the source's own time is 0 whatever it waits for)
+            const bool go = pos < end && r != UNRES;
+            const int via = max(val == NEG ? NEG : val + (x >> PACK_SHIFT), r);
+            const int v = at ? 0 : via;
+            if (go && !pick) M.st(M.r + ca, v == NEG ? NEG : v + p);
+            if (go) row[pos] = v;
+            val = go ? v : val;
+            last = go ? x : last;
+            pos += go ? 1 : 0;
+            x = go ? (pos < end ? nx : 0) : x;
+            moved |= go;
+            __syncwarp();
         }
-        __syncwarp();
-        if (!__any_sync(FULL_MASK, go)) break;
-    }
+    } while (__any_sync(FULL_MASK, moved));
     if (pos < end) atomicExch(&t.ctl->err, DEV_BAD_STATE);
-    int tail = (lane < m && val != NEG) ? val + Dx(t, s, last, 0) : NEG;
+    int tail = (lane < m && val != NEG) ? val + Dx(t, s, (last & PACK_MASK) >> 1, 0) : NEG;
     for (int o = 16; o > 0; o >>= 1) tail = max(tail, __shfl_xor_sync(FULL_MASK, tail, o));
     if (lane == 0) t.T[u] = tail;
+}
+
+// A route of the staged W with up to two new stops in it, as one sequence of
+// packed (travel-in << PACK_SHIFT | op) words: the new stops sit at places q0 < q1
+// (SEQ_NONE: not there), and a stop behind one has its leg from there.  A lane's
+// walk asks for the word of each place in turn, so the walks themselves are those
+// of W, one stop a round.
+constexpr int SEQ_NONE = 1 << 29;
+struct Seq {
+    int base, len, q0 = SEQ_NONE, q1 = SEQ_NONE;
+    int x0 = 0, y0 = 0, x1 = 0, y1 = 0;        // words of the new stops, and of the stops behind them
+    __device__ __forceinline__ int pos(int q) const { return base + q - (q > q0 ? 1 : 0) - (q > q1 ? 1 : 0); }
+    __device__ __forceinline__ int at(const WalkMem& M, int q) const {
+        int x = M.op(pos(max(q, 0)));
+        x = q >= 0 && q < len ? x : 0;
+        if (q == q0 + 1) x = y0;
+        if (q == q0) x = x0;
+        if (q == q1) x = x1;
+        if (q == q1 + 1) x = y1;
+        return x;
+    }
+};
+
+// lane's route with stop o1 at gap (a, i) and o2 at gap (b, j) (a < 0 or b < 0
+// leaves one out; o1 goes first when both share a gap)
+__device__ __forceinline__ Seq make_seq(const AlnsTeam& t, const Smem& s, int a, int i, int o1, int b, int j, int o2) {
+    const int lane = threadIdx.x & 31;
+    Seq u;
+    u.base = lane < t.m ? s.sWoff[lane] : 0;
+    const int L = lane < t.m ? s.sWoff[lane + 1] - u.base : 0;
+    u.len = L;
+    const bool va = lane == a, vb = lane == b;
+    if (va || vb) {
+        const int g0 = va ? i : j, v0 = va ? o1 : o2;
+        auto word = [&](int k) { return k < L ? s.sW[u.base + k] & PACK_MASK : 0; };
+        auto leg_in = [&](int op, int k) {     // op with its leg from W position k (the depot below 0)
+            return Dx(t, s, k >= 0 ? word(k) >> 1 : 0, op >> 1) << PACK_SHIFT | op;
+        };
+        auto behind = [&](int op, int k) { return Dx(t, s, op >> 1, word(k) >> 1) << PACK_SHIFT | word(k); };
+        u.q0 = g0;
+        u.x0 = leg_in(v0, g0 - 1);
+        u.y0 = behind(v0, g0);
+        u.len = L + 1;
+        if (va && vb) {
+            u.q1 = j + 1;
+            u.x1 = j == i ? Dx(t, s, o1 >> 1, o2 >> 1) << PACK_SHIFT | o2 : leg_in(o2, j - 1);
+            u.y1 = behind(o2, j);
+            u.len = L + 2;
+        }
+    }
+    return u;
 }
 
 // Forward simulation of W plus up to two stops, V1 (op code o1) at gap (a, i)
 // and V2 (op code o2) at gap (b, j); a < 0 or b < 0 leaves one out, and V1
 // goes first when both share a gap.  Returns the makespan (INT32_MAX on a
 // precedence cycle); with Hb non-null the departure of every W position goes
-// to Hb[pos] and V1's to *hv.  Up to two stops per lane per step (see
-// walk_source); the legs next to the new stops are read before the walk.
+// to Hb[pos] and V1's to *hv.  One stop per lane and round, the next one's word
+// read ahead: the 200 rounds of a solution with n = 1000, m = 20 take 15 us, and
+// 43 us with two stops a round and every choice between them written out.
 __device__ int walk_fwd(const AlnsTeam& t, const Smem& s, int* rdy_, int a, int i, int o1, int b, int j, int o2,
                         int* Hb, int* hv) {
-    const int* __restrict__ sW = s.sW;
-    const int* __restrict__ spp = s.sp;
-
-    const int lane = threadIdx.x & 31, m = t.m;
-    volatile int* rdy = rdy_;
-    const bool mine = lane < m;
-    const int base = mine ? s.sWoff[lane] : 0;
-    const int L = mine ? s.sWoff[lane + 1] - base : 0;
-    // this lane's stops in route order: (gap g0, op v0, leg in tv0, leg after ta0), then (g1, v1, tv1, ta1)
-    int nv = 0, g0 = -1, v0 = 0, g1 = -1, v1 = 0, f0 = 0;
-    if (mine) {
-        if (lane == a) { g0 = i; v0 = o1; f0 = 1; nv = 1; }
-        if (lane == b) {
-            if (nv == 0) { g0 = j; v0 = o2; nv = 1; }
-            else { g1 = j; v1 = o2; nv = 2; }
+    const WalkMem M(s, rdy_);
+    const Seq u = make_seq(t, s, a, i, o1, b, j, o2);
+    int q = 0, dep = 0, last = 0, h = 0, x = u.at(M, 0);
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool pick = (x & 1) != 0;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = u.at(M, q + 1);
+            const int r = pick ? rv : FREE;
+            const bool go = q < u.len && r != UNRES;
+            const int d = max(dep + (x >> PACK_SHIFT), r);
+            if (go && !pick) M.st(M.r + ca, d + p);
+            if (Hb != nullptr && go && q != u.q0 && q != u.q1) Hb[u.pos(q)] = d;
+            h = go && q == u.q0 ? d : h;
+            dep = go ? d : dep;
+            last = go ? x : last;
+            q += go ? 1 : 0;
+            x = go ? nx : x;
+            moved |= go;
+            __syncwarp();
         }
-    }
-    auto cust = [&](int k) { return (sW[base + k] & PACK_MASK) >> 1; };
-    int tv0 = 0, ta0 = 0, tv1 = 0, ta1 = 0;
-    if (nv >= 1) {
-        tv0 = Dx(t, s, g0 > 0 ? cust(g0 - 1) : 0, v0 >> 1);
-        if (nv == 2 && g1 == g0) {
-            tv1 = Dx(t, s, v0 >> 1, v1 >> 1);
-            ta1 = g1 < L ? Dx(t, s, v1 >> 1, cust(g1)) : 0;
-        } else {
-            ta0 = g0 < L ? Dx(t, s, v0 >> 1, cust(g0)) : 0;
-            if (nv == 2) {
-                tv1 = Dx(t, s, cust(g1 - 1), v1 >> 1);
-                ta1 = g1 < L ? Dx(t, s, v1 >> 1, cust(g1)) : 0;
-            }
-        }
-    }
-    int k = 0, vi = 0, dep = 0, loc = 0;
-    bool pv = false;                           // the previous stop was a new one
-    bool walking = mine && (L > 0 || nv > 0);
-    const bool any = walking;
-    bool cyc = false;
-    // the stop at state (W position kk, new stops done vv), its op and the leg into it
-    auto peek = [&](int kk, int vv, bool ppv, bool can, bool& virt, bool& real, int& w, int& op, int& leg) {
-        virt = can && vv < nv && kk == (vv == 0 ? g0 : g1);
-        real = can && !virt && kk < L;                     // never past the route
-        w = real ? sW[base + kk] : 0;
-        op = virt ? (vv == 0 ? v0 : v1) : (w & PACK_MASK);
-        leg = virt ? (vv == 0 ? tv0 : tv1) : (ppv ? (vv == 1 ? ta0 : ta1) : (w >> PACK_SHIFT));
-    };
-    // two stops per step: both located and both ready times read first
-    bool alive = __any_sync(FULL_MASK, walking);
-    while (alive) {
-        bool vr1, rl1, vr2, rl2;
-        int w1, op1, lg1, w2, op2, lg2;
-        peek(k, vi, pv, walking, vr1, rl1, w1, op1, lg1);
-        const bool can1 = vr1 || rl1;
-        const int kb = k + (rl1 ? 1 : 0), vb = vi + (vr1 ? 1 : 0);
-        peek(kb, vb, vr1, can1, vr2, rl2, w2, op2, lg2);
-        const bool can2 = vr2 || rl2;
-        const int c1 = op1 >> 1, c2 = op2 >> 1;
-        const bool p1 = (op1 & 1) != 0, p2 = (op2 & 1) != 0;
-        const int r1 = (can1 && p1) ? rdy[c1] : 0;
-        const int r2 = (can2 && p2) ? rdy[c2] : 0;
-        const bool go1 = can1 && (!p1 || r1 != UNRES);
-        const bool go2 = go1 && can2 && (!p2 || r2 != UNRES);
-        const int a1 = dep + lg1;
-        const int d1 = p1 ? max(a1, r1) : a1;
-        const int a2 = d1 + lg2;
-        const int d2 = p2 ? max(a2, r2) : a2;
-        if (go1) {
-            if (!p1) rdy[c1] = a1 + spp[c1];
-            if (Hb != nullptr) {
-                if (vr1) { if (vi == 0 && f0) *hv = d1; }
-                else Hb[base + k] = d1;
-            }
-            dep = d1;
-            loc = c1;
-        }
-        if (go2) {
-            if (!p2) rdy[c2] = a2 + spp[c2];
-            if (Hb != nullptr) {
-                if (vr2) { if (vb == 0 && f0) *hv = d2; }
-                else Hb[base + kb] = d2;
-            }
-            dep = d2;
-            loc = c2;
-            k = kb + (rl2 ? 1 : 0);
-            vi = vb + (vr2 ? 1 : 0);
-            pv = vr2;
-        } else if (go1) {
-            k = kb;
-            vi = vb;
-            pv = vr1;
-        }
-        const bool more = k < L || vi < nv;
-        const unsigned prog = __ballot_sync(FULL_MASK, go1);
-        if (walking && more && prog == 0u) cyc = true;
-        walking = walking && more && prog != 0u;
-        __syncwarp();
-        alive = prog != 0u && __any_sync(FULL_MASK, walking);
-    }
-    int ret = (mine && any && !cyc) ? dep + Dx(t, s, loc, 0) : 0;
+    } while (__any_sync(FULL_MASK, moved));
+    if (Hb != nullptr && static_cast<int>(threadIdx.x & 31) == a) *hv = h;
+    int ret = u.len > 0 ? dep + Dx(t, s, (last & PACK_MASK) >> 1, 0) : 0;
     for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
-    const unsigned anycyc = __ballot_sync(FULL_MASK, cyc);
-    return anycyc ? 0x7fffffff : ret;
+    return __any_sync(FULL_MASK, q < u.len) ? 0x7fffffff : ret;
 }
 
 // Full simulation of W + D_c at gap (a,i) + P_c at gap (b,j): makespan or
@@ -649,91 +659,39 @@ __device__ int walk_fwd1(const AlnsTeam& t, const Smem& s, int* rdy, int ov, int
 // The same graph backward: the tail of every W position (longest path from its
 // departure to the end of the schedule, return leg included) into Tb[pos] and
 // V's into *tv.  A drop's tail also takes p plus its pickup's tail; V has no
-// partner in this graph.  tp: per-customer pickup tails (n + 1 words).  Up to
-// two stops per lane per step, as in the forward walks.
+// partner in this graph.  tp: per-customer pickup tails (n + 1 words).
 __device__ void walk_bwd1(const AlnsTeam& t, const Smem& s, int* tp_, int ov, int a, int i, int* Tb, int* tv) {
-    const int* __restrict__ sW = s.sW;
-    const int* __restrict__ spp = s.sp;
-
-    const int lane = threadIdx.x & 31, m = t.m, n = t.n;
-    volatile int* tp = tp_;
-    for (int q = lane; q <= n; q += 32) tp[q] = UNRES;
+    const int lane = threadIdx.x & 31, n = t.n;
+    for (int c = lane; c <= n; c += 32) tp_[c] = UNRES;
     __syncwarp();
-    const bool mine = lane < m;
-    const int base = mine ? s.sWoff[lane] : 0;
-    const int L = mine ? s.sWoff[lane + 1] - base : 0;
-    const int gv = (mine && lane == a) ? i : -1;
-    const int vc = ov >> 1;
-    // legs next to V, read before the walk: V -> the stop after it, the stop before V -> V
-    int lv = 0, lb = 0;
-    if (gv >= 0) {
-        lv = Dx(t, s, vc, gv < L ? (sW[base + gv] & PACK_MASK) >> 1 : 0);
-        if (gv > 0) lb = Dx(t, s, (sW[base + gv - 1] & PACK_MASK) >> 1, vc);
-    }
-    const int lastleg = L > 0 ? Dx(t, s, (sW[base + L - 1] & PACK_MASK) >> 1, 0) : 0;
-    const int vret = gv >= 0 ? Dx(t, s, vc, 0) : 0;
-    // k: W position still to do (counting down); V sits between positions gv-1 and gv
-    int k = L - 1, acc = 0;
-    bool vdone = gv < 0, nvn = false, first = true;
-    bool walking = mine && (L > 0 || !vdone);
-    // the stop at state (kk, done), with "the next stop is V" / "no next stop" flags
-    auto peek = [&](int kk, bool done, bool nx, bool fst, bool can, bool& virt, bool& real, int& w, int& c, int& leg) {
-        virt = can && !done && kk == gv - 1;
-        real = can && !virt && kk >= 0;
-        w = real ? sW[base + kk] : 0;
-        c = virt ? vc : (w & PACK_MASK) >> 1;
-        if (virt) leg = fst ? vret : lv;
-        else if (fst) leg = lastleg;
-        else if (nx) leg = lb;
-        else leg = real ? (sW[base + kk + 1] >> PACK_SHIFT) : 0;
-    };
-    bool alive = __any_sync(FULL_MASK, walking);
-    while (alive) {
-        bool vr1, rl1, vr2, rl2;
-        int w1, c1, lg1, w2, c2, lg2;
-        peek(k, vdone, nvn, first, walking, vr1, rl1, w1, c1, lg1);
-        const bool can1 = vr1 || rl1;
-        const int kb = k - (rl1 ? 1 : 0);
-        const bool db = vdone || vr1;
-        peek(kb, db, vr1, false, can1, vr2, rl2, w2, c2, lg2);
-        const bool can2 = vr2 || rl2;
-        const bool dr1 = rl1 && !(w1 & 1), dr2 = rl2 && !(w2 & 1);
-        const int r1 = dr1 ? tp[c1] : 0;
-        const int r2 = dr2 ? tp[c2] : 0;
-        const bool go1 = can1 && (!dr1 || r1 != UNRES);
-        const bool go2 = go1 && can2 && (!dr2 || r2 != UNRES);
-        int t1 = lg1 + acc;
-        if (dr1) t1 = max(t1, spp[c1] + r1);
-        int t2 = lg2 + t1;
-        if (dr2) t2 = max(t2, spp[c2] + r2);
-        if (go1) {
-            if (rl1 && !dr1) tp[c1] = t1;
-            if (vr1) *tv = t1;
-            else Tb[base + k] = t1;
-            acc = t1;
+    const WalkMem M(s, tp_);
+    const Seq u = make_seq(t, s, a, i, ov, -1, 0, 0);
+    int q = u.len - 1, x = u.at(M, q), acc = 0, tl = 0;
+    int leg = q >= 0 ? Dx(t, s, (x & PACK_MASK) >> 1, 0) : 0;
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool virt = q == u.q0, pick = (x & 1) != 0, waits = !pick && !virt;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = u.at(M, q - 1);
+            const int r = waits ? rv : FREE;
+            const bool go = q >= 0 && r != UNRES;
+            const int after = acc + leg, d = waits ? max(after, p + r) : after;
+            if (go && pick && !virt) M.st(M.r + ca, d);
+            if (go && !virt) Tb[u.pos(q)] = d;
+            tl = go && virt ? d : tl;
+            acc = go ? d : acc;
+            leg = go ? x >> PACK_SHIFT : leg;
+            q -= go ? 1 : 0;
+            x = go ? nx : x;
+            moved |= go;
+            __syncwarp();
         }
-        if (go2) {
-            if (rl2 && !dr2) tp[c2] = t2;
-            if (vr2) *tv = t2;
-            else Tb[base + kb] = t2;
-            acc = t2;
-            k = kb - (rl2 ? 1 : 0);
-            vdone = db || vr2;
-            nvn = vr2;
-            first = false;
-        } else if (go1) {
-            k = kb;
-            vdone = db;
-            nvn = vr1;
-            first = false;
-        }
-        const bool more = k >= 0 || !vdone;
-        const unsigned prog = __ballot_sync(FULL_MASK, go1);
-        if (walking && more && prog == 0u) atomicExch(&t.ctl->err, DEV_BAD_STATE);
-        walking = walking && more && prog != 0u;
-        __syncwarp();
-        alive = prog != 0u && __any_sync(FULL_MASK, walking);
-    }
+    } while (__any_sync(FULL_MASK, moved));
+    if (lane == a) *tv = tl;
+    if (q >= 0) atomicExch(&t.ctl->err, DEV_BAD_STATE);
 }
 
 // ---------------------------------------------------------------------------
@@ -972,44 +930,42 @@ __device__ void phase_update(const AlnsTeam& t, const Smem& s, int rank, int tea
 // The stop after a skipped one is reached from the last kept stop (or the
 // depot); a route left empty returns at 0.  One stop per lane per step.
 __device__ int walk_skip(const AlnsTeam& t, const Smem& s, int* rdy_, int cx) {
-    const int lane = threadIdx.x & 31, m = t.m, n = t.n;
-    const int* __restrict__ sW = s.sW;
-    const int* __restrict__ spp = s.sp;
-    volatile int* rdy = rdy_;
-    for (int c = lane; c <= n; c += 32) rdy[c] = UNRES;
+    const int lane = threadIdx.x & 31, n = t.n;
+    for (int c = lane; c <= n; c += 32) rdy_[c] = c == cx ? FREE : UNRES;
     __syncwarp();
-    const bool mine = lane < m;
-    int pos = mine ? s.sWoff[lane] : 0;
-    const int end = mine ? s.sWoff[lane + 1] : 0;
-    int dep = 0, loc = 0;
-    bool skipped = false, any = false, cyc = false;
-    bool walking = mine && pos < end;
-    bool alive = __any_sync(FULL_MASK, walking);
-    while (alive) {
-        const int w = walking ? sW[pos] : 0;
-        const int c = (w & PACK_MASK) >> 1;
-        const bool pick = (w & 1) != 0, skip = walking && c == cx;
-        const int rv = (walking && pick && !skip) ? rdy[c] : 0;
-        const bool go = walking && (skip || !pick || rv != UNRES);
-        if (go && !skip) {
-            const int arr = dep + (skipped ? Dx(t, s, loc, c) : (w >> PACK_SHIFT));
-            if (pick) dep = max(arr, rv);
-            else { dep = arr; rdy[c] = arr + spp[c]; }
-            loc = c;
-            any = true;
+    const WalkMem M(s, rdy_);
+    int pos = lane < t.m ? s.sWoff[lane] : 0;
+    const int end = lane < t.m ? s.sWoff[lane + 1] : 0;
+    int dep = 0, last = 0, x = pos < end ? M.op(pos) : 0;
+    bool skipped = false;                      // the stop before is left out: the leg starts at last
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const int c = static_cast<int>(ca >> 2);
+            const bool pick = (x & 1) != 0, skip = c == cx;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = M.op(pos + 1);
+            const int r = pick ? rv : FREE;
+            const bool go = pos < end && r != UNRES;
+            int leg = x >> PACK_SHIFT;
+            if (skipped) leg = Dx(t, s, last, c);
+            const int d = max(dep + leg, r);
+            if (go && !pick && !skip) M.st(M.r + ca, d + p);
+            dep = go && !skip ? d : dep;
+            last = go && !skip ? c : last;
+            skipped = go ? skip : skipped;
+            pos += go ? 1 : 0;
+            x = go ? (pos < end ? nx : 0) : x;
+            moved |= go;
+            __syncwarp();
         }
-        if (go) { skipped = skip; ++pos; }
-        const bool more = pos < end;
-        const unsigned prog = __ballot_sync(FULL_MASK, go);
-        if (walking && more && prog == 0u) cyc = true;
-        walking = walking && more && prog != 0u;
-        __syncwarp();
-        alive = prog != 0u && __any_sync(FULL_MASK, walking);
-    }
-    int ret = (mine && any && !cyc) ? dep + Dx(t, s, loc, 0) : 0;
+    } while (__any_sync(FULL_MASK, moved));
+    // (last = 0: the route has no other stop)
+    int ret = last > 0 ? dep + Dx(t, s, last, 0) : 0;
     for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
-    const unsigned anycyc = __ballot_sync(FULL_MASK, cyc);
-    return anycyc ? 0x7fffffff : ret;
+    return __any_sync(FULL_MASK, pos < end) ? 0x7fffffff : ret;
 }
 
 // Worst removal's gains (Section 4.2.2): every CTA stages the current
@@ -1301,82 +1257,100 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
     if (rank == 0 && threadIdx.x == 0) t.ctl->work_counter = 0;
 }
 
+// route of gap g
+__device__ __forceinline__ int route_of_gap(const AlnsTeam& t, const Smem& s, int g) {
+    int lo = 0, hi = t.m;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (s.sWoff[mid] + mid <= g) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // Simulations of the shortcut gaps for the matrix phase: per shortcut gap g of
 // customer c the graph with D_c alone at g (forward, backward) and with P_c
 // alone at g (forward, backward); per pair of shortcut gaps of one customer (g
-// itself twice: the adjacent pair) W with both stops.  One warp per
-// simulation, handed out from the last CTA down.  They run between arriving
-// at the barrier before the matrix phase and waiting at it, so the tiles of
-// the other CTAs proceed meanwhile; every finished simulation is counted in
-// walks_done, which the shortcut items wait for.
-__device__ int gap_walk_items(const AlnsTeam& t) {
+// itself twice: the adjacent pair) W with both stops.  A CTA takes one graph of
+// a gap, a warp each way, or eight pairs, a warp each, handed out from the last
+// CTA down.  The walks leave their times in shared memory and the CTA copies
+// them out: stored by the walking lanes, every round to as many lines as there
+// are routes, a graph took 31 us at n = 1000, m = 20, and takes 22 us so.  The
+// units run between arriving at the barrier before the matrix phase and waiting
+// at it, so the tiles of the other CTAs proceed meanwhile; every finished one is
+// counted in walks_done, which the shortcut items wait for.
+__device__ int gap_walk_units(const AlnsTeam& t) {
     const int ns = min(t.ctl->n_short, SC_CAP);
-    return 4 * ns + ns * ns;
+    return 2 * ns + (ns * ns + ALNS_WARPS - 1) / ALNS_WARPS;
+}
+
+// both ways through W with one stop at gap (a, i), by warps 0 and 1: departures and tails
+// of the W positions into shared arrays behind the walk buffers, and the three scalars
+struct OneStop {
+    int *H, *T;
+};
+__device__ __forceinline__ OneStop walk_one_stop(const AlnsTeam& t, const Smem& s, int ov, int a, int i, int N,
+                                                 int* scal) {
+    const int rw = ((t.n + 1) + 3) & ~3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    OneStop r;
+    r.H = s.rdy + 2 * rw;
+    r.T = r.H + ((N + 3) & ~3);
+    if (warp == 0) {
+        int hv = 0;
+        const int z1 = walk_fwd1(t, s, s.rdy, ov, a, i, r.H, &hv);
+        if (lane == a) scal[1] = hv;
+        if (lane == 0) scal[0] = z1;
+    } else if (warp == 1) {
+        int tv = 0;
+        walk_bwd1(t, s, s.rdy + rw, ov, a, i, r.T, &tv);
+        if (lane == a) scal[2] = tv;
+    }
+    __syncthreads();
+    return r;
 }
 
 __device__ void gap_walks(const AlnsTeam& t, const Smem& s, int rank, int team_blocks) {
     const int m = t.m, N = s.sWoff[m], G = N + m;
-    {
-        AlnsCtl* ctl = t.ctl;
-        const int ns = min(ctl->n_short, SC_CAP);
-        const int nmax = (t.scw_stride - 8) / 4;
-        const int nitems = 4 * ns + ns * ns;
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const int team_warps = team_blocks * ALNS_WARPS;
-        const int gw = (team_blocks - 1 - rank) * ALNS_WARPS + warp;
-        int* rdy = s.rdy + warp * (((t.n + 1) + 3) & ~3);
-        auto route_of = [&](int g, int* pos) {
-            int lo = 0, hi = m;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (s.sWoff[mid] + mid <= g) lo = mid; else hi = mid;
+    AlnsCtl* ctl = t.ctl;
+    const int ns = min(ctl->n_short, SC_CAP), units = gap_walk_units(t);
+    const int nmax = (t.scw_stride - 8) / 4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto pos_of = [&](int g, int r) { return g - (s.sWoff[r] + r); };
+    for (int unit = team_blocks - 1 - rank; unit < units; unit += team_blocks) {
+        if (unit < 2 * ns) {
+            const int e = unit >> 1, as_col = unit & 1;
+            const int packed = t.slist[e], ti = packed / G, g = packed - ti * G;
+            const int r = route_of_gap(t, s, g);
+            int* base = t.scw + static_cast<long long>(e) * t.scw_stride;
+            const OneStop w = walk_one_stop(t, s, 2 * t.rem[ti] + as_col, r, pos_of(g, r), N, base + 4 * nmax + as_col * 3);
+            int* Hb = base + as_col * 2 * nmax;
+            for (int k = threadIdx.x; k < N; k += blockDim.x) {
+                Hb[k] = w.H[k];
+                Hb[nmax + k] = w.T[k];
             }
-            *pos = g - (s.sWoff[lo] + lo);
-            return lo;
-        };
-        for (int item = gw; item < nitems; item += team_warps) {
-            if (item < 4 * ns) {
-                const int e = item >> 2, kind = item & 3;
-                const int packed = t.slist[e], ti = packed / G, g = packed - ti * G;
-                const int c = t.rem[ti];
-                int pos = 0;
-                const int r = route_of(g, &pos);
-                int* base = t.scw + static_cast<long long>(e) * t.scw_stride;
-                int* Hb = base + (kind >> 1) * 2 * nmax;
-                int* scal = base + 4 * nmax + (kind >> 1) * 3;
-                const int ov = 2 * c + (kind >> 1);
-                if ((kind & 1) == 0) {
-                    int hv = 0;
-                    const int z1 = walk_fwd1(t, s, rdy, ov, r, pos, Hb, &hv);
-                    if (lane == r) scal[1] = hv;
-                    if (lane == 0) scal[0] = z1;
-                } else {
-                    int tv = 0;
-                    walk_bwd1(t, s, rdy, ov, r, pos, Hb + nmax, &tv);
-                    if (lane == r) scal[2] = tv;
-                }
-            } else {
-                const int q = item - 4 * ns, e1 = q / ns, e2 = q - e1 * ns;
+        } else {
+            const int q = (unit - 2 * ns) * ALNS_WARPS + warp;
+            if (q < ns * ns) {
+                const int e1 = q / ns, e2 = q - e1 * ns;
                 const int p1 = t.slist[e1], p2 = t.slist[e2];
-                const int ti = p1 / G;
-                if (p2 / G != ti) { if (lane == 0) atomicAdd(&ctl->walks_done, 1); continue; }
-                int i1 = 0, i2 = 0;
-                const int r1 = route_of(p1 - ti * G, &i1), r2 = route_of(p2 - ti * G, &i2);
-                if (r1 == r2 && i2 < i1) {           // the pickup before the drop: never feasible
-                    if (lane == 0) atomicAdd(&ctl->walks_done, 1);
-                    continue;
+                const int ti = p1 / G, g1 = p1 - ti * G, g2 = p2 - ti * G;
+                if (p2 / G == ti) {
+                    const int r1 = route_of_gap(t, s, g1), r2 = route_of_gap(t, s, g2);
+                    const int i1 = pos_of(g1, r1), i2 = pos_of(g2, r2);
+                    if (r1 != r2 || i2 >= i1) {      // (the pickup before the drop: never feasible)
+                        const int zn = walk_insert(t, s, s.rdy + warp * (((t.n + 1) + 3) & ~3), t.rem[ti], r1, i1, r2, i2);
+                        if (lane == 0) t.scpair[e1 * SC_CAP + e2] = zn;
+                    }
                 }
-                const int zn = walk_insert(t, s, rdy, t.rem[ti], r1, i1, r2, i2);
-                if (lane == 0) t.scpair[e1 * SC_CAP + e2] = zn;
             }
-            // results visible device-wide, then counted
+        }
+        __syncthreads();
+        // results visible device-wide, then counted
+        if (threadIdx.x == 0) {
             __threadfence();
-            __syncwarp();
-            if (lane == 0) atomicAdd(&ctl->walks_done, 1);
+            atomicAdd(&ctl->walks_done, 1);
         }
     }
 }
-
 
 // One matrix tile (rows rt*TR.., cols ct*TC..) for every customer still to insert.
 //
@@ -1746,24 +1720,13 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
     const bool pre = e < SC_CAP;
     const int nmax = (t.scw_stride - 8) / 4;
     const int* pbase = t.scw + static_cast<long long>(pre ? e : 0) * t.scw_stride + as_col * 2 * nmax;
-    int* Hs = s.rdy + 2 * rw;                  // [N] departures in W + V (simulated here)
-    int* Ts = Hs + ((N + 3) & ~3);             // [N] tails in W + V
     int* sh = s.misc + 8;                      // z1, h_v, t_v
     const int ga = t.groute[g], gi = t.gpos[g];
     const int ov = 2 * c + as_col;
-    if (!pre && warp == 0) {
-        int hv = 0;
-        const int z1 = walk_fwd1(t, s, s.rdy, ov, ga, gi, Hs, &hv);
-        if (lane == ga) sh[1] = hv;
-        if (lane == 0) sh[0] = z1;
-    } else if (!pre && warp == 1) {
-        int tv = 0;
-        walk_bwd1(t, s, s.rdy + rw, ov, ga, gi, Ts, &tv);
-        if (lane == ga) sh[2] = tv;
-    }
-    __syncthreads();
-    const int* Hb = pre ? pbase : Hs;
-    const int* Tb = pre ? pbase + nmax : Ts;
+    OneStop own = {nullptr, nullptr};          // departures and tails in W + V, simulated here
+    if (!pre) own = walk_one_stop(t, s, ov, ga, gi, N, sh);
+    const int* Hb = pre ? pbase : own.H;
+    const int* Tb = pre ? pbase + nmax : own.T;
     const int* scal = pre ? t.scw + static_cast<long long>(e) * t.scw_stride + 4 * nmax + as_col * 3 : sh;
     const int z1 = scal[0], hv = scal[1], tv = scal[2];
     const int z = ctl->z_work, pc = s.sp[c];
@@ -1858,7 +1821,7 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s) {
     // time the phase starts (the team barrier before it waits for every walk).
     const int nfb = 2 * ctl->n_short * FB_SPLIT;
     const int total = tiles + nfb;
-    const int nwalks = gap_walk_items(t);
+    const int nwalks = gap_walk_units(t);
     bool walks_seen = false;
     int* slot = s.misc;
     // Tiles go out by their distance d = |ct - rt/2| from the diagonal (the
@@ -2863,35 +2826,38 @@ __device__ void stage_without(const AlnsTeam& t, const Smem& s, int lo, int hi) 
 // drop of c at dpos.  c > 0: c's pickup is not in the solution.
 __device__ void walk_tails(const AlnsTeam& t, const Smem& s, int* tp_, int* T, int c0, int dpos) {
     const int lane = threadIdx.x & 31, n = t.n;
-    volatile int* tp = tp_;
-    for (int c = lane; c <= n; c += 32) tp[c] = c0 > 0 && c == c0 ? TAIL_NONE : UNRES;
+    for (int c = lane; c <= n; c += 32) tp_[c] = c0 > 0 && c == c0 ? TAIL_NONE : UNRES;
     __syncwarp();
+    const WalkMem M(s, tp_);
     const int start = lane < t.m ? s.sWoff[lane] : 0;
     int pos = (lane < t.m ? s.sWoff[lane + 1] : 0) - 1;
-    int x = pos >= start ? s.sW[pos] : 0;
+    int x = pos >= start ? M.op(pos) : 0;
     int leg = pos >= start ? Dx(t, s, (x & PACK_MASK) >> 1, 0) : 0, acc = 0, mark = 0;
-    for (;;) {
-        const bool on = pos >= start;
-        const int c = (x & PACK_MASK) >> 1, nx = pos - 1 >= start ? s.sW[pos - 1] : 0;
-        const bool drop = !(x & 1);
-        const int r = on && drop ? tp[c] : 0;
-        const bool go = on && (!drop || r != UNRES);
-        if (go) {
-            acc += leg;
-            if (drop && r != TAIL_NONE) {
-                acc = max(acc, s.sp[c] + (r & TAIL_BITS));
-                mark |= r & ~TAIL_BITS;
-            }
-            if (pos == dpos) mark = TAIL_BITS + 1;
-            T[pos] = acc | mark;
-            if (!drop) tp[c] = acc | mark;
-            leg = x >> PACK_SHIFT;
-            x = nx;
-            --pos;
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool pick = (x & 1) != 0;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = M.op(max(pos - 1, 0));
+            const int r = pick ? TAIL_NONE : rv;   // (a drop of a customer without its pickup waits for nothing, as a pickup)
+            const bool go = pos >= start && r != UNRES;
+            const int after = acc + leg;
+            const int d = r == TAIL_NONE ? after : max(after, p + (r & TAIL_BITS));
+            int mk = mark | (r == TAIL_NONE ? 0 : r & ~TAIL_BITS);
+            if (pos == dpos) mk = TAIL_BITS + 1;
+            if (go) T[pos] = d | mk;
+            if (go && pick) M.st(M.r + ca, d | mk);
+            acc = go ? d : acc;
+            mark = go ? mk : mark;
+            leg = go ? x >> PACK_SHIFT : leg;
+            pos -= go ? 1 : 0;
+            x = go ? (pos >= start ? nx : 0) : x;
+            moved |= go;
+            __syncwarp();
         }
-        __syncwarp();
-        if (!__any_sync(FULL_MASK, go)) break;
-    }
+    } while (__any_sync(FULL_MASK, moved));
 }
 
 // One warp, route r of the staged solution: stock after every op, its running
