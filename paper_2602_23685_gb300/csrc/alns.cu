@@ -103,12 +103,18 @@ struct AlnsCtl {
     alignas(128) unsigned bar_gen;
     alignas(128) int work_counter;
     alignas(128) int walks_done;      // shortcut simulations finished in this greedy step
+    alignas(128) int tests_done;      // CTAs that have tested their share of the matrix tiles in this step
     alignas(128) int n_short;
     int sum_load;
     alignas(128) unsigned long long entries, fallback_entries;
     unsigned long long pruned;        // tile entries skipped by the bound (counted in entries too)
     unsigned long long tiles, tiles_pruned;  // matrix tiles run, and those with no customer left to score
 };
+
+// 32-bit words of one bit per matrix tile
+__host__ __device__ inline int tile_words(int G) {
+    return (((G + TR - 1) / TR) * ((G + TC - 1) / TC) + 31) / 32;
+}
 
 struct AlnsTeam {
     // instance
@@ -148,8 +154,9 @@ struct AlnsTeam {
     unsigned long long* keys;  // [q_max][G]: per drop gap, best (dz, dt, col)
     unsigned long long* rkeys; // [q_max][32]: per drop vehicle, best (dz, dt, row)
     unsigned long long* gmin;  // [q_max][4]: per vehicle group (v mod 4), best (dz, dt) seen so far
-    int4* bands;               // [q_max][band_stride]: per 32 gaps, least row x, row w, col x, col w
+    int4* bands;               // [bands][band_stride]: per 32 gaps and customer, least row x, row w, col x, col w
     int band_stride;
+    unsigned* tmask;           // [tile_words(G)]: tiles that passed the phase's first test, in the order they go out
     unsigned char* sc;         // [q_max][G]
     int* slist;                // [q_max * G] entries t * G + g
     int* scix;                 // [q_max][G]: index in slist of a shortcut (customer, gap)
@@ -175,6 +182,7 @@ struct Smem {
     int* rowv;      // [TR][RV]
     int* colv;      // [TC][CV]
     int* misc;      // 64 ints
+    unsigned long long* counts;  // entries, pruned entries, tiles, pruned tiles of this CTA
     unsigned char* flags;  // [n + 1] removed flags / route-start bits
     int* xy;        // coordinates [n + 1][2] (when staged)
 };
@@ -218,7 +226,7 @@ __host__ __device__ inline size_t alns_smem_words(int n, int m, bool with_coords
     w += ((m + 1) + 3) & ~3;
     w += ((n + 1) + 3) & ~3;
     w += rdy_words(n);
-    w += TR * RV + TC * CV + 64;
+    w += TR * RV + TC * CV + 64 + 8;
     w += ((n + 1 + 3) / 4 + 3) & ~3;
     if (with_coords) w += ((2 * (n + 1)) + 3) & ~3;   // coordinates
     return w;
@@ -234,6 +242,7 @@ __device__ inline Smem carve(int* base, int n, int m) {
     s.rowv = q; q += TR * RV;
     s.colv = q; q += TC * CV;
     s.misc = q; q += 64;
+    s.counts = reinterpret_cast<unsigned long long*>(q); q += 8;
     s.flags = reinterpret_cast<unsigned char*>(q);
     q += ((n + 1 + 3) / 4 + 3) & ~3;
     s.xy = q;
@@ -1197,7 +1206,7 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
             const unsigned cw = __reduce_min_sync(FULL_MASK, vc.x < SKIPV ? static_cast<unsigned>(vc.w) : 0xffffffffu);
             const int lane = threadIdx.x & 31;
             if (lane == 0)
-                t.bands[static_cast<long long>(ti) * t.band_stride + (g >> 5)] =
+                t.bands[static_cast<long long>(g >> 5) * t.band_stride + ti] =
                     make_int4(static_cast<int>(rx), static_cast<int>(rw), static_cast<int>(cx), static_cast<int>(cw));
             // adjacent entries per drop vehicle: the gaps of one warp lie on
             // consecutive routes, each reduced by the whole warp
@@ -1254,7 +1263,10 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
             }
         }
     }
-    if (rank == 0 && threadIdx.x == 0) t.ctl->work_counter = 0;
+    if (rank == 0 && threadIdx.x == 0) {
+        t.ctl->work_counter = 0;
+        t.ctl->tests_done = 0;
+    }
 }
 
 // route of gap g
@@ -1352,6 +1364,64 @@ __device__ void gap_walks(const AlnsTeam& t, const Smem& s, int rank, int team_b
     }
 }
 
+// Which customers can a matrix tile change the repair operator's pick for?
+// Every entry of a customer in the tile is at least
+//     (max(least row x, least col x), least row w + least col w)
+// over the tile's rows and columns (the band minima).  The pick needs per
+// customer the best entry (greedy) and, for regret-2 and regret-3, the
+// makespans of the best two or three drop vehicles.  The best of each vehicle
+// group so far bounds the best entry and those makespans from above; an entry
+// whose drop vehicle already has an entry of no larger makespan cannot change
+// that vehicle's makespan.  Regret-m needs every vehicle's best and skips only
+// tiles without an admissible entry.  The bounds only fall as tiles are
+// scored, so a customer left out once stays out.
+struct TileBounds {
+    int4 r, c0, c1;                            // band minima: rows, columns (two bands)
+    unsigned long long gm[4];                  // best per vehicle group so far
+    unsigned long long vbest;                  // largest best makespan among the tile's drop vehicles (regret)
+};
+
+// the bounds of customer slot ti in tile (rt, ct), whose rows have drop vehicles va0..va1
+__device__ __forceinline__ TileBounds tile_bounds(const AlnsTeam& t, int ti, int rt, int ct, int va0, int va1, int kind,
+                                                  int G) {
+    TileBounds b;
+    const int4* bp = t.bands + ti;
+    b.r = bp[static_cast<long long>(rt) * t.band_stride];
+    b.c0 = bp[static_cast<long long>(2 * ct) * t.band_stride];
+    b.c1 = make_int4(0, 0, 0x7fffffff, -1);
+    if (2 * ct + 1 < ((G + 31) >> 5)) b.c1 = bp[static_cast<long long>(2 * ct + 1) * t.band_stride];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b.gm[k] = t.gmin[ti * 4 + k];
+    b.vbest = 0;
+    if (kind == 1 || kind == 2)
+        for (int v = va0; v <= va1; ++v) b.vbest = max(b.vbest, t.rkeys[ti * 32 + v] >> 32);
+    return b;
+}
+
+__device__ __forceinline__ bool tile_matters(const TileBounds& b, int kind, int z) {
+    const int lzz = max(b.r.x, min(b.c0.z, b.c1.z));
+    if (lzz >= SKIPV) return false;
+    if (kind > 2) return true;
+    const unsigned llo = static_cast<unsigned>(b.r.y) + min(static_cast<unsigned>(b.c0.w), static_cast<unsigned>(b.c1.w));
+    const unsigned long long ldz = static_cast<unsigned>(lzz - z) ^ 0x80000000u;
+    if (((ldz << 20) | (llo >> 12)) <= min(min(b.gm[0], b.gm[1]), min(b.gm[2], b.gm[3]))) return true;   // may be the best entry
+    if (kind == 0) return false;
+    // the second (regret-2) or third (regret-3) least group makespan
+    unsigned long long d[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = b.gm[k] >> 20;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3 - i; ++j) {
+            const unsigned long long lo = min(d[j], d[j + 1]), hi = max(d[j], d[j + 1]);
+            d[j] = lo;
+            d[j + 1] = hi;
+        }
+    // may lower a drop vehicle's best makespan that counts
+    return ldz <= (kind == 1 ? d[1] : d[2]) && ldz < b.vbest;
+}
+
 // One matrix tile (rows rt*TR.., cols ct*TC..) for every customer still to insert.
 //
 // Whether a (drop gap, pickup gap) pair can take a customer at all does not
@@ -1377,47 +1447,16 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
     const bool dump = t.mode == 1;
     const int nrem = ctl->nrem;
     const int z = ctl->z_work;
-    // Which customers can this tile change the repair operator's pick for?
-    // Every entry of customer c here is at least
-    //     (max(least row x, least col x), least row w + least col w)
-    // over the tile's rows and columns (the band minima).  The pick needs
-    // per customer the best entry (greedy and the local search) and, for
-    // regret-2 and regret-3, the makespans of the best two or three drop
-    // vehicles.  The best of each vehicle group so far bounds the best entry
-    // and those makespans from above; an entry whose drop vehicle already has
-    // an entry of no larger makespan cannot change that vehicle's makespan.
-    // A customer none of whose entries here can matter is not scored.
-    // Regret-m needs every vehicle's best and skips only tiles without an
-    // admissible entry.  The tiles' own scores tighten the bounds as they go.
+    // only customers whose pick the tile can change are scored (tile_matters)
     const bool prune_on = !dump && nrem <= ACT_CAP;
     int* act = s.rdy + TILE_WORDS;             // [ACT_CAP] customers to score
     int* nact = s.misc + 12;
     if (tid == 0) *nact = 0;
-    int4 bnd_r = make_int4(0, 0, 0, 0), bnd_c0 = bnd_r, bnd_c1 = make_int4(0, 0, 0x7fffffff, -1);
-    unsigned long long gm[4] = {KEY_NONE, KEY_NONE, KEY_NONE, KEY_NONE};
     const bool mine = prune_on && tid < nrem;
     const int kind = ctl->rj;
-    // drop vehicles of the tile's rows: the routes of gaps r0 and min(G, r0 + TR) - 1
-    auto route_of_gap = [&](int g) {
-        int lo = 0, hi = t.m;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (s.sWoff[mid] + mid <= g) lo = mid; else hi = mid;
-        }
-        return lo;
-    };
-    const int va0 = route_of_gap(r0), va1 = route_of_gap(min(G, r0 + TR) - 1);
-    unsigned long long vbest = 0;              // largest best makespan among those vehicles (regret)
-    if (mine) {
-        const int4* bp = t.bands + static_cast<long long>(tid) * t.band_stride;
-        bnd_r = bp[rt];
-        bnd_c0 = bp[2 * ct];
-        if (2 * ct + 1 < ((G + 31) >> 5)) bnd_c1 = bp[2 * ct + 1];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) gm[k] = t.gmin[tid * 4 + k];
-        if (kind == 1 || kind == 2)
-            for (int v = va0; v <= va1; ++v) vbest = max(vbest, t.rkeys[tid * 32 + v] >> 32);
-    }
+    TileBounds bounds;
+    if (mine)
+        bounds = tile_bounds(t, tid, rt, ct, route_of_gap(t, s, r0), route_of_gap(t, s, min(G, r0 + TR) - 1), kind, G);
     __syncthreads();                           // the previous tile is done with rowc / colc and the vectors
     for (int e = tid; e < TR * (RV / 4) + TC * (CV / 4); e += blockDim.x) {
         if (e < TR * (RV / 4)) {
@@ -1435,33 +1474,7 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
             reinterpret_cast<int4*>(colc)[e2] = v;
         }
     }
-    if (mine) {
-        const int lzz = max(bnd_r.x, min(bnd_c0.z, bnd_c1.z));
-        const unsigned llo = static_cast<unsigned>(bnd_r.y) + min(static_cast<unsigned>(bnd_c0.w), static_cast<unsigned>(bnd_c1.w));
-        bool keep = lzz < SKIPV;
-        if (keep && kind <= 2) {
-            const unsigned long long ldz = static_cast<unsigned>(lzz - z) ^ 0x80000000u;
-            const unsigned long long u = min(min(gm[0], gm[1]), min(gm[2], gm[3]));
-            keep = ((ldz << 20) | (llo >> 12)) <= u;   // may be the best entry
-            if (!keep && kind > 0) {
-                // the second (regret-2) or third (regret-3) least group makespan
-                unsigned long long d[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) d[k] = gm[k] >> 20;
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3 - i; ++j) {
-                        const unsigned long long a = min(d[j], d[j + 1]), b = max(d[j], d[j + 1]);
-                        d[j] = a;
-                        d[j + 1] = b;
-                    }
-                // may lower a drop vehicle's best makespan that counts
-                keep = ldz <= d[kind] && ldz < vbest;
-            }
-        }
-        if (keep) act[atomicAdd(nact, 1)] = tid;
-    }
+    if (mine && tile_matters(bounds, kind, z)) act[atomicAdd(nact, 1)] = tid;
     __syncthreads();
     const int na = prune_on ? *nact : nrem;
     auto cust = [&](int i) { return prune_on ? act[i] : i; };
@@ -1493,23 +1506,16 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
     const bool row_ok = ra >= 0;               // all 8 lanes of a row agree; no early exit (shuffles below)
     const int R = r0 + r;
     const unsigned ncols = static_cast<unsigned>(max(0, min(TC / 8, (G - c0 - cb + 7) / 8)));  // this thread's columns < G
-    // every entry of the tile counts, scored or not
-    const unsigned local_entries = row_ok ? static_cast<unsigned>(nrem) * ncols : 0u;
-    const unsigned local_pruned = row_ok ? static_cast<unsigned>(nrem - na) * ncols : 0u;
-    auto count_entries = [&]() {
-        const unsigned we = __reduce_add_sync(FULL_MASK, local_entries);
-        const unsigned wp = __reduce_add_sync(FULL_MASK, local_pruned);
-        if ((tid & 31) == 0 && we) atomicAdd(&ctl->entries, static_cast<unsigned long long>(we));
-        if ((tid & 31) == 0 && wp) atomicAdd(&ctl->pruned, static_cast<unsigned long long>(wp));
-    };
+    // every entry of the tile counts, scored or not; in shared memory until the
+    // run ends
     if (tid == 0) {
-        atomicAdd(&ctl->tiles, 1ull);
-        if (na == 0) atomicAdd(&ctl->tiles_pruned, 1ull);
+        const unsigned long long each = static_cast<unsigned long long>(min(TR, G - r0)) * static_cast<unsigned>(min(TC, G - c0));
+        s.counts[0] += each * static_cast<unsigned>(nrem);
+        s.counts[1] += each * static_cast<unsigned>(nrem - na);
+        s.counts[2] += 1ull;
+        s.counts[3] += na == 0 ? 1ull : 0ull;
     }
-    if (na == 0) {                             // no customer left to score: no pair work either
-        count_entries();
-        return;
-    }
+    if (na == 0) return;                       // no customer left to score: no pair work either
     int lpv[TC / 8];
     int diag = -1;                             // column slot of the coinciding gap, if in this thread's set
     // both table reads of every pair first, as predicated loads all in flight
@@ -1627,10 +1633,7 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
     for (int q = tid; q < CB * TR; q += blockDim.x) rowbest[q] = KEY_NONE;
     // a tile with no surviving pair has nothing to compute (the adjacent
     // entries were scored with the gap vectors)
-    if (total == 0) {
-        count_entries();
-        return;
-    }
+    if (total == 0) return;
     for (int tb = 0; tb < na; tb += CB) {
         const int nb = min(CB, na - tb);
         __syncthreads();                       // the list and the row slots are ready; the previous batch is flushed
@@ -1687,7 +1690,6 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
             }
         }
     }
-    count_entries();
 }
 
 // Shortcut item: every entry with one shortcut gap g for customer c (the
@@ -1810,7 +1812,116 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
     if (lane == 0 && wc) atomicAdd(&ctl->fallback_entries, static_cast<unsigned long long>(wc));
 }
 
-__device__ void phase_matrix(const AlnsTeam& t, const Smem& s) {
+// Tiles go out by their distance d = |ct - rt/2| from the diagonal (the
+// column tile that holds the row band's own gaps): the entries near it
+// (drop and pickup on one route or on neighbouring ones) are where a
+// customer's best insertion usually lies, so their scores tighten the
+// bounds before the far tiles are reached.  Per d, the tiles left of the
+// diagonal (ct = rt/2 - d, rt = 2d..RT-1), then those right of it
+// (ct = rt/2 + d, rt = 0..2(CT-d)-1).
+__device__ __forceinline__ void tile_of(int item, int RT, int CT, int* prt, int* pct) {
+    if (item < RT) { *prt = item; *pct = item >> 1; return; }
+    item -= RT;
+    for (int d = 1; d < CT; ++d) {
+        const int nl = max(0, RT - 2 * d), nr = max(0, min(RT, 2 * (CT - d)));
+        if (item < nl) { *prt = 2 * d + item; *pct = (*prt >> 1) - d; return; }
+        item -= nl;
+        if (item < nr) { *prt = item; *pct = (item >> 1) + d; return; }
+        item -= nr;
+    }
+    *prt = -1;                                 // past the last tile
+    *pct = -1;
+}
+
+// First test of all tiles at once, a warp per tile: 95 in 100 tiles can change no
+// customer's pick, and a CTA found that out one tile after another, a trip to L2
+// for the tile's number, one for its bounds and a few block barriers each.  A
+// CTA's eight tests give one byte of the bit mask of the tiles to run; the CTAs
+// that simulate shortcut gaps (the last ones) test nothing.  Matrix and selection
+// of a step at n = 1000: 41.4
+// us without it and 36.3 with it (random removal), 57.1 and 51.0 (all removals).
+// Thread w keeps word w of the mask (rows and columns fit 12 bits, so there
+// are 128 x 64 tiles at most) and the number of bits in the words before it.
+struct TileMask {
+    int count, before;
+    unsigned word;
+};
+
+__device__ __noinline__ TileMask test_tiles(const AlnsTeam& t, const Smem& s, int rank, int testers, int G) {
+    AlnsCtl* ctl = t.ctl;
+    const int RT = (G + TR - 1) / TR, CT = (G + TC - 1) / TC;
+    const int nrem = ctl->nrem, kind = ctl->rj, z = ctl->z_work;
+    const int words = tile_words(G), groups = 4 * words, want = min(groups, testers);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int* flag = s.misc + 2;                    // [ALNS_WARPS]
+    for (int gr = rank; gr < groups && rank < testers; gr += testers) {
+        int rt = -1, ct = -1;
+        tile_of(gr * ALNS_WARPS + warp, RT, CT, &rt, &ct);
+        bool any = false;
+        if (rt >= 0) {
+            const int va0 = route_of_gap(t, s, rt * TR), va1 = route_of_gap(t, s, min(G, (rt + 1) * TR) - 1);
+            for (int ti = lane; ti < nrem; ti += 32)
+                any |= tile_matters(tile_bounds(t, ti, rt, ct, va0, va1, kind, G), kind, z);
+        }
+        any = __any_sync(FULL_MASK, any);
+        // to run: -1; else the tile's entries, none of them scored
+        if (lane == 0) flag[warp] = any ? -1 : rt >= 0 ? min(TR, G - rt * TR) * min(TC, G - ct * TC) : 0;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned bits = 0, out = 0, entries = 0;
+#pragma unroll
+            for (int w = 0; w < ALNS_WARPS; ++w) {
+                const int f = flag[w];
+                bits |= (f < 0 ? 1u : 0u) << w;
+                out += f > 0 ? 1u : 0u;
+                entries += f > 0 ? static_cast<unsigned>(f) : 0u;
+            }
+            s.counts[0] += static_cast<unsigned long long>(entries) * static_cast<unsigned>(nrem);
+            s.counts[1] += static_cast<unsigned long long>(entries) * static_cast<unsigned>(nrem);
+            s.counts[2] += out;
+            s.counts[3] += out;
+            reinterpret_cast<unsigned char*>(t.tmask)[gr] = static_cast<unsigned char>(bits);
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        if (rank < want) {
+            __threadfence();
+            atomicAdd(&ctl->tests_done, 1);
+        }
+        volatile int* td = &ctl->tests_done;
+        const uint64_t t0 = global_ns();
+        while (*td < want) {
+            if (global_ns() - t0 > ctl->wait_ns) {
+                atomicExch(&ctl->err, DEV_TIMEOUT_BARRIER);
+                break;
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    TileMask r;
+    const int w = static_cast<int>(threadIdx.x);
+    r.word = w < words ? __ldcg(&t.tmask[w]) : 0u;
+    int incl = __popc(r.word);
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL_MASK, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) flag[warp] = incl;
+    __syncthreads();
+    r.count = 0;
+    r.before = incl - __popc(r.word);
+#pragma unroll
+    for (int k = 0; k < ALNS_WARPS; ++k) {
+        r.before += k < warp ? flag[k] : 0;
+        r.count += flag[k];
+    }
+    __syncthreads();
+    return r;
+}
+
+__device__ void phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int team_blocks) {
     AlnsCtl* ctl = t.ctl;
     const int N = s.sWoff[t.m], G = N + t.m;
     const int RT = (G + TR - 1) / TR, CT = (G + TC - 1) / TC;
@@ -1820,39 +1931,33 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s) {
     // would leave most of the team waiting; their simulations are done by the
     // time the phase starts (the team barrier before it waits for every walk).
     const int nfb = 2 * ctl->n_short * FB_SPLIT;
-    const int total = tiles + nfb;
     const int nwalks = gap_walk_units(t);
     bool walks_seen = false;
     int* slot = s.misc;
-    // Tiles go out by their distance d = |ct - rt/2| from the diagonal (the
-    // column tile that holds the row band's own gaps): the entries near it
-    // (drop and pickup on one route or on neighbouring ones) are where a
-    // customer's best insertion usually lies, so their scores tighten the
-    // bounds before the far tiles are reached.  Per d, the tiles left of the
-    // diagonal (ct = rt/2 - d, rt = 2d..RT-1), then those right of it
-    // (ct = rt/2 + d, rt = 0..2(CT-d)-1).
-    auto tile_of = [&](int item, int* prt, int* pct) {
-        if (item < RT) { *prt = item; *pct = item >> 1; return; }
-        item -= RT;
-        for (int d = 1; d < CT; ++d) {
-            const int nl = max(0, RT - 2 * d), nr = max(0, min(RT, 2 * (CT - d)));
-            if (item < nl) { *prt = 2 * d + item; *pct = (*prt >> 1) - d; return; }
-            item -= nl;
-            if (item < nr) { *prt = item; *pct = (item >> 1) + d; return; }
-            item -= nr;
+    const int testers = team_blocks - nwalks;
+    const bool test = t.mode != 1 && ctl->nrem <= ACT_CAP && tiles > team_blocks && 2 * testers >= team_blocks;
+    TileMask mask = {tiles, 0, 0u};
+    if (test) mask = test_tiles(t, s, rank, testers, G);
+    // the tile of the k-th bit of the mask
+    auto tested_tile = [&](int k) {
+        if (k >= mask.before && k < mask.before + __popc(mask.word)) {
+            unsigned w = mask.word;
+            for (int q = mask.before; q < k; ++q) w &= w - 1;
+            slot[2] = static_cast<int>(threadIdx.x) * 32 + __ffs(w) - 1;
         }
-        *prt = -1;                             // not reached: the counts add up to RT * CT
-        *pct = -1;
+        __syncthreads();
+        return slot[2];
     };
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) slot[0] = atomicAdd(&ctl->work_counter, 1);
-        __syncthreads();
-        const int item = slot[0];
-        if (item >= total) break;
+    const int ntiles = mask.count;
+    const int total = ntiles + nfb;
+    // The first item is the CTA's own; the rest are handed out by a counter, asked
+    // for while the item before runs (the answer takes a trip to L2).
+    int item = rank;
+    for (int turn = 0; item < total; turn ^= 1) {
+        if (threadIdx.x == 0) slot[turn] = total > team_blocks ? team_blocks + atomicAdd(&ctl->work_counter, 1) : total;
         if (item >= nfb) {
             int rt = 0, ct = 0;
-            tile_of(item - nfb, &rt, &ct);
+            tile_of(test ? tested_tile(item - nfb) : item - nfb, RT, CT, &rt, &ct);
             if (rt >= 0) matrix_tile(t, s, rt, ct, N, G);
         } else {
             if (!walks_seen) {
@@ -1874,6 +1979,8 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s) {
             }
             fallback_item(t, s, item, N, G);
         }
+        __syncthreads();                       // the next item is known, this one's buffers are free
+        item = slot[turn];
     }
 }
 
@@ -3412,6 +3519,7 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
     for (int c = threadIdx.x; c <= t.n; c += blockDim.x) s.sp[c] = t.p[c];
     if (t.coords)
         for (int i = threadIdx.x; i < 2 * (t.n + 1); i += blockDim.x) s.xy[i] = t.coords[i];
+    if (threadIdx.x < 4) s.counts[threadIdx.x] = 0ull;
     unsigned gen = 0, ggen = 0;
     __syncthreads();
 
@@ -3424,7 +3532,7 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
         team_arrive(ctl, team_blocks, gen);
         gap_walks(t, s, rank, team_blocks);
         if (!team_wait(ctl, team_blocks, gen)) return;
-        phase_matrix(t, s);
+        phase_matrix(t, s, rank, team_blocks);
         team_barrier(ctl, team_blocks, gen);
         return;
     }
@@ -3460,11 +3568,11 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
                 __syncthreads();
                 if (threadIdx.x == 0) team_s.mode = 1;
                 __syncthreads();
-                phase_matrix(t, s);
+                phase_matrix(t, s, rank, team_blocks);
                 team_barrier(ctl, team_blocks, gen);
                 return;
             }
-            phase_matrix(t, s);
+            phase_matrix(t, s, rank, team_blocks);
             if (!team_barrier_select(t, s, team_blocks, gen)) return;
         }
         return;
@@ -3538,7 +3646,7 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
             gap_walks(t, s, rank, team_blocks);
             if (!team_wait(ctl, team_blocks, gen)) return;
             mark(2);
-            phase_matrix(t, s);
+            phase_matrix(t, s, rank, team_blocks);
             if (!team_barrier_select(t, s, team_blocks, gen)) return;   // select runs inside
             mark(3);
             mark(4);
@@ -3557,6 +3665,12 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
             if (rank == 0) replica_import(t, s);
             if (!grid_barrier(t, ggen)) return;
         }
+    }
+    if (threadIdx.x == 0) {
+        if (s.counts[0]) atomicAdd(&ctl->entries, s.counts[0]);
+        if (s.counts[1]) atomicAdd(&ctl->pruned, s.counts[1]);
+        if (s.counts[2]) atomicAdd(&ctl->tiles, s.counts[2]);
+        if (s.counts[3]) atomicAdd(&ctl->tiles_pruned, s.counts[3]);
     }
 }
 
@@ -3598,6 +3712,7 @@ static size_t team_bytes(int n, int m, int qmax, int iterations, bool dump) {
     add(static_cast<size_t>(qmax) * 32, 8);
     add(static_cast<size_t>(qmax) * 4, 8);
     add(static_cast<size_t>(qmax) * ((G + 31) / 32), 16);
+    add(tile_words(static_cast<int>(G)), 4);
     add(static_cast<size_t>(qmax) * G, 1);
     add(static_cast<size_t>(qmax) * G, 4);
     add(static_cast<size_t>(qmax) * G, 4);
@@ -3637,8 +3752,9 @@ static void carve_team(AlnsTeam& t, DevBuf& B, int n, int m, int qmax, int itera
     t.keys = B.take<unsigned long long>(static_cast<size_t>(qmax) * G);
     t.rkeys = B.take<unsigned long long>(static_cast<size_t>(qmax) * 32);
     t.gmin = B.take<unsigned long long>(static_cast<size_t>(qmax) * 4);
-    t.band_stride = static_cast<int>((G + 31) / 32);
-    t.bands = B.take<int4>(static_cast<size_t>(qmax) * t.band_stride);
+    t.band_stride = qmax;
+    t.bands = B.take<int4>(static_cast<size_t>(qmax) * ((G + 31) / 32));
+    t.tmask = B.take<unsigned>(tile_words(static_cast<int>(G)));
     t.sc = B.take<unsigned char>(static_cast<size_t>(qmax) * G);
     t.slist = B.take<int>(static_cast<size_t>(qmax) * G);
     t.scix = B.take<int>(static_cast<size_t>(qmax) * G);
