@@ -1372,7 +1372,10 @@ __device__ void gap_walks(const AlnsTeam& t, const Smem& s, int rank, int team_b
 // makespans of the best two or three drop vehicles.  The best of each vehicle
 // group so far bounds the best entry and those makespans from above; an entry
 // whose drop vehicle already has an entry of no larger makespan cannot change
-// that vehicle's makespan.  Regret-m needs every vehicle's best and skips only
+// that vehicle's makespan, and one not below the bound of those makespans cannot
+// change their values (many vehicles tie at the makespan as it is, and with such
+// ties kept 170-210 of the 2048 tiles of a step at n = 1000 were run for regret-2
+// instead of 10-50: 72 us against 35 us for all its tiles).  Regret-m needs every vehicle's best and skips only
 // tiles without an admissible entry.  The bounds only fall as tiles are
 // scored, so a customer left out once stays out.
 struct TileBounds {
@@ -1419,7 +1422,7 @@ __device__ __forceinline__ bool tile_matters(const TileBounds& b, int kind, int 
             d[j + 1] = hi;
         }
     // may lower a drop vehicle's best makespan that counts
-    return ldz <= (kind == 1 ? d[1] : d[2]) && ldz < b.vbest;
+    return ldz < min(kind == 1 ? d[1] : d[2], b.vbest);
 }
 
 // One matrix tile (rows rt*TR.., cols ct*TC..) for every customer still to insert.
