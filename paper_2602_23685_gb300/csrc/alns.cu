@@ -188,10 +188,11 @@ struct Smem {
 };
 constexpr int RV = 16, CV = 12;   // row / col vector widths (ints)
 constexpr int CB = 8;             // customers per matrix batch
-// A tile's batch vectors, row minima and pair list (words), then the list of
-// the customers the tile still has to score (up to ACT_CAP of them; with more
+// A tile's two batches of vectors, (in a dump) the adjacent pairs' and two batches
+// of row minima (words), then the list of the customers the tile still has to
+// score with their best entries so far (up to ACT_CAP of them; with more
 // customers waiting, every tile scores every customer).
-constexpr int TILE_WORDS = CB * (4 * TC + 8 * TR) + 2 * TR * TC;
+constexpr int TILE_WORDS = 2 * CB * 4 * (TC + TR) + 2 * TR + 2 * CB * TR * 2;
 constexpr int ACT_CAP = 256;
 
 // Walk buffers (one ready array per warp).  The same words hold a matrix
@@ -204,9 +205,9 @@ __host__ __device__ inline size_t rdy_words(int n) {
     const size_t rw = static_cast<size_t>(((n + 1) + 3) & ~3);
     const size_t walks = static_cast<size_t>(ALNS_WARPS) * rw;
     const size_t fb = 2 * rw + 2 * ((static_cast<size_t>(2 * n) + 3) & ~static_cast<size_t>(3));
-    // tile: column and row vectors, adjacent-pair vectors and row minima per
-    // customer of a batch, then the compacted pair list (int2 per pair)
-    const size_t batch = static_cast<size_t>(TILE_WORDS) + ACT_CAP;
+    // tile: column and row vectors per customer of a batch, adjacent-pair vectors;
+    // the range tables' two buffers (512 + 4n words at most) fit in the larger of this and the walks
+    const size_t batch = static_cast<size_t>(TILE_WORDS) + 3 * ACT_CAP;
     const size_t sel = 5 * static_cast<size_t>(n) + 8;
     size_t w = walks > batch ? walks : batch;
     w = w > fb ? w : fb;
@@ -1425,6 +1426,30 @@ __device__ __forceinline__ bool tile_matters(const TileBounds& b, int kind, int 
     return ldz < min(kind == 1 ? d[1] : d[2], b.vbest);
 }
 
+// One warp: the best entries (key, KEY_NONE: none) of customer slot ti in rows R
+// (per lane, routes v in order) to the customer's keys.  One pair of atomics per
+// route among the lanes: one per row, from every tile, met on the same few words
+// (a step of regret-m at n = 1000, all tiles run: 450 us, and 110 us so).
+// A row's own key only names the column if the entry is the customer's best:
+// u, the best so far, rules the others out.
+__device__ __forceinline__ void fold_rows(const AlnsTeam& t, int ti, int G, int R, int v, unsigned long long key,
+                                          unsigned long long u) {
+    const int lane = threadIdx.x & 31;
+    if (key != KEY_NONE && (key >> 12) <= u) atomicMin(&t.keys[static_cast<long long>(ti) * G + R], key);
+    unsigned long long best = key == KEY_NONE ? KEY_NONE : ((key >> 12) << 12) | static_cast<unsigned long long>(R);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {         // over the lanes behind that have the same route
+        const unsigned long long other = __shfl_down_sync(FULL_MASK, best, o);
+        const int ov = __shfl_down_sync(FULL_MASK, v, o);
+        if (lane + o < 32 && ov == v && other < best) best = other;
+    }
+    const int pv = __shfl_up_sync(FULL_MASK, v, 1);
+    if ((lane == 0 || pv != v) && best != KEY_NONE) {
+        atomicMin(&t.rkeys[ti * 32 + v], best);
+        atomicMin(&t.gmin[ti * 4 + (v & 3)], best >> 12);
+    }
+}
+
 // One matrix tile (rows rt*TR.., cols ct*TC..) for every customer still to insert.
 //
 // Whether a (drop gap, pickup gap) pair can take a customer at all does not
@@ -1452,7 +1477,8 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
     const int z = ctl->z_work;
     // only customers whose pick the tile can change are scored (tile_matters)
     const bool prune_on = !dump && nrem <= ACT_CAP;
-    int* act = s.rdy + TILE_WORDS;             // [ACT_CAP] customers to score
+    unsigned long long* actu = reinterpret_cast<unsigned long long*>(s.rdy + TILE_WORDS);   // [ACT_CAP] their best (dz, dt) so far
+    int* act = reinterpret_cast<int*>(actu + ACT_CAP);                                      // [ACT_CAP] customers to score
     int* nact = s.misc + 12;
     if (tid == 0) *nact = 0;
     const bool mine = prune_on && tid < nrem;
@@ -1477,38 +1503,44 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
             reinterpret_cast<int4*>(colc)[e2] = v;
         }
     }
-    if (mine && tile_matters(bounds, kind, z)) act[atomicAdd(nact, 1)] = tid;
+    if (mine && tile_matters(bounds, kind, z)) {
+        const int at = atomicAdd(nact, 1);
+        act[at] = tid;
+        actu[at] = min(min(bounds.gm[0], bounds.gm[1]), min(bounds.gm[2], bounds.gm[3]));
+    }
     __syncthreads();
     const int na = prune_on ? *nact : nrem;
     auto cust = [&](int i) { return prune_on ? act[i] : i; };
     // Per customer the vectors of the tile's gaps come from the per-step arrays, CB
-    // customers per pair of block barriers, into the walk buffers (unused by tiles):
-    //   cols [CB][TC] int4, rows [CB][TR] int4, adj [CB][TR] int2.
-    int4* cvec = reinterpret_cast<int4*>(s.rdy);
-    int4* rvec = cvec + CB * TC;
-    int2* avec = reinterpret_cast<int2*>(rvec + CB * TR);
-    auto load_batch = [&](int tb, int nb) {
-        for (int it = tid; it < nb * (TR + TC); it += blockDim.x) {
-            const int k = it / (TR + TC), slot = it - k * (TR + TC);
-            const long long vb = static_cast<long long>(cust(tb + k)) * G;
-            if (slot < TR) {
-                const int Rr = r0 + slot;
-                const bool in = Rr < G;
-                rvec[k * TR + slot] = in ? t.vrow[vb + Rr] : make_int4(SKIPV, 0, 0, 0);
-                avec[k * TR + slot] = in ? t.vadj[vb + Rr] : make_int2(SKIPV, 0);
-            } else {
-                const int cc = slot - TR, Cg = c0 + cc;
-                cvec[k * TC + cc] = Cg < G ? t.vcol[vb + Cg] : make_int4(SKIPV, 0, 0, Cg);
+    // customers per batch, into the walk buffers (unused by tiles): cols [CB][TC]
+    // int4, rows [CB][TR] int4, twice: a batch is copied in, past the registers,
+    // while the one before is scored.  (Gaps past the last are not copied: no pair
+    // of theirs is one.)
+    constexpr int BATCH = CB * (TC + TR);
+    int4* vecs = reinterpret_cast<int4*>(s.rdy);
+    int2* avec = reinterpret_cast<int2*>(vecs + 2 * BATCH);        // [TR], a dump's
+    unsigned long long* rowbest = reinterpret_cast<unsigned long long*>(avec + TR);   // [2][CB][TR]
+    static_assert(BATCH % ALNS_THREADS == 0, "each thread copies as many vectors of a batch");
+    auto copy_batch = [&](int tb, int half) {
+#pragma unroll
+        for (int u = 0; u < BATCH / ALNS_THREADS; ++u) {
+            const int it = tid + u * ALNS_THREADS, k = it / (TC + TR), slot = it - k * (TC + TR);
+            const int g = slot < TC ? c0 + slot : r0 + slot - TC;
+            if (tb + k < na && g < G) {
+                const int4* src = (slot < TC ? t.vcol : t.vrow) + static_cast<long long>(cust(tb + k)) * G + g;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(vecs + half * BATCH + it)), "l"(src)
+                             : "memory");
             }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    auto copies_done = [&]() { asm volatile("cp.async.wait_all;" ::: "memory"); };
     // this thread's pairs
     const int r = tid >> 3, cb = tid & 7;
     const int* rk = rowc + r * RV;
     const int ra = rk[8];
     const bool row_ok = ra >= 0;               // all 8 lanes of a row agree; no early exit (shuffles below)
     const int R = r0 + r;
-    const unsigned ncols = static_cast<unsigned>(max(0, min(TC / 8, (G - c0 - cb + 7) / 8)));  // this thread's columns < G
     // every entry of the tile counts, scored or not; in shared memory until the
     // run ends
     if (tid == 0) {
@@ -1538,7 +1570,7 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
             rcl[kk] = okr ? t.Ms[static_cast<long long>(yb) * N + xa] : NEG;
         }
     }
-    load_batch(0, min(CB, na));
+    copy_batch(0, 0);
 #pragma unroll
     for (int kk = 0; kk < TC / 8; ++kk) {
         const int cc = cb + 8 * kk;
@@ -1569,130 +1601,92 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
         // every entry of the first customer still to insert written out
         // (parity runs): shortcut entries are left to the shortcut items,
         // excluded pairs read "infeasible"
-        for (int tb = 0; tb < min(nrem, 1); tb += CB) {
-            const int nb = 1;
-            __syncthreads();
-            if (tb > 0) load_batch(tb, nb);
-            __syncthreads();
-            for (int k = 0; k < nb; ++k) {
-                const int4 rv = rvec[k * TR + r];
-                if (!row_ok) continue;
-                const bool scR = rv.x >= SKIPV;
+        if (tid < TR) avec[tid] = r0 + tid < G ? t.vadj[r0 + tid] : make_int2(SKIPV, 0);
+        copies_done();
+        __syncthreads();
+        const int4 rv = vecs[TC + r];
+        if (!row_ok || rv.x >= SKIPV) return;
 #pragma unroll
-                for (int kk = 0; kk < TC / 8; ++kk) {
-                    const int cc = cb + 8 * kk, Cg = c0 + cc;
-                    const int4 g = cvec[k * TC + cc];
-                    if (Cg >= G || scR || g.x >= SKIPV) continue;
-                    const long long idx = static_cast<long long>(R) * G + Cg;
-                    if (cc == diag) {
-                        const int2 a = avec[k * TR + r];
-                        t.dump_delta[idx] = adj_ok ? a.x - z : 0x7fffffff;
-                        t.dump_travel[idx] = adj_ok ? static_cast<int>(static_cast<unsigned>(a.y) >> 12) - (1 << 19) : 0;
-                        continue;
-                    }
-                    const int zz = max(max(rv.x, g.x), max(rv.y + g.y, rv.z + lpv[kk] + g.z));
-                    const unsigned lo = static_cast<unsigned>(rv.w) + static_cast<unsigned>(g.w);
-                    const bool ok = lpv[kk] != SKIPV;
-                    t.dump_delta[idx] = ok ? zz - z : 0x7fffffff;
-                    t.dump_travel[idx] = ok ? static_cast<int>(lo >> 12) - (1 << 19) : 0;
-                }
+        for (int kk = 0; kk < TC / 8; ++kk) {
+            const int cc = cb + 8 * kk, Cg = c0 + cc;
+            const int4 g = vecs[cc];
+            if (Cg >= G || g.x >= SKIPV) continue;
+            const long long idx = static_cast<long long>(R) * G + Cg;
+            if (cc == diag) {
+                const int2 a = avec[r];
+                t.dump_delta[idx] = adj_ok ? a.x - z : 0x7fffffff;
+                t.dump_travel[idx] = adj_ok ? static_cast<int>(static_cast<unsigned>(a.y) >> 12) - (1 << 19) : 0;
+                continue;
             }
+            const int zz = max(max(rv.x, g.x), max(rv.y + g.y, rv.z + lpv[kk] + g.z));
+            const unsigned lo = static_cast<unsigned>(rv.w) + static_cast<unsigned>(g.w);
+            const bool ok = lpv[kk] != SKIPV;
+            t.dump_delta[idx] = ok ? zz - z : 0x7fffffff;
+            t.dump_travel[idx] = ok ? static_cast<int>(lo >> 12) - (1 << 19) : 0;
         }
         return;
     }
-    // Only part of the pairs survive (a sixth to a third at n = 1000), scattered
-    // over the tile.  They are compacted into one row-major list for the whole
-    // CTA; per batch the customers share the threads out and each thread takes
-    // an equal contiguous share of the list for its customer, keeping a running
-    // minimum per row that it folds into the row's slot in shared memory when
-    // its row changes; once per batch the row minima go to the global keys.
-    unsigned long long* rowbest = reinterpret_cast<unsigned long long*>(avec + CB * TR);   // [CB][TR]
-    int2* list = reinterpret_cast<int2*>(rowbest + CB * TR);                                // [TR * TC]
+    // Only part of the pairs survive (a sixth to a third at n = 1000), mostly in
+    // blocks, so a warp (4 rows by 8 columns at a time) passes over the column
+    // steps in which it has none and scores the rest with its pairs in registers:
+    // one 16-byte read of a column vector per entry, free of bank conflicts.  (The
+    // surviving pairs compacted into a list in shared memory, every thread walking
+    // a share of it, folding its row minima by shared atomics and sending one set
+    // of global atomics per row and customer: matrix and selection of a step under
+    // all removals and repair rules 107.8 us at n = 1000, 49.3 us now; 17.4 and
+    // 15.1 us at n = 120.)
+    // Shortcut gaps come out at or above SKIPV.
     unsigned fm = 0;
 #pragma unroll
     for (int kk = 0; kk < TC / 8; ++kk) fm |= (lpv[kk] != SKIPV ? 1u : 0u) << kk;
-    const int cnt = __popc(fm);
-    int incl = cnt;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL_MASK, incl, o);
-        if ((tid & 31) >= o) incl += y;
-    }
-    int* wsum = s.misc + 16;                   // [ALNS_WARPS] per-warp totals
-    if ((tid & 31) == 31) wsum[warp] = incl;
-    __syncthreads();
-    int woff = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < ALNS_WARPS; ++w) {
-        const int v = wsum[w];
-        woff += w < warp ? v : 0;
-        total += v;
-    }
-    {
-        int at = woff + incl - cnt;
-#pragma unroll
-        for (int kk = 0; kk < TC / 8; ++kk)
-            if ((fm >> kk) & 1u) list[at++] = make_int2(lpv[kk], (r << 8) | (cb + 8 * kk));
-    }
-    for (int q = tid; q < CB * TR; q += blockDim.x) rowbest[q] = KEY_NONE;
+    const unsigned wm = __reduce_or_sync(FULL_MASK, fm);
     // a tile with no surviving pair has nothing to compute (the adjacent
     // entries were scored with the gap vectors)
-    if (total == 0) return;
-    for (int tb = 0; tb < na; tb += CB) {
+    if (!__syncthreads_or(wm != 0)) {
+        copies_done();
+        return;
+    }
+    // the row minima of the batch at tb to the global keys, a warp per customer
+    auto flush = [&](int tb, int half) {
+        if (tb + warp >= na) return;
+        const int lane = tid & 31;
+        const unsigned long long b = rowbest[(half * CB + warp) * TR + lane];
+        unsigned long long key = KEY_NONE;
+        if (b < static_cast<unsigned long long>(SKIPV) << 32)
+            key = (static_cast<unsigned long long>(static_cast<unsigned>(static_cast<int>(b >> 32) - z) ^ 0x80000000u) << 32) |
+                  (b & 0xFFFFFFFFull);
+        fold_rows(t, cust(tb + warp), G, r0 + lane, rowc[lane * RV + 8], key, prune_on ? actu[tb + warp] : KEY_NONE);
+    };
+    int half = 0;
+    for (int tb = 0; tb < na; tb += CB, half ^= 1) {
         const int nb = min(CB, na - tb);
-        __syncthreads();                       // the list and the row slots are ready; the previous batch is flushed
-        if (tb > 0) load_batch(tb, nb);
-        __syncthreads();
-        // the batch's customers split the threads (L each, the rest idle); a
-        // thread walks a contiguous share of the list for its customer,
-        // keeping the running minimum of its current row, and folds it into
-        // the row's slot only when its row changes, so a row's slot sees a
-        // few atomics rather than one per pair and customer
-        const unsigned long long lim = static_cast<unsigned long long>(SKIPV) << 32;
-        const int L = ALNS_THREADS / nb;
-        const int k = tid / L, li = tid - k * L;
-        if (k < nb) {
-            const int qb = static_cast<int>((static_cast<long long>(li) * total) / L);
-            const int qe = static_cast<int>((static_cast<long long>(li + 1) * total) / L);
-            const int4* cv = cvec + k * TC;
-            const int4* rw = rvec + k * TR;
-            unsigned long long* rb = rowbest + k * TR;
-            int cur = -1;
-            int4 rv = make_int4(0, 0, 0, 0);
+        copies_done();
+        __syncthreads();                       // this batch is there, the one before is scored
+        if (tb + CB < na) copy_batch(tb + CB, half ^ 1);
+        if (tb > 0) flush(tb - CB, half ^ 1);
+        const int4* vec = vecs + half * BATCH;
+        for (int k = 0; k < nb; ++k, vec += TC + TR) {
+            const int4 rv = vec[TC + r];
             unsigned long long best = KEY_NONE;
-            for (int q = qb; q < qe; ++q) {
-                const int2 le = list[q];
-                const int rr = le.y >> 8;
-                if (rr != cur) {
-                    if (best < lim) atomicMin(&rb[cur], best);
-                    rv = rw[rr];
-                    best = KEY_NONE;
-                    cur = rr;
+#pragma unroll
+            for (int kk = 0; kk < TC / 8; ++kk)
+                if ((wm >> kk) & 1u) {
+                    const int4 g = vec[cb + 8 * kk];
+                    const int zz = max(max(rv.x, g.x), max(rv.y + g.y, rv.z + lpv[kk] + g.z));
+                    const unsigned lo = static_cast<unsigned>(rv.w) + static_cast<unsigned>(g.w);
+                    const unsigned long long key = (static_cast<unsigned long long>(static_cast<unsigned>(zz)) << 32) | lo;
+                    best = lpv[kk] != SKIPV && key < best ? key : best;
                 }
-                const int4 g = cv[le.y & 0xFF];
-                const int zz = max(max(rv.x, g.x), max(rv.y + g.y, rv.z + le.x + g.z));
-                const unsigned lo = static_cast<unsigned>(rv.w) + static_cast<unsigned>(g.w);
-                const unsigned long long key = (static_cast<unsigned long long>(static_cast<unsigned>(zz)) << 32) | lo;
-                best = key < best ? key : best;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {  // over the row's eight lanes
+                const unsigned long long other = __shfl_xor_sync(FULL_MASK, best, o);
+                best = other < best ? other : best;
             }
-            if (best < lim) atomicMin(&rb[cur], best);
-        }
-        __syncthreads();
-        // row minima of the batch to the global keys, slots back to empty
-        for (int q = tid; q < nb * TR; q += blockDim.x) {
-            const unsigned long long b = rowbest[q];
-            if (b != KEY_NONE) {
-                const int k = q / TR, rr = q - k * TR;
-                const int ti = cust(tb + k), Rr = r0 + rr, rra = rowc[rr * RV + 8];
-                const unsigned long long key =
-                    (static_cast<unsigned long long>(static_cast<unsigned>(static_cast<int>(b >> 32) - z) ^ 0x80000000u) << 32) |
-                    (b & 0xFFFFFFFFull);
-                atomicMin(&t.keys[static_cast<long long>(ti) * G + Rr], key);
-                atomicMin(&t.rkeys[ti * 32 + rra], ((key >> 12) << 12) | static_cast<unsigned long long>(Rr));
-                atomicMin(&t.gmin[ti * 4 + (rra & 3)], key >> 12);
-                rowbest[q] = KEY_NONE;
-            }
+            if (cb == 0) rowbest[(half * CB + k) * TR + r] = best;
         }
     }
+    __syncthreads();
+    flush((na - 1) / CB * CB, half ^ 1);
 }
 
 // Shortcut item: every entry with one shortcut gap g for customer c (the
@@ -1739,40 +1733,53 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
     const bool dump = t.mode == 1;
     unsigned cnt = 0;
     auto loc = [&](int pos) { return pos >= 0 ? (s.sW[pos] & PACK_MASK) >> 1 : 0; };
-    for (int k = piece * blockDim.x + tid; k < G && z1 != 0x7fffffff; k += FB_SPLIT * blockDim.x) {
-        if (k == g || t.sc[scrow + k]) continue;              // both gaps shortcuts: below / elsewhere
-        const int row = as_col ? k : g, col = as_col ? g : k;
-        const int a = t.groute[row], i = t.gpos[row], b = t.groute[col], j = t.gpos[col];
-        const long long idx = static_cast<long long>(row) * G + col;
-        if (a == b && j < i) {
-            if (dump) { t.dump_delta[idx] = 0x7fffffff; t.dump_travel[idx] = 0; }
-            continue;
+    const unsigned long long u = min(min(t.gmin[ti * 4], t.gmin[ti * 4 + 1]), min(t.gmin[ti * 4 + 2], t.gmin[ti * 4 + 3]));
+    unsigned long long rowkey = KEY_NONE;      // as_col = 0: the best of this thread's entries, all in row g
+    for (int k0 = piece * blockDim.x + warp * 32; k0 < G && z1 != 0x7fffffff; k0 += FB_SPLIT * blockDim.x) {
+        const int k = k0 + lane;
+        unsigned long long key = KEY_NONE;
+        const int vk = k < G ? t.groute[k] : -1;
+        if (k < G && k != g && !t.sc[scrow + k]) {            // (both gaps shortcuts: below / elsewhere)
+            const int row = as_col ? k : g, col = as_col ? g : k;
+            const int a = as_col ? vk : ga, i = t.gpos[row], b = as_col ? ga : vk, j = t.gpos[col];
+            const long long idx = static_cast<long long>(row) * G + col;
+            if (a == b && j < i) {
+                if (dump) { t.dump_delta[idx] = 0x7fffffff; t.dump_travel[idx] = 0; }
+            } else {
+                const int xa = t.gx[row], yb = t.gy[col];
+                const bool cyc = xa >= 0 && yb >= 0 && t.Ms[static_cast<long long>(yb) * N + xa] > NEG;
+                const bool ok = !cyc && entry_capacity(t, row, col, N);
+                int zn;
+                if (!as_col) {
+                    const int xb = t.gx[col];
+                    const int arr = (xb >= 0 ? Hb[xb] : 0) + Dx(t, s, loc(xb), c);
+                    const int dep = max(arr, hv + pc);
+                    zn = max(z1, dep + Dx(t, s, c, loc(yb)) + (yb >= 0 ? Tb[yb] : 0));
+                } else {
+                    const int ya = t.gy[row];
+                    const int td = (xa >= 0 ? Hb[xa] : 0) + Dx(t, s, loc(xa), c);
+                    zn = max(z1, max(td + Dx(t, s, c, loc(ya)) + (ya >= 0 ? Tb[ya] : 0), td + pc + tv));
+                }
+                ++cnt;
+                const int dt = travel_delta(t, s, c, row, col);
+                if (dump) {
+                    t.dump_delta[idx] = ok ? zn - z : 0x7fffffff;
+                    t.dump_travel[idx] = ok ? dt : 0;
+                } else if (ok) {
+                    key = pack_key(zn - z, dt, col);
+                }
+            }
         }
-        const int xa = t.gx[row], yb = t.gy[col];
-        const bool cyc = xa >= 0 && yb >= 0 && t.Ms[static_cast<long long>(yb) * N + xa] > NEG;
-        const bool ok = !cyc && entry_capacity(t, row, col, N);
-        int zn;
-        if (!as_col) {
-            const int xb = t.gx[col];
-            const int arr = (xb >= 0 ? Hb[xb] : 0) + Dx(t, s, loc(xb), c);
-            const int dep = max(arr, hv + pc);
-            zn = max(z1, dep + Dx(t, s, c, loc(yb)) + (yb >= 0 ? Tb[yb] : 0));
-        } else {
-            const int ya = t.gy[row];
-            const int td = (xa >= 0 ? Hb[xa] : 0) + Dx(t, s, loc(xa), c);
-            zn = max(z1, max(td + Dx(t, s, c, loc(ya)) + (ya >= 0 ? Tb[ya] : 0), td + pc + tv));
+        if (dump) continue;
+        if (as_col) fold_rows(t, ti, G, k, vk, key, u);
+        else rowkey = key < rowkey ? key : rowkey;
+    }
+    if (!as_col && !dump) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(FULL_MASK, rowkey, o);
+            rowkey = other < rowkey ? other : rowkey;
         }
-        ++cnt;
-        const int dt = travel_delta(t, s, c, row, col);
-        if (dump) {
-            t.dump_delta[idx] = ok ? zn - z : 0x7fffffff;
-            t.dump_travel[idx] = ok ? dt : 0;
-        } else if (ok) {
-            const unsigned long long key = pack_key(zn - z, dt, col);
-            atomicMin(&t.keys[scrow + row], key);
-            atomicMin(&t.rkeys[ti * 32 + a], ((key >> 12) << 12) | static_cast<unsigned long long>(row));
-            atomicMin(&t.gmin[ti * 4 + (a & 3)], key >> 12);
-        }
+        fold_rows(t, ti, G, g, ga, lane == 0 ? rowkey : KEY_NONE, u);
     }
     // both gaps shortcuts, from the drop gap's item: full re-simulation, one warp each
     if (!as_col) {
