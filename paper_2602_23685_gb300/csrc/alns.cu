@@ -1376,9 +1376,11 @@ __device__ void gap_walks(const AlnsTeam& t, const Smem& s, int rank, int team_b
 // that vehicle's makespan, and one not below the bound of those makespans cannot
 // change their values (many vehicles tie at the makespan as it is, and with such
 // ties kept 170-210 of the 2048 tiles of a step at n = 1000 were run for regret-2
-// instead of 10-50: 72 us against 35 us for all its tiles).  Regret-m needs every vehicle's best and skips only
-// tiles without an admissible entry.  The bounds only fall as tiles are
-// scored, so a customer left out once stays out.
+// instead of 10-50: 72 us against 35 us for all its tiles).  Regret-m needs every
+// vehicle's best makespan: a tile matters that may lower one of its own
+// vehicles' (matrix and selection of a step at n = 1000 under all repair rules
+// 47.8 us with only empty tiles left out for it, 32.1 us so).  The bounds only
+// fall as tiles are scored, so a customer left out once stays out.
 struct TileBounds {
     int4 r, c0, c1;                            // band minima: rows, columns (two bands)
     unsigned long long gm[4];                  // best per vehicle group so far
@@ -1397,7 +1399,7 @@ __device__ __forceinline__ TileBounds tile_bounds(const AlnsTeam& t, int ti, int
 #pragma unroll
     for (int k = 0; k < 4; ++k) b.gm[k] = t.gmin[ti * 4 + k];
     b.vbest = 0;
-    if (kind == 1 || kind == 2)
+    if (kind > 0)
         for (int v = va0; v <= va1; ++v) b.vbest = max(b.vbest, t.rkeys[ti * 32 + v] >> 32);
     return b;
 }
@@ -1405,11 +1407,11 @@ __device__ __forceinline__ TileBounds tile_bounds(const AlnsTeam& t, int ti, int
 __device__ __forceinline__ bool tile_matters(const TileBounds& b, int kind, int z) {
     const int lzz = max(b.r.x, min(b.c0.z, b.c1.z));
     if (lzz >= SKIPV) return false;
-    if (kind > 2) return true;
     const unsigned llo = static_cast<unsigned>(b.r.y) + min(static_cast<unsigned>(b.c0.w), static_cast<unsigned>(b.c1.w));
     const unsigned long long ldz = static_cast<unsigned>(lzz - z) ^ 0x80000000u;
     if (((ldz << 20) | (llo >> 12)) <= min(min(b.gm[0], b.gm[1]), min(b.gm[2], b.gm[3]))) return true;   // may be the best entry
     if (kind == 0) return false;
+    if (kind > 2) return ldz < b.vbest;
     // the second (regret-2) or third (regret-3) least group makespan
     unsigned long long d[4];
 #pragma unroll
