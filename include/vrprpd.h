@@ -344,7 +344,8 @@ typedef struct {
     double T_final;
     double w_destroy[8], w_repair[4];  /* final operator weights (destroy 0-5 used) */
     double device_ms;          /* wall time of the device run */
-    int64_t matrix_entries;    /* insertion-matrix entries scored by the O(1) tile formula */
+    int64_t matrix_entries;    /* insertion-matrix entries decided by the O(1) tile formula or its bound
+                                  (pruned_entries of them), and gaps the local search scored */
     int64_t fallback_entries;  /* entries with a shortcut gap: exact from simulations with one stop
                                   (both gaps shortcuts: both stops) instead of the tile formula */
     int32_t team_blocks;       /* CTAs used */
@@ -363,7 +364,7 @@ typedef struct {
                                   tile showed that none of them can be the one the repair operator
                                   picks (its per-vehicle bests, or the best, are already at or
                                   below it); the result is the same as scoring them */
-    int64_t tiles;             /* insertion-matrix tiles (32 drop gaps x 64 pickup gaps) run */
+    int64_t tiles;             /* insertion-matrix tiles (32 drop gaps x 64 pickup gaps) tested or run */
     int64_t tiles_pruned;      /* of those, tiles in which no customer was left to score */
 } vrprpd_alns_stats;
 

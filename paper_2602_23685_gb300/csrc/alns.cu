@@ -14,31 +14,34 @@
 //           builds W = current solution without them.
 // Then one insertion step per removed customer:
 //   prep    each CTA stages W in shared memory (op codes packed with their
-//           travel-in times).  After a full step, warps walk W from the depot
-//           (node times H, makespan) and from every op u (row u of the
-//           all-pairs longest-path table LP, and the tail T(u)); after a plain
-//           insertion the table is updated in place from the inserted pair
-//           instead.  Threads flag "shortcut" gaps, where d(x,c) + d(c,y) <
-//           d(x,y) because of the nint rounding;
+//           travel-in times), or carries the last insertion out on the copy it
+//           has.  After a full step, warps walk W from the depot (node times H,
+//           makespan) and from every op u (row u of the all-pairs longest-path
+//           table LP, and the tail T(u)); after a plain insertion the table is
+//           updated from the inserted pair instead.  Threads flag "shortcut"
+//           gaps, where d(x,c) + d(c,y) < d(x,y) because of the nint rounding;
 //   gaps    per-gap vectors (H of the stop before, T of the stop after, the
 //           removed leg, stock prefix/suffix extremes), per-(customer, gap)
-//           row and column vectors, and sparse tables of the stock prefix;
-//           the team then starts the shortcut simulations (schedules with the
-//           single shortcut stop added) without waiting for them;
+//           row and column vectors and their minima per 32 gaps, and sparse
+//           tables of the stock prefix; the team then starts the shortcut
+//           simulations (schedules with the single shortcut stop added) without
+//           waiting for them;
 //   matrix  32 x 64 tiles of (dropoff gap, pickup gap) entries for every
 //           customer still to insert.  Without shortcut gaps the new makespan
 //           is exactly max(z, beta, gamma, delta, epsilon): the old makespan,
 //           the longest path through the new drop only, through the new pickup
 //           only, through drop -> pickup by the processing edge, and through
 //           drop -> route -> pickup (the LP table).  Capacity and pool are O(1)
-//           from the prefix/suffix extremes.  Feasible pairs are compacted per
-//           CTA and reduced to per-row minima with shared 64-bit atomics.
-//           Entries on shortcut gaps come last, from the simulations;
+//           from the prefix/suffix extremes.  All tiles are tested against the
+//           best entries known so far first; those that may matter are scored
+//           from registers and their row minima folded by route into 64-bit
+//           atomics.  Entries on shortcut gaps come from the simulations;
 //   select  per-customer argmin of (delta z, delta travel, flat index), then
-//           the repair operator's choice across customers; the choice is
-//           applied to W.
-// Rank 0 ends the iteration: the repaired W is walked and accepted or not,
-// the temperature and weights are updated and the next operators are drawn.
+//           the repair operator's choice across customers, by the CTA that
+//           arrives last; the others carry the choice out in the next step.
+// Rank 0 ends the iteration: the repaired solution, whose makespan the last
+// insertion gave, is accepted or not, the temperature and weights are updated
+// and the next operators are drawn.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -1090,8 +1093,9 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
     // The phase has three independent parts: the per-gap constants, the
     // per-(customer, gap) vectors and the sparse tables.  The vectors take the
     // CTAs from rank 0 up; the constants and the tables take CTAs from the top
-    // of the team down, below the last four (which start the shortcut
-    // simulations right after this phase), so that no CTA does two parts.
+    // of the team down, below the last four (which, with more below them when
+    // there are many shortcut gaps, start the simulations right after this
+    // phase), so that few CTAs do two parts.
     const int npg = (G + ALNS_THREADS - 1) / ALNS_THREADS;
     const int rank_pg = ((team_blocks - 5 - rank) % team_blocks + team_blocks) % team_blocks;
     const int rank_sp = ((team_blocks - 5 - npg - rank) % team_blocks + team_blocks) % team_blocks;
@@ -1457,14 +1461,13 @@ __device__ __forceinline__ void fold_rows(const AlnsTeam& t, int ti, int G, int 
 // Whether a (drop gap, pickup gap) pair can take a customer at all does not
 // depend on the customer: every customer moves one unit of the resource, and
 // the cycle test and the longest path between the two gaps are properties of
-// W.  So each thread first settles its 16 pairs (row tid/8, columns
+// W.  So each thread first settles its 8 pairs (row tid/8, columns
 // tid%8 + 8k) into one register each: the longest-path value LP, or the
 // sentinel SKIPV when the pair is excluded (capacity, pool, a cycle, a pickup
 // gap before the drop gap on one route).  Per customer an entry is then
 //     z' = max(max(z, beta), gamma, A1 + p_c + B1, E + LP + F)
 // with the row terms in registers and the column terms one 16-byte shared
-// load; excluded pairs and shortcut gaps come out at or above SKIPV and never
-// win.  The pair in which both gaps coincide (drop and pickup back to back)
+// load; shortcut gaps come out at or above SKIPV and never win.  The pair in which both gaps coincide (drop and pickup back to back)
 // is the adjacent case, handled once per row.
 
 __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, int N, int G) {
