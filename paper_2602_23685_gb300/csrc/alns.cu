@@ -1467,8 +1467,9 @@ __device__ __forceinline__ void fold_rows(const AlnsTeam& t, int ti, int G, int 
 // gap before the drop gap on one route).  Per customer an entry is then
 //     z' = max(max(z, beta), gamma, A1 + p_c + B1, E + LP + F)
 // with the row terms in registers and the column terms one 16-byte shared
-// load; shortcut gaps come out at or above SKIPV and never win.  The pair in which both gaps coincide (drop and pickup back to back)
-// is the adjacent case, handled once per row.
+// load; shortcut gaps come out at or above SKIPV and never win.  The pair in
+// which both gaps coincide (drop and pickup back to back) is the adjacent case,
+// handled once per row.
 
 __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, int N, int G) {
     AlnsCtl* ctl = t.ctl;
