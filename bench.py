@@ -767,7 +767,7 @@ def main():
     crv, ilv = cr.view(-1, BASE_CANDS), il.view(-1, BASE_CANDS)
     coordination = {"coordination_counts": {
         "value": Bc / (co_ms / 1000.0), "unit": "candidates/s", "candidates": Bc, "ms": co_ms,
-        "kernel": "coordination_kernel", "tiles_agree": bool((crv == crv[0]).all()) and bool((ilv == ilv[0]).all()),
+        "kernel": "eval_tiles_kernel", "tiles_agree": bool((crv == crv[0]).all()) and bool((ilv == ilv[0]).all()),
         "mean_cross_pct": float(cr.double().mean()) * 100.0 / N_CUST,
         "mean_interleaved_pct": float(il.double().mean()) * 100.0 / N_CUST}}
 
