@@ -207,7 +207,7 @@ constexpr int ACT_CAP = 256;
 __host__ __device__ inline size_t rdy_words(int n) {
     const size_t rw = static_cast<size_t>(((n + 1) + 3) & ~3);
     const size_t walks = static_cast<size_t>(ALNS_WARPS) * rw;
-    const size_t fb = 2 * rw + 3 * ((static_cast<size_t>(2 * n) + 4) & ~static_cast<size_t>(3));
+    const size_t fb = 2 * rw + 2 * ((static_cast<size_t>(2 * n) + 3) & ~static_cast<size_t>(3));
     // tile: column and row vectors per customer of a batch, adjacent-pair vectors;
     // the range tables' two buffers (512 + 4n words at most) fit in the larger of this and the walks
     const size_t batch = static_cast<size_t>(TILE_WORDS) + 3 * ACT_CAP;
@@ -492,11 +492,10 @@ constexpr int FREE = INT32_MIN + 1;            // "ready time" of a stop that wa
 // as a shared-memory load, and rounds in which no lane moves change nothing.
 constexpr int WALK_ROUNDS = 4;
 
-// One warp: departures of the staged (acyclic) solution into H; its makespan.  The
-// pickup of customer cfree (0: none), whose drop is not in it, waits for nothing.
-__device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H, int cfree = 0) {
+// One warp: departures of the staged (acyclic) solution into H; its makespan.
+__device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H) {
     const int lane = threadIdx.x & 31, n = t.n;
-    for (int c = lane; c <= n; c += 32) rdy_[c] = cfree > 0 && c == cfree ? FREE : UNRES;
+    for (int c = lane; c <= n; c += 32) rdy_[c] = UNRES;
     __syncwarp();
     const WalkMem M(s, rdy_);
     int pos = lane < t.m ? s.sWoff[lane] : 0;
@@ -526,48 +525,6 @@ __device__ int walk_heads(const AlnsTeam& t, const Smem& s, int* rdy_, int* H, i
     int ret = end > start ? dep + Dx(t, s, (last & PACK_MASK) >> 1, 0) : 0;
     for (int o = 16; o > 0; o >>= 1) ret = max(ret, __shfl_xor_sync(FULL_MASK, ret, o));
     return ret;
-}
-
-constexpr int TAIL_BITS = (1 << 29) - 1;       // a tail; the bit above: the op leads to the candidate's drop
-constexpr int TAIL_NONE = INT32_MIN + 1;       // tail of a pickup that is not in the solution
-
-// One warp: the tail of every staged op (longest path from its departure to
-// the end of the schedule) into T, with the mark of the ops that lead to the
-// drop of c at dpos.  c > 0: c's pickup is not in the solution.
-__device__ void walk_tails(const AlnsTeam& t, const Smem& s, int* tp_, int* T, int c0, int dpos) {
-    const int lane = threadIdx.x & 31, n = t.n;
-    for (int c = lane; c <= n; c += 32) tp_[c] = c0 > 0 && c == c0 ? TAIL_NONE : UNRES;
-    __syncwarp();
-    const WalkMem M(s, tp_);
-    const int start = lane < t.m ? s.sWoff[lane] : 0;
-    int pos = (lane < t.m ? s.sWoff[lane + 1] : 0) - 1;
-    int x = pos >= start ? M.op(pos) : 0;
-    int leg = pos >= start ? Dx(t, s, (x & PACK_MASK) >> 1, 0) : 0, acc = 0, mark = 0;
-    bool moved;
-    do {
-        moved = false;
-#pragma unroll
-        for (int k = 0; k < WALK_ROUNDS; ++k) {
-            const unsigned ca = M.at(x);
-            const bool pick = (x & 1) != 0;
-            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = M.op(max(pos - 1, 0));
-            const int r = pick ? TAIL_NONE : rv;   // (a drop of a customer without its pickup waits for nothing, as a pickup)
-            const bool go = pos >= start && r != UNRES;
-            const int after = acc + leg;
-            const int d = r == TAIL_NONE ? after : max(after, p + (r & TAIL_BITS));
-            int mk = mark | (r == TAIL_NONE ? 0 : r & ~TAIL_BITS);
-            if (pos == dpos) mk = TAIL_BITS + 1;
-            if (go) T[pos] = d | mk;
-            if (go && pick) M.st(M.r + ca, d | mk);
-            acc = go ? d : acc;
-            mark = go ? mk : mark;
-            leg = go ? x >> PACK_SHIFT : leg;
-            pos -= go ? 1 : 0;
-            x = go ? (pos >= start ? nx : 0) : x;
-            moved |= go;
-            __syncwarp();
-        }
-    } while (__any_sync(FULL_MASK, moved));
 }
 
 // From op u: row u of LP (NEG where unreachable) and T(u).  One op per lane and
@@ -714,6 +671,58 @@ __device__ int walk_insert(const AlnsTeam& t, const Smem& s, int* rdy, int c, in
     for (int q = lane; q <= n; q += 32) rdy[q] = UNRES;
     __syncwarp();
     return walk_fwd(t, s, rdy, a, i, 2 * c, b, j, 2 * c + 1, nullptr, nullptr);
+}
+
+// W plus one stop V (op code ov) at gap (a, i), forward: the departure time of
+// every W position into Hb[pos] and of V into *hv; returns the makespan
+// (INT32_MAX on a precedence cycle).  A pickup V without its drop leaves at
+// arrival (its ready time is set to 0): the drop's edge comes with the second
+// stop, not here.
+__device__ int walk_fwd1(const AlnsTeam& t, const Smem& s, int* rdy, int ov, int a, int i, int* Hb, int* hv) {
+    const int lane = threadIdx.x & 31, n = t.n;
+    for (int q = lane; q <= n; q += 32) rdy[q] = UNRES;
+    __syncwarp();
+    if (lane == 0 && (ov & 1)) rdy[ov >> 1] = 0;
+    __syncwarp();
+    return walk_fwd(t, s, rdy, a, i, ov, -1, 0, 0, Hb, hv);
+}
+
+// The same graph backward: the tail of every W position (longest path from its
+// departure to the end of the schedule, return leg included) into Tb[pos] and
+// V's into *tv.  A drop's tail also takes p plus its pickup's tail; V has no
+// partner in this graph.  tp: per-customer pickup tails (n + 1 words).
+__device__ void walk_bwd1(const AlnsTeam& t, const Smem& s, int* tp_, int ov, int a, int i, int* Tb, int* tv) {
+    const int lane = threadIdx.x & 31, n = t.n;
+    for (int c = lane; c <= n; c += 32) tp_[c] = UNRES;
+    __syncwarp();
+    const WalkMem M(s, tp_);
+    const Seq u = make_seq(t, s, a, i, ov, -1, 0, 0);
+    int q = u.len - 1, x = u.at(M, q), acc = 0, tl = 0;
+    int leg = q >= 0 ? Dx(t, s, (x & PACK_MASK) >> 1, 0) : 0;
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool virt = q == u.q0, pick = (x & 1) != 0, waits = !pick && !virt;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = u.at(M, q - 1);
+            const int r = waits ? rv : FREE;
+            const bool go = q >= 0 && r != UNRES;
+            const int after = acc + leg, d = waits ? max(after, p + r) : after;
+            if (go && pick && !virt) M.st(M.r + ca, d);
+            if (go && !virt) Tb[u.pos(q)] = d;
+            tl = go && virt ? d : tl;
+            acc = go ? d : acc;
+            leg = go ? x >> PACK_SHIFT : leg;
+            q -= go ? 1 : 0;
+            x = go ? nx : x;
+            moved |= go;
+            __syncwarp();
+        }
+    } while (__any_sync(FULL_MASK, moved));
+    if (lane == a) *tv = tl;
+    if (q >= 0) atomicExch(&t.ctl->err, DEV_BAD_STATE);
 }
 
 // ---------------------------------------------------------------------------
@@ -1309,48 +1318,28 @@ __device__ int gap_walk_units(const AlnsTeam& t) {
     return 2 * ns + (ns * ns + ALNS_WARPS - 1) / ALNS_WARPS;
 }
 
-// Both ways through W with one stop (op code ov) at gap (a, i), by warps 0 and 1:
-// departures and tails of all positions, V's at pv, in shared arrays behind the
-// walk buffers.  A pickup V leaves at arrival and a drop V's tail has no pickup: the
-// other stop's edge comes with the other stop, not here.  The CTA lays the route
-// with V in it out in shared memory first, so the walks are those of W (with V taken in
-// place by a few selects in every round, matrix and selection of a step took 31.7
-// us at n = 1000 instead of 31.1, and 20.5 instead of 19.9 at n = 400).
+// both ways through W with one stop at gap (a, i), by warps 0 and 1: departures and tails
+// of the W positions into shared arrays behind the walk buffers, and the three scalars
 struct OneStop {
     int *H, *T;
-    int pv, z;
 };
-__device__ OneStop walk_one_stop(const AlnsTeam& t, const Smem& s, int ov, int a, int i, int N) {
-    const int rw = ((t.n + 1) + 3) & ~3, len = (N + 1 + 3) & ~3, warp = threadIdx.x >> 5;
+__device__ __forceinline__ OneStop walk_one_stop(const AlnsTeam& t, const Smem& s, int ov, int a, int i, int N,
+                                                 int* scal) {
+    const int rw = ((t.n + 1) + 3) & ~3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     OneStop r;
     r.H = s.rdy + 2 * rw;
-    r.T = r.H + len;
-    r.pv = s.sWoff[a] + i;
-    Smem v = s;
-    v.sW = r.T + len;
-    v.sWoff = s.misc + 16;                     // [m + 1]
-    int* z = s.misc + 8;
-    __syncthreads();                           // the buffers are free
-    const int c = ov >> 1, L = s.sWoff[a + 1] - s.sWoff[a];
-    for (int k = threadIdx.x; k <= N; k += blockDim.x) {
-        int x;
-        if (k == r.pv) x = Dx(t, s, i > 0 ? (s.sW[k - 1] & PACK_MASK) >> 1 : 0, c) << PACK_SHIFT | ov;
-        else {
-            x = s.sW[k - (k > r.pv ? 1 : 0)];
-            if (k == r.pv + 1 && i < L) x = Dx(t, s, c, (x & PACK_MASK) >> 1) << PACK_SHIFT | (x & PACK_MASK);
-        }
-        v.sW[k] = x;
-    }
-    if (threadIdx.x <= t.m) v.sWoff[threadIdx.x] = s.sWoff[threadIdx.x] + (a < static_cast<int>(threadIdx.x) ? 1 : 0);
-    __syncthreads();
+    r.T = r.H + ((N + 3) & ~3);
     if (warp == 0) {
-        const int z1 = walk_heads(t, v, s.rdy, r.H, (ov & 1) ? c : 0);
-        if (threadIdx.x == 0) *z = z1;
+        int hv = 0;
+        const int z1 = walk_fwd1(t, s, s.rdy, ov, a, i, r.H, &hv);
+        if (lane == a) scal[1] = hv;
+        if (lane == 0) scal[0] = z1;
     } else if (warp == 1) {
-        walk_tails(t, v, s.rdy + rw, r.T, (ov & 1) ? 0 : c, -1);
+        int tv = 0;
+        walk_bwd1(t, s, s.rdy + rw, ov, a, i, r.T, &tv);
+        if (lane == a) scal[2] = tv;
     }
     __syncthreads();
-    r.z = *z;
     return r;
 }
 
@@ -1367,18 +1356,11 @@ __device__ void gap_walks(const AlnsTeam& t, const Smem& s, int rank, int team_b
             const int packed = t.slist[e], ti = packed / G, g = packed - ti * G;
             const int r = route_of_gap(t, s, g);
             int* base = t.scw + static_cast<long long>(e) * t.scw_stride;
-            const OneStop w = walk_one_stop(t, s, 2 * t.rem[ti] + as_col, r, pos_of(g, r), N);
+            const OneStop w = walk_one_stop(t, s, 2 * t.rem[ti] + as_col, r, pos_of(g, r), N, base + 4 * nmax + as_col * 3);
             int* Hb = base + as_col * 2 * nmax;
             for (int k = threadIdx.x; k < N; k += blockDim.x) {
-                const int q = k + (k >= w.pv ? 1 : 0);
-                Hb[k] = w.H[q];
-                Hb[nmax + k] = w.T[q];
-            }
-            if (threadIdx.x == 0) {
-                int* scal = base + 4 * nmax + as_col * 3;
-                scal[0] = w.z;
-                scal[1] = w.H[w.pv];
-                scal[2] = w.T[w.pv];
+                Hb[k] = w.H[k];
+                Hb[nmax + k] = w.T[k];
             }
         } else {
             const int q = (unit - 2 * ns) * ALNS_WARPS + warp;
@@ -1758,15 +1740,15 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
     const bool pre = e < SC_CAP;
     const int nmax = (t.scw_stride - 8) / 4;
     const int* pbase = t.scw + static_cast<long long>(pre ? e : 0) * t.scw_stride + as_col * 2 * nmax;
+    int* sh = s.misc + 8;                      // z1, h_v, t_v
     const int ga = t.groute[g], gi = t.gpos[g];
     const int ov = 2 * c + as_col;
-    OneStop own = {nullptr, nullptr, 0, 0};    // departures and tails in W + V, simulated here
-    if (!pre) own = walk_one_stop(t, s, ov, ga, gi, N);
-    const int* scal = t.scw + static_cast<long long>(pre ? e : 0) * t.scw_stride + 4 * nmax + as_col * 3;
-    const int z1 = pre ? scal[0] : own.z, hv = pre ? scal[1] : own.H[own.pv], tv = pre ? scal[2] : own.T[own.pv];
-    // of the stop at W position p
-    auto Hb = [&](int p) { return pre ? pbase[p] : own.H[p + (p >= own.pv ? 1 : 0)]; };
-    auto Tb = [&](int p) { return pre ? pbase[nmax + p] : own.T[p + (p >= own.pv ? 1 : 0)]; };
+    OneStop own = {nullptr, nullptr};          // departures and tails in W + V, simulated here
+    if (!pre) own = walk_one_stop(t, s, ov, ga, gi, N, sh);
+    const int* Hb = pre ? pbase : own.H;
+    const int* Tb = pre ? pbase + nmax : own.T;
+    const int* scal = pre ? t.scw + static_cast<long long>(e) * t.scw_stride + 4 * nmax + as_col * 3 : sh;
+    const int z1 = scal[0], hv = scal[1], tv = scal[2];
     const int z = ctl->z_work, pc = s.sp[c];
     const long long scrow = static_cast<long long>(ti) * G;
     const bool dump = t.mode == 1;
@@ -1791,13 +1773,13 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
                 int zn;
                 if (!as_col) {
                     const int xb = t.gx[col];
-                    const int arr = (xb >= 0 ? Hb(xb) : 0) + Dx(t, s, loc(xb), c);
+                    const int arr = (xb >= 0 ? Hb[xb] : 0) + Dx(t, s, loc(xb), c);
                     const int dep = max(arr, hv + pc);
-                    zn = max(z1, dep + Dx(t, s, c, loc(yb)) + (yb >= 0 ? Tb(yb) : 0));
+                    zn = max(z1, dep + Dx(t, s, c, loc(yb)) + (yb >= 0 ? Tb[yb] : 0));
                 } else {
                     const int ya = t.gy[row];
-                    const int td = (xa >= 0 ? Hb(xa) : 0) + Dx(t, s, loc(xa), c);
-                    zn = max(z1, max(td + Dx(t, s, c, loc(ya)) + (ya >= 0 ? Tb(ya) : 0), td + pc + tv));
+                    const int td = (xa >= 0 ? Hb[xa] : 0) + Dx(t, s, loc(xa), c);
+                    zn = max(z1, max(td + Dx(t, s, c, loc(ya)) + (ya >= 0 ? Tb[ya] : 0), td + pc + tv));
                 }
                 ++cnt;
                 const int dt = travel_delta(t, s, c, row, col);
@@ -2845,6 +2827,8 @@ __device__ __noinline__ void replica_import(const AlnsTeam& t, const Smem& s) {
 // replicas, 40 ms of an 81 ms run, 1.0 ms now.
 enum { LS_PICKUP = 1, LS_RELOCATE = 2 };
 
+constexpr int TAIL_BITS = (1 << 29) - 1;       // a tail; the bit above: the op leads to the candidate's drop
+constexpr int TAIL_NONE = INT32_MIN + 1;       // tail of a pickup that is not in the solution
 constexpr int LS_MAX_CTAS = SC_CAP * SC_CAP / 4;
 
 // Scratch of one CTA, in words: H, T, stock after each op, packed prefix and
@@ -2951,6 +2935,45 @@ __device__ void stage_without(const AlnsTeam& t, const Smem& s, int lo, int hi) 
         W[k] = (Dx(t, s, prev, o >> 1) << PACK_SHIFT) | o;
     }
     __syncthreads();
+}
+
+// One warp: the tail of every staged op (longest path from its departure to
+// the end of the schedule) into T, with the mark of the ops that lead to the
+// drop of c at dpos.  c > 0: c's pickup is not in the solution.
+__device__ void walk_tails(const AlnsTeam& t, const Smem& s, int* tp_, int* T, int c0, int dpos) {
+    const int lane = threadIdx.x & 31, n = t.n;
+    for (int c = lane; c <= n; c += 32) tp_[c] = c0 > 0 && c == c0 ? TAIL_NONE : UNRES;
+    __syncwarp();
+    const WalkMem M(s, tp_);
+    const int start = lane < t.m ? s.sWoff[lane] : 0;
+    int pos = (lane < t.m ? s.sWoff[lane + 1] : 0) - 1;
+    int x = pos >= start ? M.op(pos) : 0;
+    int leg = pos >= start ? Dx(t, s, (x & PACK_MASK) >> 1, 0) : 0, acc = 0, mark = 0;
+    bool moved;
+    do {
+        moved = false;
+#pragma unroll
+        for (int k = 0; k < WALK_ROUNDS; ++k) {
+            const unsigned ca = M.at(x);
+            const bool pick = (x & 1) != 0;
+            const int rv = M.ld(M.r + ca), p = M.ld(M.p + ca), nx = M.op(max(pos - 1, 0));
+            const int r = pick ? TAIL_NONE : rv;   // (a drop of a customer without its pickup waits for nothing, as a pickup)
+            const bool go = pos >= start && r != UNRES;
+            const int after = acc + leg;
+            const int d = r == TAIL_NONE ? after : max(after, p + (r & TAIL_BITS));
+            int mk = mark | (r == TAIL_NONE ? 0 : r & ~TAIL_BITS);
+            if (pos == dpos) mk = TAIL_BITS + 1;
+            if (go) T[pos] = d | mk;
+            if (go && pick) M.st(M.r + ca, d | mk);
+            acc = go ? d : acc;
+            mark = go ? mk : mark;
+            leg = go ? x >> PACK_SHIFT : leg;
+            pos -= go ? 1 : 0;
+            x = go ? (pos >= start ? nx : 0) : x;
+            moved |= go;
+            __syncwarp();
+        }
+    } while (__any_sync(FULL_MASK, moved));
 }
 
 // One warp, route r of the staged solution: stock after every op, its running
