@@ -69,9 +69,9 @@ struct EvalArgs {
 // (3.9 k), where the earlier kernels issued 9.9 k and 8.4 k: one route per lane
 // runs at 81% of the issue slots and 72% of the shared-memory pipe, two routes
 // at 53% and 60%, short of warps.  262144 candidates: 2861 us before (its best
-// walk and shape), 1411 us now; n=100 m=4, 65536: 89 to 43 us; n=499 m=19,
-// 65536, a quarter of them blocked: 348 to 181 us; 32 instances of 17 to 500
-// customers, 4096 each: 298 to 135 us.
+// walk and shape), 1411 us now; n=100 m=4, 65536: 89 to 42 us; n=499 m=19,
+// 65536, a quarter of them blocked: 348 to 179 us; 32 instances of 17 to 500
+// customers, 4096 each: 298 to 137 us.
 // Tried at n=1000: the round's loads a round earlier, between the two routes'
 // steps (21% more instructions, 446 us against 365 us for 65536 candidates);
 // legs computed after the round's loads (385); groups of two warps with a
@@ -79,12 +79,12 @@ struct EvalArgs {
 // 172 us at n=499); eight code chunks in flight at 64 registers (spills, 486).
 //
 // Ready slots.  Slot c holds -(p_c + 1) until c's drop, the pickup-ready time
-// T_drop + p_c until its pickup, then PICKED.  The slots of the depot (c = 0)
-// and of code 2n+2 (c = n+1, where every code out of range ends up) start as
-// PICKED, so nothing on them is ever ready.  A lane past its route's end holds
-// code 1, "pick up at the depot": it never goes, its point is the depot, so
-// the leg it computes is the way home, and no lane state says whether the
-// route is still going on.
+// T_drop + p_c until its pickup, then PICKED for good: a drop that finds PICKED
+// stores nothing.  The slots of the depot (c = 0) and of code 2n+2 (c = n+1,
+// where every code out of range ends up) start as PICKED, so nothing on them is
+// ever ready.  A lane past its route's end holds code 1, "pick up at the depot":
+// it never goes, its point is the depot, so the leg it computes is the way home,
+// and no lane state says whether the route is still going on.
 //
 // A round with no progress in the whole warp ends the walk: every write of
 // earlier rounds was visible to this one, so nothing can go later either.
@@ -93,13 +93,21 @@ struct EvalArgs {
 // Validation without bookkeeping in the walk.  Let a candidate's offsets be in
 // order (checked first).  If no route of it is blocked, 2n ops were walked.  A
 // slot becomes PICKED only by a pickup of its customer, and a pickup goes only
-// after a drop of the same customer.  So if every customer's slot ends PICKED,
-// the 2n ops hold a drop and a pickup of each of the n customers and nothing
-// else: a permutation.  If some slot does not, an op is repeated or out of
-// range.  A candidate with a blocked route gets the full check (range and a
-// duplicate bitmap), which tells MALFORMED from CYCLE.  Whatever a repeated or
-// foreign code does to the slots on the way stays inside its own candidate,
-// and every route still ends: each round that goes on takes at least one op.
+// after a drop of the same customer: a drop stores nd - 1 - r, which is
+// T_drop + p_c over the slot's first state and between -1 and nd over a ready
+// time (nd >= r then; -1 is the first state of p_c = 0), and no nd + p_c wraps.
+// (Every leg is one of the instance's, also to and from the point of code 2n+2,
+// and no path through the walked ops passes one twice or adds a p_c twice, so
+// times stay within the (2n+1) max d + n max p that an instance keeps below
+// 2^31 - 1.)  So if every customer's slot ends PICKED, the 2n ops hold a drop
+// and a pickup of each of the n customers and nothing else: a permutation.  If
+// some slot does not, an op is repeated or out of range.  (Over PICKED the
+// drop's sum would wrap, to a ready time or, a drop later, even to PICKED: with
+// such drops stored, 2 3 2 3 4 6 passed for three customers at the depot with
+// p = 0, 1, 1.)  A candidate with a blocked route gets the full check (range and
+// a duplicate bitmap), which tells MALFORMED from CYCLE.  Whatever a repeated or
+// foreign code does to the slots on the way stays inside its own candidate, and
+// every route still ends: each round that goes on takes at least one op.
 //
 // Stock.  One word holds 2^14 - s above 2^14 + s (s the stock relative to the
 // start, |s| <= 2n < 2^13), so one add moves both and one packed maximum keeps
@@ -160,17 +168,17 @@ struct Place {
     static constexpr int BIAS = 0;
     int row;                                   // c (n+1)
     static __device__ __forceinline__ Place of(const EvalArgs& a, const int32_t*, int c) {
-        // code 2n+2 stands one past the matrix: any row will do, its candidate is malformed
-        if constexpr (DM == VRPRPD_DIST_GLOBAL16 || DM == VRPRPD_DIST_GLOBAL32) return {min(c, a.n) * a.N};
-        else return {c * a.N};
+        // code 2n+2 stands one past the matrix: the last customer's row and column will
+        // do, its candidate is malformed
+        return {min(c, a.n) * a.N};
     }
     static __device__ __forceinline__ int leg(const EvalArgs& a, const int32_t* sh, const Place& x, const Place&,
                                               int c) {
-        // shared matrices: row and column n+1 fall into the block's other data, never outside it
-        if constexpr (DM == VRPRPD_DIST_SMEM32) return sh[x.row + c];
-        else if constexpr (DM == VRPRPD_DIST_SMEM16) return reinterpret_cast<const uint16_t*>(sh)[x.row + c];
-        else if constexpr (DM == VRPRPD_DIST_GLOBAL16) return __ldg(a.d16 + x.row + min(c, a.n));
-        else return __ldg(a.d32 + x.row + min(c, a.n));
+        const int at = x.row + min(c, a.n);
+        if constexpr (DM == VRPRPD_DIST_SMEM32) return sh[at];
+        else if constexpr (DM == VRPRPD_DIST_SMEM16) return reinterpret_cast<const uint16_t*>(sh)[at];
+        else if constexpr (DM == VRPRPD_DIST_GLOBAL16) return __ldg(a.d16 + at);
+        else return __ldg(a.d32 + at);
     }
 };
 template <>
@@ -394,7 +402,7 @@ __device__ __forceinline__ void eval_tile(const EvalArgs& a, const int32_t* sh, 
                 }
                 prev[s] = go ? code[s] : prev[s];
             }
-            sts_s32_if(go, ad[s], pick ? PICKED : static_cast<int>(static_cast<unsigned>(nd) - 1u - static_cast<unsigned>(r[s])));
+            sts_s32_if(go && r[s] != PICKED, ad[s], pick ? PICKED : static_cast<int>(static_cast<unsigned>(nd) - 1u - static_cast<unsigned>(r[s])));
             any = any || go;
             if (go) {
                 dep[s] = nd - P::BIAS;
@@ -526,7 +534,7 @@ __global__ void __launch_bounds__(32 * max_warps(V)) eval_tiles_kernel(EvalArgs 
         unsigned dist_bytes = 0;
         if constexpr (DM == VRPRPD_DIST_SMEM32) dist_bytes = ((a.N * a.N * 4) + 15) & ~15;
         if constexpr (DM == VRPRPD_DIST_SMEM16) dist_bytes = ((a.N * a.N * 2) + 15) & ~15;
-        if constexpr (DM == VRPRPD_DIST_COORDS) dist_bytes = ((a.N * 8) + 15) & ~15;
+        if constexpr (DM == VRPRPD_DIST_COORDS) dist_bytes = ((a.N * 8) + 8 + 15) & ~15;
         const unsigned row_bytes = a.row_words * 4u;
         if constexpr (DM == DIST_HALF2) dist_bytes = row_bytes;
         mbar_arrive_expect_tx(&block_bar, dist_bytes + row_bytes);
@@ -759,7 +767,7 @@ static bool make_plan(const vrprpd_instance* I, int dm, int warps, int V, long l
     long long dist_words = 0;
     if (dm == VRPRPD_DIST_SMEM32) dist_words = N * N;
     if (dm == VRPRPD_DIST_SMEM16) dist_words = (N * N + 1) / 2;
-    if (dm == VRPRPD_DIST_COORDS) dist_words = 2 * N;
+    if (dm == VRPRPD_DIST_COORDS) dist_words = 2 * (N + 1);   // the point of code 2n+2 with them
     if (dm == DIST_HALF2) dist_words = a.row_words;
     a.dist_words = round4(dist_words);
     a.shared_words = a.dist_words + a.row_words;

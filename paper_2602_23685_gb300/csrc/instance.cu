@@ -228,12 +228,15 @@ static int create_from_coords(const int32_t* coords, const int32_t* p, int32_t n
     const long long dx = hi[0] - lo[0], dy = hi[1] - lo[1];
     I->coords24 = dx * dx + dy * dy < (1ll << 24);
     const bool half = dx * dx + dy * dy < EUC2D_HALF2_LIMIT;
-    const size_t c_words = (2 * N + 63) & ~static_cast<size_t>(63);
+    // one point past the last customer's, the depot's again: where the evaluator
+    // puts a code out of range (no leg is longer than the instance's own)
+    const size_t c_words = (2 * N + 2 + 63) & ~static_cast<size_t>(63);
     std::vector<int32_t> h(c_words + (half ? I->row_words : 0), 0);
     std::copy(coords, coords + 2 * N, h.begin());
-    for (int i = 0; half && i < N; ++i) {
-        const __half2 v = __floats2half2_rn(static_cast<float>(coords[2 * i] - lo[0]),
-                                            static_cast<float>(coords[2 * i + 1] - lo[1]));
+    std::copy(coords, coords + 2, h.begin() + 2 * N);
+    for (int i = 0; half && i <= N; ++i) {
+        const __half2 v = __floats2half2_rn(static_cast<float>(h[2 * i] - lo[0]),
+                                            static_cast<float>(h[2 * i + 1] - lo[1]));
         std::memcpy(&h[c_words + i], &v, 4);
     }
     int* dmax = nullptr;
