@@ -258,10 +258,12 @@ int vrprpd_multi_evaluate(vrprpd_multi* plan, void* stream);
  * every instance has them close enough together, GLOBAL16, GLOBAL32) on the
  * plan's own batches; keep the fastest. */
 int vrprpd_multi_autotune(vrprpd_multi* plan, void* stream, vrprpd_eval_config* chosen);
-/* Set the plan's shape by hand: dist_mode GLOBAL16 (every instance with a
- * 16-bit matrix) or GLOBAL32, warps_per_block 1..32, walk staged or streamed
- * with group_warps 1 (Section 4.2.1's multi-instance parallelism, the same
- * evaluation).  VRPRPD_EINVAL when the shape does not fit. */
+/* Set the plan's shape by hand, or again one that vrprpd_multi_autotune gave:
+ * dist_mode COORDS (every instance from coordinates, close enough together),
+ * GLOBAL16 (every instance with a 16-bit matrix) or GLOBAL32, warps_per_block
+ * 1..32, walk staged or streamed with group_warps 1 or 2 (Section 4.2.1's
+ * multi-instance parallelism, the same evaluation).  VRPRPD_EINVAL when the
+ * shape does not fit or an instance lacks what the mode reads. */
 int vrprpd_multi_set_config(vrprpd_multi* plan, const vrprpd_eval_config* cfg);
 void vrprpd_multi_destroy(vrprpd_multi* plan);
 

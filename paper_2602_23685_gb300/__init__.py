@@ -468,8 +468,8 @@ class MultiBatch:
         _check(lib().vrprpd_multi_autotune(self._h, _stream_ptr(stream), C.byref(cfg)))
         return _cfg_dict(cfg)
 
-    def set_config(self, dist_mode="global16", warps_per_block=8, walk="staged"):
-        cfg = EvalConfig(DIST_MODES[dist_mode], warps_per_block, 0, WALKS[walk], 1)
+    def set_config(self, dist_mode="global16", warps_per_block=8, walk="staged", group_warps=1):
+        cfg = EvalConfig(DIST_MODES[dist_mode], warps_per_block, 0, WALKS[walk], group_warps)
         _check(lib().vrprpd_multi_set_config(self._h, C.byref(cfg)))
 
     def close(self):

@@ -1380,7 +1380,8 @@ extern "C" int vrprpd_multi_autotune(vrprpd_multi* M, void* stream_, vrprpd_eval
     for (int V : {1, 2}) {
         for (int dm : {DIST_HALF2, static_cast<int>(VRPRPD_DIST_GLOBAL16), static_cast<int>(VRPRPD_DIST_GLOBAL32)}) {
             if ((dm == DIST_HALF2 && !M->all_xy) || (dm == VRPRPD_DIST_GLOBAL16 && !M->all16)) continue;
-            for (int warps : {4, 8, 12, 16, 24, 32}) {
+            for (int warps : {4, 8, 12, 16, 24, 32, 2, 1}) {
+                if (warps < 4 && best < 1e30f) continue;      // only where no larger block fits
                 if (M->accepted_words[V - 1] * 4 * warps + 64 > static_cast<long long>(M->smem_optin)) continue;
                 if (multi_layout(M, dm, warps, V) != VRPRPD_OK) continue;
                 float ms_min = 1e30f;
@@ -1414,17 +1415,22 @@ extern "C" int vrprpd_multi_autotune(vrprpd_multi* M, void* stream_, vrprpd_eval
 
 extern "C" int vrprpd_multi_set_config(vrprpd_multi* M, const vrprpd_eval_config* cfg) {
     VRP_CHECK(M && cfg, VRPRPD_EINVAL, "NULL argument");
-    VRP_CHECK(cfg->dist_mode == VRPRPD_DIST_GLOBAL16 || cfg->dist_mode == VRPRPD_DIST_GLOBAL32, VRPRPD_EINVAL,
-              "many-instance plans gather distances from L2: dist_mode must be GLOBAL16 or GLOBAL32");
-    VRP_CHECK(cfg->walk == VRPRPD_WALK_STAGED || (cfg->walk == VRPRPD_WALK_STREAMED && cfg->group_warps == 1),
-              VRPRPD_EINVAL, "walk must be staged, or streamed with one-warp groups");
+    VRP_CHECK(cfg->dist_mode == VRPRPD_DIST_GLOBAL16 || cfg->dist_mode == VRPRPD_DIST_GLOBAL32 ||
+                  cfg->dist_mode == VRPRPD_DIST_COORDS, VRPRPD_EINVAL,
+              "many-instance plans take distances from points or L2: dist_mode must be COORDS, GLOBAL16 or GLOBAL32");
+    VRP_CHECK(cfg->walk == VRPRPD_WALK_STAGED ||
+                  (cfg->walk == VRPRPD_WALK_STREAMED && (cfg->group_warps == 1 || cfg->group_warps == 2)),
+              VRPRPD_EINVAL, "walk must be staged, or streamed with group_warps 1 or 2");
+    VRP_CHECK(cfg->dist_mode != VRPRPD_DIST_COORDS || M->all_xy, VRPRPD_EINVAL,
+              "an instance has no points, or points too far apart");
     if (cfg->dist_mode == VRPRPD_DIST_GLOBAL16)
         for (auto& a : M->args[0]) VRP_CHECK(a.d16 != nullptr, VRPRPD_EINVAL, "an instance has no 16-bit matrix");
     VRP_CHECK(cfg->warps_per_block >= 1 && cfg->warps_per_block <= 32, VRPRPD_EINVAL, "bad warps_per_block");
     const bool streamed = cfg->walk == VRPRPD_WALK_STREAMED;
     VRP_CHECK(M->accepted_words[streamed] * 4 * cfg->warps_per_block + 64 <= static_cast<long long>(M->smem_optin),
               VRPRPD_EINVAL, "this layout does not fit shared memory");
-    const int rc = multi_layout(M, cfg->dist_mode, cfg->warps_per_block, 1);
+    const int rc = multi_layout(M, cfg->dist_mode == VRPRPD_DIST_COORDS ? DIST_HALF2 : cfg->dist_mode,
+                                cfg->warps_per_block, streamed ? cfg->group_warps : 1);
     VRP_CHECK(rc == VRPRPD_OK, rc, "this layout does not fit shared memory");
     return VRPRPD_OK;
 }
