@@ -277,6 +277,7 @@ __device__ __forceinline__ unsigned add_acq_rel(unsigned* p, unsigned v) {
     asm volatile("atom.acq_rel.gpu.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
 }
+// Whatever fails in a run goes through here: the barriers read the flag, not err.
 __device__ __forceinline__ void fail_run(AlnsCtl* ctl, int why) {
     atomicExch(&ctl->err, why);
     atomicOr(&ctl->bar_gen, GEN_FAILED);
@@ -724,7 +725,7 @@ __device__ void walk_bwd1(const AlnsTeam& t, const Smem& s, int* tp_, int ov, in
         }
     } while (__any_sync(FULL_MASK, moved));
     if (lane == a) *tv = tl;
-    if (q >= 0) atomicExch(&t.ctl->err, DEV_BAD_STATE);
+    if (q >= 0) fail_run(t.ctl, DEV_BAD_STATE);
 }
 
 // ---------------------------------------------------------------------------
