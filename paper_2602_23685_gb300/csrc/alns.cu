@@ -295,7 +295,7 @@ __device__ __forceinline__ bool release_team(AlnsCtl* ctl, unsigned gen) {
 // one thread: until a counter of the step has come to want (false: the wait ran out).
 // The two waits are out of line: inlined, their registers cost the tiles more spills
 // (32 replicas at n = 1000: 632 ms instead of 623).
-__device__ __noinline__ bool await_count(AlnsCtl* ctl, const int* count, int want) {
+[[nodiscard]] __device__ __noinline__ bool await_count(AlnsCtl* ctl, const int* count, int want) {
     const uint64_t t0 = global_ns();
     const unsigned long long limit = ctl->wait_ns;
     int v;
@@ -1876,6 +1876,7 @@ __device__ __forceinline__ void tile_of(int item, int RT, int CT, int* prt, int*
 // us without it and 36.3 with it (random removal), 57.1 and 51.0 (all removals).
 // Thread w keeps word w of the mask (rows and columns fit 12 bits, so there
 // are 128 x 64 tiles at most) and the number of bits in the words before it.
+// (count below 0: the wait for the other CTAs' tests ran out)
 struct TileMask {
     int count, before;
     unsigned word;
@@ -1918,12 +1919,13 @@ __device__ __noinline__ TileMask test_tiles(const AlnsTeam& t, const Smem& s, in
         }
         __syncthreads();
     }
+    bool failed = false;
     if (threadIdx.x == 0) {
         if (rank < want) add_acq_rel(reinterpret_cast<unsigned*>(&ctl->tests_done), 1u);
-        await_count(ctl, &ctl->tests_done, want);
+        failed = !await_count(ctl, &ctl->tests_done, want);
     }
-    __syncthreads();
-    TileMask r;
+    TileMask r = {-1, 0, 0u};
+    if (__syncthreads_or(failed)) return r;
     const int w = static_cast<int>(threadIdx.x);
     r.word = w < words ? __ldcg(&t.tmask[w]) : 0u;
     int incl = __popc(r.word);
@@ -1944,15 +1946,16 @@ __device__ __noinline__ TileMask test_tiles(const AlnsTeam& t, const Smem& s, in
     return r;
 }
 
-__device__ void phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int team_blocks) {
+// False when a wait for other CTAs' part ran out: the keys are incomplete then.
+__device__ bool phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int team_blocks) {
     AlnsCtl* ctl = t.ctl;
     const int N = s.sWoff[t.m], G = N + t.m;
     const int RT = (G + TR - 1) / TR, CT = (G + TC - 1) / TC;
     const int tiles = RT * CT;
     // The shortcut items go out first: each scores a whole row or column of
     // G entries, far more work than a tile, so at the end of the phase they
-    // would leave most of the team waiting; their simulations are done by the
-    // time the phase starts (the team barrier before it waits for every walk).
+    // would leave most of the team waiting.  Other CTAs may still be simulating
+    // their gaps then, so the first item of a CTA waits for walks_done.
     const int nfb = 2 * ctl->n_short * FB_SPLIT;
     const int nwalks = gap_walk_units(t);
     bool walks_seen = false;
@@ -1960,7 +1963,10 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int tea
     const int testers = team_blocks - nwalks;
     const bool test = t.mode != 1 && ctl->nrem <= ACT_CAP && tiles > team_blocks && 2 * testers >= team_blocks;
     TileMask mask = {tiles, 0, 0u};
-    if (test) mask = test_tiles(t, s, rank, testers, G);
+    if (test) {
+        mask = test_tiles(t, s, rank, testers, G);
+        if (mask.count < 0) return false;
+    }
     // the tile of the k-th bit of the mask
     auto tested_tile = [&](int k) {
         if (k >= mask.before && k < mask.before + __popc(mask.word)) {
@@ -1985,8 +1991,7 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int tea
         } else {
             if (!walks_seen) {
                 // the shortcut simulations, still running in other CTAs, must be done (bounded wait)
-                if (threadIdx.x == 0) await_count(ctl, &ctl->walks_done, nwalks);
-                __syncthreads();
+                if (__syncthreads_or(threadIdx.x == 0 && !await_count(ctl, &ctl->walks_done, nwalks))) return false;
                 walks_seen = true;
             }
             fallback_item(t, s, item, N, G);
@@ -1994,6 +1999,7 @@ __device__ void phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int tea
         __syncthreads();                       // the next item is known, this one's buffers are free
         item = slot[turn];
     }
+    return true;
 }
 
 // Insert customer c into the staged solution (s.sW, s.sWoff): its drop at
@@ -3524,7 +3530,7 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
         team_arrive(ctl, team_blocks, gen);
         gap_walks(t, s, rank, team_blocks);
         if (!team_wait(ctl, team_blocks, gen)) return;
-        phase_matrix(t, s, rank, team_blocks);
+        if (!phase_matrix(t, s, rank, team_blocks)) return;
         team_barrier(ctl, team_blocks, gen);
         return;
     }
@@ -3560,11 +3566,11 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
                 __syncthreads();
                 if (threadIdx.x == 0) team_s.mode = 1;
                 __syncthreads();
-                phase_matrix(t, s, rank, team_blocks);
+                if (!phase_matrix(t, s, rank, team_blocks)) return;
                 team_barrier(ctl, team_blocks, gen);
                 return;
             }
-            phase_matrix(t, s, rank, team_blocks);
+            if (!phase_matrix(t, s, rank, team_blocks)) return;
             if (!team_barrier_select(t, s, team_blocks, gen)) return;
         }
         return;
@@ -3638,7 +3644,7 @@ __global__ void __launch_bounds__(ALNS_THREADS, 3) alns_kernel(AlnsTeam* teams, 
             gap_walks(t, s, rank, team_blocks);
             if (!team_wait(ctl, team_blocks, gen)) return;
             mark(2);
-            phase_matrix(t, s, rank, team_blocks);
+            if (!phase_matrix(t, s, rank, team_blocks)) return;
             if (!team_barrier_select(t, s, team_blocks, gen)) return;   // select runs inside
             mark(3);
             mark(4);
