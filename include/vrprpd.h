@@ -346,10 +346,12 @@ typedef struct {
     double T_final;
     double w_destroy[8], w_repair[4];  /* final operator weights (destroy 0-5 used) */
     double device_ms;          /* wall time of the device run */
-    int64_t matrix_entries;    /* insertion-matrix entries decided by the O(1) tile formula or its bound
-                                  (pruned_entries of them), and gaps the local search scored */
+    int64_t matrix_entries;    /* insertion-matrix entries, and gaps or pairs of gaps of the local search,
+                                  decided by the O(1) formula or its bound (pruned_entries of them) */
     int64_t fallback_entries;  /* entries with a shortcut gap: exact from simulations with one stop
-                                  (both gaps shortcuts: both stops) instead of the tile formula */
+                                  (both gaps shortcuts: both stops) instead of the tile formula; in the
+                                  relocation also those that its bound rules out.  Like matrix_entries
+                                  the same on every run with the same inputs and seed */
     int32_t team_blocks;       /* CTAs used */
     double phase_ms[6];        /* wall time per phase: begin, prep, gaps, matrix, select, end */
     int64_t incremental_steps; /* greedy steps whose longest-path table was updated in O(N^2) */
@@ -365,7 +367,9 @@ typedef struct {
     int64_t pruned_entries;    /* of matrix_entries, those never scored: a lower bound over their
                                   tile showed that none of them can be the one the repair operator
                                   picks (its per-vehicle bests, or the best, are already at or
-                                  below it); the result is the same as scoring them */
+                                  below it), or a local-search pass had reached less already; the
+                                  result is the same as scoring them.  How many depends on the order
+                                  in which CTAs finish: not the same on every run */
     int64_t tiles;             /* insertion-matrix tiles (32 drop gaps x 64 pickup gaps) tested or run */
     int64_t tiles_pruned;      /* of those, tiles in which no customer was left to score */
 } vrprpd_alns_stats;

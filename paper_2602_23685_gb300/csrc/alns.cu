@@ -3063,6 +3063,13 @@ struct LsBest {
         if (h < hi || (h == hi && l < lo)) { hi = h; lo = l; }
     }
 };
+// Gaps and pairs of gaps of one pass, per thread: decided by the formula or by a
+// bound, decided through a shortcut gap, and of the first those scored.  What a
+// bound rules out depends on how far the other CTAs are; the first two do not.
+struct LsCounts {
+    unsigned long long entries = 0, shortcut = 0;
+    unsigned scored = 0;
+};
 // The least of all threads' keys, in thread 0 (sh: 2 u64 per warp).
 __device__ void ls_block_least(LsBest& b, unsigned long long* sh) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -3082,7 +3089,7 @@ __device__ void ls_block_least(LsBest& b, unsigned long long* sh) {
 
 // One candidate of pickup repositioning, the whole CTA.
 __device__ void ls_pickup_item(const AlnsTeam& t, const Smem& s, int* scr, LsRoutes* rt, int c, LsBest& best,
-                               unsigned& scored, unsigned& simulated) {
+                               LsCounts& count) {
     const int n = t.n, m = t.m, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N0 = 2 * n;
     const int rw = ((n + 1) + 3) & ~3;
     const uint16_t* place = reinterpret_cast<const uint16_t*>(t.gains);
@@ -3147,7 +3154,8 @@ __device__ void ls_pickup_item(const AlnsTeam& t, const Smem& s, int* scr, LsRou
             list[atomicAdd(&sh[1], 1)] = g;
             continue;
         }
-        ++scored;
+        ++count.entries;
+        ++count.scored;
         const int zn = max(z1, max((xo >= 0 ? H[xo] : 0) + dxc, hp) + dcy + Ty);
         if (zn < zcur) best.take(zn, len + dxc + dcy - w, c, a, ia, r, pos - (r == a ? 1 : 0));
     }
@@ -3162,7 +3170,7 @@ __device__ void ls_pickup_item(const AlnsTeam& t, const Smem& s, int* scr, LsRou
         const int zn = walk_fwd(t, s, rdy, r, pos, 2 * c + 1, -1, 0, 0, nullptr, nullptr);
         const int x = pos > 0 ? cust(off + pos - 1) : 0, y = pos < L ? cust(off + pos) : 0;
         if (lane == 0) {
-            ++simulated;
+            ++count.shortcut;
             if (zn < zcur)
                 best.take(zn, len + Dx(t, s, x, c) + Dx(t, s, c, y) - Dx(t, s, x, y), c, a, ia, r, pos - (r == a ? 1 : 0));
         }
@@ -3171,14 +3179,14 @@ __device__ void ls_pickup_item(const AlnsTeam& t, const Smem& s, int* scr, LsRou
 
 // One candidate of relocation onto the vehicles part, part + split, ..., the whole CTA.
 __device__ void ls_relocate_item(const AlnsTeam& t, const Smem& s, int* scr, LsRoutes* rt, int c, int part, int split,
-                                 LsBest& best, unsigned& scored, unsigned& simulated) {
+                                 LsBest& best, LsCounts& count) {
     const int n = t.n, m = t.m, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, N0 = 2 * n;
     const int rw = ((n + 1) + 3) & ~3;
     const uint16_t* place = reinterpret_cast<const uint16_t*>(t.gains);
     const int pd = place[2 * c], pp = place[2 * c + 1], zcur = t.ctl->z_cur, bott = t.ctl->ls_bott, pc = s.sp[c];
     int *H = scr, *T = H + N0, *S = T + N0, *PM = S + N0, *SM = PM + N0, *gC = SM + N0, *list = gC + N0 + 4;
     constexpr int SCUT = INT32_MIN;            // gC: a shortcut gap; SKIPV: one that cannot matter; else its path
-    int* sh = s.misc + 32;                     // makespan, largest shortcut, gaps that matter, their least travel
+    int* sh = s.misc + 32;                     // makespan, largest shortcut, gaps that matter, their least travel, bound, shortcut gaps
     // what the whole team's moves of this pass have reached: nothing above it
     // can be the pass's move
     volatile unsigned long long* bound = &t.ctl->ls_bound;
@@ -3246,15 +3254,24 @@ __device__ void ls_relocate_item(const AlnsTeam& t, const Smem& s, int* scr, LsR
             sh[2] = 0;
             sh[3] = INT32_MAX;
             sh[4] = static_cast<int>(min(*bound >> 32, 0x7fffffffull));
+            sh[5] = 0;
         }
         __syncthreads();
         for (int i = tid; i <= L; i += ALNS_THREADS) {
             const Gap g = gap(i);
             const int cut = g.w - g.dxc - g.dcy;
-            if (cut > 0) atomicMax(&sh[1], cut);
+            if (cut > 0) {
+                atomicMax(&sh[1], cut);
+                atomicAdd(&sh[5], 1);
+            }
             gC[i] = cut > 0 ? SCUT : g.Hx + g.dxc + g.dcy + g.Ty;
         }
         __syncthreads();
+        if (tid == 0) {                        // every pair of the route's gaps, whatever a bound leaves out below
+            const unsigned long long gaps = L + 1, plain = gaps - sh[5];
+            count.entries += plain * (plain + 1) / 2;
+            count.shortcut += gaps * (gaps + 1) / 2 - plain * (plain + 1) / 2;
+        }
         // a path through two shortcut gaps loses at most both
         const int cut = sh[1];
         if (z - 2 * cut >= zcur || z - 2 * cut > sh[4]) continue;
@@ -3263,7 +3280,7 @@ __device__ void ls_relocate_item(const AlnsTeam& t, const Smem& s, int* scr, LsR
             const Gap g = gap(i);
             if (gc != SCUT) {
                 const int zn = max(z, g.Hx + g.dxc + max(dcc, pc) + g.dcy + g.Ty);
-                ++scored;
+                ++count.scored;
                 if (zn < zcur && fits_adjacent(i)) best.take(zn, len + g.dxc + dcc + g.dcy - g.w, c, v, i, v, i);
                 if (gc - cut >= zcur) {
                     gC[i] = SKIPV;
@@ -3316,7 +3333,6 @@ __device__ void ls_relocate_item(const AlnsTeam& t, const Smem& s, int* scr, LsR
                 if (!ok) continue;
                 const int zn = walk_insert(t, s, rdy_, c, v, i, v, j);
                 if (lane == 0) {
-                    ++simulated;
                     const int di = gi.dxc + gi.dcy - gi.w;
                     if (zn < zcur)
                         best.take(zn, len + (i == j ? gi.dxc + dcc + gi.dcy - gi.w : di + gj.dxc + gj.dcy - gj.w), c, v, i, v, j);
@@ -3346,7 +3362,7 @@ __device__ void ls_relocate_item(const AlnsTeam& t, const Smem& s, int* scr, LsR
                         const int j = pos + 1 - off, gc = gC[j];
                         if (gc != SCUT && gc != SKIPV) {
                             const Gap gj = gap(j);
-                            ++scored;
+                            ++count.scored;
                             const int zn = max(max(row, gc), max(gi.Hx + gi.dxc + pc + gj.dcy + gj.Ty,
                                                                  gi.Hx + gi.dxc + gi.dcy + val + gj.dxc + gj.dcy + gj.Ty));
                             if (zn < zcur) {
@@ -3381,18 +3397,24 @@ __device__ __noinline__ void ls_pass(const AlnsTeam& t, const Smem& s, int rank,
     int* scr = ls_scratch(t, rank);
     LsRoutes* rt = reinterpret_cast<LsRoutes*>(s.rowv);
     LsBest best;
-    unsigned scored = 0, simulated = 0;
+    LsCounts count;
     if (mode == LS_PICKUP) {
-        for (int k = rank; k < ncand; k += active) ls_pickup_item(t, s, scr, rt, t.lscand[k], best, scored, simulated);
+        for (int k = rank; k < ncand; k += active) ls_pickup_item(t, s, scr, rt, t.lscand[k], best, count);
     } else {
         const int split = max(1, min(t.m - 1, active / max(ncand, 1)));
         for (int k = rank; k < ncand * split; k += active)
-            ls_relocate_item(t, s, scr, rt, t.lscand[k / split], k % split, split, best, scored, simulated);
+            ls_relocate_item(t, s, scr, rt, t.lscand[k / split], k % split, split, best, count);
     }
-    const unsigned ws = __reduce_add_sync(FULL_MASK, scored), wf = __reduce_add_sync(FULL_MASK, simulated);
-    if ((threadIdx.x & 31) == 0) {
-        if (ws) atomicAdd(&ctl->entries, static_cast<unsigned long long>(ws));
-        if (wf) atomicAdd(&ctl->fallback_entries, static_cast<unsigned long long>(wf));
+    unsigned long long we = count.entries, wf = count.shortcut, ws = count.scored;
+    for (int o = 16; o > 0; o >>= 1) {
+        we += __shfl_xor_sync(FULL_MASK, we, o);
+        wf += __shfl_xor_sync(FULL_MASK, wf, o);
+        ws += __shfl_xor_sync(FULL_MASK, ws, o);
+    }
+    if ((threadIdx.x & 31) == 0) {             // (thread 0 holds a route's entries, the others their scores: modulo 2^64)
+        if (we) atomicAdd(&ctl->entries, we);
+        if (we != ws) atomicAdd(&ctl->pruned, we - ws);
+        if (wf) atomicAdd(&ctl->fallback_entries, wf);
     }
     ls_block_least(best, reinterpret_cast<unsigned long long*>(s.colv));
     if (threadIdx.x == 0) {
