@@ -9,6 +9,7 @@
 // Plain form: one thread per candidate, Kahn order over routes, scratch in
 // global memory, distances from global memory.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "device_common.cuh"
@@ -831,6 +832,26 @@ static int plan_shape(const vrprpd_instance* I, const EvalTuning& T, long long n
     return VRPRPD_EINVAL;
 }
 
+// What a batch costs whose distances are gathered from L2, by shape (in lane
+// reads that miss the L1).  The L1 is what the blocks' shared memory leaves of an
+// SM's 256 KB, and how much of the matrix it catches decides: a turn of the SMs
+// takes a round's latency or its lanes' reads, whichever is longer.  The three
+// numbers were fitted to 2800 timings (n 240 to 1400, m 5 to 30, 512 to 32768
+// candidates, one and two routes per lane, 4 to 32 warps): the shape of the
+// least cost is 4% from the fastest one on average; the most routes in flight,
+// as for the other forms, is 18% from it and loses by 1.7 at n=500 m=20 (32768
+// candidates: two routes in 196 KB 249 us, one in 134 KB 152 us).
+static double gather_cost(const EvalArgs& a, long long resident, long long shared, double matrix, int sms) {
+    int kb = 228;
+    for (int step : {196, 164, 132, 100, 64, 32, 16, 8})
+        if (shared <= static_cast<long long>(step) << 10) kb = step;
+    const double misses = 1.0 / 12 + 1.0 - std::min(1.0, std::pow((256 - kb) * 1024.0 / matrix, 0.2));
+    auto turn = [&](double warps) { return std::max(160.0, warps * a.K * a.m * misses); };
+    const long long tiles = (a.num + a.K - 1) / a.K, all = resident * sms;
+    const double rest = static_cast<double>(tiles % all);
+    return static_cast<double>(tiles / all) * turn(static_cast<double>(resident)) + (rest > 0 ? turn(rest / sms) : 0.0);
+}
+
 // The plan when nothing is configured.
 static int auto_plan(const vrprpd_instance* I, long long num, Plan* P) {
     // Distances: points as fp16 pairs when the instance has them (a leg is 7
@@ -843,37 +864,58 @@ static int auto_plan(const vrprpd_instance* I, long long num, Plan* P) {
     else if (accepted_shared_words(I, VRPRPD_DIST_SMEM32) * 8 <= static_cast<long long>(I->smem_optin)) dm = VRPRPD_DIST_SMEM32;
     else if (I->coords24) dm = VRPRPD_DIST_COORDS;
     else if (I->has_d16) dm = VRPRPD_DIST_GLOBAL16;
+    const bool gathers = dm == VRPRPD_DIST_GLOBAL16 || dm == VRPRPD_DIST_GLOBAL32;
+    const double matrix = static_cast<double>(I->n + 1) * (I->n + 1) * (dm == VRPRPD_DIST_GLOBAL16 ? 2 : 4);
+    Plan best;
+    double least = 0;                          // its cost; 0: none yet
+    long long resident = 0;                    // its warps on an SM
+    // Warps per block: most routes in flight on an SM, the smallest block on
+    // ties (n=200 m=6: 4 warps 72 us, 24 warps 76 us), or the least gather_cost.
+    auto take = [&](int V) {
+        for (int warps : {4, 8, 12, 16, 20, 24, 28, 32, 2, 1}) {
+            if (warps > max_warps(V) || (warps < 4 && least != 0) || (warps == 20 && !gathers)) continue;
+            Plan C;
+            C.w16 = P->w16;
+            C.count = P->count;
+            if (!make_plan(I, dm, warps, V, num, &C)) continue;
+            const long long bytes = static_cast<long long>(C.smem + BLOCK_SHARED_BYTES);
+            const long long blocks = std::min<long long>(SM_SHARED_BYTES / bytes, max_warps(V) / warps);
+            const double cost = gathers ? gather_cost(C.args, warps * blocks, blocks * bytes, matrix, I->num_sms)
+                                        : 1.0 / static_cast<double>(warps * blocks * C.args.K);
+            if (least != 0 && cost >= least) continue;
+            least = cost;
+            best = C;
+            resident = warps * blocks;
+        }
+    };
+    auto tiles = [&]() { return (num + best.args.K - 1) / best.args.K; };
     // Two routes per lane when that uses the lanes better by a fifth or more
     // (m = 11, 12 and 17..21): n=499 m=19 (57 of 64 lane slots against 19 of
     // 32) 172 us against 223 us for 65536 candidates, n=1000 m=20 368 against
-    // 377; but n=200 m=6 (30 of 32 both ways) 78 us against 72 us.
-    const int m = I->m, V = 5 * (64 / m) * m >= 6 * 2 * (32 / m) * m ? 2 : 1;
-    // Warps per block: most routes in flight on an SM, the smallest block on
-    // ties (n=200 m=6: 4 warps 72 us, 24 warps 76 us); few tiles are spread
-    // over the SMs first.
-    Plan best;
-    best.w16 = P->w16;
-    best.count = P->count;
-    long long most = 0;
-    for (int warps : {4, 8, 12, 16, 24, 28, 32, 2, 1}) {
-        Plan C;
-        C.count = P->count;
-        if (warps > max_warps(V) || (warps < 4 && most) || !make_plan(I, dm, warps, V, num, &C)) continue;
-        const long long by_smem = SM_SHARED_BYTES / static_cast<long long>(C.smem + BLOCK_SHARED_BYTES);
-        const long long resident = warps * std::min<long long>(by_smem, max_warps(V) / warps);
-        if (resident * C.args.K > most) {
-            most = resident * C.args.K;
-            best.args = C.args;
-            best.dm = C.dm;
-            best.warps = warps;
-            best.V = V;
+    // 377; but n=200 m=6 (30 of 32 both ways) 78 us against 72 us.  The counts
+    // keep two rows per candidate, and two routes per lane take 1.1 to 2 times as
+    // long there (n=200 m=20, 8192: 37.8 us against 30.3), unless that saves a
+    // second turn of the SMs (n=60 m=20, 5120: 10.9 us against 12.7).
+    const int m = I->m;
+    const bool two = 5 * (64 / m) * m >= 6 * 2 * (32 / m) * m;
+    if (gathers || P->count || !two) take(1);
+    if (gathers ? !P->count : !P->count && two) take(2);
+    if (P->count && !gathers && two && resident && tiles() > resident * I->num_sms) {
+        const Plan one = best;
+        const long long before = resident;
+        least = 0;
+        take(2);
+        if (least == 0 || tiles() > resident * I->num_sms) {
+            best = one;
+            resident = before;
         }
     }
-    if (!most) {
+    if (!resident) {
         set_error("no evaluation layout fits shared memory (n=%d, m=%d)", I->n, I->m);
         return VRPRPD_EINVAL;
     }
-    const long long ntiles = (num + best.args.K - 1) / best.args.K;
+    // few tiles are spread over the SMs first
+    const long long ntiles = tiles();
     best.warps = static_cast<int>(std::max<long long>(1, std::min<long long>(best.warps, (ntiles + I->num_sms - 1) / I->num_sms)));
     best.smem = static_cast<size_t>(best.args.shared_words + static_cast<long long>(best.warps) * best.args.warp_words) * 4;
     *P = best;
