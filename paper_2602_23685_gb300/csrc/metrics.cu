@@ -2,7 +2,7 @@
 // Interleaved %) for a batch of complete solutions of one instance.
 //
 // The evaluator's walk counts them on the way (eval.cu).  The kernel here takes
-// what that walk does not: n above 2046, distances from 2^19 or processing
+// what that walk does not: n above 2047, distances from 2^19 or processing
 // times from 2^25 on.
 //
 // One warp per candidate.  A pre-pass over the ops, 32 at a time, checks op

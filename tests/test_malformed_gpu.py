@@ -61,8 +61,8 @@ def sequences(codes, length):
     return np.array(list(itertools.product(codes, repeat=length)), np.int32)
 
 
-# A drop of a customer already picked up must not leave a slot that a pickup, or
-# a later drop with travel plus processing time of 1, could turn into "picked up".
+# A drop of a customer already picked up must leave no slot that a pickup takes, or
+# that a drop with travel plus processing time of 1 turns into "picked up".
 def test_repeated_drop_behind_its_pickup(vrp):
     zo, so = check(vrp, [[2, 3, 2, 3, 4, 6]], [[0, 6]], [0, 1, 1], coords=np.zeros((4, 2), np.int32))
     assert so[0] == vrp.MALFORMED
@@ -89,8 +89,8 @@ def test_all_sequences_of_three_customers(vrp, p):
     check(vrp, ops, [[0, 3, 6], [0, 2, 6]], p, d=d)
 
 
-# the largest processing times an instance may have, where the slots come
-# closest to the words that mean "picked up" and "dropped again"
+# the largest processing times an instance may have, where a slot not dropped yet
+# comes closest to the word that means "picked up"
 @pytest.mark.parametrize("p", [(2**31 - 2,), (2**31 - 3,), (2**31 - 4,), (2**30 - 1, 2**30 - 1)])
 def test_largest_processing_times(vrp, p):
     n = len(p)
