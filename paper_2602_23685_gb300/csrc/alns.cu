@@ -105,7 +105,7 @@ struct AlnsCtl {
     alignas(128) unsigned bar_count;
     alignas(128) unsigned bar_gen;
     alignas(128) int work_counter;
-    alignas(128) int walks_done;      // shortcut simulations finished in this greedy step
+    alignas(128) int walks_done;      // CTAs that have finished their shortcut simulations in this greedy step
     alignas(128) int tests_done;      // CTAs that have tested their share of the matrix tiles in this step
     alignas(128) int n_short;
     int sum_load;
@@ -165,6 +165,7 @@ struct AlnsTeam {
     int* scix;                 // [q_max][G]: index in slist of a shortcut (customer, gap)
     int* scw;                  // [SC_CAP][scw_stride]: walks of the first SC_CAP shortcut gaps (below)
     int scw_stride;
+    int graph_warps;           // warps of a CTA that simulate a shortcut gap at once
     int* scpair;               // [SC_CAP][SC_CAP]: makespan with both stops in two shortcut gaps of one customer
     int* trace;
     int* gains;                // [n+1]: removal gain z(cur) - z(cur - c), worst removal; local search: places of the ops
@@ -1308,19 +1309,31 @@ __device__ __forceinline__ int route_of_gap(const AlnsTeam& t, const Smem& s, in
 // Simulations of the shortcut gaps for the matrix phase: per shortcut gap g of
 // customer c the graph with D_c alone at g (forward, backward) and with P_c
 // alone at g (forward, backward); per pair of shortcut gaps of one customer (g
-// itself twice: the adjacent pair) W with both stops.  A CTA takes one graph of
-// a gap, a warp each way, or eight pairs, a warp each, handed out from the last
-// CTA down.  The walks leave their times in shared memory and the CTA copies
-// them out: stored by the walking lanes, every round to as many lines as there
-// are routes, a graph took 31 us at n = 1000, m = 20, and takes 22 us so.  The
-// units run between arriving at the barrier before the matrix phase and waiting
-// at it, so the tiles of the other CTAs proceed meanwhile; every finished one is
-// counted in walks_done, which the shortcut items wait for.
-__device__ int gap_walk_units(const AlnsTeam& t) {
-    const int ns = min(t.ctl->n_short, SC_CAP);
-    return 2 * ns + (ns * ns + ALNS_WARPS - 1) / ALNS_WARPS;
+// itself twice: the adjacent pair) W with both stops.  A warp takes one graph one
+// way, as many warps at once as have room for their times in shared memory (two
+// from n = 1000 on, all eight below 300), or one pair; the CTAs are filled from
+// the last one down.  The times go out of shared memory when the walk is done:
+// stored by the walking lanes, every round to as many lines as there are routes, a
+// graph took 31 us at n = 1000, m = 20, and takes 22 us so.  The simulations run
+// between arriving at the barrier before the matrix phase and waiting at it, so the
+// tiles of the other CTAs proceed meanwhile; every CTA that has finished its share
+// is counted in walks_done, which the shortcut items wait for.  (One graph per CTA
+// at a time, and a block barrier after every eight pairs, made the gap phase of
+// small solutions with many shortcuts, as matrices without the triangle inequality
+// have, half as long again: n = 15, m = 3, one CTA, 344 steps 7.3 ms in that phase, 4.1 ms now.)
+__host__ __device__ inline int walk_words(int n) { return (((n + 1) + 3) & ~3) + ((2 * n + 3) & ~3); }
+__host__ inline int graph_warps(int n) { return std::min(ALNS_WARPS, static_cast<int>(rdy_words(n)) / walk_words(n)); }
+// CTA-sized units: of graphs, then of pairs
+__device__ __forceinline__ int2 gap_walk_units(const AlnsTeam& t) {
+    const int ns = min(t.ctl->n_short, SC_CAP), W = t.graph_warps;
+    if (ns == 0) return make_int2(0, 0);
+    return make_int2((4 * ns + W - 1) / W, (ns * ns + ALNS_WARPS - 1) / ALNS_WARPS);
 }
-
+// CTAs that have a share of them
+__device__ __forceinline__ int gap_walk_ctas(const AlnsTeam& t, int team_blocks) {
+    const int2 u = gap_walk_units(t);
+    return min(u.x + u.y, team_blocks);
+}
 // both ways through W with one stop at gap (a, i), by warps 0 and 1: departures and tails
 // of the W positions into shared arrays behind the walk buffers, and the three scalars
 struct OneStop {
@@ -1347,44 +1360,54 @@ __device__ __forceinline__ OneStop walk_one_stop(const AlnsTeam& t, const Smem& 
 }
 
 __device__ void gap_walks(const AlnsTeam& t, const Smem& s, int rank, int team_blocks) {
-    const int m = t.m, N = s.sWoff[m], G = N + m;
+    const int m = t.m, n = t.n, N = s.sWoff[m], G = N + m;
     AlnsCtl* ctl = t.ctl;
-    const int ns = min(ctl->n_short, SC_CAP), units = gap_walk_units(t);
+    const int ns = min(ctl->n_short, SC_CAP), W = t.graph_warps;
+    const int2 units = gap_walk_units(t);
     const int nmax = (t.scw_stride - 8) / 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rw = ((n + 1) + 3) & ~3;
+    const int first = team_blocks - 1 - rank;              // this CTA's first unit
+    if (first >= units.x + units.y) return;
     auto pos_of = [&](int g, int r) { return g - (s.sWoff[r] + r); };
-    for (int unit = team_blocks - 1 - rank; unit < units; unit += team_blocks) {
-        if (unit < 2 * ns) {
-            const int e = unit >> 1, as_col = unit & 1;
-            const int packed = t.slist[e], ti = packed / G, g = packed - ti * G;
-            const int r = route_of_gap(t, s, g);
-            int* base = t.scw + static_cast<long long>(e) * t.scw_stride;
-            const OneStop w = walk_one_stop(t, s, 2 * t.rem[ti] + as_col, r, pos_of(g, r), N, base + 4 * nmax + as_col * 3);
-            int* Hb = base + as_col * 2 * nmax;
-            for (int k = threadIdx.x; k < N; k += blockDim.x) {
-                Hb[k] = w.H[k];
-                Hb[nmax + k] = w.T[k];
-            }
+    for (int q = first * W + warp; warp < W && q < 4 * ns; q += team_blocks * W) {
+        const int e = q >> 2, as_col = (q >> 1) & 1, back = q & 1;
+        const int packed = t.slist[e], ti = packed / G, g = packed - ti * G;
+        const int r = route_of_gap(t, s, g), pos = pos_of(g, r), op = 2 * t.rem[ti] + as_col;
+        int* rdy = s.rdy + warp * walk_words(n);
+        int* times = rdy + rw;
+        int* base = t.scw + static_cast<long long>(e) * t.scw_stride;
+        int* scal = base + 4 * nmax + as_col * 3;
+        int v = 0;
+        if (back) {
+            walk_bwd1(t, s, rdy, op, r, pos, times, &v);
+            if (lane == r) scal[2] = v;
         } else {
-            const int q = (unit - 2 * ns) * ALNS_WARPS + warp;
-            if (q < ns * ns) {
-                const int e1 = q / ns, e2 = q - e1 * ns;
-                const int p1 = t.slist[e1], p2 = t.slist[e2];
-                const int ti = p1 / G, g1 = p1 - ti * G, g2 = p2 - ti * G;
-                if (p2 / G == ti) {
-                    const int r1 = route_of_gap(t, s, g1), r2 = route_of_gap(t, s, g2);
-                    const int i1 = pos_of(g1, r1), i2 = pos_of(g2, r2);
-                    if (r1 != r2 || i2 >= i1) {      // (the pickup before the drop: never feasible)
-                        const int zn = walk_insert(t, s, s.rdy + warp * (((t.n + 1) + 3) & ~3), t.rem[ti], r1, i1, r2, i2);
-                        if (lane == 0) t.scpair[e1 * SC_CAP + e2] = zn;
-                    }
-                }
-            }
+            const int z1 = walk_fwd1(t, s, rdy, op, r, pos, times, &v);
+            if (lane == r) scal[1] = v;
+            if (lane == 0) scal[0] = z1;
         }
-        __syncthreads();
-        // results visible device-wide, then counted
-        if (threadIdx.x == 0) add_acq_rel(reinterpret_cast<unsigned*>(&ctl->walks_done), 1u);
+        __syncwarp();
+        int* out = base + (2 * as_col + back) * nmax;
+        for (int k = lane; k < N; k += 32) out[k] = times[k];
+        __syncwarp();
     }
+    __syncthreads();                                       // the pairs' ready times overlap the graphs'
+    const int turn = units.x % team_blocks;                // unit units.x is this CTA's
+    for (int q = ((first - turn + team_blocks) % team_blocks) * ALNS_WARPS + warp; q < ns * ns; q += team_blocks * ALNS_WARPS) {
+        const int e1 = q / ns, e2 = q - e1 * ns;
+        const int p1 = t.slist[e1], p2 = t.slist[e2];
+        const int ti = p1 / G, g1 = p1 - ti * G, g2 = p2 - ti * G;
+        if (p2 / G != ti) continue;
+        const int r1 = route_of_gap(t, s, g1), r2 = route_of_gap(t, s, g2);
+        const int i1 = pos_of(g1, r1), i2 = pos_of(g2, r2);
+        if (r1 == r2 && i2 < i1) continue;                 // the pickup before the drop: never feasible
+        const int zn = walk_insert(t, s, s.rdy + warp * rw, t.rem[ti], r1, i1, r2, i2);
+        if (lane == 0) t.scpair[e1 * SC_CAP + e2] = zn;
+    }
+    __syncthreads();
+    // results visible device-wide, then counted
+    if (threadIdx.x == 0) add_acq_rel(reinterpret_cast<unsigned*>(&ctl->walks_done), 1u);
 }
 
 // Which customers can a matrix tile change the repair operator's pick for?
@@ -1731,6 +1754,7 @@ __device__ void matrix_tile(const AlnsTeam& t, const Smem& s, int rt, int ct, in
 __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N, int G) {
     AlnsCtl* ctl = t.ctl;
     const int piece = item % FB_SPLIT;
+    if (piece * static_cast<int>(blockDim.x) >= G) return;   // fewer blocks of entries than pieces
     item /= FB_SPLIT;
     const int e = item >> 1, as_col = item & 1;
     const int packed = t.slist[e];
@@ -1795,15 +1819,20 @@ __device__ void fallback_item(const AlnsTeam& t, const Smem& s, int item, int N,
             }
         }
         if (dump) continue;
-        if (as_col) fold_rows(t, ti, G, k, vk, key, u);
-        else rowkey = key < rowkey ? key : rowkey;
+        if (as_col) {
+            if (__any_sync(FULL_MASK, key != KEY_NONE)) fold_rows(t, ti, G, k, vk, key, u);
+        } else rowkey = key < rowkey ? key : rowkey;
     }
-    if (!as_col && !dump) {
+    if (!as_col && !dump && __any_sync(FULL_MASK, rowkey != KEY_NONE)) {
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long other = __shfl_xor_sync(FULL_MASK, rowkey, o);
             rowkey = other < rowkey ? other : rowkey;
         }
-        fold_rows(t, ti, G, g, ga, lane == 0 ? rowkey : KEY_NONE, u);
+        if (lane == 0) {                       // (fold_rows for a single row)
+            if ((rowkey >> 12) <= u) atomicMin(&t.keys[scrow + g], rowkey);
+            atomicMin(&t.rkeys[ti * 32 + ga], ((rowkey >> 12) << 12) | static_cast<unsigned long long>(g));
+            atomicMin(&t.gmin[ti * 4 + (ga & 3)], rowkey >> 12);
+        }
     }
     // both gaps shortcuts, from the drop gap's item: full re-simulation, one warp each
     if (!as_col) {
@@ -1957,7 +1986,7 @@ __device__ bool phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int tea
     // would leave most of the team waiting.  Other CTAs may still be simulating
     // their gaps then, so the first item of a CTA waits for walks_done.
     const int nfb = 2 * ctl->n_short * FB_SPLIT;
-    const int nwalks = gap_walk_units(t);
+    const int nwalks = gap_walk_ctas(t, team_blocks);
     bool walks_seen = false;
     int* slot = s.misc;
     const int testers = team_blocks - nwalks;
@@ -1980,10 +2009,12 @@ __device__ bool phase_matrix(const AlnsTeam& t, const Smem& s, int rank, int tea
     const int ntiles = mask.count;
     const int total = ntiles + nfb;
     // The first item is the CTA's own; the rest are handed out by a counter, asked
-    // for while the item before runs (the answer takes a trip to L2).
+    // for while the item before runs (the answer takes a trip to L2).  A CTA by
+    // itself counts on.
     int item = rank;
     for (int turn = 0; item < total; turn ^= 1) {
-        if (threadIdx.x == 0) slot[turn] = total > team_blocks ? team_blocks + atomicAdd(&ctl->work_counter, 1) : total;
+        if (threadIdx.x == 0)
+            slot[turn] = team_blocks == 1 ? item + 1 : total > team_blocks ? team_blocks + atomicAdd(&ctl->work_counter, 1) : total;
         if (item >= nfb) {
             int rt = 0, ct = 0;
             tile_of(test ? tested_tile(item - nfb) : item - nfb, RT, CT, &rt, &ct);
@@ -3779,6 +3810,7 @@ static void carve_team(AlnsTeam& t, DevBuf& B, int n, int m, int qmax, int itera
     t.slist = B.take<int>(static_cast<size_t>(qmax) * G);
     t.scix = B.take<int>(static_cast<size_t>(qmax) * G);
     t.scw_stride = static_cast<int>(4 * N + 8);
+    t.graph_warps = graph_warps(n);
     t.scw = B.take<int>(static_cast<size_t>(SC_CAP) * (4 * N + 8));
     t.scpair = B.take<int>(static_cast<size_t>(SC_CAP) * SC_CAP);
     t.trace = B.take<int>(std::max(iterations, 1));
