@@ -77,7 +77,6 @@ struct AlnsCtl {
     int z_cur, z_best, z_work, z_next;   // z_next: z_work after the insertion just selected
     unsigned st_work;
     int stagnation, repair_fail, wsel, err;
-    int pick_t, pick_row, pick_col;
     unsigned long long wait_ns;       // limit of each spin-wait; one that runs out sets err
     double T, T_init;
     double wd[8], wr[4];
@@ -86,7 +85,7 @@ struct AlnsCtl {
     int z_init;
     // set by the selection when the insertion it applied used no shortcut gap:
     // the next step updates the longest-path table in place of re-walking W.
-    // upd: c, x_a, y_a, x_b, y_b (old positions, -1 = depot), adjacent, new
+    // upd from 1 on: c, x_a, y_a, x_b, y_b (old positions, -1 = depot), adjacent, new
     // positions of D_c and P_c, old length, d(x_a,c), d(c,y_a), d(x_b,c),
     // d(c,y_b), d(c,c), p_c, routes of D_c and P_c
     int incr;
@@ -143,17 +142,17 @@ struct AlnsTeam {
     AlnsCtl* ctl;
     int *cur_ops, *cur_off, *best_ops, *best_off;
     int *W_ops[2], *W_off[2];
-    int *rem, *perm;
+    int *rem;
     int *H, *T, *Ms;
     int *H2, *T2, *Ms2;      // the other copy of each: written by the incremental update, then swapped
     int *S_, *PMINp, *PMAXp, *SMINs, *SMAXs;
     int *spmin, *spmax;      // [LOG][2n]
     int log_levels;
-    int *gx, *gy, *gHx, *gTy, *gw, *gsb, *gpmin, *gpmax, *gsmin, *gsmax, *groute, *gpos;
+    int *gx, *gy, *gw, *gsb, *gpmin, *gpmax, *gsmin, *gsmax, *groute, *gpos;
     int *rload;              // start load per route
     int *growc, *gcolc;      // [G][RV], [G][CV]: per-gap constants of the matrix tiles
     int4 *vrow, *vcol;       // [q_max][G]: per (customer, gap) row / column vectors of the matrix
-    int2 *vadj;              // [q_max][G]: per (customer, gap) adjacent-pair vector
+    int2 *vadj;              // [q_max][G]: per (customer, gap) adjacent-pair vector (null but for dumps)
     unsigned long long* keys;  // [q_max][G]: per drop gap, best (dz, dt, col)
     unsigned long long* rkeys; // [q_max][32]: per drop vehicle, best (dz, dt, row)
     unsigned long long* gmin;  // [q_max][4]: per vehicle group (v mod 4), best (dz, dt) seen so far
@@ -394,12 +393,10 @@ __device__ void stage_W(const AlnsTeam& t, const Smem& s) {
 // ---------------------------------------------------------------------------
 // walks (one warp; lane r walks route r; m <= 32)
 // ---------------------------------------------------------------------------
-// From the depot: node times H, stock prefixes, makespan, cycle flag.
-__device__ void walk_depot(const AlnsTeam& t, const Smem& s, int* rdy_, bool write_arrays, int* z_out,
-                           unsigned* st_out) {
+// From the depot: makespan and status.
+__device__ void walk_depot(const AlnsTeam& t, const Smem& s, int* rdy_, int* z_out, unsigned* st_out) {
     const int* __restrict__ sW = s.sW;
     const int* __restrict__ spp = s.sp;
-    int* const Hh = t.H;
 
     const int lane = threadIdx.x & 31, m = t.m, n = t.n;
     volatile int* rdy = rdy_;
@@ -427,7 +424,6 @@ __device__ void walk_depot(const AlnsTeam& t, const Smem& s, int* rdy_, bool wri
         const int d2 = k2 ? max(a2, r2) : a2;
         if (go1) {
             if (!k1) rdy[c1] = a1 + spp[c1];
-            if (write_arrays) Hh[pos] = d1;
             sv += k1 ? 1 : -1;
             smin = min(smin, sv);
             smax = max(smax, sv);
@@ -436,7 +432,6 @@ __device__ void walk_depot(const AlnsTeam& t, const Smem& s, int* rdy_, bool wri
         }
         if (go2) {
             if (!k2) rdy[c2] = a2 + spp[c2];
-            if (write_arrays) Hh[pos + 1] = d2;
             sv += k2 ? 1 : -1;
             smin = min(smin, sv);
             smax = max(smax, sv);
@@ -1135,8 +1130,6 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
         const int y = yo >= 0 ? (s.sW[yo] & PACK_MASK) >> 1 : 0;
         t.gx[g] = xo;
         t.gy[g] = yo;
-        t.gHx[g] = xo >= 0 ? t.H[xo] : 0;
-        t.gTy[g] = yo >= 0 ? t.T[yo] : 0;
         t.gw[g] = L == 0 ? 0 : Dx(t, s, x, y);
         t.gsb[g] = xo >= 0 ? t.S_[xo] : 0;
         t.gpmin[g] = xo >= 0 ? t.PMINp[xo] : 0;
@@ -1211,7 +1204,7 @@ __device__ void phase_gaps(const AlnsTeam& t, const Smem& s, int rank, int team_
                 vc = make_int4(shortcut ? SKIPV : Hx + Ty + delta, dcy + Ty, delta + Ty,
                                static_cast<int>((static_cast<unsigned>(delta - w) << 12) + static_cast<unsigned>(g)));
                 t.vrow[e] = vr;
-                t.vadj[e] = va;
+                if (t.vadj) t.vadj[e] = va;
                 t.vcol[e] = vc;
                 // the adjacent entry of gap g: the stock check of the drop and
                 // pickup together at g (the tiles' row constant), then its key
@@ -2181,9 +2174,6 @@ __device__ void phase_select(const AlnsTeam& t, const Smem& s) {
             sel[3] = colof(pick);
             // the entry is exact: the makespan once it is inserted
             ctl->z_next = ctl->z_work + static_cast<int>(static_cast<unsigned>(bestv[pick] >> 32) ^ 0x80000000u);
-            ctl->pick_t = sel[1];
-            ctl->pick_row = sel[2];
-            ctl->pick_col = sel[3];
         }
     }
     __syncthreads();
@@ -2212,7 +2202,6 @@ __device__ void phase_select(const AlnsTeam& t, const Smem& s) {
         // gap of this insertion was a shortcut for c
         int* up = ctl->upd;
         auto loc = [&](int pos) { return pos >= 0 ? (s.sW[pos] & PACK_MASK) >> 1 : 0; };
-        up[0] = 1;
         up[1] = c;
         up[2] = xa; up[3] = ya; up[4] = xb; up[5] = yb;
         up[6] = (a == b && ia == jb) ? 1 : 0;
@@ -2622,7 +2611,7 @@ __device__ __noinline__ void phase_end(const AlnsTeam& t, const Smem& s, bool fi
         if ((threadIdx.x >> 5) == 0) {
             int z;
             unsigned st;
-            walk_depot(t, s, s.rdy, false, &z, &st);
+            walk_depot(t, s, s.rdy, &z, &st);
             if ((threadIdx.x & 31) == 0) {
                 ctl->z_work = z;
                 ctl->st_work = st;
@@ -3749,16 +3738,16 @@ static size_t team_bytes(int n, int m, int qmax, int iterations, bool dump) {
     add(1, sizeof(AlnsCtl));
     add(N, 4); add(m + 1, 4); add(N, 4); add(m + 1, 4);
     add(N + 2, 4); add(m + 1, 4); add(N + 2, 4); add(m + 1, 4);
-    add(std::max<size_t>(n + 1, qmax), 4); add(n + 1, 4);
+    add(std::max<size_t>(n + 1, qmax), 4);
     add(N, 4); add(N, 4); add(N * N, 4);
     add(N, 4); add(N, 4); add(N * N, 4);
     for (int i = 0; i < 5; ++i) add(N, 4);
     add(levels * N, 4); add(levels * N, 4);
-    for (int i = 0; i < 12; ++i) add(G, 4);
+    for (int i = 0; i < 10; ++i) add(G, 4);
     add(m, 4);
     add(G * 16, 4); add(G * 12, 4);
     add(static_cast<size_t>(qmax) * G, 16); add(static_cast<size_t>(qmax) * G, 16);
-    add(static_cast<size_t>(qmax) * G, 8);
+    if (dump) add(static_cast<size_t>(qmax) * G, 8);
     add(static_cast<size_t>(qmax) * G, 8);
     add(static_cast<size_t>(qmax) * 32, 8);
     add(static_cast<size_t>(qmax) * 4, 8);
@@ -3786,20 +3775,20 @@ static void carve_team(AlnsTeam& t, DevBuf& B, int n, int m, int qmax, int itera
     t.best_ops = B.take<int>(N); t.best_off = B.take<int>(m + 1);
     t.W_ops[0] = B.take<int>(N + 2); t.W_off[0] = B.take<int>(m + 1);
     t.W_ops[1] = B.take<int>(N + 2); t.W_off[1] = B.take<int>(m + 1);
-    t.rem = B.take<int>(std::max(n + 1, qmax)); t.perm = B.take<int>(n + 1);
+    t.rem = B.take<int>(std::max(n + 1, qmax));
     t.H = B.take<int>(N); t.T = B.take<int>(N); t.Ms = B.take<int>(N * N);
     t.H2 = B.take<int>(N); t.T2 = B.take<int>(N); t.Ms2 = B.take<int>(N * N);
     t.S_ = B.take<int>(N); t.PMINp = B.take<int>(N); t.PMAXp = B.take<int>(N);
     t.SMINs = B.take<int>(N); t.SMAXs = B.take<int>(N);
     t.spmin = B.take<int>(levels * N); t.spmax = B.take<int>(levels * N);
     t.log_levels = levels;
-    t.gx = B.take<int>(G); t.gy = B.take<int>(G); t.gHx = B.take<int>(G); t.gTy = B.take<int>(G);
+    t.gx = B.take<int>(G); t.gy = B.take<int>(G);
     t.gw = B.take<int>(G); t.gsb = B.take<int>(G); t.gpmin = B.take<int>(G); t.gpmax = B.take<int>(G);
     t.gsmin = B.take<int>(G); t.gsmax = B.take<int>(G); t.groute = B.take<int>(G); t.gpos = B.take<int>(G);
     t.rload = B.take<int>(m);
     t.growc = B.take<int>(G * 16); t.gcolc = B.take<int>(G * 12);
     t.vrow = B.take<int4>(static_cast<size_t>(qmax) * G); t.vcol = B.take<int4>(static_cast<size_t>(qmax) * G);
-    t.vadj = B.take<int2>(static_cast<size_t>(qmax) * G);
+    t.vadj = dump ? B.take<int2>(static_cast<size_t>(qmax) * G) : nullptr;
     t.keys = B.take<unsigned long long>(static_cast<size_t>(qmax) * G);
     t.rkeys = B.take<unsigned long long>(static_cast<size_t>(qmax) * 32);
     t.gmin = B.take<unsigned long long>(static_cast<size_t>(qmax) * 4);
