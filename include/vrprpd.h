@@ -77,6 +77,9 @@ int vrprpd_instance_create(const int32_t* coords, const int32_t* p, int32_t n, i
 int vrprpd_instance_create_dist(const int32_t* d, const int32_t* p, int32_t n, int32_t m,
                                 int32_t R, int32_t Q, uint32_t flags, vrprpd_instance** out);
 
+/* Searches and start solutions take their device memory from a pool of the
+ * library's own on the current device.  It keeps up to 256 MiB of freed memory
+ * for the next call while any instance or server lives and goes with the last. */
 void vrprpd_instance_destroy(vrprpd_instance* inst);
 
 /* Copy the instance's (n+1)^2 distance matrix into host memory d_host. */
@@ -228,6 +231,8 @@ typedef struct {
 } vrprpd_eval_config;
 
 int vrprpd_eval_set_config(vrprpd_instance* inst, const vrprpd_eval_config* cfg);
+/* The shape set or tuned (as it was given: a launch may use fewer warps, see
+ * above); without one, the shape chosen for a batch of 2^20 candidates. */
 int vrprpd_eval_get_config(const vrprpd_instance* inst, vrprpd_eval_config* cfg);
 /* Time each feasible configuration on `batch` (device) and keep the fastest.
  * The choice holds for batches like the one timed: give it at least a few
@@ -578,7 +583,10 @@ typedef struct vrprpd_server vrprpd_server;
  * request is admitted (FIFO) when a slot is free, its estimated device memory
  * fits what mem_budget leaves, and its ALNS team fits the resident-CTA share;
  * admitted requests run concurrently on their own streams.  Results do not
- * depend on what else runs: every draw is counter-based. */
+ * depend on what else runs: every draw is counter-based.  Requests' memory
+ * comes from the library's pool, which keeps up to 256 MiB of what has been
+ * used (never more than was in use at once) while any instance or server
+ * lives, so that much of an earlier peak may stay held between requests. */
 int vrprpd_server_create(size_t mem_budget, int32_t max_active, vrprpd_server** out);
 /* Queue a request; VRPRPD_EBUSY if it alone exceeds the memory budget. */
 int vrprpd_server_submit(vrprpd_server* server, const vrprpd_request* req, int64_t* id);

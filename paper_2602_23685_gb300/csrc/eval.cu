@@ -66,11 +66,11 @@ struct EvalArgs {
 //   reduce  makespan, start loads and flags per candidate by shared atomics.
 //
 // What bounds it.  At n=1000 m=20 a candidate takes 1475 wavefronts of shared
-// memory with one route per lane (1206 with two) and 6.0 k warp instructions
-// (3.9 k), where the earlier kernels issued 9.9 k and 8.4 k: one route per lane
+// memory with one route per lane (1208 with two) and 6.1 k warp instructions
+// (4.0 k), where the earlier kernels issued 9.9 k and 8.4 k: one route per lane
 // runs at 81% of the issue slots and 72% of the shared-memory pipe, two routes
-// at 53% and 60%, short of warps.  262144 candidates: 2861 us before (its best
-// walk and shape), 1411 us now; n=100 m=4, 65536: 89 to 42 us; n=499 m=19,
+// at 54% and 61%, short of warps.  262144 candidates: 2861 us before (its best
+// walk and shape), 1415 us now; n=100 m=4, 65536: 89 to 42 us; n=499 m=19,
 // 65536, a quarter of them blocked: 348 to 179 us; 32 instances of 17 to 500
 // customers, 4096 each: 298 to 137 us.
 // Tried at n=1000: the round's loads a round earlier, between the two routes'
@@ -839,8 +839,8 @@ static int plan_shape(const vrprpd_instance* I, const EvalTuning& T, long long n
 // numbers were fitted to 2800 timings (n 240 to 1400, m 5 to 30, 512 to 32768
 // candidates, one and two routes per lane, 4 to 32 warps): the shape of the
 // least cost is 4% from the fastest one on average; the most routes in flight,
-// as for the other forms, is 18% from it and loses by 1.7 at n=500 m=20 (32768
-// candidates: two routes in 196 KB 249 us, one in 134 KB 152 us).
+// as for the other forms, is 18% from it (n=500 m=20, 32768 candidates: two
+// routes in 196 KB of shared memory 249 us, the shape of the least cost 182).
 static double gather_cost(const EvalArgs& a, long long resident, long long shared, double matrix, int sms) {
     int kb = 228;
     for (int step : {196, 164, 132, 100, 64, 32, 16, 8})
